@@ -166,8 +166,7 @@ typedef struct gs_bvh gs_bvh;
  *   GS_NODES_BINARY    64-byte binary nodes, FP32 child boxes; the handle
  *                      also holds 8-, 16- and 32-wide copies (one 32-byte
  *                      FP32 record per child, M + (M - 1) records at most
- *                      each, from 3, 4 and 5 binary levels) for the grouped
- *                      traversal, unless M > 2^25
+ *                      each) for the grouped traversal, unless M > 2^25
  *   GS_NODES_WIDE4     128-byte 4-wide nodes, FP32 child boxes
  *   GS_NODES_WIDE4_Q8  64-byte 4-wide nodes, child boxes quantised to 8 bits
  *                      per plane with outward rounding (a decoded box always

@@ -82,13 +82,12 @@ static void release(gs_bvh *b) {
     if (!b) return;
     void *bufs[] = {b->nodes, b->prims, b->status, b->codes[0], b->codes[1], b->vals[0],
                     b->vals[1], b->parent, b->arrive, b->aabb, b->bounds, b->hist,
-                    b->scan_tmp, b->wide, b->depth, b->wmap, b->node_depth};
+                    b->scan_tmp, b->wide, b->depth, b->wmap, b->link};
     for (void *p : bufs)
         if (p) cudaFree(p);
     for (auto &t : b->group) {
         if (t.rec) cudaFree(t.rec);
-        if (t.cnt) cudaFree(t.cnt);
-        if (t.off) cudaFree(t.off);
+        if (t.ref) cudaFree(t.ref);
     }
     void *wave[] = {b->wave_codes[0], b->wave_codes[1], b->wave_bounce, b->wave_hist, b->wave_scan};
     for (void *p : wave)
@@ -163,7 +162,7 @@ gs_status gs_build_bvh_ex(const gs_gaussians *g, const gs_build_options *opt, gs
         {(void **)&b->vals[0], (size_t)(cap > 0 ? cap : 1) * 4},
         {(void **)&b->vals[1], (size_t)(cap > 0 ? cap : 1) * 4},
         {(void **)&b->parent, (size_t)(2 * cap + 2) * 4},
-        {(void **)&b->arrive, (size_t)(cap > 0 ? cap : 1) * 4},
+        {(void **)&b->arrive, (size_t)((cap > 0 ? cap : 1) + kGroupTrees) * 4},
         {(void **)&b->aabb, (size_t)(cap > 0 ? cap : 1) * 24},
         {(void **)&b->bounds, 64},
         {(void **)&b->hist, (size_t)256 * tiles * 4},
@@ -171,16 +170,13 @@ gs_status gs_build_bvh_ex(const gs_gaussians *g, const gs_build_options *opt, gs
         {(void **)&b->wide, wide ? (size_t)nn * wide_bytes : 0},
         {(void **)&b->depth, wide ? (size_t)nn * 4 : 0},
         {(void **)&b->wmap, wide ? (size_t)nn * 4 : 0},
-        {(void **)&b->node_depth, grouped ? (size_t)nn * 4 : 0},
+        {(void **)&b->link, grouped ? (size_t)nn * sizeof(uint4) : 0},
         {(void **)&b->group[0].rec, grouped ? (size_t)recs * rec_bytes : 0},
-        {(void **)&b->group[0].cnt, grouped ? (size_t)nn * 4 : 0},
-        {(void **)&b->group[0].off, grouped ? (size_t)nn * 4 : 0},
+        {(void **)&b->group[0].ref, grouped ? (size_t)nn * 4 : 0},
         {(void **)&b->group[1].rec, grouped ? (size_t)recs * rec_bytes : 0},
-        {(void **)&b->group[1].cnt, grouped ? (size_t)nn * 4 : 0},
-        {(void **)&b->group[1].off, grouped ? (size_t)nn * 4 : 0},
+        {(void **)&b->group[1].ref, grouped ? (size_t)nn * 4 : 0},
         {(void **)&b->group[2].rec, grouped ? (size_t)recs * rec_bytes : 0},
-        {(void **)&b->group[2].cnt, grouped ? (size_t)nn * 4 : 0},
-        {(void **)&b->group[2].off, grouped ? (size_t)nn * 4 : 0},
+        {(void **)&b->group[2].ref, grouped ? (size_t)nn * 4 : 0},
     };
     int64_t total = 0;
     for (auto &r : reqs) {

@@ -310,7 +310,7 @@ __device__ void enumerate_group(const TraceArgs &a, const Ray<N> &r, const float
     for (int o = 1; o < L; o <<= 1) G = fmaxf(G, __shfl_xor_sync(gmask, G, o));
     if (!(G >= a.t_min)) return;
     int sp = 0;
-    uint32_t node = (__ldg(a.gcnt) - 1u) << kWideCountShift;
+    uint32_t node = __ldg(a.groot);
     uint32_t steps = 0;
     for (;;) {
         if (++steps > a.step_limit) {
@@ -655,9 +655,9 @@ gs_status launch_backward(const gs_bvh *b, const gs_gaussians *g, const gs_pinho
     a.status = b->status;
     a.work = b->status + 1;
     a.lpp_log2 = lanes_per_pixel_log2(spp_eff);
-    if (b->node_depth && a.lpp_log2 >= 3) {
+    if (b->link && a.lpp_log2 >= 3) {
         a.grec = b->group[a.lpp_log2 - 3].rec;
-        a.gcnt = b->group[a.lpp_log2 - 3].cnt;
+        a.groot = b->group[a.lpp_log2 - 3].ref;
         a.gq8 = b->node_format == GS_NODES_BINARY_Q8;
     }
     a.keys = const_cast<gs_sample_key *>(keys);  // read only here

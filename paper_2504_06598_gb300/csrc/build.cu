@@ -9,7 +9,9 @@
 //   k_karras      binary radix tree over the sorted codes (Karras 2012),
 //                 equal codes split by position
 //   k_leaves      per-Gaussian record in tree order, then bottom-up box
-//                 refit with one arrival counter per node
+//                 refit with one arrival counter per node; cuts the wide
+//                 hierarchies on the way
+//   k_wide_*      records of the 8-, 16- and 32-wide hierarchies
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -392,15 +394,61 @@ __device__ __forceinline__ void write_record(PrimRec *__restrict__ prims, int64_
     for (int k = 0; k < 4; ++k) dst[k] = src[k];
 }
 
+// The W-wide hierarchies (W = 8, 16, 32) are cut out of the binary tree
+// bottom-up, in the box refit: k_W(p) is the number of children that the
+// wide node holding binary node p has below p, k_W(leaf) = 1. At a node
+// whose children together exceed W, the one with more is closed: it becomes
+// a wide node of its own and counts as one (both, if that still exceeds W).
+// So every wide node but the root holds more than W / 2 children, and the
+// records are at most M + M / (W / 2). Against cutting at fixed binary
+// levels (mean 32-wide fill 6.6 children) the grouped walks take a third of
+// the steps: 1M shell at 1080p, rebuild + trace, spp 64 47.6 -> 28.0 ms,
+// N=4 spp 16 46.7 -> 33.8, 3M with 8-bit records 100.6 -> 48.7; and the cut
+// costs the refit little where listing, counting and scanning each width
+// took kernels of their own (frame at spp 1 6.65 -> 6.14 ms). Four words per internal node p, one
+// byte (bits 0-7, 8-15, 16-23) per W:
+//   x  parent
+//   y  children of its wide node left of p's within the parent (0 when p is
+//      the left child); bit 24 + w: p is closed in tree w
+//   z  k_W(p)
+//   w  children below p's left child; bit 24 + w: that child is closed,
+//      bit 27 + w: the right one is
+constexpr uint32_t kLeafCounts = 0x010101u;  // one child in each of the three
+constexpr uint32_t kRootClosed = 7u << 24;
+
+__device__ __forceinline__ uint32_t close_children(uint32_t &kl, uint32_t &kr) {
+    uint32_t closed = 0, nl = 0, nr = 0;
+#pragma unroll
+    for (int w = 0; w < kGroupTrees; ++w) {
+        const uint32_t W = 8u << w;
+        uint32_t a = (kl >> (8 * w)) & 255u, b = (kr >> (8 * w)) & 255u;
+        if (a + b > W) {
+            const bool left = a >= b;
+            if (left) a = 1; else b = 1;
+            closed |= (left ? 1u : 8u) << w;
+            if (a + b > W) {
+                if (left) b = 1; else a = 1;
+                closed |= (left ? 8u : 1u) << w;
+            }
+        }
+        nl |= a << (8 * w);
+        nr |= b << (8 * w);
+    }
+    kl = nl;
+    kr = nr;
+    return closed;  // bits 0-2: the left child, 3-5: the right one
+}
+
 // One thread per leaf (tree position i): write the Gaussian record, then
 // carry boxes towards the root; the second thread to reach a node merges
-// both child boxes and continues.
+// both child boxes, cuts the wide trees there (link != null) and continues.
 __global__ void k_leaves(int64_t n, const uint32_t *__restrict__ order,
                          const float *__restrict__ means, const float *__restrict__ log_scales,
                          const float *__restrict__ quats, const float *__restrict__ logits,
                          const float *__restrict__ aabb, PrimRec *__restrict__ prims,
                          Node *__restrict__ nodes, const uint32_t *__restrict__ parent_int,
-                         const uint32_t *__restrict__ parent_leaf, uint32_t *__restrict__ arrive) {
+                         const uint32_t *__restrict__ parent_leaf, uint32_t *__restrict__ arrive,
+                         uint4 *__restrict__ link) {
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     uint32_t g = order[i];
@@ -410,18 +458,49 @@ __global__ void k_leaves(int64_t n, const uint32_t *__restrict__ order,
     for (int k = 0; k < 6; ++k) box[k] = aabb[6 * (int64_t)g + k];
     uint32_t ref = kLeafBit | (uint32_t)i;
     uint32_t p = parent_leaf[i];
+    uint32_t counts = kLeafCounts;
     for (int guard = 0; guard < 4096; ++guard) {
         Node *nd = nodes + p;
-        int side = (__ldcg(&nd->child[0]) == ref) ? 0 : 1;
-        for (int k = 0; k < 6; ++k) __stcg(&nd->box[side][k], box[k]);
+        const uint2 child = __ldcg(reinterpret_cast<const uint2 *>(nd->child));
+        const int side = child.x == ref ? 0 : 1;
+        // a child's box is 24 bytes at an 8-byte boundary
+        float2 *mine = reinterpret_cast<float2 *>(nd->box[side]);
+        for (int k = 0; k < 3; ++k) __stcg(mine + k, make_float2(box[2 * k], box[2 * k + 1]));
+        if (link && !(ref & kLeafBit)) __stcg(&link[ref].z, counts);
         __threadfence();
         if (atomicAdd(&arrive[p], 1u) == 0u) return;
         __threadfence();
+        const float2 *other = reinterpret_cast<const float2 *>(nd->box[1 - side]);
+        float ob[6];
         for (int k = 0; k < 3; ++k) {
-            box[k] = fminf(box[k], __ldcg(&nd->box[1 - side][k]));
-            box[3 + k] = fmaxf(box[3 + k], __ldcg(&nd->box[1 - side][3 + k]));
+            const float2 v = __ldcg(other + k);
+            ob[2 * k] = v.x;
+            ob[2 * k + 1] = v.y;
         }
-        if (p == 0) return;
+        if (link) {
+            const uint32_t sib = side ? child.x : child.y;
+            const uint32_t oc = (sib & kLeafBit) ? kLeafCounts : __ldcg(&link[sib].z);
+            uint32_t kl = side ? oc : counts, kr = side ? counts : oc;
+            const uint32_t closed = close_children(kl, kr);
+            if (!(child.x & kLeafBit))
+                __stcg(reinterpret_cast<uint2 *>(link + child.x), make_uint2(p, (closed & 7u) << 24));
+            if (!(child.y & kLeafBit))
+                __stcg(reinterpret_cast<uint2 *>(link + child.y),
+                       make_uint2(p, kl | (closed >> 3) << 24));
+            __stcg(&link[p].w, kl | closed << 24);
+            counts = kl + kr;
+        }
+        for (int k = 0; k < 3; ++k) {
+            box[k] = fminf(box[k], ob[k]);
+            box[3 + k] = fmaxf(box[3 + k], ob[3 + k]);
+        }
+        if (p == 0) {
+            if (link) {
+                __stcg(reinterpret_cast<uint2 *>(link), make_uint2(0u, kRootClosed));
+                __stcg(&link[0].z, counts);
+            }
+            return;
+        }
         ref = p;
         p = parent_int[p];
     }
@@ -432,7 +511,8 @@ __global__ void k_leaves(int64_t n, const uint32_t *__restrict__ order,
 __global__ void k_single(const uint32_t *__restrict__ order, const float *__restrict__ means,
                          const float *__restrict__ log_scales, const float *__restrict__ quats,
                          const float *__restrict__ logits, const float *__restrict__ aabb,
-                         PrimRec *__restrict__ prims, Node *__restrict__ nodes) {
+                         PrimRec *__restrict__ prims, Node *__restrict__ nodes,
+                         uint4 *__restrict__ link) {
     uint32_t g = order[0];
     Activated a = activate(means, log_scales, quats, logits, g);
     write_record(prims, 0, g, a);
@@ -443,6 +523,8 @@ __global__ void k_single(const uint32_t *__restrict__ order, const float *__rest
     }
     nd.leaf_range[0] = nd.leaf_range[1] = 0;
     nodes[0] = nd;
+    // a wide root of one child (k_wide_records writes the left one only)
+    if (link) link[0] = make_uint4(0u, kRootClosed, kLeafCounts, kLeafCounts);
 }
 
 // Depth of every internal binary node (walk to the root).
@@ -549,130 +631,68 @@ __global__ void k_collapse(int64_t n_int, const Node *__restrict__ nodes,
     }
 }
 
-// The W-wide hierarchies (W = 2^LEVELS). The wide nodes sit at binary
-// internal nodes of depth 0 mod LEVELS; a wide node covering at most W
-// leaves has those leaves as its children (and no wide node below it),
-// any other has its descendants LEVELS levels down, or the leaves met
-// before. So a binary node is a wide root when it is the root, or when its
-// depth is 0 mod LEVELS and its ancestor LEVELS levels up covers more than
-// W leaves. expand_wide lists the LEVELS-level children, left to right,
-// with their boxes.
-template <int LEVELS>
-__device__ __forceinline__ int expand_wide(const Node *__restrict__ nodes, uint32_t i,
-                                           uint32_t ref[1 << LEVELS], float box[1 << LEVELS][6]) {
-    int n = 0;
-    const Node nd = nodes[i];
-    for (int sd = 0; sd < 2; ++sd) {
-        ref[n] = nd.child[sd];
-        for (int q = 0; q < 6; ++q) box[n][q] = nd.box[sd][q];
-        ++n;
-    }
-    for (int level = 1; level < LEVELS; ++level) {
-        // expand in place from the back so entries keep left-to-right order
-        int m = n;
-        for (int j = 0; j < n; ++j)
-            if (!(ref[j] & kLeafBit)) ++m;
-        for (int j = n - 1, dst = m - 1; j >= 0; --j) {
-            if (ref[j] & kLeafBit) {
-                ref[dst] = ref[j];
-                for (int q = 0; q < 6; ++q) box[dst][q] = box[j][q];
-                --dst;
-            } else {
-                const Node cn = nodes[ref[j]];
-                for (int sd = 1; sd >= 0; --sd) {
-                    ref[dst] = cn.child[sd];
-                    for (int q = 0; q < 6; ++q) box[dst][q] = cn.box[sd][q];
-                    --dst;
-                }
-            }
+// Reference of the wide node at every closed binary node: a block adds up its
+// nodes' record counts (plus `header` units each), takes its range of the
+// three trees' records with one atomic per tree, and hands it out in node
+// order. The order of the blocks' ranges varies from run to run; a reference
+// is never compared, so no result depends on it.
+struct WideRefs {
+    uint32_t *ref[kGroupTrees];
+};
+
+__global__ void __launch_bounds__(256)
+    k_wide_offsets(int64_t n_int, const uint4 *__restrict__ link, uint32_t *__restrict__ alloc,
+                   uint32_t header, const WideRefs out) {
+    constexpr int P = 4;  // consecutive nodes per thread
+    __shared__ uint32_t base[kGroupTrees];
+    __shared__ unsigned long long warp_sum[8];
+    const int64_t i0 = ((int64_t)blockIdx.x * 256 + threadIdx.x) * P;
+    uint32_t flags[P], cnt[P];
+    // 21 bits per tree: at most 1024 nodes x 34 units
+    unsigned long long local = 0;
+#pragma unroll
+    for (int j = 0; j < P; ++j) {
+        flags[j] = 0;
+        cnt[j] = 0;
+        if (i0 + j < n_int) {
+            const uint4 l = link[i0 + j];
+            flags[j] = l.y >> 24;
+            cnt[j] = l.z;
         }
-        n = m;
+#pragma unroll
+        for (int w = 0; w < kGroupTrees; ++w)
+            if ((flags[j] >> w) & 1u)
+                local += (unsigned long long)(((cnt[j] >> (8 * w)) & 255u) + header) << (21 * w);
     }
-    return n;
-}
-
-// Depth of every binary internal node (walk to the root).
-__global__ void k_node_depth(int64_t n_int, const uint32_t *__restrict__ parent_int,
-                             uint32_t *__restrict__ depth) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_int) return;
-    uint32_t d = 0, p = (uint32_t)i;
-    while (p != 0 && d < 4096) {
-        p = parent_int[p];
-        ++d;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    unsigned long long incl = local;
+    for (int off = 1; off < 32; off <<= 1) {
+        const unsigned long long u = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += u;
     }
-    depth[i] = d;
-}
-
-__device__ __forceinline__ uint32_t leaves_under(const Node &nd) {
-    return nd.leaf_range[1] - nd.leaf_range[0] + 1u;
-}
-
-// Children of the wide node at each binary internal node (0 where none);
-// the same count, plus `header` units where a node exists, seeds the
-// offsets.
-template <int LEVELS>
-__global__ void k_count_wide(int64_t n_int, const Node *__restrict__ nodes,
-                             const uint32_t *__restrict__ depth,
-                             const uint32_t *__restrict__ parent_int, uint32_t *__restrict__ cnt,
-                             uint32_t *__restrict__ off, uint32_t header) {
-    constexpr uint32_t W = 1u << LEVELS;
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_int) return;
-    uint32_t c = 0;
-    bool root = i == 0;
-    if (!root && depth[i] % (uint32_t)LEVELS == 0u) {
-        uint32_t p = (uint32_t)i;
-        for (int k = 0; k < LEVELS; ++k) p = parent_int[p];
-        root = leaves_under(nodes[p]) > W;
+    if (lane == 31) warp_sum[warp] = incl;
+    __syncthreads();
+    unsigned long long before = 0, total = 0;
+    for (int k = 0; k < 8; ++k) {
+        if (k < warp) before += warp_sum[k];
+        total += warp_sum[k];
     }
-    if (root) {
-        const uint32_t n_leaves = leaves_under(nodes[i]);
-        if (n_leaves <= W) {
-            c = n_leaves;
-        } else {
-            uint32_t ref[1 << LEVELS];
-            float box[1 << LEVELS][6];
-            c = (uint32_t)expand_wide<LEVELS>(nodes, (uint32_t)i, ref, box);
+    if (threadIdx.x < kGroupTrees) {
+        const uint32_t t = (uint32_t)(total >> (21 * threadIdx.x)) & 0x1fffffu;
+        base[threadIdx.x] = t ? atomicAdd(&alloc[threadIdx.x], t) : 0u;
+    }
+    __syncthreads();
+    const unsigned long long excl = before + incl - local;
+#pragma unroll
+    for (int w = 0; w < kGroupTrees; ++w) {
+        uint32_t run = base[w] + ((uint32_t)(excl >> (21 * w)) & 0x1fffffu);
+#pragma unroll
+        for (int j = 0; j < P; ++j) {
+            if (!((flags[j] >> w) & 1u)) continue;
+            const uint32_t c = (cnt[j] >> (8 * w)) & 255u;
+            out.ref[w][i0 + j] = (c - 1u) << kWideCountShift | run;
+            run += c + header;
         }
-    }
-    cnt[i] = c;
-    off[i] = c ? c + header : 0u;
-}
-
-// Writes the child records of every wide node at its offset.
-template <int LEVELS>
-__global__ void k_collapse_wide(int64_t n_int, const Node *__restrict__ nodes,
-                                const uint32_t *__restrict__ cnt, const uint32_t *__restrict__ off,
-                                const uint32_t *__restrict__ order, const float *__restrict__ aabb,
-                                ChildRec *__restrict__ rec) {
-    constexpr uint32_t W = 1u << LEVELS;
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_int || cnt[i] == 0u) return;
-    ChildRec *dst = rec + off[i];
-    const Node ndi = nodes[i];
-    if (leaves_under(ndi) <= W) {
-        // every leaf of the node, with the box its parent node holds for it
-        for (uint32_t k = ndi.leaf_range[0]; k <= ndi.leaf_range[1]; ++k) {
-            ChildRec c;
-            const float *b = aabb + 6 * (int64_t)order[k];
-            for (int q = 0; q < 3; ++q) { c.lo[q] = b[q]; c.hi[q] = b[3 + q]; }
-            c.child = kLeafBit | k;
-            c.reserved = 0;
-            *dst++ = c;
-        }
-        return;
-    }
-    uint32_t ref[1 << LEVELS];
-    float box[1 << LEVELS][6];
-    const int n = expand_wide<LEVELS>(nodes, (uint32_t)i, ref, box);
-    for (int j = 0; j < n; ++j) {
-        ChildRec c;
-        for (int q = 0; q < 3; ++q) { c.lo[q] = box[j][q]; c.hi[q] = box[j][3 + q]; }
-        const uint32_t r = ref[j];
-        c.child = (r & kLeafBit) ? r : (((cnt[r] - 1u) << kWideCountShift) | off[r]);
-        c.reserved = 0;
-        dst[j] = c;
     }
 }
 
@@ -717,53 +737,84 @@ __device__ __forceinline__ void quant_frame(const float lo[3], const float hi[3]
     }
 }
 
-// Writes every wide node of the 8-bit form at its offset: the header from
-// the children's union box, then one unit per child.
-template <int LEVELS>
-__global__ void k_collapse_wide_q8(int64_t n_int, const Node *__restrict__ nodes,
-                                   const uint32_t *__restrict__ cnt,
-                                   const uint32_t *__restrict__ off,
-                                   const uint32_t *__restrict__ order,
-                                   const float *__restrict__ aabb, uint4 *__restrict__ units) {
-    constexpr uint32_t W = 1u << LEVELS;
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n_int || cnt[i] == 0u) return;
-    uint4 *dst = units + off[i];
-    const Node ndi = nodes[i];
-    float ulo[3] = {INFINITY, INFINITY, INFINITY}, uhi[3] = {-INFINITY, -INFINITY, -INFINITY};
-    float origin[3], scale[3];
-    if (leaves_under(ndi) <= W) {
-        for (uint32_t k = ndi.leaf_range[0]; k <= ndi.leaf_range[1]; ++k) {
-            const float *b = aabb + 6 * (int64_t)order[k];
-            for (int q = 0; q < 3; ++q) { ulo[q] = fminf(ulo[q], b[q]); uhi[q] = fmaxf(uhi[q], b[3 + q]); }
+struct WideOut {
+    const uint32_t *ref[kGroupTrees];
+    void *rec[kGroupTrees];
+};
+
+// Writes the child records of the three wide trees, one thread per binary
+// internal node, each record by itself: the thread whose child is a leaf or
+// closed climbs to the wide node it belongs to (a few levels, one link each)
+// and adds up the children to its left on the way. All reads of its own node
+// are coalesced and nothing is kept in arrays. In the 8-bit form the planes
+// are taken against the wide node's own box, and the first child's thread
+// also writes the header.
+template <bool Q8>
+__global__ void __launch_bounds__(256)
+    k_wide_records(int64_t n_int, const Node *__restrict__ nodes, const uint4 *__restrict__ link,
+                   const WideOut out) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n_int) return;
+    const float4 *np = reinterpret_cast<const float4 *>(nodes + i);
+    const float4 b0 = __ldg(np), b1 = __ldg(np + 1), b2 = __ldg(np + 2);
+    const uint4 cref = __ldg(reinterpret_cast<const uint4 *>(np + 3));
+    const float box[2][6] = {{b0.x, b0.y, b0.z, b0.w, b1.x, b1.y},
+                             {b1.z, b1.w, b2.x, b2.y, b2.z, b2.w}};
+    uint4 l = __ldg(link + i);
+    const uint32_t left = l.w;
+    uint32_t need[2];  // trees in which the child is a record of its own
+    need[0] = (cref.x & kLeafBit) ? 7u : (left >> 24) & 7u;
+    need[1] = (cref.y & kLeafBit) ? 7u : (left >> 27) & 7u;
+    if (cref.x == cref.y) need[1] = 0u;  // a single Gaussian
+    uint32_t todo = need[0] | need[1];
+    uint32_t cur = (uint32_t)i, pos = 0;  // children left of node i, one byte per tree
+    for (int guard = 0; todo && guard < 4096; ++guard) {
+        const uint32_t here = (l.y >> 24) & todo;
+#pragma unroll
+        for (int w = 0; w < kGroupTrees; ++w) {
+            if (!((here >> w) & 1u)) continue;
+            const uint32_t first = __ldg(out.ref[w] + cur) & kWideOffsetMask;
+            float origin[3], scale[3];
+            if constexpr (Q8) {
+                const float *rb = &nodes[cur].box[0][0];
+                float lo[3], hi[3];
+                for (int q = 0; q < 3; ++q) {
+                    lo[q] = fminf(__ldg(rb + q), __ldg(rb + 6 + q));
+                    hi[q] = fmaxf(__ldg(rb + 3 + q), __ldg(rb + 9 + q));
+                }
+                quant_frame(lo, hi, origin, scale);
+            }
+#pragma unroll
+            for (int side = 0; side < 2; ++side) {
+                if (!((need[side] >> w) & 1u)) continue;
+                const uint32_t c = side ? cref.y : cref.x;
+                const uint32_t r = (c & kLeafBit) ? c : __ldg(out.ref[w] + c);
+                const uint32_t j = ((pos >> (8 * w)) & 255u) +
+                                   (side ? (left >> (8 * w)) & 255u : 0u);
+                const float *b = box[side];
+                if constexpr (Q8) {
+                    uint4 *dst = static_cast<uint4 *>(out.rec[w]) + first;
+                    uint32_t q0, q1;
+                    quant_child(b, origin, scale, q0, q1);
+                    dst[kGroupQHeaderUnits + j] = make_uint4(q0, q1, r, 0u);
+                    if (j == 0) {
+                        dst[0] = make_uint4(__float_as_uint(origin[0]), __float_as_uint(origin[1]),
+                                            __float_as_uint(origin[2]), __float_as_uint(scale[0]));
+                        dst[1] = make_uint4(__float_as_uint(scale[1]), __float_as_uint(scale[2]), 0u, 0u);
+                    }
+                } else {
+                    float4 *dst = reinterpret_cast<float4 *>(static_cast<ChildRec *>(out.rec[w]) + first + j);
+                    dst[0] = make_float4(b[0], b[1], b[2], b[3]);
+                    dst[1] = make_float4(b[4], b[5], __uint_as_float(r), 0.0f);
+                }
+            }
         }
-        quant_frame(ulo, uhi, origin, scale);
-        uint32_t j = kGroupQHeaderUnits;
-        for (uint32_t k = ndi.leaf_range[0]; k <= ndi.leaf_range[1]; ++k, ++j) {
-            const float *b = aabb + 6 * (int64_t)order[k];
-            const float bx[6] = {b[0], b[1], b[2], b[3], b[4], b[5]};
-            uint32_t q0, q1;
-            quant_child(bx, origin, scale, q0, q1);
-            dst[j] = make_uint4(q0, q1, kLeafBit | k, 0u);
-        }
-    } else {
-        uint32_t ref[1 << LEVELS];
-        float box[1 << LEVELS][6];
-        const int n = expand_wide<LEVELS>(nodes, (uint32_t)i, ref, box);
-        for (int j = 0; j < n; ++j)
-            for (int q = 0; q < 3; ++q) { ulo[q] = fminf(ulo[q], box[j][q]); uhi[q] = fmaxf(uhi[q], box[j][3 + q]); }
-        quant_frame(ulo, uhi, origin, scale);
-        for (int j = 0; j < n; ++j) {
-            uint32_t q0, q1;
-            quant_child(box[j], origin, scale, q0, q1);
-            const uint32_t r = ref[j];
-            const uint32_t c = (r & kLeafBit) ? r : (((cnt[r] - 1u) << kWideCountShift) | off[r]);
-            dst[kGroupQHeaderUnits + j] = make_uint4(q0, q1, c, 0u);
-        }
+        todo &= ~here;
+        if (!todo) break;
+        pos += l.y & 0xffffffu;  // at most W children per tree: no carry
+        cur = l.x;
+        l = __ldg(link + cur);
     }
-    dst[0] = make_uint4(__float_as_uint(origin[0]), __float_as_uint(origin[1]),
-                        __float_as_uint(origin[2]), __float_as_uint(scale[0]));
-    dst[1] = make_uint4(__float_as_uint(scale[1]), __float_as_uint(scale[2]), 0u, 0u);
 }
 
 inline unsigned grid_for(int64_t n, int threads) {
@@ -817,18 +868,20 @@ gs_status build_into(gs_bvh *b, const gs_gaussians *g, cudaStream_t s) {
     }
     b->final_buf = cur;
     const uint32_t *order = b->vals[cur];
+    // arrival counters, then the wide trees' record allocators
+    const size_t n_arrive = (size_t)M + (b->link ? kGroupTrees : 0);
+    if ((e = cudaMemsetAsync(b->arrive, 0, n_arrive * sizeof(uint32_t), s)) != cudaSuccess)
+        return cuda_fail(e, "memset arrive");
     if (M == 1) {
         k_single<<<1, 1, 0, s>>>(order, g->means, g->log_scales, g->quats, g->opacity_logits,
-                                 b->aabb, b->prims, b->nodes);
+                                 b->aabb, b->prims, b->nodes, b->link);
     } else {
         uint32_t *parent_int = b->parent, *parent_leaf = b->parent + M;
         k_karras<<<grid_for(M - 1, 256), 256, 0, s>>>(M, b->codes[cur], b->nodes, parent_int,
                                                        parent_leaf);
-        if ((e = cudaMemsetAsync(b->arrive, 0, (size_t)M * sizeof(uint32_t), s)) != cudaSuccess)
-            return cuda_fail(e, "memset arrive");
         k_leaves<<<grid_for(M, 256), 256, 0, s>>>(M, order, g->means, g->log_scales, g->quats,
                                                    g->opacity_logits, b->aabb, b->prims, b->nodes,
-                                                   parent_int, parent_leaf, b->arrive);
+                                                   parent_int, parent_leaf, b->arrive, b->link);
     }
     if (b->node_format == GS_NODES_WIDE4 || b->node_format == GS_NODES_WIDE4_Q8) {
         const int64_t n_int = b->n_nodes;
@@ -846,39 +899,20 @@ gs_status build_into(gs_bvh *b, const gs_gaussians *g, cudaStream_t s) {
             k_collapse<GS_NODES_WIDE4_Q8><<<grid_for(n_int, 256), 256, 0, s>>>(
                 n_int, b->nodes, b->depth, b->wmap, b->wide);
     }
-    if (b->node_depth) {
+    if (b->link) {
         const int64_t n_int = b->n_nodes;
         const bool q8 = b->node_format == GS_NODES_BINARY_Q8;
-        const uint32_t hdr = q8 ? (uint32_t)kGroupQHeaderUnits : 0u;
-        k_node_depth<<<grid_for(n_int, 256), 256, 0, s>>>(n_int, b->parent, b->node_depth);
-        const GroupTree *t = b->group;
-        k_count_wide<3><<<grid_for(n_int, 256), 256, 0, s>>>(n_int, b->nodes, b->node_depth, b->parent,
-                                                            t[0].cnt, t[0].off, hdr);
-        scan_exclusive(t[0].off, n_int, b->scan_tmp, s);
-        if (q8)
-            k_collapse_wide_q8<3><<<grid_for(n_int, 256), 256, 0, s>>>(
-                n_int, b->nodes, t[0].cnt, t[0].off, order, b->aabb, static_cast<uint4 *>(t[0].rec));
-        else
-            k_collapse_wide<3><<<grid_for(n_int, 256), 256, 0, s>>>(
-                n_int, b->nodes, t[0].cnt, t[0].off, order, b->aabb, static_cast<ChildRec *>(t[0].rec));
-        k_count_wide<4><<<grid_for(n_int, 128), 128, 0, s>>>(n_int, b->nodes, b->node_depth, b->parent,
-                                                            t[1].cnt, t[1].off, hdr);
-        scan_exclusive(t[1].off, n_int, b->scan_tmp, s);
-        if (q8)
-            k_collapse_wide_q8<4><<<grid_for(n_int, 128), 128, 0, s>>>(
-                n_int, b->nodes, t[1].cnt, t[1].off, order, b->aabb, static_cast<uint4 *>(t[1].rec));
-        else
-            k_collapse_wide<4><<<grid_for(n_int, 128), 128, 0, s>>>(
-                n_int, b->nodes, t[1].cnt, t[1].off, order, b->aabb, static_cast<ChildRec *>(t[1].rec));
-        k_count_wide<5><<<grid_for(n_int, 128), 128, 0, s>>>(n_int, b->nodes, b->node_depth, b->parent,
-                                                            t[2].cnt, t[2].off, hdr);
-        scan_exclusive(t[2].off, n_int, b->scan_tmp, s);
-        if (q8)
-            k_collapse_wide_q8<5><<<grid_for(n_int, 128), 128, 0, s>>>(
-                n_int, b->nodes, t[2].cnt, t[2].off, order, b->aabb, static_cast<uint4 *>(t[2].rec));
-        else
-            k_collapse_wide<5><<<grid_for(n_int, 128), 128, 0, s>>>(
-                n_int, b->nodes, t[2].cnt, t[2].off, order, b->aabb, static_cast<ChildRec *>(t[2].rec));
+        WideRefs refs;
+        WideOut out;
+        for (int w = 0; w < kGroupTrees; ++w) {
+            refs.ref[w] = b->group[w].ref;
+            out.ref[w] = b->group[w].ref;
+            out.rec[w] = b->group[w].rec;
+        }
+        k_wide_offsets<<<grid_for(n_int, 1024), 256, 0, s>>>(
+            n_int, b->link, b->arrive + M, q8 ? (uint32_t)kGroupQHeaderUnits : 0u, refs);
+        if (q8) k_wide_records<true><<<grid_for(n_int, 256), 256, 0, s>>>(n_int, b->nodes, b->link, out);
+        else k_wide_records<false><<<grid_for(n_int, 256), 256, 0, s>>>(n_int, b->nodes, b->link, out);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return cuda_fail(e, "build launch");
     return GS_OK;

@@ -80,15 +80,14 @@ constexpr int kGroupQHeaderUnits = 2;
 constexpr uint32_t kQ8Skip = 1u << 16;  // q1 flag: a child with a non-finite box
 constexpr int kWideCountShift = 26;
 constexpr uint32_t kWideOffsetMask = (1u << kWideCountShift) - 1u;
-constexpr int kGroupTrees = 3;  // W = 8 << i: collapses of 3, 4 and 5 binary levels
+constexpr int kGroupTrees = 3;  // W = 8 << i
 
 // One W-wide hierarchy: records (ChildRec, or 16-byte units of the 8-bit
-// form), and per binary internal node the child count of the wide node
-// there (0 where none) and its first record or unit.
+// form), and per binary internal node the reference of the wide node there
+// (set where one exists; the root's is at 0).
 struct GroupTree {
     void *rec;
-    uint32_t *cnt;
-    uint32_t *off;
+    uint32_t *ref;
 };
 
 // 4-wide node, 64 bytes, child boxes quantised to 8 bits per plane against
@@ -139,7 +138,7 @@ struct gs_bvh {
     unsigned long long *codes[2];
     uint32_t *vals[2];
     uint32_t *parent;   // [2M]: parents of internal nodes (0..M-2) then leaves
-    uint32_t *arrive;   // [M] refit arrival counters
+    uint32_t *arrive;   // [M + 3] refit arrival counters, then the wide record allocators
     float *aabb;        // [M][6] in Gaussian-id order
     unsigned int *bounds;  // [6] ordered-int scene bounds of the means
     uint32_t *hist;     // radix histograms [256 * tiles]
@@ -152,9 +151,9 @@ struct gs_bvh {
     uint32_t *depth;    // depth of every internal binary node
     uint32_t *wmap;     // binary internal node -> wide node index
     // W-wide hierarchies for groups of lanes sharing one ray (binary format
-    // only): W = 8, 16, 32, each at most M + (M - 1) records
+    // formats only): W = 8, 16, 32, each at most M + (M - 1) records
     gsrt::GroupTree group[gsrt::kGroupTrees];
-    uint32_t *node_depth;  // depth of every binary internal node
+    uint4 *link;  // per binary internal node: its place in the wide trees (build.cu)
     // scratch of the batched form's deferred bounce rays, grown on demand
     int64_t wave_cap;                    // sample slots (pixels x spp) held
     int64_t wave_bytes;                  // device bytes of the scratch below

@@ -275,7 +275,7 @@ void trace_layout(const gs_bvh *b, const gs_trace_params *p, int *S_out, int *sp
     *spp_eff_out = (p->spp + S - 1) / S;
     *lpp_log2_out = lanes_per_pixel_log2(*spp_eff_out);
     *grouped_out = (b->node_format == GS_NODES_BINARY || b->node_format == GS_NODES_BINARY_Q8) &&
-                   b->node_depth && *lpp_log2_out >= 3;
+                   b->link && *lpp_log2_out >= 3;
 }
 
 gs_status launch_trace(const gs_bvh *b, const gs_gaussians *g, const gs_pinhole *cam,
@@ -289,12 +289,12 @@ gs_status launch_trace(const gs_bvh *b, const gs_gaussians *g, const gs_pinhole 
     a.nodes = b->nodes;
     a.wide = b->wide;
     a.lpp_log2 = lpp_log2;
-    if (b->node_depth && a.lpp_log2 >= 3) {
+    if (b->link && a.lpp_log2 >= 3) {
         a.grec = b->group[a.lpp_log2 - 3].rec;
-        a.gcnt = b->group[a.lpp_log2 - 3].cnt;
+        a.groot = b->group[a.lpp_log2 - 3].ref;
     } else {
         a.grec = nullptr;
-        a.gcnt = nullptr;
+        a.groot = nullptr;
     }
     a.gq8 = b->node_format == GS_NODES_BINARY_Q8;
     a.prims = b->prims;

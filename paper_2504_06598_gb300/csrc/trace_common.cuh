@@ -21,7 +21,7 @@ struct TraceArgs {
     const void *wide;  // Node4 or NodeQ4 when the handle has wide nodes
     const void *grec;      // W-wide records (ChildRec, or the 8-bit units) for the
                            // launch's group size, or null
-    const uint32_t *gcnt;  // their per-node child counts (the root's at 0)
+    const uint32_t *groot; // reference of their root
     int gq8;               // 1 when grec holds the 8-bit form
     const PrimRec *prims;
     const void *sh;
@@ -919,7 +919,7 @@ __device__ __forceinline__ void traverse_group(const TraceArgs &a, Ray<N> &r, in
     for (int o = 1; o < L; o <<= 1) G = fmaxf(G, __shfl_xor_sync(gmask, G, o));
     if (!(G >= r.t_min)) return;  // no lane of the group is live
     int sp = 0;
-    uint32_t node = (__ldg(a.gcnt) - 1u) << kWideCountShift;  // the root's records start at 0
+    uint32_t node = __ldg(a.groot);
     uint32_t steps = 0;
     float node_t = r.t_min;
     for (;;) {

@@ -831,9 +831,9 @@ gs_status launch_render_views(const gs_bvh *b, const gs_gaussians *g, const gs_p
     a.status = b->status;
     a.work = b->status + 1;
     a.lpp_log2 = lanes_per_pixel_log2(a.spp);
-    if (b->node_depth && a.lpp_log2 >= 3) {
+    if (b->link && a.lpp_log2 >= 3) {
         a.grec = b->group[a.lpp_log2 - 3].rec;
-        a.gcnt = b->group[a.lpp_log2 - 3].cnt;
+        a.groot = b->group[a.lpp_log2 - 3].ref;
         a.gq8 = b->node_format == GS_NODES_BINARY_Q8;
     }
     const int tw_lg = tile_w_log2(a.lpp_log2), th_lg = 5 - a.lpp_log2 - tw_lg;

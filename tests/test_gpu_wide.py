@@ -1,0 +1,51 @@
+"""The wide hierarchies against the binary one: the grouped traversals (8, 16
+and 32 lanes on a pixel) must return the hits of the per-lane packets, which
+read the binary nodes, at the sizes where the cut of the wide nodes changes
+(one node, exactly full, one more, two levels) and on trees of equal codes."""
+import numpy as np
+import pytest
+
+import scenes
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+SIZES = (1, 2, 3, 8, 9, 16, 17, 32, 33, 65, 257, 1024, 1025, 7000)
+
+
+@pytest.fixture(scope="module")
+def gs():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2504_06598_gb300 as m
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA device required for gpu tests")
+    return m
+
+
+def _cloud(M, coincident):
+    cloud = scenes.tiny_cloud(M, M=M)
+    cloud.log_scales[:] += 1.0
+    if coincident:
+        cloud.means[M // 2:] = cloud.means[0]
+    return cloud
+
+
+@pytest.mark.parametrize("fmt", ["binary", "binary_q8"])
+@pytest.mark.parametrize("coincident", [False, True])
+def test_grouped_hits_equal_packet_hits(gs, fmt, coincident):
+    cam = scenes.Pinhole(width=21, height=13, eye=(0.4, 0.3, 2.8))
+    for M in SIZES:
+        g = gs.Gaussians.from_cloud(_cloud(M, coincident))
+        bvh = gs.build_bvh(g, node_format=fmt)
+        for lanes in (8, 16, 32):
+            kw = dict(seed=M, spp=lanes, want_hits=True)
+            assert gs.trace_layout(bvh, spp=lanes, samples_per_lane=1)["grouped"]
+            _, a, ta = gs.trace_stochastic(bvh, g, cam, samples_per_lane=1, **kw)
+            # eight samples per lane: fewer than eight lanes a pixel; an
+            # explicit stack depth keeps the per-lane walk of the binary nodes
+            _, b, tb = gs.trace_stochastic(bvh, g, cam, samples_per_lane=8, stack_depth=96, **kw)
+            bvh.sync_status()
+            assert torch.equal(a, b) and torch.equal(ta, tb), (M, lanes)
+        assert M < 100 or (a >= 0).any()
+        bvh.free()
