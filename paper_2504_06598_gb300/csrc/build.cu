@@ -804,8 +804,14 @@ __global__ void __launch_bounds__(256)
                     }
                 } else {
                     float4 *dst = reinterpret_cast<float4 *>(static_cast<ChildRec *>(out.rec[w]) + first + j);
-                    dst[0] = make_float4(b[0], b[1], b[2], b[3]);
-                    dst[1] = make_float4(b[4], b[5], __uint_as_float(r), 0.0f);
+                    // planes within +-1e30, so that sums and differences of
+                    // them are numbers (NaN boxes, never hit, stay NaN)
+                    float v[6];
+#pragma unroll
+                    for (int q = 0; q < 6; ++q)
+                        v[q] = b[q] < -1e30f ? -1e30f : (b[q] > 1e30f ? 1e30f : b[q]);
+                    dst[0] = make_float4(v[0], v[1], v[2], v[3]);
+                    dst[1] = make_float4(v[4], v[5], __uint_as_float(r), 0.0f);
                 }
             }
         }

@@ -47,6 +47,9 @@ namespace {
 // GS_NODES_*.
 constexpr int kFmtGroup = 8;
 constexpr int kFmtGroupQ8 = 16;
+// Tile traversal of the 32-wide records by a warp of camera rays.
+constexpr int kFmtTile = 6, kFmtTileQ8 = 7;
+__host__ __device__ constexpr bool is_tile_fmt(int f) { return f == kFmtTile || f == kFmtTileQ8; }
 __host__ __device__ constexpr bool is_group_fmt(int f) { return f >= kFmtGroup + 3; }
 __host__ __device__ constexpr bool is_group_q8(int f) { return f >= kFmtGroupQ8 + 3; }
 
@@ -64,7 +67,7 @@ constexpr int group_min_blocks(int n) { return n >= 8 ? 5 : (n >= 4 ? 7 : kGroup
 template <int N, bool COUNT, int FMT>
 __global__ void __launch_bounds__(kThreads, is_group_fmt(FMT) ? group_min_blocks(N)
                                                                : (N >= 8 ? 6 : 8))
-    k_trace(const TraceArgs a) {
+    k_trace(const __grid_constant__ TraceArgs a) {
     const int lane = threadIdx.x & 31;
     const uint32_t kAll = 0xffffffffu;
     const int lg = a.lpp_log2, L = 1 << lg;
@@ -79,14 +82,19 @@ __global__ void __launch_bounds__(kThreads, is_group_fmt(FMT) ? group_min_blocks
     uint32_t err = 0;
     Counts cnt;
     unsigned long long n_shaded = 0, n_rays = 0;
-    // group stacks: each warp's pool split evenly among its groups
-    constexpr bool grouped = is_group_fmt(FMT);
-    constexpr int LG = grouped ? (FMT & 7) : 3;
-    __shared__ uint32_t s_ref[grouped ? kThreads / 32 : 1][grouped ? kGroupPool : 1];
-    __shared__ float s_t[grouped ? kThreads / 32 : 1][grouped ? kGroupPool : 1];
+    // group stacks: each warp's pool split evenly among its groups (a tile's
+    // warp is one group)
+    constexpr bool grouped = is_group_fmt(FMT), tiled = is_tile_fmt(FMT);
+    constexpr int LG = grouped ? (FMT & 7) : 5;
+    constexpr bool pooled = grouped || tiled;
+    constexpr int pool = tiled ? kTilePool : grouped ? kGroupPool : 1;
+    __shared__ uint32_t s_ref[pooled ? kThreads / 32 : 1][pool];
+    __shared__ float s_t[pooled ? kThreads / 32 : 1][pool];
+    __shared__ __align__(16) float s_pyr[tiled ? kThreads / 32 : 1][tiled ? kTileFloats : 4];
     const int grp_off = grouped ? (lane >> LG) * (kGroupPool >> (5 - LG)) : 0;
-    uint32_t *grp_ref = s_ref[grouped ? threadIdx.x >> 5 : 0] + grp_off;
-    float *grp_t = s_t[grouped ? threadIdx.x >> 5 : 0] + grp_off;
+    uint32_t *grp_ref = s_ref[pooled ? threadIdx.x >> 5 : 0] + grp_off;
+    float *grp_t = s_t[pooled ? threadIdx.x >> 5 : 0] + grp_off;
+    float *pyr = s_pyr[tiled ? threadIdx.x >> 5 : 0];
     for (;;) {
         uint32_t tile = 0;
         if (lane == 0) tile = atomicAdd(a.work, 1u);
@@ -107,6 +115,7 @@ __global__ void __launch_bounds__(kThreads, is_group_fmt(FMT) ? group_min_blocks
         r.t_min = a.t_min;
         r.t_max = a.t_max;
         r.any_hit = false;
+        if constexpr (tiled) tile_pyramid(r.d, valid, pyr);
         float acc[3] = {0.0f, 0.0f, 0.0f};
         const int n_rounds = (a.spp + L - 1) >> lg;
         for (int j = 0; j < n_rounds; ++j) {
@@ -115,14 +124,29 @@ __global__ void __launch_bounds__(kThreads, is_group_fmt(FMT) ? group_min_blocks
             const int s0 = pass * N;
             // an unused slot (sample index beyond the pixel's count) sits
             // at -inf: no candidate is closer, and it never sets the clip
+            auto reset = [&](Ray<N> &q) {
 #pragma unroll
-            for (int k = 0; k < N; ++k)
-                r.slot[k] = s0 + k < a.n_samples ? Slot{INFINITY, 0.0f, 0xffffffffu}
-                                                 : Slot{-INFINITY, 0.0f, 0xffffffffu};
-            update_clip(r, a.t_max);
-            if (!live) r.t_far = -INFINITY;  // lanes off the image never hit
+                for (int k = 0; k < N; ++k)
+                    q.slot[k] = s0 + k < a.n_samples ? Slot{INFINITY, 0.0f, 0xffffffffu}
+                                                     : Slot{-INFINITY, 0.0f, 0xffffffffu};
+                update_clip(q, a.t_max);
+                if (!live) q.t_far = -INFINITY;  // lanes off the image never hit
+            };
+            reset(r);
             if (a.n_nodes > 0) {
-                if constexpr (grouped)
+                if constexpr (tiled) {
+                    if (!traverse_tile<N, FMT == kFmtTileQ8>(a, r, pass, a.eye, pyr, grp_ref, grp_t,
+                                                             err)) {
+                        Ray<N> again = r;
+                        set_ray(again, a.eye, r.d);
+                        reset(again);
+                        uint32_t err2 = 0;
+                        tile_fallback<N>(a, again, pass, err2);
+                        err |= err2;
+#pragma unroll
+                        for (int k = 0; k < N; ++k) r.slot[k] = again.slot[k];
+                    }
+                } else if constexpr (grouped)
                     traverse_group<N, COUNT, LG, true, is_group_q8(FMT)>(a, r, pass, grp_ref,
                                                                           grp_t, err, cnt);
                 else if constexpr (FMT == GS_NODES_BINARY)
@@ -198,7 +222,7 @@ gs_status launch_nf(const TraceArgs &a, bool count, cudaStream_t s) {
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
-        e = count ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_trace<N, true, FMT>, kThreads, 0)
+        e = count ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_trace<N, !is_tile_fmt(FMT), FMT>, kThreads, 0)
                   : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_trace<N, false, FMT>, kThreads, 0);
     if (e != cudaSuccess) return cuda_fail(e, "trace launch setup");
     // one resident grid; warps take tiles until none is left
@@ -211,13 +235,15 @@ gs_status launch_nf(const TraceArgs &a, bool count, cudaStream_t s) {
     if (blocks > max_blocks) blocks = max_blocks;
     if ((e = cudaMemsetAsync(a.work, 0, sizeof(uint32_t), s)) != cudaSuccess)
         return cuda_fail(e, "reset work counter");
-    if (count) k_trace<N, true, FMT><<<blocks, kThreads, 0, s>>>(a);
+    if (count) k_trace<N, !is_tile_fmt(FMT), FMT><<<blocks, kThreads, 0, s>>>(a);
     else k_trace<N, false, FMT><<<blocks, kThreads, 0, s>>>(a);
     return GS_OK;
 }
 
 template <int N>
 gs_status launch_n(const TraceArgs &a, int format, bool count, cudaStream_t s) {
+    if (a.trec != nullptr)
+        return a.gq8 ? launch_nf<N, kFmtTileQ8>(a, false, s) : launch_nf<N, kFmtTile>(a, false, s);
     // groups of 8 or more lanes on one pixel take the cooperative form
     if (format == GS_NODES_BINARY && a.grec != nullptr) {
         if (a.lpp_log2 == 5) return launch_nf<N, kFmtGroup + 5>(a, count, s);
@@ -297,6 +323,12 @@ gs_status launch_trace(const gs_bvh *b, const gs_gaussians *g, const gs_pinhole 
         a.groot = nullptr;
     }
     a.gq8 = b->node_format == GS_NODES_BINARY_Q8;
+    // the tile traversal: fewer than 8 lanes a pixel, depths along the ray
+    // from the eye, and none of the options that are about the per-lane walk
+    const bool tile = b->link && a.lpp_log2 < 3 && p->t_min >= 0.0f && p->depth_mode == 0 &&
+                      p->rng_mode == 0 && p->stack_depth == 0 && p->counters == nullptr;
+    a.trec = tile ? b->group[2].rec : nullptr;
+    a.troot = tile ? b->group[2].ref : nullptr;
     a.prims = b->prims;
     a.sh = g->sh;
     a.n_nodes = b->n_nodes;

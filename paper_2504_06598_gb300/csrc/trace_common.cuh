@@ -23,6 +23,8 @@ struct TraceArgs {
                            // launch's group size, or null
     const uint32_t *groot; // reference of their root
     int gq8;               // 1 when grec holds the 8-bit form
+    const void *trec;       // the 32-wide records and the reference of their root,
+    const uint32_t *troot;  // for the tile traversal
     const PrimRec *prims;
     const void *sh;
     int64_t n_nodes;
@@ -1056,6 +1058,237 @@ __device__ __forceinline__ void traverse_group(const TraceArgs &a, Ray<N> &r, in
         }
         if (!found) break;
     }
+}
+
+// ---------------------------------------------------------------- tiles
+// A warp's rays through one apex (camera rays through the eye; shadow rays
+// through their light) as a narrow pyramid: an orthonormal frame (r, u, f)
+// with f inside the rays, and the largest |x / z| and |y / z| of a ray in it.
+// Kept in shared memory, 20 floats per warp: r, |r|, u, |u|, f, |f|, tx, ty.
+constexpr int kTileFloats = 20;
+constexpr int kTilePool = 256;  // stack entries per warp
+
+// Fills the warp's pyramid from each lane's direction d (away from the apex,
+// any length; `in` marks the lanes that count). false when the rays spread
+// too far for it (or none counts): the caller then traverses otherwise.
+__device__ __forceinline__ bool tile_pyramid(const float d[3], bool in, float *pyr) {
+    const uint32_t kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const float n = rsqrtf(fmaf(d[0], d[0], fmaf(d[1], d[1], d[2] * d[2])));
+    float f[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        f[i] = in ? d[i] * n : 0.0f;
+#pragma unroll
+        for (int o = 16; o >= 1; o >>= 1) f[i] += __shfl_xor_sync(kAll, f[i], o);
+    }
+    const float nf = rsqrtf(fmaf(f[0], f[0], fmaf(f[1], f[1], f[2] * f[2])));
+#pragma unroll
+    for (int i = 0; i < 3; ++i) f[i] *= nf;
+    // r perpendicular to f through the axis f is smallest on
+    const float af[3] = {fabsf(f[0]), fabsf(f[1]), fabsf(f[2])};
+    const int ax = af[0] <= af[1] ? (af[0] <= af[2] ? 0 : 2) : (af[1] <= af[2] ? 1 : 2);
+    float r[3] = {ax == 0 ? 1.0f : 0.0f, ax == 1 ? 1.0f : 0.0f, ax == 2 ? 1.0f : 0.0f};
+    const float rf = ax == 0 ? f[0] : ax == 1 ? f[1] : f[2];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) r[i] = fmaf(-rf, f[i], r[i]);
+    const float nr = rsqrtf(fmaf(r[0], r[0], fmaf(r[1], r[1], r[2] * r[2])));
+#pragma unroll
+    for (int i = 0; i < 3; ++i) r[i] *= nr;
+    const float u[3] = {fmaf(r[1], f[2], -r[2] * f[1]), fmaf(r[2], f[0], -r[0] * f[2]),
+                        fmaf(r[0], f[1], -r[1] * f[0])};
+    const float z = fmaf(d[0], f[0], fmaf(d[1], f[1], d[2] * f[2])) * n;
+    const float x = fabsf(fmaf(d[0], r[0], fmaf(d[1], r[1], d[2] * r[2]))) * n;
+    const float y = fabsf(fmaf(d[0], u[0], fmaf(d[1], u[1], d[2] * u[2]))) * n;
+    // every counting ray well inside the half space of f (this also fails
+    // for a NaN frame)
+    const bool narrow = __all_sync(kAll, !in || z > 0.5f);
+    float tx = in ? x / z : 0.0f, ty = in ? y / z : 0.0f;
+#pragma unroll
+    for (int o = 16; o >= 1; o >>= 1) {
+        tx = fmaxf(tx, __shfl_xor_sync(kAll, tx, o));
+        ty = fmaxf(ty, __shfl_xor_sync(kAll, ty, o));
+    }
+    // 2^-17 of the distance outward: the roundings here and in the box test
+    // stay below 2^-20 of it
+    tx += 0x1p-17f;
+    ty += 0x1p-17f;
+    __syncwarp();
+    if (lane == 0) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            pyr[i] = narrow ? r[i] : 0.0f;
+            pyr[3 + i] = narrow ? fabsf(r[i]) : 0.0f;
+            pyr[6 + i] = narrow ? u[i] : 0.0f;
+            pyr[9 + i] = narrow ? fabsf(u[i]) : 0.0f;
+            pyr[12 + i] = narrow ? f[i] : 0.0f;
+            pyr[15 + i] = narrow ? fabsf(f[i]) : 0.0f;
+        }
+        pyr[18] = narrow ? tx : 0.0f;
+        pyr[19] = narrow ? ty : 0.0f;
+    }
+    __syncwarp();
+}
+
+// Whether a box (planes relative to the apex) can meet the pyramid nearer
+// than the clip (squared, g2), and its squared distance from the apex. With
+// c twice the centre and e twice the half extents in the pyramid's frame,
+// the box reaches in front of the apex if cz + ez >= 0 and into the pyramid
+// if |cx| <= ex + tx (cz + ez), likewise y. A NaN box never does.
+__device__ __forceinline__ bool tile_box(const float lo[3], const float hi[3], const float *pyr,
+                                         float g2, float &d2) {
+    const float4 *p = reinterpret_cast<const float4 *>(pyr);
+    const float4 p0 = p[0], p1 = p[1], p2 = p[2], p3 = p[3], p4 = p[4];
+    float c[3], e[3], m[3];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        c[i] = lo[i] + hi[i];
+        e[i] = hi[i] - lo[i];
+        m[i] = fmaxf(fmaxf(lo[i], -hi[i]), 0.0f);
+    }
+    d2 = fmaf(m[0], m[0], fmaf(m[1], m[1], m[2] * m[2]));
+    const float cx = fmaf(p0.x, c[0], fmaf(p0.y, c[1], p0.z * c[2]));
+    const float ex = fmaf(p0.w, e[0], fmaf(p1.x, e[1], p1.y * e[2]));
+    const float cy = fmaf(p1.z, c[0], fmaf(p1.w, c[1], p2.x * c[2]));
+    const float ey = fmaf(p2.y, e[0], fmaf(p2.z, e[1], p2.w * e[2]));
+    const float cz = fmaf(p3.x, c[0], fmaf(p3.y, c[1], p3.z * c[2]));
+    const float s = cz + fmaf(p3.w, e[0], fmaf(p4.x, e[1], p4.y * e[2]));
+    return s >= 0.0f && fabsf(cx) <= fmaf(p4.z, s, ex) && fabsf(cy) <= fmaf(p4.w, s, ey) && d2 <= g2;
+}
+
+// Child `sub` of wide node `node` of the 32-wide copy against the pyramid.
+template <bool Q8>
+__device__ __forceinline__ bool tile_child(const void *grec, uint32_t node, int sub,
+                                           const float apex[3], const float *pyr, float g2,
+                                           uint32_t &ref, float &d2) {
+    float lo[3], hi[3];
+    bool ok = true;
+    if constexpr (!Q8) {
+        const float4 *cp = reinterpret_cast<const float4 *>(
+            static_cast<const ChildRec *>(grec) + (node & kWideOffsetMask) + sub);
+        const float4 q0 = __ldg(cp), q1 = __ldg(cp + 1);
+        lo[0] = q0.x; lo[1] = q0.y; lo[2] = q0.z;
+        hi[0] = q0.w; hi[1] = q1.x; hi[2] = q1.y;
+        ref = __float_as_uint(q1.z);
+    } else {
+        const uint4 *u = static_cast<const uint4 *>(grec) + (node & kWideOffsetMask);
+        const float4 h0 = __ldg(reinterpret_cast<const float4 *>(u));
+        const float4 h1 = __ldg(reinterpret_cast<const float4 *>(u) + 1);
+        const uint4 c = __ldg(u + kGroupQHeaderUnits + sub);
+        ref = c.z;
+        ok = !(c.y & kQ8Skip);
+        // plane q is origin + q * scale rounded once, as the build checked it
+        lo[0] = fmaf((float)(c.x & 255u), h0.w, h0.x);
+        lo[1] = fmaf((float)((c.x >> 8) & 255u), h1.x, h0.y);
+        lo[2] = fmaf((float)((c.x >> 16) & 255u), h1.y, h0.z);
+        hi[0] = fmaf((float)(c.x >> 24), h0.w, h0.x);
+        hi[1] = fmaf((float)(c.y & 255u), h1.x, h0.y);
+        hi[2] = fmaf((float)((c.y >> 8) & 255u), h1.y, h0.z);
+    }
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        lo[i] -= apex[i];
+        hi[i] -= apex[i];
+    }
+    return tile_box(lo, hi, pyr, g2, d2) && ok;
+}
+
+// Traversal of the 32-wide copy by a warp whose rays share an apex: per step
+// lane k tests child k against the pyramid of all the rays, one test for 32
+// boxes and 32 rays where the binary packet makes one per box and ray. A
+// box's distance from the apex bounds the depth of every hit in it from
+// below (directions are unit length), so boxes beyond the farthest clip of
+// the warp are dropped; inner children go nearest first. Each surviving
+// leaf, nearest box first, is evaluated by every lane for its own ray and
+// samples (Alg. 1, whose ellipsoid test decides; the box only saves work),
+// so per-lane results are those of an independent traversal. For shadow rays
+// the apex is the far end: their clip bounds the distance from it as well.
+// Returns false when the stack is full (the caller starts over otherwise).
+template <int N, bool Q8>
+__device__ __forceinline__ bool traverse_tile(const TraceArgs &a, Ray<N> &r, int pass,
+                                              const float apex[3], const float *pyr,
+                                              uint32_t *s_ref, float *s_t, uint32_t &err) {
+    const uint32_t kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    unsigned long long draws = 0;
+    // clips are not negative here (t_min >= 0), so their bits order them
+    uint32_t gb = __reduce_max_sync(kAll, r.t_far >= r.t_min ? __float_as_uint(fmaxf(r.t_far, 0.0f)) : 0u);
+    if (!__any_sync(kAll, r.t_far >= r.t_min)) return true;
+    float g2 = __uint_as_float(gb) * __uint_as_float(gb);
+    int sp = 0;
+    uint32_t node = __ldg(a.troot), steps = 0;
+    for (;;) {
+        if (++steps > a.step_limit) {
+            err |= kErrSteps;
+            break;
+        }
+        const int n_child = (int)((node >> kWideCountShift) & 31u) + 1;
+        uint32_t ref = kEmpty;
+        float d2 = INFINITY;
+        bool hit = false;
+        if (lane < n_child) hit = tile_child<Q8>(a.trec, node, lane, apex, pyr, g2, ref, d2);
+        const bool leaf = (ref & kLeafBit) != 0u;
+        const uint32_t key = (__float_as_uint(d2) & ~31u) | (uint32_t)lane;
+        bool pending = hit && leaf;
+        while (__any_sync(kAll, pending)) {
+            const uint32_t best = __reduce_min_sync(kAll, pending ? key : 0xffffffffu);
+            const int src = (int)(best & 31u);
+            // (cleared low bits: never above the distance itself)
+            if (__uint_as_float(best & ~31u) > g2) break;
+            if (lane == src) pending = false;
+            const uint32_t idx = __shfl_sync(kAll, ref, src) & ~kLeafBit;
+            const float far0 = r.t_far;
+            intersect<N, false>(a, r, idx, pass, draws);
+            if (__any_sync(kAll, r.t_far != far0)) {
+                gb = __reduce_max_sync(kAll, __float_as_uint(fmaxf(r.t_far, 0.0f)));
+                g2 = __uint_as_float(gb) * __uint_as_float(gb);
+            }
+        }
+        const bool inner = hit && !leaf && d2 <= g2;
+        const uint32_t im = __ballot_sync(kAll, inner);
+        if (im) {
+            const int nj = (int)(__reduce_min_sync(kAll, inner ? key : 0xffffffffu) & 31u);
+            const uint32_t next = __shfl_sync(kAll, ref, nj);
+            const uint32_t others = im & ~(1u << nj);
+            const int npush = __popc(others);
+            if (sp + npush > kTilePool) return false;
+            __syncwarp();  // earlier reads of these entries are done
+            if (inner && lane != nj) {
+                const int pos = sp + __popc(others & ((1u << lane) - 1u));
+                s_ref[pos] = ref;
+                s_t[pos] = d2;
+            }
+            sp += npush;
+            __syncwarp();
+            node = next;
+            continue;
+        }
+        // the topmost entry within the clip, 32 entries at a time
+        bool found = false;
+        while (sp > 0) {
+            const int k = sp - 1 - lane;
+            const uint32_t okm = __ballot_sync(kAll, k >= 0 && s_t[k >= 0 ? k : 0] <= g2);
+            if (okm) {
+                sp -= __ffs(okm);  // the lowest lane holds the topmost
+                node = s_ref[sp];
+                found = true;
+                break;
+            }
+            sp = sp > 32 ? sp - 32 : 0;
+        }
+        if (!found) break;
+    }
+    return true;
+}
+
+// The same rays through the binary nodes, for a tile whose stack does not do:
+// out of line, so that the common path keeps its registers.
+template <int N>
+__device__ __noinline__ void tile_fallback(const TraceArgs &a, Ray<N> &r, int pass, uint32_t &err) {
+    uint32_t stack[kMaxStack];
+    float stack_t[kMaxStack];
+    Counts cnt;
+    traverse_packet<N, false>(a, r, pass, stack, stack_t, err, cnt);
 }
 
 }  // namespace

@@ -49,3 +49,29 @@ def test_grouped_hits_equal_packet_hits(gs, fmt, coincident):
             assert torch.equal(a, b) and torch.equal(ta, tb), (M, lanes)
         assert M < 100 or (a >= 0).any()
         bvh.free()
+
+
+@pytest.mark.parametrize("fmt", ["binary", "binary_q8"])
+@pytest.mark.parametrize("spp,spl", [(1, 0), (3, 1), (5, 2), (7, 0), (16, 0), (32, 8)])
+def test_tile_hits_equal_packet_hits(gs, fmt, spp, spl):
+    """The tile traversal against the binary walk: an eye inside the cloud,
+    a view so wide that a tile has no pyramid, one pixel, odd sizes, a range
+    and a range that ends before everything."""
+    cams = [scenes.Pinhole(width=37, height=19, eye=(0.4, 0.3, 2.8)),
+            scenes.Pinhole(width=41, height=23, eye=(0.05, 0.02, 0.1), look_at=(1.0, 0.3, -0.4)),
+            scenes.Pinhole(width=5, height=3, eye=(0.0, 0.0, 0.5), fov_y_deg=170.0),
+            scenes.Pinhole(width=1, height=1, eye=(0.3, 0.1, 2.0)),
+            scenes.Pinhole(width=33, height=9, eye=(0.0, 3.0, 0.0), up=(0.0, 0.0, 1.0))]
+    for M, coincident in ((1, False), (2, False), (33, True), (1025, False), (7000, True)):
+        g = gs.Gaussians.from_cloud(_cloud(M, coincident))
+        bvh = gs.build_bvh(g, node_format=fmt)
+        for cam in cams:
+            for lim in ({}, dict(t_min=1.5, t_max=3.0), dict(t_max=1e-3)):
+                kw = dict(seed=M, spp=spp, samples_per_lane=spl, want_hits=True, **lim)
+                assert gs.trace_layout(bvh, spp=spp, samples_per_lane=spl)["lanes_per_pixel"] < 8
+                rgb, a, ta = gs.trace_stochastic(bvh, g, cam, **kw)
+                ref, b, tb = gs.trace_stochastic(bvh, g, cam, stack_depth=96, **kw)
+                bvh.sync_status()
+                assert torch.equal(a, b) and torch.equal(ta, tb), (M, cam)
+                assert torch.equal(rgb, ref)
+        bvh.free()
