@@ -82,7 +82,7 @@ static void release(gs_bvh *b) {
     if (!b) return;
     void *bufs[] = {b->nodes, b->prims, b->status, b->codes[0], b->codes[1], b->vals[0],
                     b->vals[1], b->parent, b->arrive, b->aabb, b->bounds, b->hist,
-                    b->scan_tmp, b->wide, b->depth, b->wmap, b->link};
+                    b->scan_tmp, b->wide, b->depth, b->wmap, b->link, b->grad};
     for (void *p : bufs)
         if (p) cudaFree(p);
     for (auto &t : b->group) {
@@ -171,6 +171,7 @@ gs_status gs_build_bvh_ex(const gs_gaussians *g, const gs_build_options *opt, gs
         {(void **)&b->depth, wide ? (size_t)nn * 4 : 0},
         {(void **)&b->wmap, wide ? (size_t)nn * 4 : 0},
         {(void **)&b->link, grouped ? (size_t)nn * sizeof(uint4) : 0},
+        {(void **)&b->grad, grouped ? (size_t)cap * 10 * sizeof(float) : 0},
         {(void **)&b->group[0].rec, grouped ? (size_t)recs * rec_bytes : 0},
         {(void **)&b->group[0].ref, grouped ? (size_t)nn * 4 : 0},
         {(void **)&b->group[1].rec, grouped ? (size_t)recs * rec_bytes : 0},

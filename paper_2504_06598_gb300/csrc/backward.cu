@@ -108,6 +108,29 @@ __device__ __forceinline__ Cand eval_cand(const TraceArgs &a, const float o[3], 
     return c;
 }
 
+// Gradient with respect to an unnormalised quaternion qr (w, x, y, z) from
+// the one with respect to its rotation matrix.
+__device__ __forceinline__ void quat_gradient(const float4 qr, const float dR[9], float out[4]) {
+    const float n = sqrtf(qr.x * qr.x + qr.y * qr.y + qr.z * qr.z + qr.w * qr.w);
+    const float w = qr.x / n, x = qr.y / n, y = qr.z / n, z = qr.w / n;
+    const float Dw[9] = {0.0f, -2 * z, 2 * y, 2 * z, 0.0f, -2 * x, -2 * y, 2 * x, 0.0f};
+    const float Dx[9] = {0.0f, 2 * y, 2 * z, 2 * y, -4 * x, -2 * w, 2 * z, 2 * w, -4 * x};
+    const float Dy[9] = {-4 * y, 2 * x, 2 * w, 2 * x, 0.0f, 2 * z, -2 * w, 2 * z, -4 * y};
+    const float Dz[9] = {-4 * z, -2 * w, 2 * x, 2 * w, -4 * z, 2 * y, 2 * x, 2 * y, 0.0f};
+    float gq[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+    for (int e = 0; e < 9; ++e) {
+        gq[0] = fmaf(dR[e], Dw[e], gq[0]);
+        gq[1] = fmaf(dR[e], Dx[e], gq[1]);
+        gq[2] = fmaf(dR[e], Dy[e], gq[2]);
+        gq[3] = fmaf(dR[e], Dz[e], gq[3]);
+    }
+    const float qh[4] = {w, x, y, z};
+    const float dot = gq[0] * w + gq[1] * x + gq[2] * y + gq[3] * z;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) out[k] = (gq[k] - dot * qh[k]) / n;
+}
+
 // d alpha / d(mu, log s, quat, logit) of one candidate; alpha = o exp(-q/2),
 // q = |u|^2 with u = S^-1 R_q^T v, and t held at the 1D mean (dq/dt = 0).
 template <bool RELOAD>
@@ -142,25 +165,10 @@ __device__ void grad_alpha(const TraceArgs &a, const Cand &c, float out[11]) {
     for (int j = 0; j < 3; ++j)
 #pragma unroll
         for (int k = 0; k < 3; ++k) dR[3 * j + k] = 2.0f * c.v[j] * c.u[k] * inv_s[k];
-    const float4 qr = __ldg(reinterpret_cast<const float4 *>(a.quats) + c.gid);
-    const float n = sqrtf(qr.x * qr.x + qr.y * qr.y + qr.z * qr.z + qr.w * qr.w);
-    const float w = qr.x / n, x = qr.y / n, y = qr.z / n, z = qr.w / n;
-    const float Dw[9] = {0.0f, -2 * z, 2 * y, 2 * z, 0.0f, -2 * x, -2 * y, 2 * x, 0.0f};
-    const float Dx[9] = {0.0f, 2 * y, 2 * z, 2 * y, -4 * x, -2 * w, 2 * z, 2 * w, -4 * x};
-    const float Dy[9] = {-4 * y, 2 * x, 2 * w, 2 * x, 0.0f, 2 * z, -2 * w, 2 * z, -4 * y};
-    const float Dz[9] = {-4 * z, -2 * w, 2 * x, 2 * w, -4 * z, 2 * y, 2 * x, 2 * y, 0.0f};
-    float gq[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    float gq[4];
+    quat_gradient(__ldg(reinterpret_cast<const float4 *>(a.quats) + c.gid), dR, gq);
 #pragma unroll
-    for (int e = 0; e < 9; ++e) {
-        gq[0] = fmaf(dR[e], Dw[e], gq[0]);
-        gq[1] = fmaf(dR[e], Dx[e], gq[1]);
-        gq[2] = fmaf(dR[e], Dy[e], gq[2]);
-        gq[3] = fmaf(dR[e], Dz[e], gq[3]);
-    }
-    const float qh[4] = {w, x, y, z};
-    const float dot = gq[0] * w + gq[1] * x + gq[2] * y + gq[3] * z;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) out[6 + k] = dadq * (gq[k] - dot * qh[k]) / n;
+    for (int k = 0; k < 4; ++k) out[6 + k] = dadq * gq[k];
     out[10] = c.alpha * (1.0f - opacity);
 }
 
@@ -551,6 +559,362 @@ __global__ void __launch_bounds__(kThreads, LG >= 3 ? (N >= 4 ? 7 : kGroupMinBlo
     if (err) atomicOr(a.status, err);
 }
 
+// ---------------------------------------------------------------- tiles
+// Tile form (camera rays of one eye, see traverse_tile): every lane of a warp
+// evaluates the same candidate for its own ray. What a lane contributes to a
+// Gaussian's eleven parameters is linear in ten sums over the lanes, with
+// w = sum over its slots of g . (c_i - c_k) / (1 - alpha) and u = M v:
+//   sum w alpha,  sum w alpha u (3),  sum w alpha u u^T (6)
+// (v = R S u, so the rotation's outer product v u^T follows from u u^T). The
+// warp reduces these ten and adds them to the Gaussian's row with one
+// reduction instruction of ten lanes; k_chain applies the chain rule once per
+// Gaussian after the launch instead of once per ray and Gaussian.
+constexpr int kStats = 10;
+
+// Sums of v[0..9] over the warp: lane L returns sum stat_of(L).
+__device__ __forceinline__ float reduce_stats(const float v[kStats], int lane) {
+    const uint32_t kAll = 0xffffffffu;
+    const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4, b1 = lane & 2;
+    float x[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) {
+        const float keep = b4 ? v[5 + i] : v[i], give = b4 ? v[i] : v[5 + i];
+        x[i] = keep + __shfl_xor_sync(kAll, give, 16);
+    }
+    float y[3];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const float keep = b3 ? x[2 + i] : x[i], give = b3 ? x[i] : x[2 + i];
+        y[i] = keep + __shfl_xor_sync(kAll, give, 8);
+    }
+    y[2] = x[4] + __shfl_xor_sync(kAll, x[4], 8);
+    const float z0 = (b2 ? y[1] : y[0]) + __shfl_xor_sync(kAll, b2 ? y[0] : y[1], 4);
+    const float z1 = y[2] + __shfl_xor_sync(kAll, y[2], 4);
+    const float t = (b1 ? z1 : z0) + __shfl_xor_sync(kAll, b1 ? z0 : z1, 2);
+    return t + __shfl_xor_sync(kAll, t, 1);
+}
+
+// The sum lane L holds after reduce_stats, or -1 where another lane has it.
+__device__ __forceinline__ int stat_of(int lane) {
+    if (lane & 1) return -1;
+    const int hi = (lane & 16) ? 5 : 0;
+    if (lane & 2) return (lane & 12) ? -1 : hi + 4;
+    return hi + ((lane & 8) ? 2 : 0) + ((lane & 4) ? 1 : 0);
+}
+
+// One candidate (record idx, the same for the warp) against every lane's
+// slots; gck[k] = g . c_k of slot k's winner.
+template <int N>
+__device__ __forceinline__ void tile_gradient(const TraceArgs &a, const Ray<N> &r, uint32_t idx,
+                                              const float gck[N], const float g[3]) {
+    const uint32_t kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const Cand c = eval_cand<true>(a, r.o, r.d, idx);
+    float n_front = 0.0f, behind = 0.0f;
+    if (c.valid && c.t <= r.t_far) {
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+            if (lex_closer(c.tc, c.tau, c.gid, r.slot[k])) {
+                n_front += 1.0f;
+                behind += gck[k];
+            }
+    }
+    if (!__any_sync(kAll, n_front > 0.0f)) return;
+    float wa = 0.0f;
+    if (n_front > 0.0f) {
+        float Y[16], ci[3];
+        sh_basis(a.sh_degree, r.d, Y);
+        sh_colour(a, c.gid, Y, ci);
+        const float gci = fmaf(g[0], ci[0], fmaf(g[1], ci[1], g[2] * ci[2]));
+        // a rejected hit has alpha <= xi < 1
+        wa = fmaf(n_front, gci, -behind) / (1.0f - c.alpha) * c.alpha;
+    }
+    const bool add = wa != 0.0f;
+    if (!__any_sync(kAll, add)) return;
+    float v[kStats];
+    v[0] = wa;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) v[1 + i] = add ? wa * c.u[i] : 0.0f;
+    v[4] = v[1] * (add ? c.u[0] : 0.0f);
+    v[5] = v[2] * (add ? c.u[1] : 0.0f);
+    v[6] = v[3] * (add ? c.u[2] : 0.0f);
+    v[7] = v[1] * (add ? c.u[1] : 0.0f);
+    v[8] = v[1] * (add ? c.u[2] : 0.0f);
+    v[9] = v[2] * (add ? c.u[2] : 0.0f);
+    const float sum = reduce_stats(v, lane);
+    const int which = stat_of(lane);
+    if (which >= 0) atomicAdd(a.g_stats + (int64_t)idx * kStats + which, sum);
+}
+
+// Every Gaussian a ray of the warp reaches before its farthest winner. The
+// order does not matter and nothing is clipped, so a stack entry is a wide
+// node with the inner children still to visit, one per level of the 32-wide
+// tree: at most the 95 levels of the binary one.
+constexpr int kTileLevels = 128;
+
+template <int N, bool Q8>
+__device__ __forceinline__ void enumerate_tile(const TraceArgs &a, const Ray<N> &r,
+                                               const float gck[N], const float g[3],
+                                               const float *pyr, uint2 *stack, uint32_t &err) {
+    const uint32_t kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const bool live = r.t_far >= a.t_min;
+    if (!__any_sync(kAll, live)) return;
+    const float G = __uint_as_float(
+        __reduce_max_sync(kAll, live ? __float_as_uint(fmaxf(r.t_far, 0.0f)) : 0u));
+    const float g2 = G * G;
+    int sp = 0;
+    uint32_t node = __ldg(a.troot), steps = 0;
+    for (;;) {
+        if (++steps > a.step_limit) {
+            err |= kErrSteps;
+            break;
+        }
+        const int n_child = (int)((node >> kWideCountShift) & 31u) + 1;
+        uint32_t ref = kEmpty;
+        float d2 = INFINITY;
+        bool hit = false;
+        if (lane < n_child) hit = tile_child<Q8>(a.trec, node, lane, a.eye, pyr, g2, ref, d2);
+        const bool leaf = (ref & kLeafBit) != 0u;
+        for (uint32_t lm = __ballot_sync(kAll, hit && leaf); lm; lm &= lm - 1u) {
+            const uint32_t idx = __shfl_sync(kAll, ref, __ffs(lm) - 1) & ~kLeafBit;
+            tile_gradient<N>(a, r, idx, gck, g);
+        }
+        uint32_t im = __ballot_sync(kAll, hit && !leaf);
+        if (im) {
+            const int j = __ffs(im) - 1;
+            im &= im - 1u;
+            if (im) {
+                if (sp >= kTileLevels) {
+                    err |= kErrStack;
+                    break;
+                }
+                __syncwarp();
+                if (lane == 0) stack[sp] = make_uint2(node, im);
+                __syncwarp();
+                ++sp;
+            }
+            node = __shfl_sync(kAll, ref, j);
+            continue;
+        }
+        if (sp == 0) break;
+        const uint2 top = stack[sp - 1];
+        const int j = __ffs(top.y) - 1;
+        const uint32_t rest = top.y & (top.y - 1u);
+        __syncwarp();
+        if (rest == 0) --sp;
+        else if (lane == 0) stack[sp - 1].y = rest;
+        __syncwarp();
+        const uint32_t at = (top.x & kWideOffsetMask) + (uint32_t)j;
+        if constexpr (Q8)
+            node = __ldg(&static_cast<const ChildQ8 *>(a.trec)[at + kGroupQHeaderUnits].child);
+        else
+            node = __ldg(&static_cast<const ChildRec *>(a.trec)[at].child);
+    }
+}
+
+// dLoss/dk of one winner, counted `mult` times: 12 or 3 reductions of four
+// coefficients where the rows start on 16 bytes, else one each.
+__device__ __forceinline__ void add_sh_gradient(const TraceArgs &a, uint32_t gid, const float gm[3],
+                                                const float Y[16]) {
+    const int K = (a.sh_degree + 1) * (a.sh_degree + 1);
+    float *dst = a.g_sh + (int64_t)gid * K * 3;
+    if (a.sh_vec && K == 16) {
+#pragma unroll
+        for (int q = 0; q < 12; ++q)
+            atomicAdd(reinterpret_cast<float4 *>(dst) + q,
+                      make_float4(gm[(4 * q) % 3] * Y[(4 * q) / 3], gm[(4 * q + 1) % 3] * Y[(4 * q + 1) / 3],
+                                  gm[(4 * q + 2) % 3] * Y[(4 * q + 2) / 3],
+                                  gm[(4 * q + 3) % 3] * Y[(4 * q + 3) / 3]));
+        return;
+    }
+    for (int ch = 0; ch < 3; ++ch)
+        if (gm[ch] != 0.0f)
+            for (int i = 0; i < K; ++i) atomicAdd(dst + 3 * i + ch, gm[ch] * Y[i]);
+}
+
+template <int N, bool Q8, bool KEYS>
+__global__ void __launch_bounds__(kThreads, N >= 8 ? 4 : 5)
+    k_backward_tile(const __grid_constant__ TraceArgs a) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const uint32_t kAll = 0xffffffffu;
+    __shared__ __align__(16) float s_pyr[kThreads / 32][kTileFloats];
+    __shared__ uint2 s_lvl[kThreads / 32][kTileLevels];
+    // the forward traversal's stack, where the winners are traced again
+    __shared__ uint32_t s_ref[KEYS ? 1 : kThreads / 32][KEYS ? 1 : kTilePool];
+    __shared__ float s_t[KEYS ? 1 : kThreads / 32][KEYS ? 1 : kTilePool];
+    float *pyr = s_pyr[warp];
+    const int lg = a.lpp_log2, L = 1 << lg;
+    const int tw_lg = tile_w_log2(lg), th_lg = 5 - lg - tw_lg;
+    const int sub = lane & (L - 1), pl = lane >> lg;
+    const uint32_t tiles_x = (uint32_t)((a.width + (1 << tw_lg) - 1) >> tw_lg);
+    const uint32_t tiles_y = (uint32_t)((a.height + (1 << th_lg) - 1) >> th_lg);
+    const uint32_t n_tiles = tiles_x * tiles_y;
+    uint32_t err = 0;
+    for (;;) {
+        uint32_t tile = 0;
+        if (lane == 0) tile = atomicAdd(a.work, 1u);
+        tile = __shfl_sync(kAll, tile, 0);
+        if (tile >= n_tiles) break;
+        const int x = (int)(((tile % tiles_x) << tw_lg) + (pl & ((1 << tw_lg) - 1)));
+        const int y = (int)(((tile / tiles_x) << th_lg) + (pl >> tw_lg));
+        const bool valid = x < a.width && y < a.height;
+        const int64_t pix = valid ? (int64_t)y * a.width + x : 0;
+        Ray<N> r;
+        {
+            float d[3];
+            camera_ray(a, valid ? x : 0, valid ? y : 0, d);
+            for (int i = 0; i < 3; ++i) {
+                r.o[i] = a.eye[i];
+                r.d[i] = d[i];
+            }
+        }
+        r.ray_id = a.ray_id_offset + (uint32_t)pix;
+        r.stream_tag = a.stream_tag;
+        r.t_min = a.t_min;
+        r.t_max = a.t_max;
+        r.any_hit = false;
+        tile_pyramid(r.d, valid, pyr);
+        const float inv_s = 1.0f / (float)a.n_samples;
+        float g[3] = {0.0f, 0.0f, 0.0f};
+        if (valid)
+            for (int ch = 0; ch < 3; ++ch) g[ch] = a.d_rgb[3 * pix + ch] * inv_s;
+        const int n_rounds = (a.spp + L - 1) >> lg;
+        for (int j = 0; j < n_rounds; ++j) {
+            const int pass = (j << lg) + sub;
+            const bool live = valid && pass < a.spp;
+            // unused slots (sample index past the pixel's count) at -inf:
+            // nothing is in front of them and they never set the clip
+            auto reset = [&](Ray<N> &q) {
+#pragma unroll
+                for (int k = 0; k < N; ++k)
+                    q.slot[k] = pass * N + k < a.n_samples ? Slot{INFINITY, 0.0f, 0xffffffffu}
+                                                           : Slot{-INFINITY, 0.0f, 0xffffffffu};
+                update_clip(q, a.t_max);
+                if (!live) q.t_far = -INFINITY;
+            };
+            reset(r);
+            // 1) the winners: the rendering's stored payloads, or the forward
+            // traversal again with the same keys (same winners)
+            if constexpr (KEYS) {
+                if (live) {
+                    const gs_sample_key *kp = a.keys + pix * a.n_samples + pass * N;
+#pragma unroll
+                    for (int k = 0; k < N; ++k) {
+                        if (pass * N + k >= a.n_samples) continue;
+                        const float tc = __ldg(&kp[k].tc), tau = __ldg(&kp[k].tau);
+                        const uint32_t gid = __ldg(&kp[k].gid);
+                        if (gid == 0xffffffffu || gid < a.n_gauss) {
+                            r.slot[k] = Slot{tc, tau, gid};
+                        } else {
+                            err |= kErrKeys;  // names no Gaussian: no hit
+                        }
+                    }
+                }
+            } else {
+                if (!traverse_tile<N, Q8>(a, r, pass, a.eye, pyr, s_ref[warp], s_t[warp], err)) {
+                    Ray<N> again = r;
+                    set_ray(again, a.eye, r.d);
+                    reset(again);
+                    uint32_t err2 = 0;
+                    tile_fallback<N>(a, again, pass, err2);
+                    err |= err2;
+#pragma unroll
+                    for (int k = 0; k < N; ++k) r.slot[k] = again.slot[k];
+                }
+            }
+            // 2) colours of the winners; dLoss/dk of the selected Gaussians,
+            // once for the slots of a lane that hold the same one
+            float gck[N];
+            {
+                float Y[16];
+                sh_basis(a.sh_degree, r.d, Y);
+#pragma unroll
+                for (int k = 0; k < N; ++k) {
+                    const uint32_t wid = live ? r.slot[k].gid : 0xffffffffu;
+                    float ck[3] = {a.bg[0], a.bg[1], a.bg[2]};
+                    if (wid != 0xffffffffu) {
+                        float raw[3];
+                        sh_colour_raw(a, wid, Y, raw);
+                        bool first = true;
+                        float mult = 1.0f;
+#pragma unroll
+                        for (int q = 0; q < N; ++q) {
+                            if (q < k && r.slot[q].gid == wid) first = false;
+                            if (q > k && r.slot[q].gid == wid) mult += 1.0f;
+                        }
+                        float gm[3];
+                        for (int ch = 0; ch < 3; ++ch) {
+                            ck[ch] = fmaxf(raw[ch], 0.0f);
+                            gm[ch] = raw[ch] > 0.0f ? mult * g[ch] : 0.0f;
+                        }
+                        if (first && (gm[0] != 0.0f || gm[1] != 0.0f || gm[2] != 0.0f))
+                            add_sh_gradient(a, wid, gm, Y);
+                    }
+                    gck[k] = fmaf(g[0], ck[0], fmaf(g[1], ck[1], g[2] * ck[2]));
+                }
+            }
+            // 3) every Gaussian in front of a winner
+            update_clip(r, a.t_max);
+            if (!live) r.t_far = -INFINITY;
+            __syncwarp();
+            enumerate_tile<N, Q8>(a, r, gck, g, pyr, s_lvl[warp], err);
+            __syncwarp();
+        }
+    }
+    if (err) atomicOr(a.status, err);
+}
+
+// The chain rule from each Gaussian's ten sums (in record order) to its
+// parameters' gradients.
+__global__ void __launch_bounds__(256) k_chain(const __grid_constant__ TraceArgs a) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (int64_t)a.n_gauss) return;
+    const float2 *sp = reinterpret_cast<const float2 *>(a.g_stats + i * kStats);
+    float s[kStats];
+    bool any = false;
+#pragma unroll
+    for (int k = 0; k < kStats / 2; ++k) {
+        const float2 v = sp[k];
+        s[2 * k] = v.x;
+        s[2 * k + 1] = v.y;
+        any = any || v.x != 0.0f || v.y != 0.0f;
+    }
+    if (!any) return;
+    const float4 *pp = reinterpret_cast<const float4 *>(a.prims + i);
+    const float4 p0 = __ldg(pp), p1 = __ldg(pp + 1), p2 = __ldg(pp + 2), p3 = __ldg(pp + 3);
+    const float m[9] = {p1.x, p1.y, p1.z, p1.w, p2.x, p2.y, p2.z, p2.w, p3.x};
+    const int64_t gid = __float_as_uint(p3.y);
+    const float P[3][3] = {{s[4], s[7], s[8]}, {s[7], s[5], s[9]}, {s[8], s[9], s[6]}};
+    // dalpha/dq = -alpha / 2; dq/dmu = -2 M^T u, dq/dlog s_k = -2 u_k^2
+    for (int j = 0; j < 3; ++j) {
+        atomicAdd(a.g_means + 3 * gid + j, fmaf(m[j], s[1], fmaf(m[3 + j], s[2], m[6 + j] * s[3])));
+        atomicAdd(a.g_log_scales + 3 * gid + j, P[j][j]);
+    }
+    // dq/dR_jk = 2 v_j u_k / s_k with v = R S u and (R S)_jl = M_lj s_l^2
+    float inv_s[3], s2[3];
+    for (int k = 0; k < 3; ++k) {
+        const float ls = __ldg(a.log_scales + 3 * gid + k);
+        inv_s[k] = expf(-ls);
+        const float e = expf(ls);
+        s2[k] = e * e;
+    }
+    float dR[9];
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+        const float rs[3] = {m[j] * s2[0], m[3 + j] * s2[1], m[6 + j] * s2[2]};
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            dR[3 * j + k] =
+                2.0f * fmaf(rs[0], P[0][k], fmaf(rs[1], P[1][k], rs[2] * P[2][k])) * inv_s[k];
+    }
+    const float4 qr = __ldg(reinterpret_cast<const float4 *>(a.quats) + gid);
+    float gq[4];
+    quat_gradient(qr, dR, gq);
+    for (int k = 0; k < 4; ++k) atomicAdd(a.g_quats + 4 * gid + k, -0.5f * gq[k]);
+    atomicAdd(a.g_logits + gid, s[0] * (1.0f - p0.w));
+}
+
 template <int N, int LG, bool Q8, bool KEYS>
 gs_status launch_backward_nl(const TraceArgs &a, cudaStream_t s) {
     int dev = 0, sms = 0, per = 0;
@@ -573,8 +937,35 @@ gs_status launch_backward_nl(const TraceArgs &a, cudaStream_t s) {
 }
 
 // Groups of 8 or more lanes on one pixel use the wide copy of their width.
+template <int N, bool Q8, bool KEYS>
+gs_status launch_backward_tile(const TraceArgs &a, cudaStream_t s) {
+    int dev = 0, sms = 0, per = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_backward_tile<N, Q8, KEYS>,
+                                                          kThreads, 0);
+    if (e != cudaSuccess) return cuda_fail(e, "backward launch setup");
+    const int tw_lg = tile_w_log2(a.lpp_log2), th_lg = 5 - a.lpp_log2 - tw_lg;
+    const uint32_t tiles = (uint32_t)(((a.width + (1 << tw_lg) - 1) >> tw_lg) *
+                                      ((a.height + (1 << th_lg) - 1) >> th_lg));
+    uint32_t blocks = (uint32_t)sms * (uint32_t)(per > 0 ? per : 1);
+    const uint32_t max_blocks = (tiles + kThreads / 32 - 1) / (kThreads / 32);
+    if (blocks > max_blocks) blocks = max_blocks;
+    if ((e = cudaMemsetAsync(a.work, 0, sizeof(uint32_t), s)) != cudaSuccess)
+        return cuda_fail(e, "reset work counter");
+    if ((e = cudaMemsetAsync(a.g_stats, 0, (size_t)a.n_gauss * kStats * sizeof(float), s)) != cudaSuccess)
+        return cuda_fail(e, "reset gradient sums");
+    k_backward_tile<N, Q8, KEYS><<<blocks, kThreads, 0, s>>>(a);
+    k_chain<<<(unsigned)((a.n_gauss + 255) / 256), 256, 0, s>>>(a);
+    return GS_OK;
+}
+
 template <int N, bool KEYS>
 gs_status launch_backward_nk(const TraceArgs &a, cudaStream_t s) {
+    if (a.trec != nullptr)
+        return a.gq8 ? launch_backward_tile<N, true, KEYS>(a, s)
+                     : launch_backward_tile<N, false, KEYS>(a, s);
     if (a.grec != nullptr && a.gq8) {
         switch (a.lpp_log2) {
             case 5: return launch_backward_nl<N, 5, true, KEYS>(a, s);
@@ -608,9 +999,10 @@ gs_status launch_backward_n(const TraceArgs &a, cudaStream_t s) {
 // 15.0, per-lane packets), else K = 2 (spp 16: 49.4 -> 46.0, spp 64:
 // 104.8 -> 59.8, 16- and 32-lane groups); never fewer than n_hits (N = 4
 // at spp 4 and 16 keeps S = 1: 48.1 and 77.8 ms against 50.1 and 103.8).
-static int auto_backward_samples_per_lane(int spp, int n_hits) {
+static int auto_backward_samples_per_lane(int spp, int n_hits, bool tile) {
     const int64_t T = (int64_t)spp * n_hits;
     int K = T <= 2 ? (int)T : (T < 16 ? 4 : 2);
+    if (tile) K = T <= 2 ? (int)T : (T < 8 ? 4 : 8);
     if (K < n_hits) K = n_hits;
     return K / n_hits;
 }
@@ -621,8 +1013,9 @@ gs_status launch_backward(const gs_bvh *b, const gs_gaussians *g, const gs_pinho
                           float *d_sh, cudaStream_t s) {
     // a lane carries S consecutive samples: ceil(spp / S) passes of
     // n_hits * S slots, the same sample indices and keys as the forward
+    const bool tile = b->link && p->t_min >= 0.0f && p->stack_depth == 0;
     int S = p->samples_per_lane > 0 ? p->samples_per_lane
-                                    : auto_backward_samples_per_lane(p->spp, p->n_hits);
+                                    : auto_backward_samples_per_lane(p->spp, p->n_hits, tile);
     while (S > 1 && S > p->spp) S >>= 1;
     const int spp_eff = (p->spp + S - 1) / S;
     TraceArgs a = {};
@@ -659,6 +1052,13 @@ gs_status launch_backward(const gs_bvh *b, const gs_gaussians *g, const gs_pinho
         a.grec = b->group[a.lpp_log2 - 3].rec;
         a.groot = b->group[a.lpp_log2 - 3].ref;
         a.gq8 = b->node_format == GS_NODES_BINARY_Q8;
+    }
+    if (tile) {
+        a.trec = b->group[2].rec;
+        a.troot = b->group[2].ref;
+        a.gq8 = b->node_format == GS_NODES_BINARY_Q8;
+        a.g_stats = b->grad;
+        a.sh_vec = ((uintptr_t)d_sh & 15u) == 0;
     }
     a.keys = const_cast<gs_sample_key *>(keys);  // read only here
     a.n_gauss = (uint32_t)b->M;

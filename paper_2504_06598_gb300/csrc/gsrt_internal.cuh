@@ -154,6 +154,7 @@ struct gs_bvh {
     // formats only): W = 8, 16, 32, each at most M + (M - 1) records
     gsrt::GroupTree group[gsrt::kGroupTrees];
     uint4 *link;  // per binary internal node: its place in the wide trees (build.cu)
+    float *grad;  // [M][10] sums of a gradient launch (backward.cu)
     // scratch of the batched form's deferred bounce rays, grown on demand
     int64_t wave_cap;                    // sample slots (pixels x spp) held
     int64_t wave_bytes;                  // device bytes of the scratch below

@@ -61,6 +61,8 @@ struct TraceArgs {
     const float *log_scales;   // raw parameters, for the scale and rotation
     const float *quats;        // derivatives
     float *g_means, *g_log_scales, *g_quats, *g_logits, *g_sh;
+    float *g_stats;  // tile form: ten sums per Gaussian, in record order
+    int sh_vec;      // 1 when g_sh starts on 16 bytes
 };
 
 // A warp traces a tile of 32 >> lpp_log2 pixels, each pixel on 1 << lpp_log2
