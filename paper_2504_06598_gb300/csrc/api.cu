@@ -81,15 +81,14 @@ static gs_status check_gaussians_device(const gs_gaussians *g, bool need_sh) {
 static void release(gs_bvh *b) {
     if (!b) return;
     void *bufs[] = {b->nodes, b->prims, b->status, b->codes[0], b->codes[1], b->vals[0],
-                    b->vals[1], b->parent, b->arrive, b->aabb, b->bounds, b->hist,
-                    b->scan_tmp, b->wide, b->depth, b->wmap, b->link, b->grad};
+                    b->vals[1], b->parent, b->aabb, b->zero, b->scan_tmp, b->wide, b->depth, b->wmap, b->link, b->grad};
     for (void *p : bufs)
         if (p) cudaFree(p);
     for (auto &t : b->group) {
         if (t.rec) cudaFree(t.rec);
         if (t.ref) cudaFree(t.ref);
     }
-    void *wave[] = {b->wave_codes[0], b->wave_codes[1], b->wave_bounce, b->wave_hist, b->wave_scan};
+    void *wave[] = {b->wave_codes[0], b->wave_codes[1], b->wave_bounce, b->wave_sort};
     for (void *p : wave)
         if (p) cudaFree(p);
     free(b);
@@ -141,8 +140,6 @@ gs_status gs_build_bvh_ex(const gs_gaussians *g, const gs_build_options *opt, gs
     const int64_t M = g->M;
     const int64_t cap = M > 0 ? M : 0;
     const int64_t nn = M > 1 ? M - 1 : 1;
-    const int64_t tiles = radix_tiles(cap > 0 ? cap : 1);
-    const int64_t scan_n = 256 * tiles > nn ? 256 * tiles : nn;
     const bool q8 = format == GS_NODES_BINARY_Q8;
     const bool wide = format == GS_NODES_WIDE4 || format == GS_NODES_WIDE4_Q8;
     const size_t wide_bytes = format == GS_NODES_WIDE4 ? sizeof(Node4) : sizeof(NodeQ4);
@@ -162,11 +159,9 @@ gs_status gs_build_bvh_ex(const gs_gaussians *g, const gs_build_options *opt, gs
         {(void **)&b->vals[0], (size_t)(cap > 0 ? cap : 1) * 4},
         {(void **)&b->vals[1], (size_t)(cap > 0 ? cap : 1) * 4},
         {(void **)&b->parent, (size_t)(2 * cap + 2) * 4},
-        {(void **)&b->arrive, (size_t)((cap > 0 ? cap : 1) + kGroupTrees) * 4},
         {(void **)&b->aabb, (size_t)(cap > 0 ? cap : 1) * 24},
-        {(void **)&b->bounds, 64},
-        {(void **)&b->hist, (size_t)256 * tiles * 4},
-        {(void **)&b->scan_tmp, (size_t)scan_tmp_entries(scan_n) * 4},
+        {(void **)&b->zero, build_scratch_bytes(cap > 0 ? cap : 1)},
+        {(void **)&b->scan_tmp, wide ? (size_t)scan_tmp_entries(nn) * 4 : 0},
         {(void **)&b->wide, wide ? (size_t)nn * wide_bytes : 0},
         {(void **)&b->depth, wide ? (size_t)nn * 4 : 0},
         {(void **)&b->wmap, wide ? (size_t)nn * 4 : 0},
@@ -190,7 +185,6 @@ gs_status gs_build_bvh_ex(const gs_gaussians *g, const gs_build_options *opt, gs
         total += (int64_t)r.bytes;
     }
     b->capacity = cap;
-    b->hist_len = 256 * tiles;
     b->device_bytes = total;
     cudaError_t e = cudaMemsetAsync(b->status, 0, 16, (cudaStream_t)stream);
     if (e != cudaSuccess) {

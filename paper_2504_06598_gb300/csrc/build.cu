@@ -5,7 +5,8 @@
 //   k_morton      63-bit key: Morton code of each mean in the scene bounds
 //                 with a size class of the Gaussian's box below the top
 //                 two octree levels
-//   radix sort    stable LSD sort of (code, id), 8 passes of 8 bits
+//   k_radix_pass  stable LSD sort of (code, id), 8 digits of 8 bits, one
+//                 pass over the keys each
 //   k_karras      binary radix tree over the sorted codes (Karras 2012),
 //                 equal codes split by position
 //   k_leaves      per-Gaussian record in tree order, then bottom-up box
@@ -23,8 +24,10 @@ namespace {
 constexpr int kSortThreads = 256;
 constexpr int kSortItems = 8;
 constexpr int kSortTile = kSortThreads * kSortItems;
+constexpr int kSortPasses = 8;  // 8-bit digits of a 64-bit key
 
-// Order-preserving map float -> uint32 (for atomicMin / atomicMax).
+// Order-preserving map float -> uint32 (for atomicMax; a minimum is kept as
+// the maximum of the complement, so that zero starts both).
 __device__ __forceinline__ unsigned int f2ord(float f) {
     unsigned int u = __float_as_uint(f);
     return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
@@ -97,7 +100,7 @@ __device__ __forceinline__ void ellipsoid_box(const Activated &a, float box[6]) 
     }
 }
 
-__global__ void k_preprocess(int64_t M, const float *__restrict__ means,
+__global__ void __launch_bounds__(256) k_preprocess(int64_t M, const float *__restrict__ means,
                              const float *__restrict__ log_scales, const float *__restrict__ quats,
                              const float *__restrict__ logits, float *__restrict__ aabb,
                              unsigned int *__restrict__ bounds, uint32_t *__restrict__ status) {
@@ -122,17 +125,30 @@ __global__ void k_preprocess(int64_t M, const float *__restrict__ means,
         }
         for (int k = 0; k < 6; ++k) aabb[6 * g + k] = box[k];
     }
-    // warp reduction of the finite means, then one atomic per warp
+    // reduction of the finite means over the block, then six atomics: one per
+    // warp made the kernel wait on its six addresses (1M: 131 us)
+    __shared__ float s_lo[3][8], s_hi[3][8];
     for (int k = 0; k < 3; ++k) {
         for (int off = 16; off > 0; off >>= 1) {
             lo[k] = fminf(lo[k], __shfl_xor_sync(0xffffffffu, lo[k], off));
             hi[k] = fmaxf(hi[k], __shfl_xor_sync(0xffffffffu, hi[k], off));
         }
+        if ((threadIdx.x & 31) == 0) {
+            s_lo[k][threadIdx.x >> 5] = lo[k];
+            s_hi[k][threadIdx.x >> 5] = hi[k];
+        }
     }
-    if ((threadIdx.x & 31) == 0 && lo[0] <= hi[0]) {
-        for (int k = 0; k < 3; ++k) {
-            atomicMin(&bounds[k], f2ord(lo[k]));
-            atomicMax(&bounds[3 + k], f2ord(hi[k]));
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        const int k = threadIdx.x;
+        float l = INFINITY, h = -INFINITY;
+        for (int w = 0; w < 8; ++w) {
+            l = fminf(l, s_lo[k][w]);
+            h = fmaxf(h, s_hi[k][w]);
+        }
+        if (l <= h) {
+            atomicMax(&bounds[k], ~f2ord(l));
+            atomicMax(&bounds[3 + k], f2ord(h));
         }
     }
 }
@@ -158,15 +174,13 @@ __device__ __forceinline__ unsigned long long spread3(unsigned long long v) {
 constexpr int kKeyTopBits = 6;
 constexpr int kKeySizeBits = 4;
 
-__global__ void k_morton(int64_t M, const float *__restrict__ means,
-                         const unsigned int *__restrict__ bounds, const float *__restrict__ aabb,
-                         unsigned long long *__restrict__ codes, uint32_t *__restrict__ vals) {
-    int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= M) return;
+__device__ __forceinline__ unsigned long long sort_code(int64_t g, const float *__restrict__ means,
+                                                        const unsigned int *__restrict__ bounds,
+                                                        const float *__restrict__ aabb) {
     unsigned long long q[3];
     float scene = 0.0f, edge = 0.0f;
     for (int k = 0; k < 3; ++k) {
-        float lo = ord2f(bounds[k]), hi = ord2f(bounds[3 + k]);
+        float lo = ord2f(~bounds[k]), hi = ord2f(bounds[3 + k]);
         float ext = hi - lo;
         scene = fmaxf(scene, ext);
         edge = fmaxf(edge, aabb[6 * g + 3 + k] - aabb[6 * g + k]);
@@ -184,25 +198,54 @@ __global__ void k_morton(int64_t M, const float *__restrict__ means,
     const int low = 63 - kKeyTopBits - kKeySizeBits;
     const unsigned long long top = morton >> (63 - kKeyTopBits);
     const unsigned long long rest = (morton & ((1ull << (63 - kKeyTopBits)) - 1ull)) >> kKeySizeBits;
-    codes[g] = (top << (63 - kKeyTopBits)) | ((unsigned long long)cls << low) | rest;
-    vals[g] = (uint32_t)g;
+    return (top << (63 - kKeyTopBits)) | ((unsigned long long)cls << low) | rest;
+}
+
+// Codes and ids, and the histograms of every sort digit (kSortTile codes a
+// block).
+__global__ void __launch_bounds__(kSortThreads)
+    k_morton(int64_t M, const float *__restrict__ means, const unsigned int *__restrict__ bounds,
+             const float *__restrict__ aabb, unsigned long long *__restrict__ codes,
+             uint32_t *__restrict__ vals, uint32_t *__restrict__ hist) {
+    __shared__ uint32_t h[kSortPasses][256];
+    for (int p = 0; p < kSortPasses; ++p) h[p][threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t base = (int64_t)blockIdx.x * kSortTile;
+    for (int r = 0; r < kSortItems; ++r) {
+        const int64_t g = base + r * kSortThreads + threadIdx.x;
+        if (g >= M) break;
+        const unsigned long long c = sort_code(g, means, bounds, aabb);
+        codes[g] = c;
+        vals[g] = (uint32_t)g;
+        for (int p = 0; p < kSortPasses; ++p) atomicAdd(&h[p][(uint32_t)(c >> (8 * p)) & 255u], 1u);
+    }
+    __syncthreads();
+    for (int p = 0; p < kSortPasses; ++p) {
+        const uint32_t v = h[p][threadIdx.x];
+        if (v) atomicAdd(&hist[256 * p + threadIdx.x], v);
+    }
 }
 
 // ---------------------------------------------------------------- radix sort
 
+// Histograms of the digits of bits [8 * first, 64) (n below 2^32).
 __global__ void __launch_bounds__(kSortThreads)
-    k_radix_hist(int64_t n, const unsigned long long *__restrict__ keys, int shift,
-                 uint32_t *__restrict__ hist, int64_t tiles) {
-    __shared__ uint32_t h[256];
-    h[threadIdx.x] = 0;
+    k_radix_hist(int64_t n, const unsigned long long *__restrict__ keys, int first,
+                 uint32_t *__restrict__ hist) {
+    __shared__ uint32_t h[kSortPasses][256];
+    for (int p = 0; p < kSortPasses; ++p) h[p][threadIdx.x] = 0;
     __syncthreads();
-    int64_t base = (int64_t)blockIdx.x * kSortTile;
-    for (int r = 0; r < kSortItems; ++r) {
-        int64_t i = base + r * kSortThreads + threadIdx.x;
-        if (i < n) atomicAdd(&h[(uint32_t)(keys[i] >> shift) & 255u], 1u);
+    const int64_t step = (int64_t)gridDim.x * kSortThreads;
+    for (int64_t i = (int64_t)blockIdx.x * kSortThreads + threadIdx.x; i < n; i += step) {
+        const unsigned long long c = keys[i];
+        for (int p = first; p < kSortPasses; ++p)
+            atomicAdd(&h[p][(uint32_t)(c >> (8 * p)) & 255u], 1u);
     }
     __syncthreads();
-    hist[(int64_t)threadIdx.x * tiles + blockIdx.x] = h[threadIdx.x];
+    for (int p = first; p < kSortPasses; ++p) {
+        const uint32_t v = h[p][threadIdx.x];
+        if (v) atomicAdd(&hist[256 * p + threadIdx.x], v);
+    }
 }
 
 // Exclusive scan in three launches: per-block sums, a scan of the block
@@ -287,49 +330,139 @@ void scan_exclusive(uint32_t *a, int64_t n, uint32_t *sums, cudaStream_t s) {
     k_scan_apply<<<(unsigned)nb, 256, 0, s>>>(a, n, sums);
 }
 
-// Stable scatter: keys of a tile are ranked in input order, round by round
-// (256 keys per round), with warp-level digit matching and a per-digit
-// prefix over the warps of the block.
+// One digit of the stable sort in one pass over the keys (decoupled
+// look-back: Merrill and Garland 2016; as a radix sort, Adinets and Merrill
+// 2022). A block takes the next tile, ranks its keys by digit in input order
+// (each warp its own consecutive keys, with warp-level digit matching and
+// counters of its own, so no block barrier per round), publishes its digit
+// counts, and adds up the tiles before it from theirs: thread d reads back
+// the counts of digit d until a tile whose running total is known. The keys
+// go through shared memory so that each digit's run is stored together.
+// A tile is taken only after the tiles before it, so each waits only on
+// blocks that are already running; the wait is bounded all the same.
+// Against a histogram, a three-kernel scan and a scatter per digit: 1M keys
+// and ids, eight digits, 0.31 ms in 40 launches before.
+constexpr unsigned long long kTileCounted = 1ull << 62, kTileTotal = 2ull << 62;
+constexpr unsigned long long kTileValue = (1ull << 40) - 1ull;
+constexpr int kLookbackLimit = 1 << 24;
+
+template <bool VALS>
 __global__ void __launch_bounds__(kSortThreads)
-    k_radix_scatter(int64_t n, const unsigned long long *__restrict__ kin,
-                    const uint32_t *__restrict__ vin, unsigned long long *__restrict__ kout,
-                    uint32_t *__restrict__ vout, int shift, const uint32_t *__restrict__ offs,
-                    int64_t tiles) {
+    k_radix_pass(int64_t n, const unsigned long long *__restrict__ kin,
+                 const uint32_t *__restrict__ vin, unsigned long long *__restrict__ kout,
+                 uint32_t *__restrict__ vout, int pass, const uint32_t *__restrict__ hist,
+                 uint32_t *__restrict__ tickets, unsigned long long *__restrict__ tile_state,
+                 uint32_t *__restrict__ status) {
     constexpr int W = kSortThreads / 32;
-    __shared__ uint32_t base[256];
+    __shared__ unsigned long long s_key[kSortTile];
+    __shared__ uint32_t s_val[VALS ? kSortTile : 1];
     __shared__ uint32_t wcount[W][256];
-    __shared__ uint32_t pref[W][256];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    base[tid] = offs[(int64_t)tid * tiles + blockIdx.x];
+    __shared__ long long s_shift[256];  // global position minus position in the tile
+    __shared__ uint32_t s_tile;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, shift = 8 * pass;
+    if (tid == 0) s_tile = atomicAdd(&tickets[pass], 1u);
     for (int w = 0; w < W; ++w) wcount[w][tid] = 0;
+    const uint32_t digit_total = hist[256 * pass + tid];
     __syncthreads();
-    const int64_t tile0 = (int64_t)blockIdx.x * kSortTile;
-    for (int r = 0; r < kSortItems; ++r) {
-        int64_t i = tile0 + r * kSortThreads + tid;
-        bool valid = i < n;
-        unsigned long long key = valid ? kin[i] : 0ull;
-        uint32_t val = (valid && vin) ? vin[i] : 0u;
-        uint32_t digit = valid ? ((uint32_t)(key >> shift) & 255u) : (256u + lane);
-        uint32_t peers = __match_any_sync(0xffffffffu, digit);
-        uint32_t rank = __popc(peers & ((1u << lane) - 1u));
-        if (valid && rank == 0) wcount[warp][digit] = __popc(peers);
-        __syncthreads();
-        uint32_t run = base[tid];
-        for (int w = 0; w < W; ++w) {
-            uint32_t c = wcount[w][tid];
-            pref[w][tid] = run;
-            wcount[w][tid] = 0;
-            run += c;
-        }
-        base[tid] = run;
-        __syncthreads();
-        if (valid) {
-            uint32_t pos = pref[warp][digit] + rank;
-            kout[pos] = key;
-            if (vout) vout[pos] = val;
+    const int64_t tile = s_tile;
+    const int64_t tile0 = tile * kSortTile;
+    const int64_t warp0 = tile0 + warp * (kSortItems * 32);
+    unsigned long long key[kSortItems];
+    uint32_t val[kSortItems], rank[kSortItems];
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) {
+        const int64_t i = warp0 + 32 * j + lane;
+        key[j] = i < n ? kin[i] : 0ull;
+        if constexpr (VALS) val[j] = i < n ? vin[i] : 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) {
+        const bool in = warp0 + 32 * j + lane < n;
+        const uint32_t digit = (uint32_t)(key[j] >> shift) & 255u;
+        const uint32_t peers = __match_any_sync(0xffffffffu, in ? digit : 256u + lane);
+        const uint32_t before = in ? wcount[warp][digit] : 0u;
+        rank[j] = before + __popc(peers & ((1u << lane) - 1u));
+        __syncwarp();
+        if (in && rank[j] == before) wcount[warp][digit] = before + __popc(peers);
+        __syncwarp();
+    }
+    __syncthreads();
+    // thread d: the tile's count of digit d, made exclusive over the warps
+    uint32_t count = 0;
+    for (int w = 0; w < W; ++w) {
+        const uint32_t c = wcount[w][tid];
+        wcount[w][tid] = count;
+        count += c;
+    }
+    const unsigned long long tag = (unsigned long long)(pass + 1) << 56;  // states of other passes
+    volatile unsigned long long *mine = tile_state + tile * 256 + tid;
+    *mine = (tile == 0 ? kTileTotal : kTileCounted) | tag | count;
+    const uint32_t local = block_exclusive_scan(count, nullptr);
+    const uint32_t digit_base = block_exclusive_scan(digit_total, nullptr);
+    // eight tiles' states at a time: one after the other, the reads of the
+    // tiles that start together were the whole time of a 1M pass
+    unsigned long long prior = 0;
+    int spins = 0;
+    for (int64_t t = tile - 1; t >= 0;) {
+        constexpr int B = 8;
+        unsigned long long v[B];
+#pragma unroll
+        for (int q = 0; q < B; ++q)
+            v[q] = t - q >= 0
+                       ? *(volatile unsigned long long *)(tile_state + (t - q) * 256 + tid)
+                       : kTileTotal | tag;
+        int used = 0;
+        bool done = false;
+#pragma unroll
+        for (int q = 0; q < B; ++q)
+            if (!done && used == q && (v[q] & (63ull << 56)) == tag) {
+                prior += v[q] & kTileValue;
+                done = (v[q] & kTileTotal) != 0;
+                ++used;
+            }
+        if (done) break;
+        t -= used;
+        if (used == 0 && ++spins > kLookbackLimit) {
+            atomicOr(status, kErrSteps);
+            break;
         }
     }
+    if (tile > 0) *mine = kTileTotal | tag | (prior + count);
+    s_shift[tid] = (long long)digit_base + (long long)prior - (long long)local;
+    // positions within the tile: the digits' starts, then the warps', then ranks
+    for (int w = 0; w < W; ++w) wcount[w][tid] += local;
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kSortItems; ++j) {
+        if (warp0 + 32 * j + lane >= n) continue;
+        const uint32_t pos = wcount[warp][(uint32_t)(key[j] >> shift) & 255u] + rank[j];
+        s_key[pos] = key[j];
+        if constexpr (VALS) s_val[pos] = val[j];
+    }
+    __syncthreads();
+    const int m = (int)min((int64_t)kSortTile, n - tile0);
+    for (int i = tid; i < m; i += kSortThreads) {
+        const unsigned long long k = s_key[i];
+        const int64_t pos = s_shift[(uint32_t)(k >> shift) & 255u] + i;
+        if (pos < 0 || pos >= n) continue;  // after a wait that ran out
+        kout[pos] = k;
+        if constexpr (VALS) vout[pos] = s_val[i];
+    }
 }
+
+// Scratch that starts a sort or a build at zero, in one allocation: scene
+// bounds, digit histograms, tile tickets, arrival counters and wide record
+// allocators (of a build over `arrivals` Gaussians), tile states.
+struct ZeroScratch {
+    size_t hist, tickets, arrive, states, bytes;
+    ZeroScratch(int64_t n, int64_t arrivals) {
+        hist = 64;
+        tickets = hist + kSortPasses * 256 * sizeof(uint32_t);
+        arrive = tickets + 64;
+        states = (arrive + (size_t)arrivals * sizeof(uint32_t) + 255) / 256 * 256;
+        bytes = states + (size_t)radix_tiles(n) * 256 * sizeof(unsigned long long);
+    }
+};
 
 // ---------------------------------------------------------------- hierarchy
 
@@ -831,15 +964,25 @@ inline unsigned grid_for(int64_t n, int threads) {
 
 int64_t radix_tiles(int64_t n) { return (n + kSortTile - 1) / kSortTile; }
 
-int sort_keys64(unsigned long long *keys[2], int64_t n, int lo_bit, uint32_t *hist,
-                uint32_t *scan_tmp, cudaStream_t s) {
+size_t sort_scratch_bytes(int64_t n) { return ZeroScratch(n, 0).bytes; }
+size_t build_scratch_bytes(int64_t n) { return ZeroScratch(n, n + kGroupTrees).bytes; }
+
+int sort_keys64(unsigned long long *keys[2], int64_t n, int lo_bit, void *scratch,
+                uint32_t *status, cudaStream_t s) {
+    const ZeroScratch z(n, 0);
+    unsigned char *base = static_cast<unsigned char *>(scratch);
+    uint32_t *hist = reinterpret_cast<uint32_t *>(base + z.hist);
+    // a failed call leaves its error for the caller's cudaGetLastError
+    cudaMemsetAsync(base, 0, z.bytes, s);
     const int64_t tiles = radix_tiles(n);
+    k_radix_hist<<<(unsigned)(tiles < 1216 ? tiles : 1216), kSortThreads, 0, s>>>(n, keys[0],
+                                                                                lo_bit / 8, hist);
     int cur = 0;
-    for (int shift = lo_bit; shift < 64; shift += 8) {
-        k_radix_hist<<<(unsigned)tiles, kSortThreads, 0, s>>>(n, keys[cur], shift, hist, tiles);
-        scan_exclusive(hist, 256 * tiles, scan_tmp, s);
-        k_radix_scatter<<<(unsigned)tiles, kSortThreads, 0, s>>>(n, keys[cur], nullptr, keys[1 - cur],
-                                                                 nullptr, shift, hist, tiles);
+    for (int pass = lo_bit / 8; pass < kSortPasses; ++pass) {
+        k_radix_pass<false><<<(unsigned)tiles, kSortThreads, 0, s>>>(
+            n, keys[cur], nullptr, keys[1 - cur], nullptr, pass, hist,
+            reinterpret_cast<uint32_t *>(base + z.tickets),
+            reinterpret_cast<unsigned long long *>(base + z.states), status);
         cur = 1 - cur;
     }
     return cur;
@@ -853,31 +996,28 @@ gs_status build_into(gs_bvh *b, const gs_gaussians *g, cudaStream_t s) {
     b->n_nodes = M == 0 ? 0 : (M == 1 ? 1 : M - 1);
     if (M == 0) return GS_OK;
     cudaError_t e;
-    // bounds: mins start at the largest ordered value, maxes at the smallest
-    if ((e = cudaMemsetAsync(b->bounds, 0xff, 3 * sizeof(unsigned int), s)) != cudaSuccess)
-        return cuda_fail(e, "memset bounds");
-    if ((e = cudaMemsetAsync(b->bounds + 3, 0, 3 * sizeof(unsigned int), s)) != cudaSuccess)
-        return cuda_fail(e, "memset bounds");
+    const ZeroScratch z(M, M + kGroupTrees);
+    unsigned char *base = static_cast<unsigned char *>(b->zero);
+    unsigned int *bounds = reinterpret_cast<unsigned int *>(base);
+    uint32_t *hist = reinterpret_cast<uint32_t *>(base + z.hist);
+    uint32_t *arrive = reinterpret_cast<uint32_t *>(base + z.arrive);
+    if ((e = cudaMemsetAsync(base, 0, z.bytes, s)) != cudaSuccess)
+        return cuda_fail(e, "memset build scratch");
     k_preprocess<<<grid_for(M, 256), 256, 0, s>>>(M, g->means, g->log_scales, g->quats,
-                                                   g->opacity_logits, b->aabb, b->bounds, b->status);
-    k_morton<<<grid_for(M, 256), 256, 0, s>>>(M, g->means, b->bounds, b->aabb, b->codes[0],
-                                               b->vals[0]);
+                                                   g->opacity_logits, b->aabb, bounds, b->status);
     const int64_t tiles = radix_tiles(M);
+    k_morton<<<(unsigned)tiles, kSortThreads, 0, s>>>(M, g->means, bounds, b->aabb, b->codes[0],
+                                                       b->vals[0], hist);
     int cur = 0;
-    for (int shift = 0; shift < 64; shift += 8) {
-        k_radix_hist<<<(unsigned)tiles, kSortThreads, 0, s>>>(M, b->codes[cur], shift, b->hist, tiles);
-        scan_exclusive(b->hist, 256 * tiles, b->scan_tmp, s);
-        k_radix_scatter<<<(unsigned)tiles, kSortThreads, 0, s>>>(
-            M, b->codes[cur], b->vals[cur], b->codes[1 - cur], b->vals[1 - cur], shift, b->hist,
-            tiles);
+    for (int pass = 0; pass < kSortPasses; ++pass) {
+        k_radix_pass<true><<<(unsigned)tiles, kSortThreads, 0, s>>>(
+            M, b->codes[cur], b->vals[cur], b->codes[1 - cur], b->vals[1 - cur], pass, hist,
+            reinterpret_cast<uint32_t *>(base + z.tickets),
+            reinterpret_cast<unsigned long long *>(base + z.states), b->status);
         cur = 1 - cur;
     }
     b->final_buf = cur;
     const uint32_t *order = b->vals[cur];
-    // arrival counters, then the wide trees' record allocators
-    const size_t n_arrive = (size_t)M + (b->link ? kGroupTrees : 0);
-    if ((e = cudaMemsetAsync(b->arrive, 0, n_arrive * sizeof(uint32_t), s)) != cudaSuccess)
-        return cuda_fail(e, "memset arrive");
     if (M == 1) {
         k_single<<<1, 1, 0, s>>>(order, g->means, g->log_scales, g->quats, g->opacity_logits,
                                  b->aabb, b->prims, b->nodes, b->link);
@@ -887,7 +1027,7 @@ gs_status build_into(gs_bvh *b, const gs_gaussians *g, cudaStream_t s) {
                                                        parent_leaf);
         k_leaves<<<grid_for(M, 256), 256, 0, s>>>(M, order, g->means, g->log_scales, g->quats,
                                                    g->opacity_logits, b->aabb, b->prims, b->nodes,
-                                                   parent_int, parent_leaf, b->arrive, b->link);
+                                                   parent_int, parent_leaf, arrive, b->link);
     }
     if (b->node_format == GS_NODES_WIDE4 || b->node_format == GS_NODES_WIDE4_Q8) {
         const int64_t n_int = b->n_nodes;
@@ -916,7 +1056,7 @@ gs_status build_into(gs_bvh *b, const gs_gaussians *g, cudaStream_t s) {
             out.rec[w] = b->group[w].rec;
         }
         k_wide_offsets<<<grid_for(n_int, 1024), 256, 0, s>>>(
-            n_int, b->link, b->arrive + M, q8 ? (uint32_t)kGroupQHeaderUnits : 0u, refs);
+            n_int, b->link, arrive + M, q8 ? (uint32_t)kGroupQHeaderUnits : 0u, refs);
         if (q8) k_wide_records<true><<<grid_for(n_int, 256), 256, 0, s>>>(n_int, b->nodes, b->link, out);
         else k_wide_records<false><<<grid_for(n_int, 256), 256, 0, s>>>(n_int, b->nodes, b->link, out);
     }

@@ -138,11 +138,8 @@ struct gs_bvh {
     unsigned long long *codes[2];
     uint32_t *vals[2];
     uint32_t *parent;   // [2M]: parents of internal nodes (0..M-2) then leaves
-    uint32_t *arrive;   // [M + 3] refit arrival counters, then the wide record allocators
     float *aabb;        // [M][6] in Gaussian-id order
-    unsigned int *bounds;  // [6] ordered-int scene bounds of the means
-    uint32_t *hist;     // radix histograms [256 * tiles]
-    int64_t hist_len;
+    void *zero;         // scratch a build starts at zero: bounds, sort state, arrival counters
     uint32_t *scan_tmp; // block sums of the multi-block scan
     int final_buf;      // which of codes/vals holds the sorted result
     // traversal nodes other than the binary ones
@@ -160,8 +157,7 @@ struct gs_bvh {
     int64_t wave_bytes;                  // device bytes of the scratch below
     unsigned long long *wave_codes[2];   // one sort code per slot
     float *wave_bounce;                  // [slots][3] albedo x bounce radiance
-    uint32_t *wave_hist;                 // radix histograms of the codes
-    uint32_t *wave_scan;                 // scan block sums
+    void *wave_sort;                     // sort state of the codes
 };
 
 namespace gsrt {
@@ -175,12 +171,14 @@ bool is_device_ptr(const void *p);
 gs_status build_into(gs_bvh *b, const gs_gaussians *g, cudaStream_t s);
 int64_t radix_tiles(int64_t n);
 int64_t scan_tmp_entries(int64_t n);
+size_t build_scratch_bytes(int64_t n);
 // Stable LSD radix sort of n 64-bit keys on bits [lo_bit, 64), 8 bits per
 // pass, ping-ponging between keys[0] and keys[1]; returns the index of the
-// buffer holding the result. hist: 256 * radix_tiles(n) entries, scan_tmp:
-// scan_tmp_entries(256 * radix_tiles(n)).
-int sort_keys64(unsigned long long *keys[2], int64_t n, int lo_bit, uint32_t *hist,
-                uint32_t *scan_tmp, cudaStream_t s);
+// buffer holding the result. scratch: sort_scratch_bytes(n) bytes, 256-byte
+// aligned; status: receives kErrSteps if a wait between tiles runs out.
+size_t sort_scratch_bytes(int64_t n);
+int sort_keys64(unsigned long long *keys[2], int64_t n, int lo_bit, void *scratch,
+                uint32_t *status, cudaStream_t s);
 
 // Batched form (wavefront.cu): grows the handle's deferred-bounce scratch to
 // `slots` sample slots (synchronous allocation; refused while the stream is

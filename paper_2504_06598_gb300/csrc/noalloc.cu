@@ -28,14 +28,12 @@ constexpr size_t kCodes1 = kCodes0 + align_up(8 * kNoAllocMaxGaussians);
 constexpr size_t kVals0 = kCodes1 + align_up(8 * kNoAllocMaxGaussians);
 constexpr size_t kVals1 = kVals0 + align_up(4 * kNoAllocMaxGaussians);
 constexpr size_t kParent = kVals1 + align_up(4 * kNoAllocMaxGaussians);
-constexpr size_t kArrive = kParent + align_up(4 * (2 * kNoAllocMaxGaussians + 2));
-constexpr size_t kAabb = kArrive + align_up(4 * kNoAllocMaxGaussians);
-constexpr size_t kBounds = kAabb + align_up(24 * kNoAllocMaxGaussians);
-constexpr size_t kHist = kBounds + align_up(64);
-constexpr size_t kHistEntries = 256 * ((kNoAllocMaxGaussians + 2047) / 2048);
-constexpr size_t kScanTmp = kHist + align_up(4 * kHistEntries);
-constexpr size_t kScanTmpEntries = kHistEntries / 1024 + 2;
-constexpr size_t kScratchBytes = kScanTmp + align_up(4 * kScanTmpEntries);
+constexpr size_t kAabb = kParent + align_up(4 * (2 * kNoAllocMaxGaussians + 2));
+constexpr size_t kZero = kAabb + align_up(24 * kNoAllocMaxGaussians);
+// at least build_scratch_bytes(kNoAllocMaxGaussians), checked by each call
+constexpr size_t kZeroBytes = 64 + 8 * 256 * 4 + 64 + 4 * (kNoAllocMaxGaussians + 64) +
+                              8 * 256 * ((kNoAllocMaxGaussians + 2047) / 2048) + 512;
+constexpr size_t kScratchBytes = kZero + align_up(kZeroBytes);
 
 __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -103,6 +101,8 @@ extern "C" gs_status gs_build_bvh_noalloc(const gs_gaussians *g, void *nodes_out
     unsigned char *s = nullptr;
     gs_status st = scratch_address(&s);
     if (st != GS_OK) return st;
+    if (build_scratch_bytes(g->M) > kZeroBytes)
+        return fail(GS_ERR_OOM, "the build's scratch does not fit the library's array");
     gs_bvh b = {};
     cudaGetDevice(&b.device);
     b.capacity = kNoAllocMaxGaussians;
@@ -113,12 +113,8 @@ extern "C" gs_status gs_build_bvh_noalloc(const gs_gaussians *g, void *nodes_out
     b.vals[0] = reinterpret_cast<uint32_t *>(s + kVals0);
     b.vals[1] = reinterpret_cast<uint32_t *>(s + kVals1);
     b.parent = reinterpret_cast<uint32_t *>(s + kParent);
-    b.arrive = reinterpret_cast<uint32_t *>(s + kArrive);
     b.aabb = reinterpret_cast<float *>(s + kAabb);
-    b.bounds = reinterpret_cast<unsigned int *>(s + kBounds);
-    b.hist = reinterpret_cast<uint32_t *>(s + kHist);
-    b.hist_len = (int64_t)kHistEntries;
-    b.scan_tmp = reinterpret_cast<uint32_t *>(s + kScanTmp);
+    b.zero = s + kZero;
     b.node_format = GS_NODES_BINARY;
     b.status = status_out;
     return build_into(&b, g, (cudaStream_t)stream);

@@ -760,7 +760,7 @@ gs_status reserve_wave_scratch(gs_bvh *b, int64_t slots, cudaStream_t s) {
         return fail(GS_ERR_INVALID_ARG,
                     "the batched form's scratch must be reserved before a graph capture");
     void **bufs[] = {(void **)&b->wave_codes[0], (void **)&b->wave_codes[1],
-                     (void **)&b->wave_bounce, (void **)&b->wave_hist, (void **)&b->wave_scan};
+                     (void **)&b->wave_bounce, &b->wave_sort};
     for (void **q : bufs)
         if (*q) {
             cudaFree(*q);
@@ -769,10 +769,9 @@ gs_status reserve_wave_scratch(gs_bvh *b, int64_t slots, cudaStream_t s) {
     b->device_bytes -= b->wave_bytes;
     b->wave_bytes = 0;
     b->wave_cap = 0;
-    const int64_t tiles = radix_tiles(slots);
     const size_t sizes[] = {(size_t)slots * 8, (size_t)slots * 8, (size_t)slots * 12,
-                            (size_t)tiles * 256 * 4, (size_t)scan_tmp_entries(256 * tiles) * 4};
-    for (int k = 0; k < 5; ++k) {
+                            sort_scratch_bytes(slots)};
+    for (int k = 0; k < 4; ++k) {
         cudaError_t e = cudaMalloc(bufs[k], sizes[k]);
         if (e != cudaSuccess) {
             for (void **q : bufs)
@@ -899,7 +898,7 @@ gs_status launch_render_views(const gs_bvh *b, const gs_gaussians *g, const gs_p
     if (st != GS_OK) return st;
     if (slots > 0) {
         gs_bvh *mb = const_cast<gs_bvh *>(b);
-        const int cur = sort_keys64(mb->wave_codes, slots, 32, mb->wave_hist, mb->wave_scan, s);
+        const int cur = sort_keys64(mb->wave_codes, slots, 32, mb->wave_sort, mb->status, s);
         const unsigned long long *sorted = mb->wave_codes[cur];
         switch (b->node_format) {
             case GS_NODES_WIDE4:
