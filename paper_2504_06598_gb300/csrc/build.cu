@@ -100,31 +100,37 @@ __device__ __forceinline__ void ellipsoid_box(const Activated &a, float box[6]) 
     }
 }
 
+// Box of Gaussian g into aabb; a finite mean widens lo and hi.
+__device__ __forceinline__ void gaussian_box(int64_t g, const float *means, const float *log_scales,
+                                             const float *quats, const float *logits,
+                                             float *__restrict__ aabb, uint32_t *status,
+                                             float lo[3], float hi[3]) {
+    const Activated a = activate(means, log_scales, quats, logits, g);
+    float box[6];
+    if (a.finite) {
+        ellipsoid_box(a, box);
+        for (int k = 0; k < 3; ++k) {
+            lo[k] = fminf(lo[k], a.mu[k]);
+            hi[k] = fmaxf(hi[k], a.mu[k]);
+        }
+    } else {
+        // A non-finite Gaussian gets an empty box: it is never hit.
+        for (int k = 0; k < 3; ++k) {
+            box[k] = NAN;
+            box[3 + k] = NAN;
+        }
+        atomicOr(status, kErrNonfinite);
+    }
+    for (int k = 0; k < 6; ++k) aabb[6 * g + k] = box[k];
+}
+
 __global__ void __launch_bounds__(256) k_preprocess(int64_t M, const float *__restrict__ means,
                              const float *__restrict__ log_scales, const float *__restrict__ quats,
                              const float *__restrict__ logits, float *__restrict__ aabb,
                              unsigned int *__restrict__ bounds, uint32_t *__restrict__ status) {
     int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
-    if (g < M) {
-        Activated a = activate(means, log_scales, quats, logits, g);
-        float box[6];
-        if (a.finite) {
-            ellipsoid_box(a, box);
-            for (int k = 0; k < 3; ++k) {
-                lo[k] = a.mu[k];
-                hi[k] = a.mu[k];
-            }
-        } else {
-            // A non-finite Gaussian gets an empty box: it is never hit.
-            for (int k = 0; k < 3; ++k) {
-                box[k] = NAN;
-                box[3 + k] = NAN;
-            }
-            atomicOr(status, kErrNonfinite);
-        }
-        for (int k = 0; k < 6; ++k) aabb[6 * g + k] = box[k];
-    }
+    if (g < M) gaussian_box(g, means, log_scales, quats, logits, aabb, status, lo, hi);
     // reduction of the finite means over the block, then six atomics: one per
     // warp made the kernel wait on its six addresses (1M: 131 us)
     __shared__ float s_lo[3][8], s_hi[3][8];
@@ -174,9 +180,9 @@ __device__ __forceinline__ unsigned long long spread3(unsigned long long v) {
 constexpr int kKeyTopBits = 6;
 constexpr int kKeySizeBits = 4;
 
-__device__ __forceinline__ unsigned long long sort_code(int64_t g, const float *__restrict__ means,
-                                                        const unsigned int *__restrict__ bounds,
-                                                        const float *__restrict__ aabb) {
+__device__ __forceinline__ unsigned long long sort_code(int64_t g, const float *means,
+                                                        const unsigned int *bounds,
+                                                        const float *aabb) {
     unsigned long long q[3];
     float scene = 0.0f, edge = 0.0f;
     for (int k = 0; k < 3; ++k) {
@@ -468,7 +474,7 @@ struct ZeroScratch {
 
 // Common-prefix length of sorted keys i and j, extended by the index bits
 // when the codes are equal; -1 outside [0, n).
-__device__ __forceinline__ int delta(const unsigned long long *__restrict__ codes, int64_t n,
+__device__ __forceinline__ int delta(const unsigned long long *codes, int64_t n,
                                      int64_t i, int64_t j) {
     if (j < 0 || j >= n) return -1;
     unsigned long long a = codes[i], b = codes[j];
@@ -476,11 +482,11 @@ __device__ __forceinline__ int delta(const unsigned long long *__restrict__ code
     return __clzll(a ^ b);
 }
 
-__global__ void k_karras(int64_t n, const unsigned long long *__restrict__ codes,
-                         Node *__restrict__ nodes, uint32_t *__restrict__ parent_int,
-                         uint32_t *__restrict__ parent_leaf) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n - 1) return;
+// Internal node i of the binary radix tree over n sorted codes.
+__device__ __forceinline__ void karras_node(int64_t i, int64_t n, const unsigned long long *codes,
+                                            Node *__restrict__ nodes,
+                                            uint32_t *__restrict__ parent_int,
+                                            uint32_t *__restrict__ parent_leaf) {
     int d = (delta(codes, n, i, i + 1) - delta(codes, n, i, i - 1)) >= 0 ? 1 : -1;
     int dmin = delta(codes, n, i, i - d);
     int64_t lmax = 2;
@@ -507,6 +513,111 @@ __global__ void k_karras(int64_t n, const unsigned long long *__restrict__ codes
     nd.leaf_range[1] = (uint32_t)hi;
     if (left & kLeafBit) parent_leaf[gamma] = (uint32_t)i; else parent_int[gamma] = (uint32_t)i;
     if (right & kLeafBit) parent_leaf[gamma + 1] = (uint32_t)i; else parent_int[gamma + 1] = (uint32_t)i;
+}
+
+__global__ void k_karras(int64_t n, const unsigned long long *__restrict__ codes,
+                         Node *__restrict__ nodes, uint32_t *__restrict__ parent_int,
+                         uint32_t *__restrict__ parent_leaf) {
+    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n - 1) karras_node(i, n, codes, nodes, parent_int, parent_leaf);
+}
+
+// Up to kSmallMax Gaussians: boxes, bounds, codes, the sort and the tree in
+// one launch of one block, everything between them in its shared memory. The
+// eleven launches it stands for cost more than their work: 1,000 Gaussians
+// rebuilt and traced at 64x64. Each digit is ranked as in
+// k_radix_pass, the keys moving within shared memory.
+constexpr int kSmallThreads = 1024, kSmallItems = 8;
+constexpr int kSmallMax = kSmallThreads * kSmallItems;
+constexpr size_t kSmallBytes = (size_t)kSmallMax * 12 + (size_t)(kSmallThreads / 32) * 256 * 4;
+
+__global__ void __launch_bounds__(kSmallThreads, 1)
+    k_small(int n, const float *__restrict__ means, const float *__restrict__ log_scales,
+            const float *__restrict__ quats, const float *__restrict__ logits,
+            float *__restrict__ aabb, unsigned long long *__restrict__ codes,
+            uint32_t *__restrict__ vals, Node *__restrict__ nodes,
+            uint32_t *__restrict__ parent_int, uint32_t *__restrict__ parent_leaf,
+            uint32_t *__restrict__ arrive, int n_arrive, uint32_t *__restrict__ status) {
+    constexpr int W = kSmallThreads / 32;
+    extern __shared__ unsigned long long small_smem[];
+    unsigned long long *s_key = small_smem;
+    uint32_t *s_val = reinterpret_cast<uint32_t *>(s_key + kSmallMax);
+    uint32_t(*wcount)[256] = reinterpret_cast<uint32_t(*)[256]>(s_val + kSmallMax);
+    __shared__ unsigned int s_bounds[6];
+    __shared__ uint32_t s_base[256];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid < 6) s_bounds[tid] = 0;
+    for (int i = tid; i < n_arrive; i += kSmallThreads) arrive[i] = 0;
+    __syncthreads();
+    {
+        float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+        for (int g = tid; g < n; g += kSmallThreads) gaussian_box(g, means, log_scales, quats, logits, aabb, status, lo, hi);
+        for (int k = 0; k < 3; ++k) {
+            for (int off = 16; off > 0; off >>= 1) {
+                lo[k] = fminf(lo[k], __shfl_xor_sync(0xffffffffu, lo[k], off));
+                hi[k] = fmaxf(hi[k], __shfl_xor_sync(0xffffffffu, hi[k], off));
+            }
+            if (lane == 0 && lo[k] <= hi[k]) {
+                atomicMax(&s_bounds[k], ~f2ord(lo[k]));
+                atomicMax(&s_bounds[3 + k], f2ord(hi[k]));
+            }
+        }
+    }
+    __syncthreads();
+    for (int g = tid; g < n; g += kSmallThreads) {
+        s_key[g] = sort_code(g, means, s_bounds, aabb);
+        s_val[g] = (uint32_t)g;
+    }
+    const int J = (n + kSmallThreads - 1) / kSmallThreads;  // keys per thread
+    const int first = warp * J * 32 + lane;
+    for (int shift = 0; shift < 64; shift += 8) {
+        for (int i = tid; i < W * 256; i += kSmallThreads) (&wcount[0][0])[i] = 0;
+        __syncthreads();
+        unsigned long long key[kSmallItems];
+        uint32_t val[kSmallItems], rank[kSmallItems];
+#pragma unroll
+        for (int j = 0; j < kSmallItems; ++j) {
+            if (j >= J) break;
+            const int i = first + 32 * j;
+            const bool in = i < n;
+            key[j] = in ? s_key[i] : 0ull;
+            val[j] = in ? s_val[i] : 0u;
+            const uint32_t digit = (uint32_t)(key[j] >> shift) & 255u;
+            const uint32_t peers = __match_any_sync(0xffffffffu, in ? digit : 256u + lane);
+            const uint32_t before = in ? wcount[warp][digit] : 0u;
+            rank[j] = before + __popc(peers & ((1u << lane) - 1u));
+            __syncwarp();
+            if (in && rank[j] == before) wcount[warp][digit] = before + __popc(peers);
+            __syncwarp();
+        }
+        __syncthreads();
+        uint32_t count = 0;
+        if (tid < 256)
+            for (int w = 0; w < W; ++w) {
+                const uint32_t c = wcount[w][tid];
+                wcount[w][tid] = count;
+                count += c;
+            }
+        const uint32_t base = block_exclusive_scan(count, nullptr);
+        if (tid < 256) s_base[tid] = base;
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < kSmallItems; ++j) {
+            if (j >= J) break;
+            if (first + 32 * j < n) {
+                const uint32_t digit = (uint32_t)(key[j] >> shift) & 255u;
+                const uint32_t pos = s_base[digit] + wcount[warp][digit] + rank[j];
+                s_key[pos] = key[j];
+                s_val[pos] = val[j];
+            }
+        }
+        __syncthreads();
+    }
+    for (int i = tid; i < n; i += kSmallThreads) {
+        codes[i] = s_key[i];
+        vals[i] = s_val[i];
+        if (i < n - 1) karras_node(i, n, s_key, nodes, parent_int, parent_leaf);
+    }
 }
 
 __device__ __forceinline__ void write_record(PrimRec *__restrict__ prims, int64_t i, uint32_t g,
@@ -1001,20 +1112,31 @@ gs_status build_into(gs_bvh *b, const gs_gaussians *g, cudaStream_t s) {
     unsigned int *bounds = reinterpret_cast<unsigned int *>(base);
     uint32_t *hist = reinterpret_cast<uint32_t *>(base + z.hist);
     uint32_t *arrive = reinterpret_cast<uint32_t *>(base + z.arrive);
-    if ((e = cudaMemsetAsync(base, 0, z.bytes, s)) != cudaSuccess)
-        return cuda_fail(e, "memset build scratch");
-    k_preprocess<<<grid_for(M, 256), 256, 0, s>>>(M, g->means, g->log_scales, g->quats,
-                                                   g->opacity_logits, b->aabb, bounds, b->status);
-    const int64_t tiles = radix_tiles(M);
-    k_morton<<<(unsigned)tiles, kSortThreads, 0, s>>>(M, g->means, bounds, b->aabb, b->codes[0],
-                                                       b->vals[0], hist);
+    uint32_t *parent_int = b->parent, *parent_leaf = b->parent + M;
     int cur = 0;
-    for (int pass = 0; pass < kSortPasses; ++pass) {
-        k_radix_pass<true><<<(unsigned)tiles, kSortThreads, 0, s>>>(
-            M, b->codes[cur], b->vals[cur], b->codes[1 - cur], b->vals[1 - cur], pass, hist,
-            reinterpret_cast<uint32_t *>(base + z.tickets),
-            reinterpret_cast<unsigned long long *>(base + z.states), b->status);
-        cur = 1 - cur;
+    const bool small = M > 1 && M <= kSmallMax;
+    if (small) {
+        if ((e = cudaFuncSetAttribute(k_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)kSmallBytes)) != cudaSuccess)
+            return cuda_fail(e, "small build setup");
+        k_small<<<1, kSmallThreads, kSmallBytes, s>>>(
+            (int)M, g->means, g->log_scales, g->quats, g->opacity_logits, b->aabb, b->codes[0],
+            b->vals[0], b->nodes, parent_int, parent_leaf, arrive, (int)M + kGroupTrees, b->status);
+    } else {
+        if ((e = cudaMemsetAsync(base, 0, z.bytes, s)) != cudaSuccess)
+            return cuda_fail(e, "memset build scratch");
+        k_preprocess<<<grid_for(M, 256), 256, 0, s>>>(M, g->means, g->log_scales, g->quats,
+                                                       g->opacity_logits, b->aabb, bounds, b->status);
+        const int64_t tiles = radix_tiles(M);
+        k_morton<<<(unsigned)tiles, kSortThreads, 0, s>>>(M, g->means, bounds, b->aabb, b->codes[0],
+                                                           b->vals[0], hist);
+        for (int pass = 0; pass < kSortPasses; ++pass) {
+            k_radix_pass<true><<<(unsigned)tiles, kSortThreads, 0, s>>>(
+                M, b->codes[cur], b->vals[cur], b->codes[1 - cur], b->vals[1 - cur], pass, hist,
+                reinterpret_cast<uint32_t *>(base + z.tickets),
+                reinterpret_cast<unsigned long long *>(base + z.states), b->status);
+            cur = 1 - cur;
+        }
     }
     b->final_buf = cur;
     const uint32_t *order = b->vals[cur];
@@ -1022,9 +1144,9 @@ gs_status build_into(gs_bvh *b, const gs_gaussians *g, cudaStream_t s) {
         k_single<<<1, 1, 0, s>>>(order, g->means, g->log_scales, g->quats, g->opacity_logits,
                                  b->aabb, b->prims, b->nodes, b->link);
     } else {
-        uint32_t *parent_int = b->parent, *parent_leaf = b->parent + M;
-        k_karras<<<grid_for(M - 1, 256), 256, 0, s>>>(M, b->codes[cur], b->nodes, parent_int,
-                                                       parent_leaf);
+        if (!small)
+            k_karras<<<grid_for(M - 1, 256), 256, 0, s>>>(M, b->codes[cur], b->nodes, parent_int,
+                                                           parent_leaf);
         k_leaves<<<grid_for(M, 256), 256, 0, s>>>(M, order, g->means, g->log_scales, g->quats,
                                                    g->opacity_logits, b->aabb, b->prims, b->nodes,
                                                    parent_int, parent_leaf, arrive, b->link);
