@@ -454,11 +454,15 @@ __device__ __forceinline__ void bounce_finish(const WaveArgs &w, const Ray<1> &b
 }
 
 // One step of traverse_lane's walk of the binary nodes, its state (node,
-// stack depth, steps) held by the caller: false once the walk has ended.
+// stack depth, steps) held by the caller: false once the walk has no node
+// left. Leaves the ray reaches are handed to the caller (their records, the
+// farther one first), at most two a step, instead of being evaluated here.
 template <bool COUNT>
-__device__ __forceinline__ bool lane_step(const TraceArgs &a, Ray<1> &r, int pass, uint32_t &node,
+__device__ __forceinline__ bool lane_step(const TraceArgs &a, const Ray<1> &r, uint32_t &node,
                                           int &sp, uint32_t &steps, uint32_t *stack,
-                                          float *stack_t, uint32_t &err, Counts &cnt) {
+                                          float *stack_t, uint32_t leaves[2], int &n_leaves,
+                                          uint32_t &err, Counts &cnt) {
+    n_leaves = 0;
     if (++steps > a.step_limit) {
         err |= kErrSteps;
         return false;
@@ -476,26 +480,24 @@ __device__ __forceinline__ bool lane_step(const TraceArgs &a, Ray<1> &r, int pas
     bool hL = slab(boxL, r.inv, r.oinv, r.t_min, r.t_far, tL);
     bool hR = slab(boxR, r.inv, r.oinv, r.t_min, r.t_far, tR);
     const bool leafL = (cref.x & kLeafBit) != 0u, leafR = (cref.y & kLeafBit) != 0u;
-    if ((leafL && hL) || (leafR && hR)) {
-        const bool swap = leafL && leafR && hR && (!hL || tR < tL);
-        for (int li = 0; li < 2; ++li) {
-            const bool right = (li == 0) == swap;
-            if (!(right ? leafR : leafL) || !(right ? hR : hL)) continue;
-            if (COUNT) {
-                ++cnt.prims;
-                ++cnt.prim_fetch;
-            }
-            intersect<1, COUNT>(a, r, (right ? cref.y : cref.x) & ~kLeafBit, pass, cnt.draws);
+    const bool left_first = tL <= tR;
+    {
+        const bool l = leafL && hL, q = leafR && hR;
+        n_leaves = (int)l + (int)q;
+        leaves[0] = l && (!q || !left_first) ? cref.x : cref.y;
+        leaves[1] = left_first ? cref.x : cref.y;
+        if (COUNT) {
+            cnt.prims += n_leaves;
+            cnt.prim_fetch += n_leaves;
         }
     }
-    hL = hL && !leafL && tL <= r.t_far;
-    hR = hR && !leafR && tR <= r.t_far;
+    hL = hL && !leafL;
+    hR = hR && !leafR;
     if (hL && hR) {
         if (sp >= a.stack_depth) {
             err |= kErrStack;
             return false;
         }
-        const bool left_first = tL <= tR;
         stack[sp] = left_first ? cref.y : cref.x;
         stack_t[sp] = left_first ? tR : tL;
         ++sp;
@@ -527,10 +529,19 @@ __device__ __forceinline__ bool lane_step(const TraceArgs &a, Ray<1> &r, int pas
 // lane whose ray has ended takes the next code from the queue at once
 // (lanes that need one share an atomic): a warp's lanes stay busy instead
 // of waiting for its longest walk (the persistent traversal with ray
-// replacement of Aila and Laine, HPG 2009). Each lane shades its ray when
-// the walk ends and writes albedo x radiance to the sample's slot. On
+// replacement of Aila and Laine, HPG 2009). A leaf reached is not evaluated
+// at once: about one lane in six reaches one per step, and the warp would run
+// Alg. 1 (two to three times a node step's instructions) for those few. A
+// lane keeps up to kPending of them and walks on while there is room; the
+// warp evaluates one per lane when kEvalLanes lanes hold some, or when no lane
+// can walk on. A clip that moves later than it could only costs node steps:
+// the order of candidates does not change a sample's hit. Each lane shades
+// its ray when the walk ends and writes albedo x radiance to the sample's slot. On
 // 4-wide nodes a warp takes 32 consecutive codes and walks them as a
 // packet.
+constexpr int kPending = 4;
+constexpr int kEvalLanes = 20;
+
 template <int FMT, int STACK, bool COUNT>
 __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
     k_bounce(const WaveArgs w, const unsigned long long *__restrict__ codes, int64_t n_slots) {
@@ -544,12 +555,15 @@ __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
     if constexpr (FMT == GS_NODES_BINARY || FMT == GS_NODES_BINARY_Q8) {
         // the work counter counts codes; the launcher keeps n_slots + the
         // launch's threads below 2^32
-        bool active = false, more = true;
+        bool active = false, walking = false, more = true;
         int64_t gpix = 0;
         int s = 0;
         Ray<1> br;
         uint32_t node = 0, steps = 0;
-        int sp = 0;
+        int sp = 0, np = 0;
+        uint32_t pend[kPending];
+#pragma unroll
+        for (int k = 0; k < kPending; ++k) pend[k] = 0;
         for (;;) {
             const uint32_t idle = __ballot_sync(kAll, !active && more);
             if (idle) {
@@ -567,13 +581,36 @@ __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
                         node = 0;
                         sp = 0;
                         steps = 0;
-                        active = a.n_nodes > 0 && br.t_far >= br.t_min;
+                        np = 0;
+                        walking = active = a.n_nodes > 0 && br.t_far >= br.t_min;
                         if (!active) bounce_finish(w, br, gpix, s);
                     }
                 }
             }
             if (!__any_sync(kAll, active) && !__any_sync(kAll, more)) break;
-            if (active && !lane_step<COUNT>(a, br, s, node, sp, steps, stack, stack_t, err, cnt)) {
+            const bool room = walking && np <= kPending - 2;
+            const uint32_t holding = __ballot_sync(kAll, np > 0);
+            if (__popc(holding) >= kEvalLanes || !__any_sync(kAll, room)) {
+                if (np > 0) {
+                    uint32_t leaf = pend[0];
+#pragma unroll
+                    for (int k = 1; k < kPending; ++k)
+                        if (k == np - 1) leaf = pend[k];
+                    --np;
+                    intersect<1, COUNT>(a, br, leaf & ~kLeafBit, s, cnt.draws);
+                }
+            } else if (room) {
+                uint32_t leaves[2];
+                int nl;
+                walking = lane_step<COUNT>(a, br, node, sp, steps, stack, stack_t, leaves, nl, err, cnt);
+#pragma unroll
+                for (int k = 0; k < kPending; ++k) {
+                    if (nl > 0 && k == np) pend[k] = leaves[0];
+                    if (nl > 1 && k == np + 1) pend[k] = leaves[1];
+                }
+                np += nl;
+            }
+            if (active && !walking && np == 0) {
                 active = false;
                 bounce_finish(w, br, gpix, s);
             }
