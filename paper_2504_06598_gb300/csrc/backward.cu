@@ -785,15 +785,12 @@ __global__ void __launch_bounds__(kThreads, N >= 8 ? 4 : 5)
             const bool live = valid && pass < a.spp;
             // unused slots (sample index past the pixel's count) at -inf:
             // nothing is in front of them and they never set the clip
-            auto reset = [&](Ray<N> &q) {
 #pragma unroll
-                for (int k = 0; k < N; ++k)
-                    q.slot[k] = pass * N + k < a.n_samples ? Slot{INFINITY, 0.0f, 0xffffffffu}
-                                                           : Slot{-INFINITY, 0.0f, 0xffffffffu};
-                update_clip(q, a.t_max);
-                if (!live) q.t_far = -INFINITY;
-            };
-            reset(r);
+            for (int k = 0; k < N; ++k)
+                r.slot[k] = pass * N + k < a.n_samples ? Slot{INFINITY, 0.0f, 0xffffffffu}
+                                                       : Slot{-INFINITY, 0.0f, 0xffffffffu};
+            update_clip(r, a.t_max);
+            if (!live) r.t_far = -INFINITY;
             // 1) the winners: the rendering's stored payloads, or the forward
             // traversal again with the same keys (same winners)
             if constexpr (KEYS) {
@@ -812,16 +809,7 @@ __global__ void __launch_bounds__(kThreads, N >= 8 ? 4 : 5)
                     }
                 }
             } else {
-                if (!traverse_tile<N, Q8>(a, r, pass, a.eye, pyr, s_ref[warp], s_t[warp], err)) {
-                    Ray<N> again = r;
-                    set_ray(again, a.eye, r.d);
-                    reset(again);
-                    uint32_t err2 = 0;
-                    tile_fallback<N>(a, again, pass, err2);
-                    err |= err2;
-#pragma unroll
-                    for (int k = 0; k < N; ++k) r.slot[k] = again.slot[k];
-                }
+                trace_tile<N, Q8>(a, r, pass, a.eye, pyr, s_ref[warp], s_t[warp], err);
             }
             // 2) colours of the winners; dLoss/dk of the selected Gaussians,
             // once for the slots of a lane that hold the same one

@@ -124,28 +124,15 @@ __global__ void __launch_bounds__(kThreads, is_group_fmt(FMT) ? group_min_blocks
             const int s0 = pass * N;
             // an unused slot (sample index beyond the pixel's count) sits
             // at -inf: no candidate is closer, and it never sets the clip
-            auto reset = [&](Ray<N> &q) {
 #pragma unroll
-                for (int k = 0; k < N; ++k)
-                    q.slot[k] = s0 + k < a.n_samples ? Slot{INFINITY, 0.0f, 0xffffffffu}
-                                                     : Slot{-INFINITY, 0.0f, 0xffffffffu};
-                update_clip(q, a.t_max);
-                if (!live) q.t_far = -INFINITY;  // lanes off the image never hit
-            };
-            reset(r);
+            for (int k = 0; k < N; ++k)
+                r.slot[k] = s0 + k < a.n_samples ? Slot{INFINITY, 0.0f, 0xffffffffu}
+                                                 : Slot{-INFINITY, 0.0f, 0xffffffffu};
+            update_clip(r, a.t_max);
+            if (!live) r.t_far = -INFINITY;  // lanes off the image never hit
             if (a.n_nodes > 0) {
                 if constexpr (tiled) {
-                    if (!traverse_tile<N, FMT == kFmtTileQ8>(a, r, pass, a.eye, pyr, grp_ref, grp_t,
-                                                             err)) {
-                        Ray<N> again = r;
-                        set_ray(again, a.eye, r.d);
-                        reset(again);
-                        uint32_t err2 = 0;
-                        tile_fallback<N>(a, again, pass, err2);
-                        err |= err2;
-#pragma unroll
-                        for (int k = 0; k < N; ++k) r.slot[k] = again.slot[k];
-                    }
+                    trace_tile<N, FMT == kFmtTileQ8>(a, r, pass, a.eye, pyr, grp_ref, grp_t, err);
                 } else if constexpr (grouped)
                     traverse_group<N, COUNT, LG, true, is_group_q8(FMT)>(a, r, pass, grp_ref,
                                                                           grp_t, err, cnt);

@@ -1293,5 +1293,27 @@ __device__ __noinline__ void tile_fallback(const TraceArgs &a, Ray<N> &r, int pa
     traverse_packet<N, false>(a, r, pass, stack, stack_t, err, cnt);
 }
 
+// traverse_tile, started over on the binary nodes where its stack is full:
+// every slot but the unused ones (at -inf with no Gaussian) is emptied again.
+template <int N, bool Q8>
+__device__ __forceinline__ void trace_tile(const TraceArgs &a, Ray<N> &r, int pass,
+                                           const float apex[3], const float *pyr, uint32_t *s_ref,
+                                           float *s_t, uint32_t &err) {
+    if (traverse_tile<N, Q8>(a, r, pass, apex, pyr, s_ref, s_t, err)) return;
+    Ray<N> again = r;
+    set_ray(again, r.o, r.d);
+#pragma unroll
+    for (int k = 0; k < N; ++k)
+        if (!(r.slot[k].gid == 0xffffffffu && r.slot[k].tc == -INFINITY))
+            again.slot[k] = Slot{INFINITY, 0.0f, 0xffffffffu};
+    update_clip(again, r.t_max);
+    if (!(again.t_far > -INFINITY)) again.t_far = -INFINITY;
+    uint32_t err2 = 0;
+    tile_fallback<N>(a, again, pass, err2);
+    err |= err2;
+#pragma unroll
+    for (int k = 0; k < N; ++k) r.slot[k] = again.slot[k];
+}
+
 }  // namespace
 }  // namespace gsrt

@@ -144,12 +144,18 @@ __device__ __forceinline__ void trace_own_ray(const TraceArgs &a, Ray<1> &r, int
 
 // Camera and shadow rays are one ray for all lanes of a pixel: with groups
 // of 2^GLG >= 8 lanes they take the grouped traversal of the wide copy.
+// GLG = kTileWarp: a warp's rays of one apex take the tile traversal.
+constexpr int kTileWarp = 1;
+
 template <int FMT, int GLG, bool COUNT, int K = 1>
 __device__ __forceinline__ void trace_pixel_ray(const TraceArgs &a, Ray<K> &r, int pass,
+                                                const float apex[3], const float *pyr,
                                                 uint32_t *stack, float *stack_t, uint32_t *g_ref,
                                                 float *g_t, uint32_t &err, Counts &cnt) {
     if (a.n_nodes == 0) return;
-    if constexpr (GLG >= 3)
+    if constexpr (GLG == kTileWarp) {
+        trace_tile<K, FMT == GS_NODES_BINARY_Q8>(a, r, pass, apex, pyr, g_ref, g_t, err);
+    } else if constexpr (GLG >= 3)
         traverse_group<K, COUNT, GLG, false, FMT == GS_NODES_BINARY_Q8>(a, r, pass, g_ref, g_t, err,
                                                                         cnt);
     else trace_packet<FMT, COUNT, K>(a, r, pass, stack, stack_t, err, cnt);
@@ -184,18 +190,24 @@ constexpr int kWaveMinBlocks = 4;
 // 386.9 and 747.4 with three blocks; 423.7 with two at spp 16).
 template <int FMT, int STACK, bool COUNT, int GLG, int K = 1>
 __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
-    k_render_views(const WaveArgs w) {
+    k_render_views(const __grid_constant__ WaveArgs w) {
     const TraceArgs &a = w.t;
     const int lane = threadIdx.x & 31;
     const uint32_t kAll = 0xffffffffu;
     extern __shared__ uint32_t wave_smem[];
     uint32_t *g_ref = nullptr;
     float *g_t = nullptr;
+    float *pyr = nullptr;
     if constexpr (GLG >= 3) {
         uint32_t *pool = wave_smem + (size_t)(threadIdx.x >> 5) * 2 * kGroupPool;
         const int off = (lane >> GLG) * (kGroupPool >> (5 - GLG));
         g_ref = pool + off;
         g_t = reinterpret_cast<float *>(pool + kGroupPool) + off;
+    } else if constexpr (GLG == kTileWarp) {
+        uint32_t *pool = wave_smem + (size_t)(threadIdx.x >> 5) * (2 * kTilePool + kTileFloats);
+        g_ref = pool;
+        g_t = reinterpret_cast<float *>(pool + kTilePool);
+        pyr = reinterpret_cast<float *>(pool + 2 * kTilePool);
     }
     const int lg = a.lpp_log2, L = 1 << lg;
     const int tw_lg = tile_w_log2(lg), th_lg = 5 - lg - tw_lg;
@@ -254,7 +266,9 @@ __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
             reset_live_slots<K>(r, pass, S, live);
             update_clip(r, r.t_max);
             if (!live[0]) r.t_far = -INFINITY;
-            trace_pixel_ray<FMT, GLG, COUNT, K>(a, r, pass, stack, stack_t, g_ref, g_t, err, cnt);
+            if constexpr (GLG == kTileWarp) tile_pyramid(d0, valid, pyr);
+            trace_pixel_ray<FMT, GLG, COUNT, K>(a, r, pass, vw.eye, pyr, stack, stack_t, g_ref, g_t,
+                                                err, cnt);
             float c[K][3];
             bool on_ground[K];
             int32_t diag_cam[K], diag_bounce[K], diag_vis[K];
@@ -305,7 +319,12 @@ __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
                 reset_live_slots<K>(sr, pass, S, need);
                 update_clip(sr, sr.t_max);
                 if (!any_need) sr.t_far = -INFINITY;
-                trace_pixel_ray<FMT, GLG, COUNT, K>(a, sr, pass, stack, stack_t, g_ref, g_t, err, cnt);
+                if constexpr (GLG == kTileWarp) {
+                    const float away[3] = {-omega[0], -omega[1], -omega[2]};
+                    tile_pyramid(away, any_need, pyr);
+                }
+                trace_pixel_ray<FMT, GLG, COUNT, K>(a, sr, pass, w.light_pos[l], pyr, stack, stack_t,
+                                                    g_ref, g_t, err, cnt);
 #pragma unroll
                 for (int k = 0; k < K; ++k) {
                     n_shadow += need[k];
@@ -700,7 +719,9 @@ gs_status launch_bounce_f(const WaveArgs &w, const unsigned long long *codes, in
 template <int FMT, int STACK, bool COUNT, int GLG, int K = 1>
 gs_status launch_views(const WaveArgs &w, int threads, cudaStream_t s) {
     int dev = 0, sms = 0, per = 0;
-    const size_t smem = GLG >= 3 ? (size_t)(threads / 32) * 2 * kGroupPool * sizeof(uint32_t) : 0;
+    const size_t smem =
+        (size_t)(threads / 32) * sizeof(uint32_t) *
+        (GLG >= 3 ? 2 * kGroupPool : GLG == kTileWarp ? 2 * kTilePool + kTileFloats : 0);
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
@@ -721,6 +742,15 @@ gs_status launch_views(const WaveArgs &w, int threads, cudaStream_t s) {
 template <int FMT, int GLG>
 gs_status launch_views_g(const WaveArgs &w, int threads, int stack, cudaStream_t s) {
     const bool count = w.counters != nullptr;
+    if constexpr (GLG == kTileWarp) {
+        // (no per-lane stacks but the fallback's own)
+        switch (w.spl) {
+            case 8: return launch_views<FMT, 48, false, GLG, 8>(w, threads, s);
+            case 4: return launch_views<FMT, 48, false, GLG, 4>(w, threads, s);
+            case 2: return launch_views<FMT, 48, false, GLG, 2>(w, threads, s);
+            default: return launch_views<FMT, 48, false, GLG, 1>(w, threads, s);
+        }
+    }
     // several samples per lane: packets only (fewer than 8 lanes a pixel),
     // never with counters
     if constexpr (GLG == 0) {
@@ -749,6 +779,7 @@ gs_status launch_views_f(const WaveArgs &w, int threads, int stack, cudaStream_t
 // Binary handles with wide copies: pixels with 8 or more lanes group.
 template <>
 gs_status launch_views_f<GS_NODES_BINARY>(const WaveArgs &w, int threads, int stack, cudaStream_t s) {
+    if (w.t.trec != nullptr) return launch_views_g<GS_NODES_BINARY, kTileWarp>(w, threads, stack, s);
     if (w.t.grec != nullptr) {
         switch (w.t.lpp_log2) {
             case 5: return launch_views_g<GS_NODES_BINARY, 5>(w, threads, stack, s);
@@ -765,6 +796,8 @@ gs_status launch_views_f<GS_NODES_BINARY>(const WaveArgs &w, int threads, int st
 template <>
 gs_status launch_views_f<GS_NODES_BINARY_Q8>(const WaveArgs &w, int threads, int stack,
                                              cudaStream_t s) {
+    if (w.t.trec != nullptr)
+        return launch_views_g<GS_NODES_BINARY_Q8, kTileWarp>(w, threads, stack, s);
     if (w.t.grec != nullptr) {
         switch (w.t.lpp_log2) {
             case 5: return launch_views_g<GS_NODES_BINARY_Q8, 5>(w, threads, stack, s);
@@ -871,6 +904,14 @@ gs_status launch_render_views(const gs_bvh *b, const gs_gaussians *g, const gs_p
         a.grec = b->group[a.lpp_log2 - 3].rec;
         a.groot = b->group[a.lpp_log2 - 3].ref;
         a.gq8 = b->node_format == GS_NODES_BINARY_Q8;
+    }
+    // the tile traversal: fewer than 8 lanes a pixel, camera depths from the
+    // eye, no counters, and no option about the per-lane walk; an inline
+    // bounce keeps the per-lane form
+    if (b->link && a.lpp_log2 < 3 && p->t_min >= 0.0f && p->stack_depth == 0 &&
+        counters == nullptr && !inline_bounce) {
+        a.trec = b->group[2].rec;
+        a.troot = b->group[2].ref;
     }
     const int tw_lg = tile_w_log2(a.lpp_log2), th_lg = 5 - a.lpp_log2 - tw_lg;
     uint32_t tiles = 0;
