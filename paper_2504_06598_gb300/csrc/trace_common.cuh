@@ -419,6 +419,35 @@ __device__ __forceinline__ bool cand_alpha(const TraceArgs &a, const Ray<N> &r, 
     return true;
 }
 
+// Eq. 4 with the slots' draws at hand: accepted slots are replaced (Eq. 6)
+// and the traversal range is clipped.
+template <int N>
+__device__ __forceinline__ void apply_draws(const TraceArgs &a, Ray<N> &r, const bool closer[N],
+                                            const uint32_t bits[N], float key_tc, float key_tau,
+                                            float alpha, uint32_t gid) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        if (!closer[k]) continue;
+        if (lane_to_unit(bits[k]) < alpha) {
+            r.slot[k].tc = key_tc;
+            r.slot[k].tau = key_tau;
+            r.slot[k].gid = gid;
+        }
+    }
+    if (r.any_hit) {
+        // a sample's visibility is known at its first accepted hit: that
+        // slot stops holding the clip and nothing is closer than it
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+            if (r.slot[k].gid != 0xffffffffu) r.slot[k].tc = -INFINITY;
+    }
+    update_clip(r, r.t_max);
+    if (r.any_hit && !(r.t_far > -INFINITY)) r.t_far = -INFINITY;  // every sample known
+    // A projected-centre depth is not a ray parameter, so it cannot clip the
+    // box tests: every box on the ray stays open and order is decided here.
+    if (a.depth_mode == 1) r.t_far = r.t_max;
+}
+
 // Eq. 4 for the slots that the candidate is closer than: accept iff
 // xi < alpha, replacing the slot (Eq. 6) and clipping the traversal range.
 template <int N, bool COUNT>
@@ -448,29 +477,10 @@ __device__ __forceinline__ void accept(const TraceArgs &a, Ray<N> &r, int pass, 
     u0 = philox10_rk(make_uint4(r.ray_id, gid, s0 >> 2, r.stream_tag), a.rk);
     if (N == 8) u1 = philox10_rk(make_uint4(r.ray_id, gid, (s0 >> 2) + 1, r.stream_tag), a.rk);
     if (COUNT) n_draws += 1 + (N == 8);
+    uint32_t bits[N];
 #pragma unroll
-    for (int k = 0; k < N; ++k) {
-        if (!closer[k]) continue;
-        const uint32_t s = s0 + k;
-        const uint32_t bits = (N == 8 && k >= 4) ? pick(u1, s & 3) : pick(u0, s & 3);
-        if (lane_to_unit(bits) < alpha) {
-            r.slot[k].tc = key_tc;
-            r.slot[k].tau = key_tau;
-            r.slot[k].gid = gid;
-        }
-    }
-    if (r.any_hit) {
-        // a sample's visibility is known at its first accepted hit: that
-        // slot stops holding the clip and nothing is closer than it
-#pragma unroll
-        for (int k = 0; k < N; ++k)
-            if (r.slot[k].gid != 0xffffffffu) r.slot[k].tc = -INFINITY;
-    }
-    update_clip(r, r.t_max);
-    if (r.any_hit && !(r.t_far > -INFINITY)) r.t_far = -INFINITY;  // every sample known
-    // A projected-centre depth is not a ray parameter, so it cannot clip the
-    // box tests: every box on the ray stays open and order is decided here.
-    if (a.depth_mode == 1) r.t_far = r.t_max;
+    for (int k = 0; k < N; ++k) bits[k] = pick(N == 8 && k >= 4 ? u1 : u0, (s0 + k) & 3);
+    apply_draws<N>(a, r, closer, bits, key_tc, key_tau, alpha, gid);
 }
 
 // Which slots a candidate at depth key (key_tc, key_tau) is closer than,
@@ -965,24 +975,79 @@ __device__ __forceinline__ void traverse_group(const TraceArgs &a, Ray<N> &r, in
                 // a lane takes a candidate only at t <= its own clip <= G
                 ok = ok && ct <= G;
             }
-            const float far0 = r.t_far;
-            // every lane: its own draws against each candidate
-            for (uint32_t cm = (__ballot_sync(gmask, ok) >> base) & kLaneBits; cm; cm &= cm - 1u) {
-                const int src = base + __ffs(cm) - 1;
-                const float t = __shfl_sync(gmask, ct, src);
-                const float key_tc = __shfl_sync(gmask, ck1, src);
-                const float key_tau = __shfl_sync(gmask, ck2, src);
-                const float alpha = __shfl_sync(gmask, cal, src);
-                const uint32_t gid = __shfl_sync(gmask, cgid, src);
-                bool closer[N];
-                if (closer_slots<N>(r, t, key_tc, key_tau, gid, closer))
-                    accept<N, COUNT>(a, r, pass, closer, t, key_tc, key_tau, alpha, gid, cnt.draws);
-            }
-            // the group clip moves only when some lane's clip did
-            if (__any_sync(gmask, r.t_far != far0)) {
-                G = r.t_far >= r.t_min ? r.t_far : -INFINITY;
+            auto group_clip = [&]() {
+                const float c = r.t_far >= r.t_min ? r.t_far : -INFINITY;
+                const uint32_t b = __float_as_uint(c);
+                const uint32_t o =
+                    __reduce_max_sync(gmask, b ^ ((uint32_t)((int32_t)b >> 31) | 0x80000000u));
+                return __uint_as_float(o ^ ((o & 0x80000000u) ? 0x80000000u : 0xffffffffu));
+            };
+            bool paired = false;
+            if constexpr (N == 2 && !COUNT) paired = a.rng_mode == 0;
+            if (paired) {
+                // Two slots a lane use half of a Philox call: lanes 2i and
+                // 2i + 1 need the same one. So candidates go two at a time,
+                // the even lanes drawing for the first and the odd lanes for
+                // the second, and the pair swaps halves. Nearest first: a
+                // candidate accepted early drops those behind the new clip.
+                for (;;) {
+                    const uint32_t depth = __float_as_uint(fmaxf(ct, 0.0f)) & ~31u;
+                    const uint32_t k0 = __reduce_min_sync(gmask, ok ? depth | (uint32_t)sub : 0xffffffffu);
+                    if (k0 == 0xffffffffu) break;
+                    const int j0 = (int)(k0 & 31u);
+                    if (sub == j0) ok = false;
+                    const uint32_t k1 = __reduce_min_sync(gmask, ok ? depth | (uint32_t)sub : 0xffffffffu);
+                    const bool two = k1 != 0xffffffffu;
+                    const int j1 = two ? (int)(k1 & 31u) : j0;
+                    if (sub == j1) ok = false;
+                    const uint32_t gid0 = __shfl_sync(gmask, cgid, base + j0);
+                    const uint32_t gid1 = __shfl_sync(gmask, cgid, base + j1);
+                    const uint4 u = philox10_rk(
+                        make_uint4(r.ray_id, (sub & 1) ? gid1 : gid0, (uint32_t)pass >> 1, r.stream_tag),
+                        a.rk);
+                    const uint32_t x0 = __shfl_xor_sync(gmask, (sub & 1) ? u.x : u.z, 1);
+                    const uint32_t x1 = __shfl_xor_sync(gmask, (sub & 1) ? u.y : u.w, 1);
+                    const float far0 = r.t_far;
 #pragma unroll
-                for (int o = 1; o < L; o <<= 1) G = fmaxf(G, __shfl_xor_sync(gmask, G, o));
+                    for (int q = 0; q < 2; ++q) {
+                        if (q == 1 && !two) break;
+                        const int src = base + (q ? j1 : j0);
+                        const float t = __shfl_sync(gmask, ct, src);
+                        const float key_tc = __shfl_sync(gmask, ck1, src);
+                        const float key_tau = __shfl_sync(gmask, ck2, src);
+                        const float alpha = __shfl_sync(gmask, cal, src);
+                        const uint32_t gid = q ? gid1 : gid0;
+                        bool closer[N];
+                        if (closer_slots<N>(r, t, key_tc, key_tau, gid, closer)) {
+                            // an even lane's samples take words 0 and 1
+                            uint32_t bits[N];
+                            const bool own = (sub & 1) == q;
+                            bits[0] = own ? ((sub & 1) ? u.z : u.x) : x0;
+                            bits[N - 1] = own ? ((sub & 1) ? u.w : u.y) : x1;
+                            apply_draws<N>(a, r, closer, bits, key_tc, key_tau, alpha, gid);
+                        }
+                    }
+                    if (__any_sync(gmask, r.t_far != far0)) {
+                        G = group_clip();
+                        ok = ok && ct <= G;
+                    }
+                }
+            } else {
+                const float far0 = r.t_far;
+                // every lane: its own draws against each candidate
+                for (uint32_t cm = (__ballot_sync(gmask, ok) >> base) & kLaneBits; cm; cm &= cm - 1u) {
+                    const int src = base + __ffs(cm) - 1;
+                    const float t = __shfl_sync(gmask, ct, src);
+                    const float key_tc = __shfl_sync(gmask, ck1, src);
+                    const float key_tau = __shfl_sync(gmask, ck2, src);
+                    const float alpha = __shfl_sync(gmask, cal, src);
+                    const uint32_t gid = __shfl_sync(gmask, cgid, src);
+                    bool closer[N];
+                    if (closer_slots<N>(r, t, key_tc, key_tau, gid, closer))
+                        accept<N, COUNT>(a, r, pass, closer, t, key_tc, key_tau, alpha, gid, cnt.draws);
+                }
+                // the group clip moves only when some lane's clip did
+                if (__any_sync(gmask, r.t_far != far0)) G = group_clip();
             }
         }
         const bool inner = hit && !leaf && te <= G;
