@@ -1004,6 +1004,16 @@ gs_status launch_backward(const gs_bvh *b, const gs_gaussians *g, const gs_pinho
     const bool tile = b->link && p->t_min >= 0.0f && p->stack_depth == 0;
     int S = p->samples_per_lane > 0 ? p->samples_per_lane
                                     : auto_backward_samples_per_lane(p->spp, p->n_hits, tile);
+    if (tile && p->samples_per_lane == 0) {
+        // fewer warps than the chip holds: more lanes a pixel, fewer samples
+        // each, so that a tile covers fewer pixels
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        const int64_t pix = (int64_t)cam->width * cam->height;
+        while (S > 1 && (pix << lanes_per_pixel_log2((p->spp + S - 1) / S)) < (int64_t)sms * 16 * 32)
+            S >>= 1;
+    }
     while (S > 1 && S > p->spp) S >>= 1;
     const int spp_eff = (p->spp + S - 1) / S;
     TraceArgs a = {};

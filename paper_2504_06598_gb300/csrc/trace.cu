@@ -133,9 +133,16 @@ __global__ void __launch_bounds__(kThreads, is_group_fmt(FMT) ? group_min_blocks
             if (a.n_nodes > 0) {
                 if constexpr (tiled) {
                     trace_tile<N, FMT == kFmtTileQ8>(a, r, pass, a.eye, pyr, grp_ref, grp_t, err);
-                } else if constexpr (grouped)
+                } else if constexpr (grouped) {
+                    uint32_t e = 0;
                     traverse_group<N, COUNT, LG, true, is_group_q8(FMT)>(a, r, pass, grp_ref,
-                                                                          grp_t, err, cnt);
+                                                                          grp_t, e, cnt);
+                    if (!COUNT && __any_sync(kAll, e & kErrStack)) {
+                        e &= ~kErrStack;
+                        start_over<N>(a, r, pass, e);
+                    }
+                    err |= e;
+                }
                 else if constexpr (FMT == GS_NODES_BINARY)
                     traverse_packet<N, COUNT>(a, r, pass, stack, stack_t, err, cnt);
                 else
@@ -277,6 +284,20 @@ int auto_samples_per_lane(int spp, int n_hits, int node_format) {
 
 }  // namespace
 
+static int64_t tile_warps(int width, int height, int lpp_log2) {
+    const int tw_lg = tile_w_log2(lpp_log2), th_lg = 5 - lpp_log2 - tw_lg;
+    return (int64_t)((width + (1 << tw_lg) - 1) >> tw_lg) * ((height + (1 << th_lg) - 1) >> th_lg);
+}
+
+// Warps the current device holds at once at 64 registers a thread.
+static int64_t resident_warps() {
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return 0;
+    return (int64_t)sms * 32;
+}
+
 void trace_layout(const gs_bvh *b, const gs_trace_params *p, int *S_out, int *spp_eff_out,
                   int *lpp_log2_out, bool *grouped_out) {
     // A lane carries S consecutive samples: the launch runs ceil(spp / S)
@@ -298,6 +319,22 @@ gs_status launch_trace(const gs_bvh *b, const gs_gaussians *g, const gs_pinhole 
     bool grouped = false;
     trace_layout(b, p, &S, &spp_eff, &lpp_log2, &grouped);
     const int n_eff = p->n_hits * S;
+    // the tile traversal: fewer than 8 lanes a pixel, depths along the ray
+    // from the eye, and none of the options that are about the per-lane walk
+    bool tile = b->link && lpp_log2 < 3 && p->t_min >= 0.0f && p->depth_mode == 0 &&
+                p->rng_mode == 0 && p->stack_depth == 0 && p->counters == nullptr;
+    if (tile && tile_warps(cam->width, cam->height, lpp_log2) < resident_warps()) {
+        // Too few tiles to fill the chip once: the time is the longest walk
+        // of a warp, which evaluates its tile's Gaussians one after the other.
+        // A whole warp per pixel then (most lanes without a sample, helping in
+        // the walk) evaluates 32 at a time. us, tile -> warp per pixel: 1k
+        // Gaussians, 64x64, spp 1 89 -> 31; 90k, 96x72, spp 1 2662 -> 126 and
+        // spp 16 3350 -> 199; 411x307, spp 1 774 -> 516 (3,900 tiles); above
+        // one wave the tiles win (411x307, spp 16, 7,900 tiles 1004 against
+        // 1204; 1M at 1080p, spp 1 3.1 ms against 13.6).
+        tile = false;
+        lpp_log2 = 5;
+    }
     TraceArgs a;
     a.nodes = b->nodes;
     a.wide = b->wide;
@@ -310,10 +347,6 @@ gs_status launch_trace(const gs_bvh *b, const gs_gaussians *g, const gs_pinhole 
         a.groot = nullptr;
     }
     a.gq8 = b->node_format == GS_NODES_BINARY_Q8;
-    // the tile traversal: fewer than 8 lanes a pixel, depths along the ray
-    // from the eye, and none of the options that are about the per-lane walk
-    const bool tile = b->link && a.lpp_log2 < 3 && p->t_min >= 0.0f && p->depth_mode == 0 &&
-                      p->rng_mode == 0 && p->stack_depth == 0 && p->counters == nullptr;
     a.trec = tile ? b->group[2].rec : nullptr;
     a.troot = tile ? b->group[2].ref : nullptr;
     a.prims = b->prims;

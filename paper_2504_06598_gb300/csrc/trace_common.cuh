@@ -1358,13 +1358,10 @@ __device__ __noinline__ void tile_fallback(const TraceArgs &a, Ray<N> &r, int pa
     traverse_packet<N, false>(a, r, pass, stack, stack_t, err, cnt);
 }
 
-// traverse_tile, started over on the binary nodes where its stack is full:
-// every slot but the unused ones (at -inf with no Gaussian) is emptied again.
-template <int N, bool Q8>
-__device__ __forceinline__ void trace_tile(const TraceArgs &a, Ray<N> &r, int pass,
-                                           const float apex[3], const float *pyr, uint32_t *s_ref,
-                                           float *s_t, uint32_t &err) {
-    if (traverse_tile<N, Q8>(a, r, pass, apex, pyr, s_ref, s_t, err)) return;
+// A walk whose stack was full started over on the binary nodes: every slot but
+// the unused ones (at -inf with no Gaussian) is emptied again.
+template <int N>
+__device__ __forceinline__ void start_over(const TraceArgs &a, Ray<N> &r, int pass, uint32_t &err) {
     Ray<N> again = r;
     set_ray(again, r.o, r.d);
 #pragma unroll
@@ -1378,6 +1375,13 @@ __device__ __forceinline__ void trace_tile(const TraceArgs &a, Ray<N> &r, int pa
     err |= err2;
 #pragma unroll
     for (int k = 0; k < N; ++k) r.slot[k] = again.slot[k];
+}
+
+template <int N, bool Q8>
+__device__ __forceinline__ void trace_tile(const TraceArgs &a, Ray<N> &r, int pass,
+                                           const float apex[3], const float *pyr, uint32_t *s_ref,
+                                           float *s_t, uint32_t &err) {
+    if (!traverse_tile<N, Q8>(a, r, pass, apex, pyr, s_ref, s_t, err)) start_over<N>(a, r, pass, err);
 }
 
 }  // namespace

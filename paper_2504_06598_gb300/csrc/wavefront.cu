@@ -156,9 +156,15 @@ __device__ __forceinline__ void trace_pixel_ray(const TraceArgs &a, Ray<K> &r, i
     if constexpr (GLG == kTileWarp) {
         trace_tile<K, FMT == GS_NODES_BINARY_Q8>(a, r, pass, apex, pyr, g_ref, g_t, err);
     } else if constexpr (GLG >= 3)
-        traverse_group<K, COUNT, GLG, false, FMT == GS_NODES_BINARY_Q8>(a, r, pass, g_ref, g_t, err,
-                                                                        cnt);
-    else trace_packet<FMT, COUNT, K>(a, r, pass, stack, stack_t, err, cnt);
+    {
+        uint32_t e = 0;
+        traverse_group<K, COUNT, GLG, false, FMT == GS_NODES_BINARY_Q8>(a, r, pass, g_ref, g_t, e, cnt);
+        if (!COUNT && __any_sync(0xffffffffu, e & kErrStack)) {
+            e &= ~kErrStack;
+            start_over<K>(a, r, pass, e);
+        }
+        err |= e;
+    } else trace_packet<FMT, COUNT, K>(a, r, pass, stack, stack_t, err, cnt);
 }
 
 // Slots of pass `pass` of a lane carrying K samples: sample pass * K + k is
@@ -751,8 +757,13 @@ gs_status launch_views_g(const WaveArgs &w, int threads, int stack, cudaStream_t
             default: return launch_views<FMT, 48, false, GLG, 1>(w, threads, s);
         }
     }
-    // several samples per lane: packets only (fewer than 8 lanes a pixel),
-    // never with counters
+    // several samples per lane: fewer than 8 lanes a pixel, or a warp per
+    // pixel with most lanes idle; never with counters
+    if constexpr (GLG == 5) {
+        if (!count && w.spl == 8) return launch_views<FMT, 48, false, GLG, 8>(w, threads, s);
+        if (!count && w.spl == 4) return launch_views<FMT, 48, false, GLG, 4>(w, threads, s);
+        if (!count && w.spl == 2) return launch_views<FMT, 48, false, GLG, 2>(w, threads, s);
+    }
     if constexpr (GLG == 0) {
         if (!count && w.spl == 8)
             return stack == 48 ? launch_views<FMT, 48, false, 0, 8>(w, threads, s)
@@ -885,9 +896,23 @@ gs_status launch_render_views(const gs_bvh *b, const gs_gaussians *g, const gs_p
     // spp 32 806 (one) -> 770 (eight).
     const int64_t bounce_slots = wave_slots(cams, n_views, ex, p);
     const bool inline_bounce = ex && ex->bounce && ex->has_ground && bounce_slots == 0;
+    int sms = 0, dev = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    int64_t all_pix = 0;
+    for (int v = 0; v < n_views; ++v) all_pix += (int64_t)cams[v].width * cams[v].height;
+    // the tile traversal: fewer than 8 lanes a pixel, camera depths from the
+    // eye, no counters, and no option about the per-lane walk; an inline
+    // bounce keeps the per-lane form
+    const bool tiles_ok = b->link && p->t_min >= 0.0f && p->stack_depth == 0 &&
+                          counters == nullptr && !inline_bounce;
     int K = 1;
     if (counters == nullptr && !inline_bounce && p->spp >= 2 && p->spp < 64)
         K = p->spp >= 8 ? 8 : (p->spp >= 4 ? 4 : 2);
+    // too few tiles to fill the chip once: a warp per pixel (see launch_trace)
+    const int lanes_lg = lanes_per_pixel_log2((p->spp + K - 1) / K);
+    const bool whole_warp =
+        tiles_ok && lanes_lg < 3 && (all_pix << lanes_lg) < (int64_t)sms * 32 * 32;
     w.spl = K;
     a.spp = (p->spp + K - 1) / K;
     a.n_samples = p->spp;
@@ -899,17 +924,13 @@ gs_status launch_render_views(const gs_bvh *b, const gs_gaussians *g, const gs_p
     a.rgb = rgb;
     a.status = b->status;
     a.work = b->status + 1;
-    a.lpp_log2 = lanes_per_pixel_log2(a.spp);
+    a.lpp_log2 = whole_warp ? 5 : lanes_per_pixel_log2(a.spp);
     if (b->link && a.lpp_log2 >= 3) {
         a.grec = b->group[a.lpp_log2 - 3].rec;
         a.groot = b->group[a.lpp_log2 - 3].ref;
         a.gq8 = b->node_format == GS_NODES_BINARY_Q8;
     }
-    // the tile traversal: fewer than 8 lanes a pixel, camera depths from the
-    // eye, no counters, and no option about the per-lane walk; an inline
-    // bounce keeps the per-lane form
-    if (b->link && a.lpp_log2 < 3 && p->t_min >= 0.0f && p->stack_depth == 0 &&
-        counters == nullptr && !inline_bounce) {
+    if (tiles_ok && a.lpp_log2 < 3) {
         a.trec = b->group[2].rec;
         a.troot = b->group[2].ref;
     }
