@@ -210,6 +210,342 @@ __global__ void __launch_bounds__(kThreads, is_group_fmt(FMT) ? group_min_blocks
     }
 }
 
+// ---------------------------------------------------------------- shared walks
+// Above 32 samples a pixel: a warp holds a 2x2 tile, walks the 32-wide copy
+// once for its four pixels (the pyramid test of traverse_tile), evaluates the
+// surviving Gaussians with a lane per (pixel, Gaussian) pair, eight Gaussians
+// for the four pixels at a time, and then draws for one pixel after the
+// other, all 32 lanes with two samples each. A pixel's 64 samples are kept in
+// shared memory (three words each) between its turns. The grouped form (one
+// pixel a warp) spent more on its walk than on its draws (1M shell at 1080p:
+// 13.6 ms of 23.0 at spp 64); evaluating per lane as the tiles do repeats
+// each evaluation on the pixel's lanes.
+constexpr int kSharedPx = 4;
+constexpr int kSharedPool = 192;  // stack entries per warp
+
+struct __align__(16) SharedWarp {
+    float pyr[kTileFloats];
+    float2 tc[kSharedPx][32], tau[kSharedPx][32];
+    uint2 gid[kSharedPx][32];
+    float dir[kSharedPx][4];
+    union {
+        uint32_t ref[kSharedPool];  // during a walk
+        float colour[3][64];        // after it: of one pixel's samples
+    };
+    float t[kSharedPool];
+    uint32_t leaves[32];
+    float acc[kSharedPx][3][32];  // partial sums
+};
+
+__device__ __forceinline__ void load_slots(const SharedWarp &m, int p, int lane, Ray<2> &r) {
+    const float2 tc = m.tc[p][lane], tau = m.tau[p][lane];
+    const uint2 gid = m.gid[p][lane];
+    r.slot[0] = Slot{tc.x, tau.x, gid.x};
+    r.slot[1] = Slot{tc.y, tau.y, gid.y};
+}
+
+__device__ __forceinline__ void store_slots(SharedWarp &m, int p, int lane, const Ray<2> &r) {
+    m.tc[p][lane] = make_float2(r.slot[0].tc, r.slot[1].tc);
+    m.tau[p][lane] = make_float2(r.slot[0].tau, r.slot[1].tau);
+    m.gid[p][lane] = make_uint2(r.slot[0].gid, r.slot[1].gid);
+}
+
+// The largest clip of the warp's lanes (-inf where none is in range).
+__device__ __forceinline__ float warp_clip(float t_far, float t_min) {
+    const uint32_t b = t_far >= t_min ? __float_as_uint(fmaxf(t_far, 0.0f)) + 1u : 0u;
+    const uint32_t m = __reduce_max_sync(0xffffffffu, b);
+    return m ? __uint_as_float(m - 1u) : -INFINITY;
+}
+
+// Two candidates of pixel p at a time, nearest first, as in traverse_group:
+// an even lane draws for the first, an odd lane for the second, and the two
+// swap the halves. ok: this lane holds a candidate (of its own pixel).
+__device__ __forceinline__ float shared_draws(const TraceArgs &a, SharedWarp &m, int p, int lane,
+                                              uint32_t ray_id, uint32_t counter, bool ok, float ct,
+                                              float ck1, float ck2, float cal, uint32_t cgid,
+                                              float G) {
+    const uint32_t kAll = 0xffffffffu;
+    const bool odd = lane & 1;
+    Ray<2> r;
+    load_slots(m, p, lane, r);
+    r.t_min = a.t_min;
+    r.t_max = a.t_max;
+    r.any_hit = false;
+    update_clip(r, a.t_max);
+    const uint32_t depth = (__float_as_uint(fmaxf(ct, 0.0f)) & ~31u) | (uint32_t)lane;
+    bool drawn = false;
+    for (;;) {
+        const uint32_t k0 = __reduce_min_sync(kAll, ok ? depth : 0xffffffffu);
+        if (k0 == 0xffffffffu) break;
+        const int j0 = (int)(k0 & 31u);
+        if (lane == j0) ok = false;
+        const uint32_t k1 = __reduce_min_sync(kAll, ok ? depth : 0xffffffffu);
+        const bool two = k1 != 0xffffffffu;
+        const int j1 = two ? (int)(k1 & 31u) : j0;
+        if (lane == j1) ok = false;
+        const uint32_t gid0 = __shfl_sync(kAll, cgid, j0), gid1 = __shfl_sync(kAll, cgid, j1);
+        const uint4 u = philox10_rk(make_uint4(ray_id, odd ? gid1 : gid0, counter, a.stream_tag), a.rk);
+        const uint32_t x0 = __shfl_xor_sync(kAll, odd ? u.x : u.z, 1);
+        const uint32_t x1 = __shfl_xor_sync(kAll, odd ? u.y : u.w, 1);
+        const float far0 = r.t_far;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            if (q == 1 && !two) break;
+            const int src = q ? j1 : j0;
+            const float t = __shfl_sync(kAll, ct, src);
+            const float key_tc = __shfl_sync(kAll, ck1, src);
+            const float key_tau = __shfl_sync(kAll, ck2, src);
+            const float alpha = __shfl_sync(kAll, cal, src);
+            bool closer[2];
+            if (closer_slots<2>(r, t, key_tc, key_tau, q ? gid1 : gid0, closer)) {
+                drawn = true;
+                const bool own = odd == (q == 1);
+                uint32_t bits[2];
+                bits[0] = own ? (odd ? u.z : u.x) : x0;
+                bits[1] = own ? (odd ? u.w : u.y) : x1;
+                apply_draws<2>(a, r, closer, bits, key_tc, key_tau, alpha, q ? gid1 : gid0);
+            }
+        }
+        if (__any_sync(kAll, r.t_far != far0)) {
+            G = warp_clip(r.t_far, a.t_min);
+            ok = ok && ct <= G;
+        }
+    }
+    if (drawn) store_slots(m, p, lane, r);
+    return G;
+}
+
+template <bool Q8>
+__global__ void __launch_bounds__(kThreads, 8) k_trace_shared(const __grid_constant__ TraceArgs a) {
+    __shared__ SharedWarp s_warp[kThreads / 32];
+    const uint32_t kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    SharedWarp &m = s_warp[threadIdx.x >> 5];
+    const int ep = lane >> 3;  // the pixel this lane evaluates for
+    const uint32_t tiles_x = (uint32_t)((a.width + 1) >> 1);
+    const uint32_t n_tiles = tiles_x * (uint32_t)((a.height + 1) >> 1);
+    const int64_t npix = (int64_t)a.width * a.height;
+    uint32_t err = 0;
+    for (;;) {
+        uint32_t tile = 0;
+        if (lane == 0) tile = atomicAdd(a.work, 1u);
+        tile = __shfl_sync(kAll, tile, 0);
+        if (tile >= n_tiles) break;
+        const int x0 = (int)(tile % tiles_x) * 2, y0 = (int)(tile / tiles_x) * 2;
+        Ray<1> er;  // the ray this lane evaluates along
+        const bool valid = x0 + (ep & 1) < a.width && y0 + (ep >> 1) < a.height;
+        camera_ray(a, valid ? x0 + (ep & 1) : 0, valid ? y0 + (ep >> 1) : 0, er.d);
+        for (int i = 0; i < 3; ++i) er.o[i] = a.eye[i];
+        er.t_min = a.t_min;
+        er.t_max = a.t_max;
+        tile_pyramid(er.d, valid, m.pyr);
+        if ((lane & 7) < 3) m.dir[ep][lane & 7] = (lane & 7) == 0 ? er.d[0] : (lane & 7) == 1 ? er.d[1] : er.d[2];
+        for (int base = 0; base < a.n_samples; base += 64) {
+            const int s0 = base + 2 * lane;
+            float G;
+            {
+                Ray<1> all;
+                all.slot[0] = Slot{INFINITY, 0.0f, 0xffffffffu};
+                update_clip(all, a.t_max);
+                G = valid ? all.t_far : -INFINITY;
+            }
+#pragma unroll
+            for (int p = 0; p < kSharedPx; ++p) {
+                m.tc[p][lane] = make_float2(s0 < a.n_samples ? INFINITY : -INFINITY,
+                                            s0 + 1 < a.n_samples ? INFINITY : -INFINITY);
+                m.tau[p][lane] = make_float2(0.0f, 0.0f);
+                m.gid[p][lane] = make_uint2(0xffffffffu, 0xffffffffu);
+            }
+            __syncwarp();
+            float g = warp_clip(G, a.t_min), g2 = g * g;
+            bool full = false;
+            int sp = 0;
+            uint32_t node = a.n_nodes > 0 ? __ldg(a.troot) : 0u, steps = 0;
+            bool walk = a.n_nodes > 0 && g >= a.t_min;
+            while (walk) {
+                if (++steps > a.step_limit) {
+                    err |= kErrSteps;
+                    break;
+                }
+                const int n_child = (int)((node >> kWideCountShift) & 31u) + 1;
+                uint32_t ref = kEmpty;
+                float d2 = INFINITY;
+                bool hit = false;
+                if (lane < n_child) hit = tile_child<Q8>(a.trec, node, lane, a.eye, m.pyr, g2, ref, d2);
+                const bool leaf = (ref & kLeafBit) != 0u;
+                const uint32_t lm = __ballot_sync(kAll, hit && leaf);
+                if (lm) {
+                    if (hit && leaf) m.leaves[__popc(lm & ((1u << lane) - 1u))] = ref & ~kLeafBit;
+                    __syncwarp();
+                    const int n_leaf = __popc(lm);
+                    for (int b = 0; b < n_leaf; b += 8) {
+                        const int c = b + (lane & 7);
+                        float ct = 0.0f, ck1 = 0.0f, ck2 = 0.0f, cal = 0.0f;
+                        uint32_t cgid = 0;
+                        bool ok = false;
+                        if (c < n_leaf && G >= a.t_min) {
+                            CandGeom cg;
+                            ok = cand_depth<1, true>(a, er, m.leaves[c], cg) && cg.t <= G &&
+                                 cand_alpha<1, true>(a, er, cg, cal);
+                            ct = cg.t;
+                            ck1 = cg.key_tc;
+                            ck2 = cg.key_tau;
+                            cgid = cg.gid;
+                        }
+                        uint32_t okm = __ballot_sync(kAll, ok);
+                        while (okm) {
+                            const int p = (__ffs(okm) - 1) >> 3;
+                            okm &= ~(0xffu << (8 * p));
+                            const uint32_t id = a.ray_id_offset +
+                                                (uint32_t)((int64_t)(y0 + (p >> 1)) * a.width + x0 + (p & 1));
+                            const float Gp = __shfl_sync(kAll, G, 8 * p);
+                            const float Gn =
+                                shared_draws(a, m, p, lane, id, (uint32_t)(base >> 2) + (lane >> 1),
+                                             ok && ep == p, ct, ck1, ck2, cal, cgid, Gp);
+                            if (ep == p) G = Gn;
+                        }
+                    }
+                    g = warp_clip(G, a.t_min);
+                    g2 = g * g;
+                    if (!(g >= a.t_min)) break;
+                    __syncwarp();
+                }
+                const bool inner = hit && !leaf && d2 <= g2;
+                const uint32_t im = __ballot_sync(kAll, inner);
+                if (im) {
+                    const uint32_t key = (__float_as_uint(d2) & ~31u) | (uint32_t)lane;
+                    const int nj = (int)(__reduce_min_sync(kAll, inner ? key : 0xffffffffu) & 31u);
+                    const uint32_t next = __shfl_sync(kAll, ref, nj);
+                    const uint32_t others = im & ~(1u << nj);
+                    const int npush = __popc(others);
+                    if (sp + npush > kSharedPool) {
+                        full = true;
+                        break;
+                    }
+                    __syncwarp();
+                    if (inner && lane != nj) {
+                        const int pos = sp + __popc(others & ((1u << lane) - 1u));
+                        m.ref[pos] = ref;
+                        m.t[pos] = d2;
+                    }
+                    sp += npush;
+                    __syncwarp();
+                    node = next;
+                    continue;
+                }
+                walk = false;
+                while (sp > 0) {
+                    const int k = sp - 1 - lane;
+                    const uint32_t okm = __ballot_sync(kAll, k >= 0 && m.t[k >= 0 ? k : 0] <= g2);
+                    if (okm) {
+                        sp -= __ffs(okm);  // the lowest lane holds the topmost
+                        node = m.ref[sp];
+                        walk = true;
+                        break;
+                    }
+                    sp = sp > 32 ? sp - 32 : 0;
+                }
+            }
+            // shade each slot once (Eq. 6) and accumulate (Eq. 7)
+#pragma unroll 1
+            for (int p = 0; p < kSharedPx; ++p) {
+                const int x = x0 + (p & 1), y = y0 + (p >> 1);
+                if (x >= a.width || y >= a.height) continue;
+                const int64_t pix = (int64_t)y * a.width + x;
+                Ray<2> r;
+                load_slots(m, p, lane, r);
+                for (int i = 0; i < 3; ++i) r.d[i] = m.dir[p][i];
+                if (full) {
+                    // (the stack did not do: this pixel's samples again)
+                    for (int i = 0; i < 3; ++i) r.o[i] = a.eye[i];
+                    r.ray_id = a.ray_id_offset + (uint32_t)pix;
+                    r.stream_tag = a.stream_tag;
+                    r.t_min = a.t_min;
+                    r.t_max = a.t_max;
+                    r.any_hit = false;
+                    start_over<2>(a, r, s0 >> 1, err);
+                }
+                float Y[16];
+                sh_basis(a.sh_degree, r.d, Y);
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {
+                    if (s0 + k >= a.n_samples) continue;
+                    float c[3];
+                    if (r.slot[k].gid != 0xffffffffu) {
+                        sh_colour(a, r.slot[k].gid, Y, c);
+                    } else {
+                        c[0] = a.bg[0]; c[1] = a.bg[1]; c[2] = a.bg[2];
+                    }
+                    for (int i = 0; i < 3; ++i) m.colour[i][2 * lane + k] = c[i];
+                    if (a.hit_id) {
+                        const int64_t o = ((int64_t)s0 + k) * npix + pix;
+                        a.hit_id[o] = r.slot[k].gid == 0xffffffffu ? -1 : (int32_t)r.slot[k].gid;
+                        a.hit_t[o] = r.slot[k].t();
+                    }
+                    if (a.keys) {
+                        gs_sample_key *key = a.keys + pix * a.n_samples + s0 + k;
+                        key->tc = r.slot[k].tc;
+                        key->tau = r.slot[k].tau;
+                        key->gid = r.slot[k].gid;
+                    }
+                }
+                __syncwarp();
+                // the sums of k_trace's lanes (passes of 2^k samples, 2^l
+                // lanes a pixel), in their order: the same image bit for bit
+                float acc[3];
+                for (int i = 0; i < 3; ++i) acc[i] = base > 0 ? m.acc[p][i][lane] : 0.0f;
+                const int L = 1 << a.lpp_log2, end = min(base + 64, a.n_samples);
+                if (lane < L) {
+                    int pass = base >> a.k_log2;
+                    pass += (lane - pass) & (L - 1);
+                    for (; pass << a.k_log2 < end; pass += L)
+                        for (int s = pass << a.k_log2; s < min((pass + 1) << a.k_log2, end); ++s)
+                            for (int i = 0; i < 3; ++i) acc[i] += m.colour[i][s - base];
+                }
+                for (int i = 0; i < 3; ++i) m.acc[p][i][lane] = acc[i];
+                __syncwarp();
+            }
+            __syncwarp();
+        }
+#pragma unroll 1
+        for (int p = 0; p < kSharedPx; ++p) {
+            const int x = x0 + (p & 1), y = y0 + (p >> 1);
+            if (x >= a.width || y >= a.height) continue;
+            float acc[3];
+            for (int i = 0; i < 3; ++i) acc[i] = m.acc[p][i][lane];
+            for (int o = (1 << a.lpp_log2) >> 1; o >= 1; o >>= 1) {
+                acc[0] += __shfl_xor_sync(kAll, acc[0], o);
+                acc[1] += __shfl_xor_sync(kAll, acc[1], o);
+                acc[2] += __shfl_xor_sync(kAll, acc[2], o);
+            }
+            if (lane == 0) {
+                const float inv_n = 1.0f / (float)a.n_samples;
+                const int64_t pix = (int64_t)y * a.width + x;
+                for (int i = 0; i < 3; ++i) a.rgb[3 * pix + i] = acc[i] * inv_n;
+            }
+        }
+        __syncwarp();
+    }
+    if (err) atomicOr(a.status, err);
+}
+
+template <bool Q8>
+gs_status launch_shared(const TraceArgs &a, cudaStream_t s) {
+    int dev = 0, sms = 0, per = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e == cudaSuccess)
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_trace_shared<Q8>, kThreads, 0);
+    if (e != cudaSuccess) return cuda_fail(e, "trace launch setup");
+    const int64_t tiles = (int64_t)((a.width + 1) >> 1) * ((a.height + 1) >> 1);
+    const int64_t need = (tiles + kThreads / 32 - 1) / (kThreads / 32);
+    const int64_t fit = (int64_t)sms * (per > 0 ? per : 1);
+    if ((e = cudaMemsetAsync(a.work, 0, sizeof(uint32_t), s)) != cudaSuccess)
+        return cuda_fail(e, "reset work counter");
+    k_trace_shared<Q8><<<(unsigned)(need < fit ? need : fit), kThreads, 0, s>>>(a);
+    return GS_OK;
+}
+
 template <int N, int FMT>
 gs_status launch_nf(const TraceArgs &a, bool count, cudaStream_t s) {
     int dev = 0, sms = 0, per = 0;
@@ -321,8 +657,10 @@ gs_status launch_trace(const gs_bvh *b, const gs_gaussians *g, const gs_pinhole 
     const int n_eff = p->n_hits * S;
     // the tile traversal: fewer than 8 lanes a pixel, depths along the ray
     // from the eye, and none of the options that are about the per-lane walk
-    bool tile = b->link && lpp_log2 < 3 && p->t_min >= 0.0f && p->depth_mode == 0 &&
-                p->rng_mode == 0 && p->stack_depth == 0 && p->counters == nullptr;
+    const bool plain = b->link && p->t_min >= 0.0f && p->depth_mode == 0 && p->rng_mode == 0 &&
+                       p->stack_depth == 0 && p->counters == nullptr;
+    const bool shared = plain && p->samples_per_lane == 0 && (int64_t)p->spp * p->n_hits > 32;
+    bool tile = plain && !shared && lpp_log2 < 3;
     if (tile && tile_warps(cam->width, cam->height, lpp_log2) < resident_warps()) {
         // Too few tiles to fill the chip once: the time is the longest walk
         // of a warp, which evaluates its tile's Gaussians one after the other.
@@ -347,8 +685,8 @@ gs_status launch_trace(const gs_bvh *b, const gs_gaussians *g, const gs_pinhole 
         a.groot = nullptr;
     }
     a.gq8 = b->node_format == GS_NODES_BINARY_Q8;
-    a.trec = tile ? b->group[2].rec : nullptr;
-    a.troot = tile ? b->group[2].ref : nullptr;
+    a.trec = tile || shared ? b->group[2].rec : nullptr;
+    a.troot = tile || shared ? b->group[2].ref : nullptr;
     a.prims = b->prims;
     a.sh = g->sh;
     a.n_nodes = b->n_nodes;
@@ -369,6 +707,8 @@ gs_status launch_trace(const gs_bvh *b, const gs_gaussians *g, const gs_pinhole 
     philox_round_keys(a.key0, a.key1, a.rk);
     a.stream_tag = p->stream_tag;
     a.spp = spp_eff;
+    a.k_log2 = 0;
+    while ((1 << a.k_log2) < n_eff) ++a.k_log2;
     a.n_samples = p->spp * p->n_hits;
     a.t_min = p->t_min;
     a.t_max = p->t_max;
@@ -397,6 +737,13 @@ gs_status launch_trace(const gs_bvh *b, const gs_gaussians *g, const gs_pinhole 
     }
     const bool count = p->counters != nullptr;
     gs_status st;
+    if (shared) {
+        st = a.gq8 ? launch_shared<true>(a, s) : launch_shared<false>(a, s);
+        if (st != GS_OK) return st;
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return cuda_fail(e, "trace launch");
+        return GS_OK;
+    }
     switch (n_eff) {
         case 1: st = launch_n<1>(a, b->node_format, count, s); break;
         case 2: st = launch_n<2>(a, b->node_format, count, s); break;

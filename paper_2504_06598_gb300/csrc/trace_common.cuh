@@ -53,6 +53,7 @@ struct TraceArgs {
     uint32_t *status;
     uint32_t *work;  // tile counter of the persistent launch
     int lpp_log2;    // log2 of the lanes that trace samples of one pixel
+    int k_log2;      // log2 of the slots of a pass (shared walks)
     int depth_mode;  // 0: 1D mean; 1: centre projected on fwd (camera rays)
     int rng_mode;    // 0: Philox; 1: trigonometric hash of the hit point
     float fwd[3];    // camera forward axis (depth_mode 1)

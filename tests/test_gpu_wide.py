@@ -85,3 +85,28 @@ def test_tile_hits_equal_packet_hits(gs, fmt, spp, spl):
                 # sums of spp colours in another order
                 assert (rgb - ref).abs().max() <= 2 * spp * 2.0 ** -24 * ref.abs().max()
         bvh.free()
+
+
+@pytest.mark.parametrize("fmt", ["binary", "binary_q8"])
+@pytest.mark.parametrize("spp,n_hits", [(33, 1), (64, 1), (65, 1), (200, 1), (16, 4), (17, 8)])
+def test_shared_walk_hits_equal_packet_hits(gs, fmt, spp, n_hits):
+    """Above 32 samples a pixel the library's own choice walks once for four
+    pixels: against one pixel at a time, with odd image sizes, sample counts
+    around 64, a range, and the stored payloads."""
+    for cams, M, coincident in ((SMALL, 1, False), (SMALL, 2, False), (SMALL, 33, True),
+                                (SMALL, 1025, False), (SMALL, 7000, True)):
+        g = gs.Gaussians.from_cloud(_cloud(M, coincident))
+        bvh = gs.build_bvh(g, node_format=fmt)
+        for cam in cams:
+            for lim in ({}, dict(t_min=1.5, t_max=3.0)):
+                kw = dict(seed=M, spp=spp, n_hits=n_hits, **lim)
+                rgb, a, ta = gs.trace_stochastic(bvh, g, cam, want_hits=True, **kw)
+                ref, b, tb = gs.trace_stochastic(bvh, g, cam, want_hits=True, stack_depth=96, **kw)
+                keys = gs.sample_keys(cam, spp, n_hits)
+                again = gs.trace_stochastic(bvh, g, cam, keys=keys, **kw)
+                bvh.sync_status()
+                assert torch.equal(a, b) and torch.equal(ta, tb), (M, cam)
+                assert torch.equal(again, rgb) and torch.equal(ref, rgb)
+                gid = gs.decode_keys(keys)[2].reshape(cam.height, cam.width, spp, n_hits)
+                assert torch.equal(gid.permute(2, 3, 0, 1), a.long())
+        bvh.free()
