@@ -171,8 +171,6 @@ gs_status gs_build_bvh_ex(const gs_gaussians *g, const gs_build_options *opt, gs
         {(void **)&b->group[0].ref, grouped ? (size_t)nn * 4 : 0},
         {(void **)&b->group[1].rec, grouped ? (size_t)recs * rec_bytes : 0},
         {(void **)&b->group[1].ref, grouped ? (size_t)nn * 4 : 0},
-        {(void **)&b->group[2].rec, grouped ? (size_t)recs * rec_bytes : 0},
-        {(void **)&b->group[2].ref, grouped ? (size_t)nn * 4 : 0},
     };
     int64_t total = 0;
     for (auto &r : reqs) {

@@ -1047,13 +1047,13 @@ gs_status launch_backward(const gs_bvh *b, const gs_gaussians *g, const gs_pinho
     a.work = b->status + 1;
     a.lpp_log2 = lanes_per_pixel_log2(spp_eff);
     if (b->link && a.lpp_log2 >= 3) {
-        a.grec = b->group[a.lpp_log2 - 3].rec;
-        a.groot = b->group[a.lpp_log2 - 3].ref;
+        a.grec = b->group[group_tree(a.lpp_log2)].rec;
+        a.groot = b->group[group_tree(a.lpp_log2)].ref;
         a.gq8 = b->node_format == GS_NODES_BINARY_Q8;
     }
     if (tile) {
-        a.trec = b->group[2].rec;
-        a.troot = b->group[2].ref;
+        a.trec = b->group[kWarpTree].rec;
+        a.troot = b->group[kWarpTree].ref;
         a.gq8 = b->node_format == GS_NODES_BINARY_Q8;
         a.g_stats = b->grad;
         a.sh_vec = ((uintptr_t)d_sh & 15u) == 0;

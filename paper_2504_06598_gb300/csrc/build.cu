@@ -12,7 +12,7 @@
 //   k_leaves      per-Gaussian record in tree order, then bottom-up box
 //                 refit with one arrival counter per node; cuts the wide
 //                 hierarchies on the way
-//   k_wide_*      records of the 8-, 16- and 32-wide hierarchies
+//   k_wide_*      records of the 8- and 32-wide hierarchies
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -352,8 +352,10 @@ constexpr unsigned long long kTileCounted = 1ull << 62, kTileTotal = 2ull << 62;
 constexpr unsigned long long kTileValue = (1ull << 40) - 1ull;
 constexpr int kLookbackLimit = 1 << 24;
 
+// Four blocks per SM, so that the tiles of 1M keys run at once (three, at 74
+// registers, left a second wave: 21 us a pass).
 template <bool VALS>
-__global__ void __launch_bounds__(kSortThreads)
+__global__ void __launch_bounds__(kSortThreads, 4)
     k_radix_pass(int64_t n, const unsigned long long *__restrict__ kin,
                  const uint32_t *__restrict__ vin, unsigned long long *__restrict__ kout,
                  uint32_t *__restrict__ vout, int pass, const uint32_t *__restrict__ hist,
@@ -474,8 +476,8 @@ struct ZeroScratch {
 
 // Common-prefix length of sorted keys i and j, extended by the index bits
 // when the codes are equal; -1 outside [0, n).
-__device__ __forceinline__ int delta(const unsigned long long *codes, int64_t n,
-                                     int64_t i, int64_t j) {
+template <typename I>
+__device__ __forceinline__ int delta(const unsigned long long *codes, I n, I i, I j) {
     if (j < 0 || j >= n) return -1;
     unsigned long long a = codes[i], b = codes[j];
     if (a == b) return 64 + __clz((uint32_t)(i ^ j));
@@ -483,27 +485,28 @@ __device__ __forceinline__ int delta(const unsigned long long *codes, int64_t n,
 }
 
 // Internal node i of the binary radix tree over n sorted codes.
-__device__ __forceinline__ void karras_node(int64_t i, int64_t n, const unsigned long long *codes,
+template <typename I>
+__device__ __forceinline__ void karras_node(I i, I n, const unsigned long long *codes,
                                             Node *__restrict__ nodes,
                                             uint32_t *__restrict__ parent_int,
                                             uint32_t *__restrict__ parent_leaf) {
     int d = (delta(codes, n, i, i + 1) - delta(codes, n, i, i - 1)) >= 0 ? 1 : -1;
     int dmin = delta(codes, n, i, i - d);
-    int64_t lmax = 2;
+    I lmax = 2;
     while (delta(codes, n, i, i + lmax * d) > dmin) lmax <<= 1;
-    int64_t l = 0;
-    for (int64_t t = lmax >> 1; t >= 1; t >>= 1)
+    I l = 0;
+    for (I t = lmax >> 1; t >= 1; t >>= 1)
         if (delta(codes, n, i, i + (l + t) * d) > dmin) l += t;
-    int64_t j = i + l * d;
+    const I j = i + l * d;
     int dnode = delta(codes, n, i, j);
-    int64_t s = 0;
-    for (int64_t div = 2;; div <<= 1) {
-        int64_t t = (l + div - 1) / div;
+    I s = 0;
+    for (I div = 2;; div <<= 1) {
+        const I t = (l + div - 1) / div;
         if (delta(codes, n, i, i + (s + t) * d) > dnode) s += t;
         if (t <= 1) break;
     }
-    int64_t gamma = i + s * d + (d < 0 ? -1 : 0);
-    int64_t lo = i < j ? i : j, hi = i < j ? j : i;
+    const I gamma = i + s * d + (d < 0 ? -1 : 0);
+    const I lo = i < j ? i : j, hi = i < j ? j : i;
     uint32_t left = (lo == gamma) ? (kLeafBit | (uint32_t)gamma) : (uint32_t)gamma;
     uint32_t right = (hi == gamma + 1) ? (kLeafBit | (uint32_t)(gamma + 1)) : (uint32_t)(gamma + 1);
     Node &nd = nodes[i];
@@ -515,11 +518,14 @@ __device__ __forceinline__ void karras_node(int64_t i, int64_t n, const unsigned
     if (right & kLeafBit) parent_leaf[gamma + 1] = (uint32_t)i; else parent_int[gamma + 1] = (uint32_t)i;
 }
 
-__global__ void k_karras(int64_t n, const unsigned long long *__restrict__ codes,
+// I: int where no index can pass 2^31 (n below 2^30), else 64 bits.
+template <typename I>
+__global__ void __launch_bounds__(256)
+    k_karras(I n, const unsigned long long *__restrict__ codes,
                          Node *__restrict__ nodes, uint32_t *__restrict__ parent_int,
                          uint32_t *__restrict__ parent_leaf) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n - 1) karras_node(i, n, codes, nodes, parent_int, parent_leaf);
+    const I i = (I)blockIdx.x * 256 + (I)threadIdx.x;
+    if (i < n - 1) karras_node<I>(i, n, codes, nodes, parent_int, parent_leaf);
 }
 
 // Up to kSmallMax Gaussians: boxes, bounds, codes, the sort and the tree in
@@ -616,7 +622,7 @@ __global__ void __launch_bounds__(kSmallThreads, 1)
     for (int i = tid; i < n; i += kSmallThreads) {
         codes[i] = s_key[i];
         vals[i] = s_val[i];
-        if (i < n - 1) karras_node(i, n, s_key, nodes, parent_int, parent_leaf);
+        if (i < n - 1) karras_node<int>(i, n, s_key, nodes, parent_int, parent_leaf);
     }
 }
 
@@ -638,7 +644,7 @@ __device__ __forceinline__ void write_record(PrimRec *__restrict__ prims, int64_
     for (int k = 0; k < 4; ++k) dst[k] = src[k];
 }
 
-// The W-wide hierarchies (W = 8, 16, 32) are cut out of the binary tree
+// The W-wide hierarchies (W = 8, 32) are cut out of the binary tree
 // bottom-up, in the box refit: k_W(p) is the number of children that the
 // wide node holding binary node p has below p, k_W(leaf) = 1. At a node
 // whose children together exceed W, the one with more is closed: it becomes
@@ -650,21 +656,21 @@ __device__ __forceinline__ void write_record(PrimRec *__restrict__ prims, int64_
 // N=4 spp 16 46.7 -> 33.8, 3M with 8-bit records 100.6 -> 48.7; and the cut
 // costs the refit little where listing, counting and scanning each width
 // took kernels of their own (frame at spp 1 6.65 -> 6.14 ms). Four words per internal node p, one
-// byte (bits 0-7, 8-15, 16-23) per W:
+// byte (bits 0-7, 8-15) per W:
 //   x  parent
 //   y  children of its wide node left of p's within the parent (0 when p is
 //      the left child); bit 24 + w: p is closed in tree w
 //   z  k_W(p)
 //   w  children below p's left child; bit 24 + w: that child is closed,
 //      bit 27 + w: the right one is
-constexpr uint32_t kLeafCounts = 0x010101u;  // one child in each of the three
-constexpr uint32_t kRootClosed = 7u << 24;
+constexpr uint32_t kLeafCounts = 0x0101u;  // one child in each of the two
+constexpr uint32_t kRootClosed = 3u << 24;
 
 __device__ __forceinline__ uint32_t close_children(uint32_t &kl, uint32_t &kr) {
     uint32_t closed = 0, nl = 0, nr = 0;
 #pragma unroll
     for (int w = 0; w < kGroupTrees; ++w) {
-        const uint32_t W = 8u << w;
+        const uint32_t W = group_width(w);
         uint32_t a = (kl >> (8 * w)) & 255u, b = (kr >> (8 * w)) & 255u;
         if (a + b > W) {
             const bool left = a >= b;
@@ -683,37 +689,163 @@ __device__ __forceinline__ uint32_t close_children(uint32_t &kl, uint32_t &kr) {
     return closed;  // bits 0-2: the left child, 3-5: the right one
 }
 
-// One thread per leaf (tree position i): write the Gaussian record, then
-// carry boxes towards the root; the second thread to reach a node merges
-// both child boxes, cuts the wide trees there (link != null) and continues.
-__global__ void k_leaves(int64_t n, const uint32_t *__restrict__ order,
-                         const float *__restrict__ means, const float *__restrict__ log_scales,
-                         const float *__restrict__ quats, const float *__restrict__ logits,
-                         const float *__restrict__ aabb, PrimRec *__restrict__ prims,
-                         Node *__restrict__ nodes, const uint32_t *__restrict__ parent_int,
-                         const uint32_t *__restrict__ parent_leaf, uint32_t *__restrict__ arrive,
-                         uint4 *__restrict__ link) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    uint32_t g = order[i];
-    Activated a = activate(means, log_scales, quats, logits, g);
-    write_record(prims, i, g, a);
+// Wide tree links of node p once both children are known (kl, kr: their
+// counts); returns p's own counts.
+__device__ __forceinline__ uint32_t cut_node(uint32_t p, uint2 child, uint32_t kl, uint32_t kr,
+                                             uint4 *__restrict__ link) {
+    const uint32_t closed = close_children(kl, kr);
+    if (!(child.x & kLeafBit))
+        __stcg(reinterpret_cast<uint2 *>(link + child.x), make_uint2(p, (closed & 7u) << 24));
+    if (!(child.y & kLeafBit))
+        __stcg(reinterpret_cast<uint2 *>(link + child.y), make_uint2(p, kl | (closed >> 3) << 24));
+    if (p == 0) __stcg(reinterpret_cast<uint2 *>(link), make_uint2(0u, kRootClosed));
+    __stcg(reinterpret_cast<uint2 *>(link + p) + 1, make_uint2(kl + kr, kl | closed << 24));
+    return kl + kr;
+}
+
+// Records in tree order, box refit and the cut of the wide trees (link !=
+// null). A Karras node is numbered by one end of its leaf range, so the nodes
+// over leaves of one block lie among that block's node numbers: those (more
+// than 9 of 10) are refitted in shared memory, in rounds: a round's ready
+// nodes are listed densely, one thread each, and a node is ready when its
+// second child arrives. (A thread per leaf that climbs while it arrives second
+// leaves one lane in ten working.) What leaves the block is listed for
+// k_climb.
+constexpr int kLeafThreads = 256;
+
+__global__ void __launch_bounds__(kLeafThreads)
+    k_leaves(int64_t n, const uint32_t *__restrict__ order, const float *__restrict__ means,
+             const float *__restrict__ log_scales, const float *__restrict__ quats,
+             const float *__restrict__ logits, const float *__restrict__ aabb,
+             PrimRec *__restrict__ prims, Node *__restrict__ nodes,
+             const uint32_t *__restrict__ parent_int, const uint32_t *__restrict__ parent_leaf,
+             uint4 *__restrict__ link, uint32_t *__restrict__ exits,
+             uint32_t *__restrict__ n_exits) {
+    __shared__ uint2 s_child[kLeafThreads];
+    __shared__ uint32_t s_parent[kLeafThreads];
+    __shared__ uint32_t s_arrive[kLeafThreads];
+    __shared__ uint32_t s_counts[kLeafThreads][2];
+    __shared__ float s_box[kLeafThreads][2][6];
+    __shared__ bool s_near[kLeafThreads];  // the node covers leaves of this block only
+    __shared__ uint16_t s_ready[2][kLeafThreads];
+    __shared__ uint32_t s_exit[kLeafThreads];
+    __shared__ uint32_t s_n[2], s_n_exit;
+    const int tid = threadIdx.x;
+    const uint32_t b0 = blockIdx.x * kLeafThreads;
+    const int64_t i = (int64_t)b0 + tid;
+    {
+        bool near = false;
+        if (i < n - 1) {
+            const uint4 c = *reinterpret_cast<const uint4 *>(nodes[i].child);  // children, range
+            s_child[tid] = make_uint2(c.x, c.y);
+            s_parent[tid] = parent_int[i];
+            near = c.z >= b0 && c.w < b0 + kLeafThreads;
+        }
+        s_near[tid] = near;
+        s_arrive[tid] = 0;
+        if (tid < 2) s_n[tid] = 0;
+        if (tid == 2) s_n_exit = 0;
+    }
+    __syncthreads();
+    // hands a finished child (its box, counts) to its parent q
+    auto arrive_at = [&](uint32_t ref, uint32_t q, const float box[6], uint32_t counts, int next) {
+        const uint32_t j = q - b0;
+        if (j < (uint32_t)kLeafThreads && s_near[j]) {
+            const int side = s_child[j].x == ref ? 0 : 1;
+            for (int k = 0; k < 6; ++k) s_box[j][side][k] = box[k];
+            s_counts[j][side] = counts;
+            __threadfence_block();
+            if (atomicAdd(&s_arrive[j], 1u) == 1u) s_ready[next][atomicAdd(&s_n[next], 1u)] = (uint16_t)j;
+        } else {
+            s_exit[atomicAdd(&s_n_exit, 1u)] = ref;
+        }
+    };
+    if (i < n) {
+        const uint32_t g = order[i];
+        const Activated a = activate(means, log_scales, quats, logits, g);
+        write_record(prims, i, g, a);
+        float box[6];
+        for (int k = 0; k < 6; ++k) box[k] = aabb[6 * (int64_t)g + k];
+        arrive_at(kLeafBit | (uint32_t)i, parent_leaf[i], box, kLeafCounts, 0);
+    }
+    __syncthreads();
+    for (int now = 0;; now ^= 1) {
+        const uint32_t n_ready = s_n[now];
+        __syncthreads();
+        if (n_ready == 0) break;
+        if (tid == 0) s_n[now] = 0;
+        if (tid < (int)n_ready) {
+            const int j = s_ready[now][tid];
+            const uint32_t p = b0 + (uint32_t)j;
+            const volatile float *l = s_box[j][0], *r = s_box[j][1];
+            float bl[6], br[6], box[6];
+            for (int k = 0; k < 6; ++k) {
+                bl[k] = l[k];
+                br[k] = r[k];
+            }
+            for (int k = 0; k < 3; ++k) {
+                box[k] = fminf(bl[k], br[k]);
+                box[3 + k] = fmaxf(bl[3 + k], br[3 + k]);
+            }
+            float4 *out = reinterpret_cast<float4 *>(nodes[p].box);
+            out[0] = make_float4(bl[0], bl[1], bl[2], bl[3]);
+            out[1] = make_float4(bl[4], bl[5], br[0], br[1]);
+            out[2] = make_float4(br[2], br[3], br[4], br[5]);
+            uint32_t counts = kLeafCounts;
+            if (link) counts = cut_node(p, s_child[j], s_counts[j][0], s_counts[j][1], link);
+            if (p != 0) arrive_at(p, s_parent[j], box, counts, now ^ 1);
+        }
+        __syncthreads();
+    }
+    // a block lists at most one exit per leaf
+    if (tid == 0) s_n[0] = s_n_exit ? atomicAdd(n_exits, s_n_exit) : 0u;
+    __syncthreads();
+    if (tid < (int)s_n_exit) exits[s_n[0] + tid] = s_exit[tid];
+}
+
+// The exits of k_leaves, one thread each, carried to the root: the second to
+// reach a node merges both boxes and continues. A launch of its own: climbing
+// at the end of k_leaves, a few threads held their block's place on the SM
+// through a dozen meetings in memory each.
+__device__ __forceinline__ uint32_t arrive_acq_rel(uint32_t *counter) {
+    uint32_t old;
+    asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], 1;" : "=r"(old) : "l"(counter) : "memory");
+    return old;
+}
+
+__global__ void __launch_bounds__(64)
+    k_climb(const uint32_t *__restrict__ exits, const uint32_t *__restrict__ n_exits,
+            const uint32_t *__restrict__ order, const float *__restrict__ aabb,
+            Node *__restrict__ nodes, const uint32_t *__restrict__ parent_int,
+            const uint32_t *__restrict__ parent_leaf, uint32_t *__restrict__ arrive,
+            uint4 *__restrict__ link) {
+    const uint32_t e = blockIdx.x * 64 + threadIdx.x;
+    if (e >= *n_exits) return;
+    uint32_t ref = exits[e], p, counts = kLeafCounts;
     float box[6];
-    for (int k = 0; k < 6; ++k) box[k] = aabb[6 * (int64_t)g + k];
-    uint32_t ref = kLeafBit | (uint32_t)i;
-    uint32_t p = parent_leaf[i];
-    uint32_t counts = kLeafCounts;
+    if (ref & kLeafBit) {
+        const uint32_t leaf = ref & ~kLeafBit;
+        const int64_t g = order[leaf];
+        for (int k = 0; k < 6; ++k) box[k] = aabb[6 * g + k];
+        p = parent_leaf[leaf];
+    } else {
+        const float *l = nodes[ref].box[0], *r = nodes[ref].box[1];
+        for (int k = 0; k < 3; ++k) {
+            box[k] = fminf(l[k], r[k]);
+            box[3 + k] = fmaxf(l[3 + k], r[3 + k]);
+        }
+        if (link) counts = link[ref].z;
+        p = parent_int[ref];
+    }
     for (int guard = 0; guard < 4096; ++guard) {
         Node *nd = nodes + p;
         const uint2 child = __ldcg(reinterpret_cast<const uint2 *>(nd->child));
+        const uint32_t next = parent_int[p];
         const int side = child.x == ref ? 0 : 1;
         // a child's box is 24 bytes at an 8-byte boundary
         float2 *mine = reinterpret_cast<float2 *>(nd->box[side]);
         for (int k = 0; k < 3; ++k) __stcg(mine + k, make_float2(box[2 * k], box[2 * k + 1]));
-        if (link && !(ref & kLeafBit)) __stcg(&link[ref].z, counts);
-        __threadfence();
-        if (atomicAdd(&arrive[p], 1u) == 0u) return;
-        __threadfence();
+        if (arrive_acq_rel(&arrive[p]) == 0u) return;
         const float2 *other = reinterpret_cast<const float2 *>(nd->box[1 - side]);
         float ob[6];
         for (int k = 0; k < 3; ++k) {
@@ -724,29 +856,15 @@ __global__ void k_leaves(int64_t n, const uint32_t *__restrict__ order,
         if (link) {
             const uint32_t sib = side ? child.x : child.y;
             const uint32_t oc = (sib & kLeafBit) ? kLeafCounts : __ldcg(&link[sib].z);
-            uint32_t kl = side ? oc : counts, kr = side ? counts : oc;
-            const uint32_t closed = close_children(kl, kr);
-            if (!(child.x & kLeafBit))
-                __stcg(reinterpret_cast<uint2 *>(link + child.x), make_uint2(p, (closed & 7u) << 24));
-            if (!(child.y & kLeafBit))
-                __stcg(reinterpret_cast<uint2 *>(link + child.y),
-                       make_uint2(p, kl | (closed >> 3) << 24));
-            __stcg(&link[p].w, kl | closed << 24);
-            counts = kl + kr;
+            counts = cut_node(p, child, side ? oc : counts, side ? counts : oc, link);
         }
         for (int k = 0; k < 3; ++k) {
             box[k] = fminf(box[k], ob[k]);
             box[3 + k] = fmaxf(box[3 + k], ob[3 + k]);
         }
-        if (p == 0) {
-            if (link) {
-                __stcg(reinterpret_cast<uint2 *>(link), make_uint2(0u, kRootClosed));
-                __stcg(&link[0].z, counts);
-            }
-            return;
-        }
+        if (p == 0) return;
         ref = p;
-        p = parent_int[p];
+        p = next;
     }
 }
 
@@ -877,7 +995,7 @@ __global__ void k_collapse(int64_t n_int, const Node *__restrict__ nodes,
 
 // Reference of the wide node at every closed binary node: a block adds up its
 // nodes' record counts (plus `header` units each), takes its range of the
-// three trees' records with one atomic per tree, and hands it out in node
+// trees' records with one atomic per tree, and hands it out in node
 // order. The order of the blocks' ranges varies from run to run; a reference
 // is never compared, so no result depends on it.
 struct WideRefs {
@@ -986,7 +1104,7 @@ struct WideOut {
     void *rec[kGroupTrees];
 };
 
-// Writes the child records of the three wide trees, one thread per binary
+// Writes the child records of the wide trees, one thread per binary
 // internal node, each record by itself: the thread whose child is a leaf or
 // closed climbs to the wide node it belongs to (a few levels, one link each)
 // and adds up the children to its left on the way. All reads of its own node
@@ -1007,8 +1125,8 @@ __global__ void __launch_bounds__(256)
     uint4 l = __ldg(link + i);
     const uint32_t left = l.w;
     uint32_t need[2];  // trees in which the child is a record of its own
-    need[0] = (cref.x & kLeafBit) ? 7u : (left >> 24) & 7u;
-    need[1] = (cref.y & kLeafBit) ? 7u : (left >> 27) & 7u;
+    need[0] = (cref.x & kLeafBit) ? 3u : (left >> 24) & 3u;
+    need[1] = (cref.y & kLeafBit) ? 3u : (left >> 27) & 3u;
     if (cref.x == cref.y) need[1] = 0u;  // a single Gaussian
     uint32_t todo = need[0] | need[1];
     uint32_t cur = (uint32_t)i, pos = 0;  // children left of node i, one byte per tree
@@ -1076,7 +1194,10 @@ inline unsigned grid_for(int64_t n, int threads) {
 int64_t radix_tiles(int64_t n) { return (n + kSortTile - 1) / kSortTile; }
 
 size_t sort_scratch_bytes(int64_t n) { return ZeroScratch(n, 0).bytes; }
-size_t build_scratch_bytes(int64_t n) { return ZeroScratch(n, n + kGroupTrees).bytes; }
+// (arrival counters, the wide record allocators, the number of exits)
+constexpr int kBuildCounters = kGroupTrees + 1;
+
+size_t build_scratch_bytes(int64_t n) { return ZeroScratch(n, n + kBuildCounters).bytes; }
 
 int sort_keys64(unsigned long long *keys[2], int64_t n, int lo_bit, void *scratch,
                 uint32_t *status, cudaStream_t s) {
@@ -1107,7 +1228,7 @@ gs_status build_into(gs_bvh *b, const gs_gaussians *g, cudaStream_t s) {
     b->n_nodes = M == 0 ? 0 : (M == 1 ? 1 : M - 1);
     if (M == 0) return GS_OK;
     cudaError_t e;
-    const ZeroScratch z(M, M + kGroupTrees);
+    const ZeroScratch z(M, M + kBuildCounters);
     unsigned char *base = static_cast<unsigned char *>(b->zero);
     unsigned int *bounds = reinterpret_cast<unsigned int *>(base);
     uint32_t *hist = reinterpret_cast<uint32_t *>(base + z.hist);
@@ -1121,7 +1242,7 @@ gs_status build_into(gs_bvh *b, const gs_gaussians *g, cudaStream_t s) {
             return cuda_fail(e, "small build setup");
         k_small<<<1, kSmallThreads, kSmallBytes, s>>>(
             (int)M, g->means, g->log_scales, g->quats, g->opacity_logits, b->aabb, b->codes[0],
-            b->vals[0], b->nodes, parent_int, parent_leaf, arrive, (int)M + kGroupTrees, b->status);
+            b->vals[0], b->nodes, parent_int, parent_leaf, arrive, (int)M + kBuildCounters, b->status);
     } else {
         if ((e = cudaMemsetAsync(base, 0, z.bytes, s)) != cudaSuccess)
             return cuda_fail(e, "memset build scratch");
@@ -1144,12 +1265,20 @@ gs_status build_into(gs_bvh *b, const gs_gaussians *g, cudaStream_t s) {
         k_single<<<1, 1, 0, s>>>(order, g->means, g->log_scales, g->quats, g->opacity_logits,
                                  b->aabb, b->prims, b->nodes, b->link);
     } else {
-        if (!small)
-            k_karras<<<grid_for(M - 1, 256), 256, 0, s>>>(M, b->codes[cur], b->nodes, parent_int,
-                                                           parent_leaf);
-        k_leaves<<<grid_for(M, 256), 256, 0, s>>>(M, order, g->means, g->log_scales, g->quats,
+        if (!small && M < (int64_t)1 << 30)
+            k_karras<int><<<grid_for(M - 1, 256), 256, 0, s>>>((int)M, b->codes[cur], b->nodes,
+                                                                parent_int, parent_leaf);
+        else if (!small)
+            k_karras<int64_t><<<grid_for(M - 1, 256), 256, 0, s>>>(M, b->codes[cur], b->nodes,
+                                                                    parent_int, parent_leaf);
+        k_leaves<<<grid_for(M, kLeafThreads), kLeafThreads, 0, s>>>(M, order, g->means, g->log_scales, g->quats,
                                                    g->opacity_logits, b->aabb, b->prims, b->nodes,
-                                                   parent_int, parent_leaf, arrive, b->link);
+                                                   parent_int, parent_leaf, b->link,
+                                                   b->vals[1 - cur], arrive + M + kGroupTrees);
+        if (M > kLeafThreads)
+            k_climb<<<grid_for(M, 64), 64, 0, s>>>(b->vals[1 - cur], arrive + M + kGroupTrees, order,
+                                                   b->aabb, b->nodes, parent_int, parent_leaf, arrive,
+                                                   b->link);
     }
     if (b->node_format == GS_NODES_WIDE4 || b->node_format == GS_NODES_WIDE4_Q8) {
         const int64_t n_int = b->n_nodes;

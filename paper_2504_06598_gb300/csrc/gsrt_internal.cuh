@@ -43,8 +43,8 @@ struct __align__(16) Node4 {
 };
 static_assert(sizeof(Node4) == 128, "Node4 must be 128 bytes");
 
-// Child record of the W-wide hierarchies (W = 8, 16, 32) that groups of W
-// lanes traverse, 32 bytes, one lane's load. A wide node is the run of its
+// Child record of the W-wide hierarchies (W = 8, 32) that groups of lanes
+// and warps traverse, 32 bytes, one lane's load. A wide node is the run of its
 // children's records (2 to W) at its offset; an internal child is
 // referenced as (count - 1) << 26 | offset, a leaf as kLeafBit | primitive
 // index.
@@ -80,7 +80,14 @@ constexpr int kGroupQHeaderUnits = 2;
 constexpr uint32_t kQ8Skip = 1u << 16;  // q1 flag: a child with a non-finite box
 constexpr int kWideCountShift = 26;
 constexpr uint32_t kWideOffsetMask = (1u << kWideCountShift) - 1u;
-constexpr int kGroupTrees = 3;  // W = 8 << i
+constexpr int kGroupTrees = 2;
+// Their widths: 8 for groups of 8 and 16 lanes, 32 for whole warps. (A 16-wide
+// tree served only groups of 16 lanes, which the library's own choices no
+// longer form; a 4-wide one for rays walked by a lane each made the batched
+// frame slower, 427 ms against 353 on the binary nodes.)
+__host__ __device__ constexpr uint32_t group_width(int tree) { return tree == 0 ? 8u : 32u; }
+constexpr int kWarpTree = 1;
+constexpr int group_tree(int lanes_log2) { return lanes_log2 >= 5 ? kWarpTree : 0; }
 
 // One W-wide hierarchy: records (ChildRec, or 16-byte units of the 8-bit
 // form), and per binary internal node the reference of the wide node there
@@ -148,7 +155,7 @@ struct gs_bvh {
     uint32_t *depth;    // depth of every internal binary node
     uint32_t *wmap;     // binary internal node -> wide node index
     // W-wide hierarchies for groups of lanes sharing one ray (binary format
-    // formats only): W = 8, 16, 32, each at most M + (M - 1) records
+    // formats only): W = 8, 32, each at most M + (M - 1) records
     gsrt::GroupTree group[gsrt::kGroupTrees];
     uint4 *link;  // per binary internal node: its place in the wide trees (build.cu)
     float *grad;  // [M][10] sums of a gradient launch (backward.cu)

@@ -272,6 +272,7 @@ __device__ __forceinline__ float shared_draws(const TraceArgs &a, SharedWarp &m,
     r.t_max = a.t_max;
     r.any_hit = false;
     update_clip(r, a.t_max);
+    if (!(r.t_far > -INFINITY)) r.t_far = -INFINITY;  // no sample here
     const uint32_t depth = (__float_as_uint(fmaxf(ct, 0.0f)) & ~31u) | (uint32_t)lane;
     bool drawn = false;
     for (;;) {
@@ -463,6 +464,8 @@ __global__ void __launch_bounds__(kThreads, 8) k_trace_shared(const __grid_const
                     r.t_min = a.t_min;
                     r.t_max = a.t_max;
                     r.any_hit = false;
+                    update_clip(r, a.t_max);
+                    if (!(r.t_far > -INFINITY)) r.t_far = -INFINITY;
                     start_over<2>(a, r, s0 >> 1, err);
                 }
                 float Y[16];
@@ -678,15 +681,15 @@ gs_status launch_trace(const gs_bvh *b, const gs_gaussians *g, const gs_pinhole 
     a.wide = b->wide;
     a.lpp_log2 = lpp_log2;
     if (b->link && a.lpp_log2 >= 3) {
-        a.grec = b->group[a.lpp_log2 - 3].rec;
-        a.groot = b->group[a.lpp_log2 - 3].ref;
+        a.grec = b->group[group_tree(a.lpp_log2)].rec;
+        a.groot = b->group[group_tree(a.lpp_log2)].ref;
     } else {
         a.grec = nullptr;
         a.groot = nullptr;
     }
     a.gq8 = b->node_format == GS_NODES_BINARY_Q8;
-    a.trec = tile || shared ? b->group[2].rec : nullptr;
-    a.troot = tile || shared ? b->group[2].ref : nullptr;
+    a.trec = tile || shared ? b->group[kWarpTree].rec : nullptr;
+    a.troot = tile || shared ? b->group[kWarpTree].ref : nullptr;
     a.prims = b->prims;
     a.sh = g->sh;
     a.n_nodes = b->n_nodes;

@@ -1139,7 +1139,7 @@ constexpr int kTilePool = 256;  // stack entries per warp
 // Fills the warp's pyramid from each lane's direction d (away from the apex,
 // any length; `in` marks the lanes that count). false when the rays spread
 // too far for it (or none counts): the caller then traverses otherwise.
-__device__ __forceinline__ bool tile_pyramid(const float d[3], bool in, float *pyr) {
+__device__ __forceinline__ void tile_pyramid(const float d[3], bool in, float *pyr) {
     const uint32_t kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const float n = rsqrtf(fmaf(d[0], d[0], fmaf(d[1], d[1], d[2] * d[2])));
@@ -1359,18 +1359,12 @@ __device__ __noinline__ void tile_fallback(const TraceArgs &a, Ray<N> &r, int pa
     traverse_packet<N, false>(a, r, pass, stack, stack_t, err, cnt);
 }
 
-// A walk whose stack was full started over on the binary nodes: every slot but
-// the unused ones (at -inf with no Gaussian) is emptied again.
+// A walk whose stack was full, again on the binary nodes. The slots stay: a
+// Gaussian met a second time is not closer than the hit it made.
 template <int N>
 __device__ __forceinline__ void start_over(const TraceArgs &a, Ray<N> &r, int pass, uint32_t &err) {
     Ray<N> again = r;
     set_ray(again, r.o, r.d);
-#pragma unroll
-    for (int k = 0; k < N; ++k)
-        if (!(r.slot[k].gid == 0xffffffffu && r.slot[k].tc == -INFINITY))
-            again.slot[k] = Slot{INFINITY, 0.0f, 0xffffffffu};
-    update_clip(again, r.t_max);
-    if (!(again.t_far > -INFINITY)) again.t_far = -INFINITY;
     uint32_t err2 = 0;
     tile_fallback<N>(a, again, pass, err2);
     err |= err2;

@@ -926,13 +926,13 @@ gs_status launch_render_views(const gs_bvh *b, const gs_gaussians *g, const gs_p
     a.work = b->status + 1;
     a.lpp_log2 = whole_warp ? 5 : lanes_per_pixel_log2(a.spp);
     if (b->link && a.lpp_log2 >= 3) {
-        a.grec = b->group[a.lpp_log2 - 3].rec;
-        a.groot = b->group[a.lpp_log2 - 3].ref;
+        a.grec = b->group[group_tree(a.lpp_log2)].rec;
+        a.groot = b->group[group_tree(a.lpp_log2)].ref;
         a.gq8 = b->node_format == GS_NODES_BINARY_Q8;
     }
     if (tiles_ok && a.lpp_log2 < 3) {
-        a.trec = b->group[2].rec;
-        a.troot = b->group[2].ref;
+        a.trec = b->group[kWarpTree].rec;
+        a.troot = b->group[kWarpTree].ref;
     }
     const int tw_lg = tile_w_log2(a.lpp_log2), th_lg = 5 - a.lpp_log2 - tw_lg;
     uint32_t tiles = 0;
