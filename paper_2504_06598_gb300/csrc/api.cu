@@ -81,7 +81,7 @@ static gs_status check_gaussians_device(const gs_gaussians *g, bool need_sh) {
 static void release(gs_bvh *b) {
     if (!b) return;
     void *bufs[] = {b->nodes, b->prims, b->status, b->codes[0], b->codes[1], b->vals[0],
-                    b->vals[1], b->parent, b->aabb, b->zero, b->scan_tmp, b->wide, b->depth, b->wmap, b->link, b->grad};
+                    b->vals[1], b->parent, b->aabb, b->zero, b->scan_tmp, b->wide, b->depth, b->wmap, b->link, b->grad, b->regions};
     for (void *p : bufs)
         if (p) cudaFree(p);
     for (auto &t : b->group) {
@@ -166,6 +166,7 @@ gs_status gs_build_bvh_ex(const gs_gaussians *g, const gs_build_options *opt, gs
         {(void **)&b->depth, wide ? (size_t)nn * 4 : 0},
         {(void **)&b->wmap, wide ? (size_t)nn * 4 : 0},
         {(void **)&b->link, grouped ? (size_t)nn * sizeof(uint4) : 0},
+        {(void **)&b->regions, grouped ? (size_t)2 * 4096 * 4 : 0},
         {(void **)&b->grad, grouped ? (size_t)cap * 10 * sizeof(float) : 0},
         {(void **)&b->group[0].rec, grouped ? (size_t)recs * rec_bytes : 0},
         {(void **)&b->group[0].ref, grouped ? (size_t)nn * 4 : 0},
@@ -188,6 +189,11 @@ gs_status gs_build_bvh_ex(const gs_gaussians *g, const gs_build_options *opt, gs
     if (e != cudaSuccess) {
         release(b);
         return cuda_fail(e, "memset status");
+    }
+    if (b->regions &&
+        (e = cudaMemsetAsync(b->regions, 0, 2 * 4096 * 4, (cudaStream_t)stream)) != cudaSuccess) {
+        release(b);
+        return cuda_fail(e, "memset regions");
     }
     st = build_into(b, g, (cudaStream_t)stream);
     if (st != GS_OK) {

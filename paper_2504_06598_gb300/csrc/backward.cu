@@ -17,10 +17,11 @@
 // traversal clipped at the winners' depths enumerates the Gaussians in
 // front of them. Gradients are accumulated with atomics: in
 // the per-lane form reduced across the warp for the warp's shared leaf; in
-// the grouped form (8 or more lanes on one pixel, the wide copy of that
-// width) the chain rule runs once per Gaussian and group on the lanes'
-// summed weights, and lanes whose slot holds the same Gaussian add its
-// colour gradient once.
+// the grouped form (8 or more lanes on one pixel) the chain rule runs once per
+// Gaussian and group on the lanes' summed weights, and lanes whose slot holds
+// the same Gaussian add its colour gradient once; the tile form (a warp of
+// camera rays, the usual one) reduces ten sums per Gaussian and applies the
+// chain rule after the launch.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -296,7 +297,7 @@ __device__ void enumerate_packet(const TraceArgs &a, const Ray<N> &r, const floa
 }
 
 // Grouped enumeration (groups of L = 2^LG lanes sharing one ray, the
-// W-wide copy with W = L): the same leaves as enumerate_packet for each
+// wide copy of at most L children): the same leaves as enumerate_packet for each
 // lane, visited once per group. The lane holding a hit leaf evaluates the
 // candidate and its colour; every lane adds its own samples' weight
 // sum_k g . (c_i - c_k) over the slots the candidate is in front of; the
@@ -733,8 +734,10 @@ __device__ __forceinline__ void add_sh_gradient(const TraceArgs &a, uint32_t gid
             for (int i = 0; i < K; ++i) atomicAdd(dst + 3 * i + ch, gm[ch] * Y[i]);
 }
 
+// Built for five blocks per SM with eight slots (four: 1M at 1080p, spp 16,
+// rebuild + image + gradients 17.6 -> 16.9 ms) and six with fewer.
 template <int N, bool Q8, bool KEYS>
-__global__ void __launch_bounds__(kThreads, N >= 8 ? 4 : 5)
+__global__ void __launch_bounds__(kThreads, N >= 8 ? 5 : 6)
     k_backward_tile(const __grid_constant__ TraceArgs a) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t kAll = 0xffffffffu;
@@ -753,9 +756,9 @@ __global__ void __launch_bounds__(kThreads, N >= 8 ? 4 : 5)
     uint32_t err = 0;
     for (;;) {
         uint32_t tile = 0;
-        if (lane == 0) tile = atomicAdd(a.work, 1u);
-        tile = __shfl_sync(kAll, tile, 0);
-        if (tile >= n_tiles) break;
+        const int more = next_tile(a, tiles_x, n_tiles, tile);
+        if (more == 0) break;
+        if (more < 0) continue;
         const int x = (int)(((tile % tiles_x) << tw_lg) + (pl & ((1 << tw_lg) - 1)));
         const int y = (int)(((tile / tiles_x) << th_lg) + (pl >> tw_lg));
         const bool valid = x < a.width && y < a.height;
@@ -924,7 +927,7 @@ gs_status launch_backward_nl(const TraceArgs &a, cudaStream_t s) {
     return GS_OK;
 }
 
-// Groups of 8 or more lanes on one pixel use the wide copy of their width.
+// Groups of 8 or more lanes on one pixel use the widest copy that fits them.
 template <int N, bool Q8, bool KEYS>
 gs_status launch_backward_tile(const TraceArgs &a, cudaStream_t s) {
     int dev = 0, sms = 0, per = 0;
@@ -940,7 +943,8 @@ gs_status launch_backward_tile(const TraceArgs &a, cudaStream_t s) {
     uint32_t blocks = (uint32_t)sms * (uint32_t)(per > 0 ? per : 1);
     const uint32_t max_blocks = (tiles + kThreads / 32 - 1) / (kThreads / 32);
     if (blocks > max_blocks) blocks = max_blocks;
-    if ((e = cudaMemsetAsync(a.work, 0, sizeof(uint32_t), s)) != cudaSuccess)
+    if (a.order == nullptr &&
+        (e = cudaMemsetAsync(a.work, 0, sizeof(uint32_t), s)) != cudaSuccess)
         return cuda_fail(e, "reset work counter");
     if ((e = cudaMemsetAsync(a.g_stats, 0, (size_t)a.n_gauss * kStats * sizeof(float), s)) != cudaSuccess)
         return cuda_fail(e, "reset gradient sums");
@@ -987,6 +991,10 @@ gs_status launch_backward_n(const TraceArgs &a, cudaStream_t s) {
 // 15.0, per-lane packets), else K = 2 (spp 16: 49.4 -> 46.0, spp 64:
 // 104.8 -> 59.8, 16- and 32-lane groups); never fewer than n_hits (N = 4
 // at spp 4 and 16 keeps S = 1: 48.1 and 77.8 ms against 50.1 and 103.8).
+// The tile form evaluates a Gaussian once per lane whatever the lane carries,
+// so a lane takes as many samples as it can: K = 4 below T = 8, else 8 (1M at
+// 1080p, spp 16, from stored payloads 19.5 ms grouped with two -> 6.3 with
+// eight).
 static int auto_backward_samples_per_lane(int spp, int n_hits, bool tile) {
     const int64_t T = (int64_t)spp * n_hits;
     int K = T <= 2 ? (int)T : (T < 16 ? 4 : 2);
@@ -1068,6 +1076,13 @@ gs_status launch_backward(const gs_bvh *b, const gs_gaussians *g, const gs_pinho
     a.g_quats = d_quats;
     a.g_logits = d_logits;
     a.g_sh = d_sh;
+    if (tile) {
+        int dev = 0, sms = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (((int64_t)a.width * a.height << a.lpp_log2) > (int64_t)sms * 3 * 16 * 32)
+            order_regions(b, a, tile_w_log2(a.lpp_log2), 5 - a.lpp_log2 - tile_w_log2(a.lpp_log2), s);
+    }
     gs_status st;
     switch (p->n_hits * S) {
         case 1: st = launch_backward_n<1>(a, s); break;

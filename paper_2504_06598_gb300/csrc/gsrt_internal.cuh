@@ -158,6 +158,7 @@ struct gs_bvh {
     // formats only): W = 8, 32, each at most M + (M - 1) records
     gsrt::GroupTree group[gsrt::kGroupTrees];
     uint4 *link;  // per binary internal node: its place in the wide trees (build.cu)
+    uint32_t *regions;  // [2][4096] counts (zero between launches) and order of image regions
     float *grad;  // [M][10] sums of a gradient launch (backward.cu)
     // scratch of the batched form's deferred bounce rays, grown on demand
     int64_t wave_cap;                    // sample slots (pixels x spp) held

@@ -6,9 +6,11 @@
 // sub, sub + L, ... of the same camera ray (L the largest power of two not
 // above the passes, at most 32), so they share their ray and differ only in
 // the random draws and the clips they cause; with one pass per pixel the
-// tile is 8x4 pixels. With 8 or more lanes on a pixel the group walks the
-// L-wide copy together (traverse_group), otherwise the warp traverses as a
-// packet (traverse_packet). Each pass is one traversal of the hierarchy
+// tile is 8x4 pixels. With 8 or more lanes on a pixel the group walks a wide
+// copy together (traverse_group), otherwise the warp traverses as a tile
+// (traverse_tile) or, for the options that are about the per-lane walk, as a
+// packet (traverse_packet). Above 32 samples a pixel one walk serves four
+// pixels (k_trace_shared). Each pass is one traversal of the hierarchy
 // (Sec. 3.2) keeping its closest accepted intersections (Sec. 3.5). At every
 // leaf the intersection routine of Alg. 1 runs:
 //   t    mean of the 1D Gaussian along the ray (Sec. 3.1)
@@ -41,8 +43,8 @@
 namespace gsrt {
 namespace {
 
-// Template values of FMT for the cooperative traversal of the W-wide records
-// by groups of W = 8, 16, 32 lanes on one pixel: kFmtGroup + log2 W for the
+// Template values of FMT for the cooperative traversal of the wide records by
+// groups of L = 8, 16, 32 lanes on one pixel: kFmtGroup + log2 L for the
 // FP32 records, kFmtGroupQ8 + log2 W for the 8-bit ones; the others are
 // GS_NODES_*.
 constexpr int kFmtGroup = 8;
@@ -97,9 +99,9 @@ __global__ void __launch_bounds__(kThreads, is_group_fmt(FMT) ? group_min_blocks
     float *pyr = s_pyr[tiled ? threadIdx.x >> 5 : 0];
     for (;;) {
         uint32_t tile = 0;
-        if (lane == 0) tile = atomicAdd(a.work, 1u);
-        tile = __shfl_sync(kAll, tile, 0);
-        if (tile >= n_tiles) break;
+        const int more = next_tile(a, tiles_x, n_tiles, tile);
+        if (more == 0) break;
+        if (more < 0) continue;
         const int x = (int)(((tile % tiles_x) << tw_lg) + (pl & ((1 << tw_lg) - 1)));
         const int y = (int)(((tile / tiles_x) << th_lg) + (pl >> tw_lg));
         const bool valid = x < a.width && y < a.height;
@@ -329,9 +331,9 @@ __global__ void __launch_bounds__(kThreads, 8) k_trace_shared(const __grid_const
     uint32_t err = 0;
     for (;;) {
         uint32_t tile = 0;
-        if (lane == 0) tile = atomicAdd(a.work, 1u);
-        tile = __shfl_sync(kAll, tile, 0);
-        if (tile >= n_tiles) break;
+        const int more = next_tile(a, tiles_x, n_tiles, tile);
+        if (more == 0) break;
+        if (more < 0) continue;
         const int x0 = (int)(tile % tiles_x) * 2, y0 = (int)(tile / tiles_x) * 2;
         Ray<1> er;  // the ray this lane evaluates along
         const bool valid = x0 + (ep & 1) < a.width && y0 + (ep >> 1) < a.height;
@@ -543,7 +545,8 @@ gs_status launch_shared(const TraceArgs &a, cudaStream_t s) {
     const int64_t tiles = (int64_t)((a.width + 1) >> 1) * ((a.height + 1) >> 1);
     const int64_t need = (tiles + kThreads / 32 - 1) / (kThreads / 32);
     const int64_t fit = (int64_t)sms * (per > 0 ? per : 1);
-    if ((e = cudaMemsetAsync(a.work, 0, sizeof(uint32_t), s)) != cudaSuccess)
+    if (a.order == nullptr &&
+        (e = cudaMemsetAsync(a.work, 0, sizeof(uint32_t), s)) != cudaSuccess)
         return cuda_fail(e, "reset work counter");
     k_trace_shared<Q8><<<(unsigned)(need < fit ? need : fit), kThreads, 0, s>>>(a);
     return GS_OK;
@@ -566,7 +569,8 @@ gs_status launch_nf(const TraceArgs &a, bool count, cudaStream_t s) {
     uint32_t blocks = (uint32_t)sms * (uint32_t)(per > 0 ? per : 1);
     const uint32_t max_blocks = (warps_needed + kThreads / 32 - 1) / (kThreads / 32);
     if (blocks > max_blocks) blocks = max_blocks;
-    if ((e = cudaMemsetAsync(a.work, 0, sizeof(uint32_t), s)) != cudaSuccess)
+    if (a.order == nullptr &&
+        (e = cudaMemsetAsync(a.work, 0, sizeof(uint32_t), s)) != cudaSuccess)
         return cuda_fail(e, "reset work counter");
     if (count) k_trace<N, !is_tile_fmt(FMT), FMT><<<blocks, kThreads, 0, s>>>(a);
     else k_trace<N, false, FMT><<<blocks, kThreads, 0, s>>>(a);
@@ -740,6 +744,13 @@ gs_status launch_trace(const gs_bvh *b, const gs_gaussians *g, const gs_pinhole 
     }
     const bool count = p->counters != nullptr;
     gs_status st;
+    a.order = nullptr;
+    // below three waves the longest tile decides, whatever the order (90k at
+    // 411x307, 1.6 waves: 1119 us by rows, 1147 ordered)
+    if (shared ? (int64_t)((a.width + 1) >> 1) * ((a.height + 1) >> 1) > 3 * resident_warps()
+               : tile && tile_warps(a.width, a.height, a.lpp_log2) > 3 * resident_warps())
+        order_regions(b, a, shared ? 1 : tile_w_log2(a.lpp_log2),
+                      shared ? 1 : 5 - a.lpp_log2 - tile_w_log2(a.lpp_log2), s);
     if (shared) {
         st = a.gq8 ? launch_shared<true>(a, s) : launch_shared<false>(a, s);
         if (st != GS_OK) return st;

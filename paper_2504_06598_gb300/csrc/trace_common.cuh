@@ -52,6 +52,9 @@ struct TraceArgs {
     unsigned long long *counters;
     uint32_t *status;
     uint32_t *work;  // tile counter of the persistent launch
+    // heaviest regions first (or null: tiles row by row); see order_regions
+    const uint32_t *order;
+    int region_log2, regions_x, n_regions;
     int lpp_log2;    // log2 of the lanes that trace samples of one pixel
     int k_log2;      // log2 of the slots of a pass (shared walks)
     int depth_mode;  // 0: 1D mean; 1: centre projected on fwd (camera rays)
@@ -1377,6 +1380,110 @@ __device__ __forceinline__ void trace_tile(const TraceArgs &a, Ray<N> &r, int pa
                                            const float apex[3], const float *pyr, uint32_t *s_ref,
                                            float *s_t, uint32_t &err) {
     if (!traverse_tile<N, Q8>(a, r, pass, apex, pyr, s_ref, s_t, err)) start_over<N>(a, r, pass, err);
+}
+
+// ---------------------------------------------------------------- regions
+// The order in which a persistent launch takes its tiles. Row by row, the
+// tiles of a dense cluster met last kept a quarter of the chip idle at the end
+// (1M shell at 1080p, spp 1). So the image is cut into at most 4,096 regions of
+// 2^region_log2 x 2^region_log2 tiles, each counts the Gaussians whose mean
+// projects into it, and regions are taken by falling count (longest first):
+// rebuild + trace at spp 1 4.76 -> 4.34 ms, spp 16 10.5 -> 10.0, a fitting step
+// at spp 16 18.2 -> 17.6.
+// Tickets of a region's tiles off the image are passed over.
+constexpr int kMaxRegions = 4096;
+
+__global__ void __launch_bounds__(256)
+    k_region_cost(const __grid_constant__ TraceArgs a, int64_t n, int tile_w_lg, int tile_h_lg,
+                  uint32_t *__restrict__ cost) {
+    const int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    if (i >= n) return;
+    float f[3], r[3], u[3];
+    for (int k = 0; k < 3; ++k) f[k] = a.look_at[k] - a.eye[k];
+    normalise_rn(f);
+    cross_rn(f, a.up, r);
+    normalise_rn(r);
+    cross_rn(r, f, u);
+    const float4 p = __ldg(reinterpret_cast<const float4 *>(a.prims + i));
+    const float v[3] = {p.x - a.eye[0], p.y - a.eye[1], p.z - a.eye[2]};
+    const float z = (v[0] * f[0] + v[1] * f[1] + v[2] * f[2]) * a.tan_half / (float)a.height;
+    if (!(z > 0.0f)) return;
+    const float x = 0.5f * ((v[0] * r[0] + v[1] * r[1] + v[2] * r[2]) / z + (float)a.width);
+    const float y = 0.5f * ((float)a.height - (v[0] * u[0] + v[1] * u[1] + v[2] * u[2]) / z);
+    if (!(x >= 0.0f && x < (float)a.width && y >= 0.0f && y < (float)a.height)) return;
+    const int rx = min((int)x >> (tile_w_lg + a.region_log2), a.regions_x - 1);
+    const int ry = (int)y >> (tile_h_lg + a.region_log2);
+    const int at = ry * a.regions_x + rx;
+    if (at < a.n_regions) atomicAdd(&cost[at], 1u);
+}
+
+// Regions by falling count, ties by number; the counts and the tile counter
+// go back to zero.
+__global__ void __launch_bounds__(1024)
+    k_region_order(int n, uint32_t *__restrict__ cost, uint32_t *__restrict__ order,
+                   uint32_t *__restrict__ work) {
+    __shared__ uint32_t key[kMaxRegions];
+    const int tid = threadIdx.x;
+    for (int i = tid; i < kMaxRegions; i += 1024) {
+        uint32_t k = 0xffffffffu;
+        if (i < n) {
+            k = (0xfffffu - min(cost[i], 0xfffffu)) << 12 | (uint32_t)i;
+            cost[i] = 0;
+        }
+        key[i] = k;
+    }
+    if (tid == 0) *work = 0;
+    __syncthreads();
+    for (int size = 2; size <= kMaxRegions; size <<= 1)
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            for (int t = tid; t < kMaxRegions / 2; t += 1024) {
+                const int i = 2 * t - (t & (stride - 1)), j = i + stride;
+                const uint32_t x = key[i], y = key[j];
+                if ((x > y) == ((i & size) == 0)) {
+                    key[i] = y;
+                    key[j] = x;
+                }
+            }
+            __syncthreads();
+        }
+    for (int i = tid; i < n; i += 1024) order[i] = key[i] & (kMaxRegions - 1);
+}
+
+// Orders the launch's tiles (of 2^tile_w_lg x 2^tile_h_lg pixels) and resets
+// its tile counter.
+inline void order_regions(const gs_bvh *b, TraceArgs &a, int tile_w_lg, int tile_h_lg, cudaStream_t s) {
+    const int64_t tx = ((int64_t)a.width + (1 << tile_w_lg) - 1) >> tile_w_lg;
+    const int64_t ty = ((int64_t)a.height + (1 << tile_h_lg) - 1) >> tile_h_lg;
+    int lg = 0;
+    while (((tx + (1 << lg) - 1) >> lg) * ((ty + (1 << lg) - 1) >> lg) > kMaxRegions) ++lg;
+    a.region_log2 = lg;
+    a.regions_x = (int)((tx + (1 << lg) - 1) >> lg);
+    a.n_regions = a.regions_x * (int)((ty + (1 << lg) - 1) >> lg);
+    a.order = b->regions + kMaxRegions;
+    k_region_cost<<<(unsigned)((b->M + 255) / 256), 256, 0, s>>>(a, b->M, tile_w_lg, tile_h_lg,
+                                                                b->regions);
+    k_region_order<<<1, 1024, 0, s>>>(a.n_regions, b->regions, b->regions + kMaxRegions, a.work);
+}
+
+// Takes the next tile; 0: none left, 1: `tile` (row by row number) is set, -1:
+// the ticket was off the image.
+__device__ __forceinline__ int next_tile(const TraceArgs &a, uint32_t tiles_x, uint32_t n_tiles,
+                                         uint32_t &tile) {
+    uint32_t t = 0;
+    if ((threadIdx.x & 31) == 0) t = atomicAdd(a.work, 1u);
+    t = __shfl_sync(0xffffffffu, t, 0);
+    if (a.order == nullptr) {
+        tile = t;
+        return t < n_tiles;
+    }
+    const int lg = a.region_log2;
+    if (t >> (2 * lg) >= (uint32_t)a.n_regions) return 0;
+    const uint32_t region = __ldg(a.order + (t >> (2 * lg)));
+    const uint32_t m = (1u << lg) - 1u;
+    const uint32_t x = ((region % (uint32_t)a.regions_x) << lg) + (t & m);
+    const uint32_t y = ((region / (uint32_t)a.regions_x) << lg) + ((t >> lg) & m);
+    tile = y * tiles_x + x;
+    return x < tiles_x && tile < n_tiles ? 1 : -1;
 }
 
 }  // namespace
