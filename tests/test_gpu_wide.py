@@ -110,3 +110,50 @@ def test_shared_walk_hits_equal_packet_hits(gs, fmt, spp, n_hits):
                 gid = gs.decode_keys(keys)[2].reshape(cam.height, cam.width, spp, n_hits)
                 assert torch.equal(gid.permute(2, 3, 0, 1), a.long())
         bvh.free()
+
+
+@pytest.mark.parametrize("M", [1023, 1025, 8192, 8193, 10240, 10241, 70001])
+@pytest.mark.parametrize("coincident", [False, True])
+def test_sort_is_stable_and_complete(gs, M, coincident):
+    """The one-block build up to 8,192 Gaussians and the tiled sort above:
+    at the limit, at whole tiles of 2,048 keys and one past them, with half of
+    the codes equal."""
+    bvh = gs.build_bvh(gs.Gaussians.from_cloud(_cloud(M, coincident)))
+    bvh.sync_status()
+    ex = bvh.export()
+    bvh.free()
+    codes, order = ex["codes"], ex["order"].astype(np.int64)
+    assert np.all(codes[1:] >= codes[:-1])
+    eq = codes[1:] == codes[:-1]
+    assert np.all(order[1:][eq] > order[:-1][eq])
+    assert eq.any() or not coincident
+    assert np.array_equal(np.sort(order), np.arange(M))
+
+
+@pytest.mark.parametrize("fmt", ["binary", "binary_q8"])
+@pytest.mark.parametrize("spp,n_hits,degree", [(1, 1, 0), (3, 1, 1), (16, 1, 3), (5, 4, 2), (70, 1, 3)])
+def test_tile_gradients_equal_packet_gradients(gs, fmt, spp, n_hits, degree):
+    """Gradients of the tile form (ten sums, one chain rule per Gaussian)
+    against those of the per-lane form, which an explicit stack depth keeps:
+    small images, and one with more tiles than a wave. Both add the same terms
+    in float32 in different orders: the bound is that of the parity tests."""
+    cams = SMALL[:2] + (LARGE[:1] if spp <= 16 else [])
+    for M in (2, 33, 1025):
+        cloud = scenes.shell_cloud(M, M=M, n_clusters=4, sh_degree=degree)
+        cloud.log_scales[:] += 1.5
+        g = gs.Gaussians.from_cloud(cloud)
+        bvh = gs.build_bvh(g, node_format=fmt)
+        for cam in cams:
+            d = torch.randn((cam.height, cam.width, 3), device="cuda",
+                            generator=torch.Generator("cuda").manual_seed(M))
+            kw = dict(seed=M, spp=spp, n_hits=n_hits, bg=(0.2, 0.1, 0.4))
+            keys = gs.sample_keys(cam, spp, n_hits)
+            gs.trace_stochastic(bvh, g, cam, keys=keys, **kw)
+            ref = gs.trace_backward(bvh, g, cam, d, stack_depth=96, **kw)
+            for k in (None, keys):
+                got = gs.trace_backward(bvh, g, cam, d, keys=k, **kw)
+                bvh.sync_status()
+                for name in ref:
+                    bound = 1e-4 * ref[name].abs().max() + 1e-6
+                    assert (got[name] - ref[name]).abs().max() <= bound, (name, M, cam)
+        bvh.free()
