@@ -805,11 +805,10 @@ def main():
 
     rays_step = npix * SPP_N1 * world
     value = rays_step / (r1["ms_per_step"] * 1e-3) / 1e6
-    # this library's kernels per step: the rebuild (preprocess, key, 8 radix
-    # passes of histogram + 3-kernel scan + scatter, Karras, leaves, node
-    # depths, and count + 3-kernel scan + collapse for each of the three
-    # wide copies) and one trace
-    launches_per_step = 2 + 8 * 5 + 2 + 1 + 3 * 5 + 1
+    # this library's kernels per step: the rebuild (preprocess, codes, 8 digits
+    # of the sort, Karras, leaves, climb, and places and records of the wide
+    # copies) and one trace (region counts, region order, trace)
+    launches_per_step = 2 + 8 + 3 + 2 + 3
 
     line = {
         "metric": "Mrays/s at 1M Gaussians 1080p (N=1,4); RMSE vs exact blend at equal time",

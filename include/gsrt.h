@@ -164,7 +164,7 @@ typedef struct gs_bvh gs_bvh;
 
 /* Node format the traversal reads (the binary tree is always built too).
  *   GS_NODES_BINARY    64-byte binary nodes, FP32 child boxes; the handle
- *                      also holds 8-, 16- and 32-wide copies (one 32-byte
+ *                      also holds 8- and 32-wide copies (one 32-byte
  *                      FP32 record per child, M + (M - 1) records at most
  *                      each) for the grouped traversal, unless M > 2^25
  *   GS_NODES_WIDE4     128-byte 4-wide nodes, FP32 child boxes
@@ -172,7 +172,7 @@ typedef struct gs_bvh gs_bvh;
  *                      per plane with outward rounding (a decoded box always
  *                      contains the FP32 box, so no hit is lost and every
  *                      result equals the FP32 traversal's)
- *   GS_NODES_BINARY_Q8 binary nodes as GS_NODES_BINARY, with the 8-, 16- and
+ *   GS_NODES_BINARY_Q8 binary nodes as GS_NODES_BINARY, with the 8- and
  *                      32-wide copies in 8-bit form: per wide node a 32-byte
  *                      header (origin, power-of-two scale per axis), then 16
  *                      bytes per child (six 8-bit planes rounded outward
@@ -268,10 +268,15 @@ gs_status gs_bvh_export_wide(const gs_bvh *bvh, void *out, int64_t capacity, int
  * The 32 lanes of a warp split into pixels x samples: the L lanes of a pixel
  * (L the largest power of two not above ceil(spp / S), at most 32, S =
  * samples_per_lane) trace passes j*L + lane of the same ray. With L >= 8 and a GS_NODES_BINARY handle a
- * group of L lanes traverses the L-wide copy together (each lane tests one
+ * group of L lanes traverses a wide copy together (each lane tests one
  * child box, evaluates one hit Gaussian's depth and alpha, and draws for its
  * own samples); otherwise each lane traverses the nodes of the handle's
- * format in a warp packet. Every form returns the same hits.
+ * format in a warp packet. On binary handles with t_min >= 0 and none of
+ * counters, stack_depth, depth_mode and rng_mode set, the warp packet gives
+ * way to a tile walk of the 32-wide copy (in small images to a warp per
+ * pixel), and above 32 samples with samples_per_lane = 0 one walk serves four
+ * pixels. Every form returns the same hits, and the same image for the same
+ * S and L.
  * Deterministic: identical inputs give bit-identical outputs. Traces that use
  * the same handle share its tile counter and status word, so they must not
  * overlap on the GPU: issue them on one stream (or order their streams). */
@@ -308,7 +313,7 @@ gs_status gs_trace_stochastic_keys(const gs_bvh *bvh, const gs_gaussians *g,
 /* How gs_trace_stochastic(bvh, ..., p, ...) maps samples to lanes (host
  * call, nothing is enqueued). layout_out (host int32[4]) receives
  * {samples per lane S, lanes per pixel L, passes ceil(spp / S) of
- * n_hits * S slots each, 1 if a group of L lanes walks the L-wide copy
+ * n_hits * S slots each, 1 if a group of L lanes walks a wide copy
  * together else 0}: one walk
  * of the hierarchy serves L * S samples of one ray when grouped, S samples
  * otherwise. Returns GS_ERR_INVALID_ARG for NULL pointers or options
