@@ -346,8 +346,9 @@ void scan_exclusive(uint32_t *a, int64_t n, uint32_t *sums, cudaStream_t s) {
 // go through shared memory so that each digit's run is stored together.
 // A tile is taken only after the tiles before it, so each waits only on
 // blocks that are already running; the wait is bounded all the same.
-// Against a histogram, a three-kernel scan and a scatter per digit: 1M keys
-// and ids, eight digits, 0.31 ms in 40 launches before.
+// Against a histogram, a three-kernel scan and a scatter per digit (40
+// launches for eight digits): the whole rebuild 806 -> 557 us at 1M, 272 -> 132
+// at 1,000. Bound by the chain of a tile, about 20 us a digit at 1M.
 constexpr unsigned long long kTileCounted = 1ull << 62, kTileTotal = 2ull << 62;
 constexpr unsigned long long kTileValue = (1ull << 40) - 1ull;
 constexpr int kLookbackLimit = 1 << 24;
@@ -530,8 +531,9 @@ __global__ void __launch_bounds__(256)
 
 // Up to kSmallMax Gaussians: boxes, bounds, codes, the sort and the tree in
 // one launch of one block, everything between them in its shared memory. The
-// eleven launches it stands for cost more than their work: 1,000 Gaussians
-// rebuilt and traced at 64x64. Each digit is ranked as in
+// eleven launches it stands for cost more than their work: a rebuild of 1,000
+// Gaussians 132 -> 72 us, of 5,000 156 either way but 17 us of host time
+// instead of 36; above, one block is the slower. Each digit is ranked as in
 // k_radix_pass, the keys moving within shared memory.
 constexpr int kSmallThreads = 1024, kSmallItems = 8;
 constexpr int kSmallMax = kSmallThreads * kSmallItems;

@@ -2,8 +2,8 @@
 //
 // Same kernels and results as gs_build_bvh, for callers that must not call
 // cudaMalloc: the caller passes the output buffers, and the build scratch
-// (sort keys and ids, parents, arrival counters, boxes, histograms, scan
-// block sums) lives in one file-scope __device__ array sized for at most
+// (sort keys and ids, parents, arrival counters, boxes, histograms, tile
+// states of the sort) lives in one file-scope __device__ array sized for at most
 // kNoAllocMaxGaussians Gaussians. Every GPU that loads this library holds
 // that array (about 4 MB) until the process exits. The caller's status word
 // receives the build's error bits, so it is required: with no word of its

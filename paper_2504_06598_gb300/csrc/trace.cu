@@ -220,8 +220,8 @@ __global__ void __launch_bounds__(kThreads, is_group_fmt(FMT) ? group_min_blocks
 // other, all 32 lanes with two samples each. A pixel's 64 samples are kept in
 // shared memory (three words each) between its turns. The grouped form (one
 // pixel a warp) spent more on its walk than on its draws (1M shell at 1080p:
-// 13.6 ms of 23.0 at spp 64); evaluating per lane as the tiles do repeats
-// each evaluation on the pixel's lanes.
+// 13.6 ms of 23.0 at spp 64; now 17.8, issue 77%); evaluating per lane as the
+// tiles do repeats each evaluation on the pixel's lanes.
 constexpr int kSharedPx = 4;
 constexpr int kSharedPool = 192;  // stack entries per warp
 

@@ -1274,6 +1274,9 @@ __device__ __forceinline__ bool tile_child(const void *grec, uint32_t node, int 
 // samples (Alg. 1, whose ellipsoid test decides; the box only saves work),
 // so per-lane results are those of an independent traversal. For shadow rays
 // the apex is the far end: their clip bounds the distance from it as well.
+// Trace alone, 1M shell at 1080p: spp 1 4.34 -> 3.7 ms, spp 16 11.7 -> 9.1
+// against the packet. Bound by the evaluations: at spp 1 a tile makes 147, of
+// which half are behind every lane's hit and 23 valid and nearer for some lane.
 // Returns false when the stack is full (the caller starts over otherwise).
 template <int N, bool Q8>
 __device__ __forceinline__ bool traverse_tile(const TraceArgs &a, Ray<N> &r, int pass,
