@@ -434,11 +434,13 @@ __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
 }
 
 // The bounce ray of a deferred sample code: the sample's ground point and
-// bounce direction rebuilt with the camera pass's arithmetic.
-__device__ __forceinline__ void bounce_ray(const WaveArgs &w, unsigned long long code, Ray<1> &br,
+// bounce direction rebuilt with the camera pass's arithmetic. false for a code
+// that names no sample of the frame (nothing is stored for it).
+__device__ __forceinline__ bool bounce_ray(const WaveArgs &w, unsigned long long code, Ray<1> &br,
                                            int64_t &gpix, int &s) {
     gpix = (int64_t)((code >> 10) & 0xffffffull);
     s = (int)(code & 1023ull);
+    if (gpix >= w.n_pix || s >= w.t.n_samples) return false;
     int v = 0;
     while (v + 1 < w.n_views && w.views[v + 1].pix_begin <= gpix) ++v;
     const ViewDesc &vw = w.views[v];
@@ -461,6 +463,7 @@ __device__ __forceinline__ void bounce_ray(const WaveArgs &w, unsigned long long
     br.any_hit = false;
     reset_slots(br);
     update_clip(br, br.t_max);
+    return true;
 }
 
 // Shades a finished bounce ray and writes albedo x radiance to its slot.
@@ -603,8 +606,7 @@ __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
                     const unsigned long long code = i < n_slots ? codes[i] : ~0ull;
                     if (code == ~0ull) {
                         more = false;
-                    } else {
-                        bounce_ray(w, code, br, gpix, s);
+                    } else if (bounce_ray(w, code, br, gpix, s)) {
                         node = 0;
                         sp = 0;
                         steps = 0;
@@ -650,14 +652,12 @@ __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
             if ((int64_t)tile * 32 >= n_slots) break;
             const int64_t i = (int64_t)tile * 32 + lane;
             const unsigned long long code = i < n_slots ? codes[i] : ~0ull;
-            const bool valid = code != ~0ull;
-            if (!__any_sync(kAll, valid)) break;
+            if (!__any_sync(kAll, code != ~0ull)) break;
             int64_t gpix = 0;
             int s = 0;
             Ray<1> br;
-            if (valid) {
-                bounce_ray(w, code, br, gpix, s);
-            } else {
+            const bool valid = code != ~0ull && bounce_ray(w, code, br, gpix, s);
+            if (!valid) {
                 const float p[3] = {0.0f, w.ground_y, 0.0f}, db[3] = {0.0f, 1.0f, 0.0f};
                 set_ray(br, p, db);
                 br.ray_id = 0;
@@ -777,6 +777,9 @@ gs_status launch_views_g(const WaveArgs &w, int threads, int stack, cudaStream_t
             return stack == 48 ? launch_views<FMT, 48, false, 0, 2>(w, threads, s)
                                : launch_views<FMT, 96, false, 0, 2>(w, threads, s);
     }
+    if (w.spl != 1)
+        return fail(GS_ERR_INVALID_ARG, "no form of %d lanes a pixel carries %d samples a lane",
+                    1 << w.t.lpp_log2, w.spl);
     if (stack == 48)
         return count ? launch_views<FMT, 48, true, GLG>(w, threads, s)
                      : launch_views<FMT, 48, false, GLG>(w, threads, s);
@@ -911,10 +914,13 @@ gs_status launch_render_views(const gs_bvh *b, const gs_gaussians *g, const gs_p
     int K = 1;
     if (counters == nullptr && !inline_bounce && p->spp >= 2 && p->spp < 64)
         K = p->spp >= 8 ? 8 : (p->spp >= 4 ? 4 : 2);
-    // too few tiles to fill the chip once: a warp per pixel (see launch_trace)
+    // the grouped walks of 8 and 16 lanes carry one sample a lane, so several
+    // samples a lane (8 to 63 samples: up to 8 lanes) are never theirs
     const int lanes_lg = lanes_per_pixel_log2((p->spp + K - 1) / K);
+    const bool ungrouped = lanes_lg < 3 || K > 1;
+    // too few tiles to fill the chip once: a warp per pixel (see launch_trace)
     const bool whole_warp =
-        tiles_ok && lanes_lg < 3 && (all_pix << lanes_lg) < (int64_t)sms * 32 * 32;
+        tiles_ok && ungrouped && (all_pix << lanes_lg) < (int64_t)sms * 32 * 32;
     w.spl = K;
     a.spp = (p->spp + K - 1) / K;
     a.n_samples = p->spp;
@@ -926,13 +932,13 @@ gs_status launch_render_views(const gs_bvh *b, const gs_gaussians *g, const gs_p
     a.rgb = rgb;
     a.status = b->status;
     a.work = b->status + 1;
-    a.lpp_log2 = whole_warp ? 5 : lanes_per_pixel_log2(a.spp);
-    if (b->link && a.lpp_log2 >= 3) {
+    a.lpp_log2 = whole_warp ? 5 : lanes_lg;
+    if (b->link && (whole_warp || !ungrouped)) {
         a.grec = b->group[group_tree(a.lpp_log2)].rec;
         a.groot = b->group[group_tree(a.lpp_log2)].ref;
         a.gq8 = b->node_format == GS_NODES_BINARY_Q8;
     }
-    if (tiles_ok && a.lpp_log2 < 3) {
+    if (tiles_ok && ungrouped && !whole_warp) {
         a.trec = b->group[kWarpTree].rec;
         a.troot = b->group[kWarpTree].ref;
     }

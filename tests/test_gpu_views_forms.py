@@ -1,0 +1,48 @@
+"""The forms of the batched launch against one another: which of them a frame
+takes follows from its size, its samples and the handle's nodes, and must not
+show in any sample's outcome. The 4-wide handles, whose camera and shadow rays
+walk as per-lane packets, are the other side."""
+import numpy as np
+import pytest
+
+import scenes
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gs():
+    import __graft_entry__
+    __graft_entry__.build()
+    import paper_2504_06598_gb300 as m
+    if not torch.cuda.is_available():
+        pytest.fail("CUDA device required for gpu tests")
+    return m
+
+
+def _render(gs, g, cams, ex, fmt, **kw):
+    bvh = gs.build_bvh(g, node_format=fmt)
+    rgb, smp = gs.render_views(bvh, g, cams, ex, seed=5, want_samples=True, **kw)
+    bvh.sync_status()
+    bvh.free()
+    return rgb, smp
+
+
+@pytest.mark.parametrize("fmt", ["binary", "binary_q8"])
+@pytest.mark.parametrize("spp", [56, 57, 60, 63, 64])
+@pytest.mark.parametrize("size", [(23, 17), (171, 120)])
+def test_samples_up_to_64(gs, fmt, spp, size):
+    """Eight samples a lane make eight passes from 57 samples on: a warp per
+    pixel in the small frame, tiles in the large one, packets with an explicit
+    stack depth."""
+    g = gs.Gaussians.from_cloud(scenes.shell_cloud(7, M=6000))
+    cams = scenes.wavefront_views(1, seed=2, fixed_res=size)
+    ex = scenes.ground_and_lights(2, seed=1)
+    ref, smp = _render(gs, g, cams, ex, "wide4", spp=spp)
+    assert (smp[..., 0] == -2).any() and (smp[..., 0] >= 0).any() and (smp[..., 1] >= 0).any()
+    for depth in (0, 96):
+        rgb, got = _render(gs, g, cams, ex, fmt, spp=spp, stack_depth=depth)
+        assert torch.equal(got, smp)
+        # sums of spp colours in another order
+        assert (rgb - ref).abs().max() <= 2 * spp * 2.0 ** -24 * ref.abs().max()
