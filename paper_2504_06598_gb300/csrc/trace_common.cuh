@@ -1453,8 +1453,10 @@ __global__ void __launch_bounds__(1024)
 }
 
 // Orders the launch's tiles (of 2^tile_w_lg x 2^tile_h_lg pixels) and resets
-// its tile counter.
+// its tile counter; a handle that holds no Gaussian has nothing to order
+// (a.order stays null).
 inline void order_regions(const gs_bvh *b, TraceArgs &a, int tile_w_lg, int tile_h_lg, cudaStream_t s) {
+    if (b->M == 0) return;
     const int64_t tx = ((int64_t)a.width + (1 << tile_w_lg) - 1) >> tile_w_lg;
     const int64_t ty = ((int64_t)a.height + (1 << tile_h_lg) - 1) >> tile_h_lg;
     int lg = 0;

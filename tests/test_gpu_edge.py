@@ -217,3 +217,24 @@ def test_mean_converges_to_exact_blend(gs):
     p3 = 0.0027
     assert fails <= n * p3 + 3 * np.sqrt(n * p3 * (1 - p3)) + 1
     assert abs(zs.mean()) < 4 / np.sqrt(n)
+
+
+@pytest.mark.parametrize("fmt", ["binary", "binary_q8", "wide4"])
+def test_rebuild_to_nothing_is_background(gs, fmt):
+    """A handle rebuilt for no Gaussians renders the background at every size
+    and sample count, and takes Gaussians again afterwards."""
+    cloud = scenes.tiny_cloud(1, M=50)
+    g = gs.Gaussians.from_cloud(cloud)
+    empty = gs.Gaussians.from_cloud(cloud.subset(np.arange(0)))
+    bvh = gs.build_bvh(g, node_format=fmt)
+    bg = (0.25, 0.5, 0.75)
+    for cam in (scenes.default_camera(40, 30), scenes.default_camera(1920, 1080)):
+        before = gs.trace_stochastic(bvh, g, cam, seed=1, spp=2, bg=bg)
+        bvh.rebuild(empty)
+        for spp in (1, 16, 64):
+            rgb = gs.trace_stochastic(bvh, empty, cam, seed=1, spp=spp, bg=bg)
+            assert (rgb.reshape(-1, 3) == torch.tensor(bg, device="cuda")).all(), (cam, spp)
+        bvh.rebuild(g)
+        assert torch.equal(gs.trace_stochastic(bvh, g, cam, seed=1, spp=2, bg=bg), before)
+    bvh.sync_status()
+    bvh.free()
