@@ -606,31 +606,38 @@ __device__ __forceinline__ int stat_of(int lane) {
 }
 
 // One candidate (record idx, the same for the warp) against every lane's
-// slots; gck[k] = g . c_k of slot k's winner.
+// slots. ck: the colours of the slots' winners, [slot and channel][lane] in
+// shared memory (in registers, 24 more at eight slots, they would spill). The
+// difference of the colours comes before the product with g: as the difference
+// of the two products the weight had up to 4e-6 of itself in rounding where
+// colours differ by a hundredth, and no exact 0 where they are equal. 1M at
+// 1080p, spp 16, rebuild + image + gradients 19.79 -> 20.15 ms (the same box).
 template <int N>
 __device__ __forceinline__ void tile_gradient(const TraceArgs &a, const Ray<N> &r, uint32_t idx,
-                                              const float gck[N], const float g[3]) {
+                                              const float (*ck)[32], const float g[3]) {
     const uint32_t kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const Cand c = eval_cand<true>(a, r.o, r.d, idx);
-    float n_front = 0.0f, behind = 0.0f;
+    uint32_t front = 0;
     if (c.valid && c.t <= r.t_far) {
 #pragma unroll
         for (int k = 0; k < N; ++k)
-            if (lex_closer(c.tc, c.tau, c.gid, r.slot[k])) {
-                n_front += 1.0f;
-                behind += gck[k];
-            }
+            if (lex_closer(c.tc, c.tau, c.gid, r.slot[k])) front |= 1u << k;
     }
-    if (!__any_sync(kAll, n_front > 0.0f)) return;
+    if (!__any_sync(kAll, front != 0u)) return;
     float wa = 0.0f;
-    if (n_front > 0.0f) {
+    if (front) {
         float Y[16], ci[3];
         sh_basis(a.sh_degree, r.d, Y);
         sh_colour(a, c.gid, Y, ci);
-        const float gci = fmaf(g[0], ci[0], fmaf(g[1], ci[1], g[2] * ci[2]));
+        float coef = 0.0f;
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+            if ((front >> k) & 1u)
+                coef += fmaf(g[0], ci[0] - ck[3 * k][lane],
+                             fmaf(g[1], ci[1] - ck[3 * k + 1][lane], g[2] * (ci[2] - ck[3 * k + 2][lane])));
         // a rejected hit has alpha <= xi < 1
-        wa = fmaf(n_front, gci, -behind) / (1.0f - c.alpha) * c.alpha;
+        wa = coef / (1.0f - c.alpha) * c.alpha;
     }
     const bool add = wa != 0.0f;
     if (!__any_sync(kAll, add)) return;
@@ -657,7 +664,7 @@ constexpr int kTileLevels = 128;
 
 template <int N, bool Q8>
 __device__ __forceinline__ void enumerate_tile(const TraceArgs &a, const Ray<N> &r,
-                                               const float gck[N], const float g[3],
+                                               const float (*ck)[32], const float g[3],
                                                const float *pyr, uint2 *stack, uint32_t &err) {
     const uint32_t kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -681,7 +688,7 @@ __device__ __forceinline__ void enumerate_tile(const TraceArgs &a, const Ray<N> 
         const bool leaf = (ref & kLeafBit) != 0u;
         for (uint32_t lm = __ballot_sync(kAll, hit && leaf); lm; lm &= lm - 1u) {
             const uint32_t idx = __shfl_sync(kAll, ref, __ffs(lm) - 1) & ~kLeafBit;
-            tile_gradient<N>(a, r, idx, gck, g);
+            tile_gradient<N>(a, r, idx, ck, g);
         }
         uint32_t im = __ballot_sync(kAll, hit && !leaf);
         if (im) {
@@ -745,6 +752,7 @@ __global__ void __launch_bounds__(kThreads, N >= 8 ? 5 : 6)
     const uint32_t kAll = 0xffffffffu;
     __shared__ __align__(16) float s_pyr[kThreads / 32][kTileFloats];
     __shared__ uint2 s_lvl[kThreads / 32][kTileLevels];
+    __shared__ float s_ck[kThreads / 32][3 * N][32];
     // the forward traversal's stack, where the winners are traced again
     __shared__ uint32_t s_ref[KEYS ? 1 : kThreads / 32][KEYS ? 1 : kTilePool];
     __shared__ float s_t[KEYS ? 1 : kThreads / 32][KEYS ? 1 : kTilePool];
@@ -818,7 +826,6 @@ __global__ void __launch_bounds__(kThreads, N >= 8 ? 5 : 6)
             }
             // 2) colours of the winners; dLoss/dk of the selected Gaussians,
             // once for the slots of a lane that hold the same one
-            float gck[N];
             {
                 float Y[16];
                 sh_basis(a.sh_degree, r.d, Y);
@@ -844,14 +851,14 @@ __global__ void __launch_bounds__(kThreads, N >= 8 ? 5 : 6)
                         if (first && (gm[0] != 0.0f || gm[1] != 0.0f || gm[2] != 0.0f))
                             add_sh_gradient(a, wid, gm, Y);
                     }
-                    gck[k] = fmaf(g[0], ck[0], fmaf(g[1], ck[1], g[2] * ck[2]));
+                    for (int ch = 0; ch < 3; ++ch) s_ck[warp][3 * k + ch][lane] = ck[ch];
                 }
             }
             // 3) every Gaussian in front of a winner
             update_clip(r, a.t_max);
             if (!live) r.t_far = -INFINITY;
             __syncwarp();
-            enumerate_tile<N, Q8>(a, r, gck, g, pyr, s_lvl[warp], err);
+            enumerate_tile<N, Q8>(a, r, s_ck[warp], g, pyr, s_lvl[warp], err);
             __syncwarp();
         }
     }

@@ -306,3 +306,29 @@ def test_keys_full_size(gs):
         scale = float(a[k].abs().max())
         assert scale > 0, k
         assert float((a[k] - b[k]).abs().max()) <= 1e-4 * scale, k
+
+
+@pytest.mark.parametrize("spp,n_hits", [(1, 1), (3, 1), (5, 1), (8, 1), (16, 1), (4, 4)])
+def test_equal_colours_have_no_geometry_gradient(gs, spp, n_hits):
+    """Where every Gaussian and the background have one colour no term
+    g . (c_i - c_k) is other than 0, so the geometry's gradients are 0 to the
+    last bit."""
+    cloud = scenes.shell_cloud(2, M=3000, n_clusters=6, sh_degree=0)
+    cloud.log_scales[:] += 1.0
+    colour = (0.3, 0.7, 0.55)
+    cloud.sh[:] = np.float32(colour)
+    g = gs.Gaussians.from_cloud(cloud)
+    bvh = gs.build_bvh(g)
+    for cam in (scenes.default_camera(48, 36), scenes.default_camera(500, 300)):
+        d = torch.randn((cam.height, cam.width, 3), device="cuda",
+                        generator=torch.Generator("cuda").manual_seed(spp))
+        kw = dict(seed=3, spp=spp, n_hits=n_hits, bg=colour)
+        keys = gs.sample_keys(cam, spp, n_hits)
+        gs.trace_stochastic(bvh, g, cam, keys=keys, **kw)
+        for k in (None, keys):
+            got = gs.trace_backward(bvh, g, cam, d, keys=k, **kw)
+            assert got["sh"].abs().max() > 0
+            for name in ("means", "log_scales", "quats", "opacity_logits"):
+                assert int((got[name] != 0).sum()) == 0, name
+    bvh.sync_status()
+    bvh.free()
