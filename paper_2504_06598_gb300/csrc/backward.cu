@@ -891,18 +891,19 @@ __global__ void __launch_bounds__(256) k_chain(const __grid_constant__ TraceArgs
         atomicAdd(a.g_means + 3 * gid + j, fmaf(m[j], s[1], fmaf(m[3 + j], s[2], m[6 + j] * s[3])));
         atomicAdd(a.g_log_scales + 3 * gid + j, P[j][j]);
     }
-    // dq/dR_jk = 2 v_j u_k / s_k with v = R S u and (R S)_jl = M_lj s_l^2
-    float inv_s[3], s2[3];
+    // dq/dR_jk = 2 v_j u_k / s_k with v = R S u and (R S)_jl = (M_lj s_l) s_l
+    // (M s is of a rotation's size: s^2 by itself leaves float32 above a
+    // log-scale of 44)
+    float inv_s[3], sc[3];
     for (int k = 0; k < 3; ++k) {
         const float ls = __ldg(a.log_scales + 3 * gid + k);
         inv_s[k] = expf(-ls);
-        const float e = expf(ls);
-        s2[k] = e * e;
+        sc[k] = expf(ls);
     }
     float dR[9];
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-        const float rs[3] = {m[j] * s2[0], m[3 + j] * s2[1], m[6 + j] * s2[2]};
+        const float rs[3] = {m[j] * sc[0] * sc[0], m[3 + j] * sc[1] * sc[1], m[6 + j] * sc[2] * sc[2]};
 #pragma unroll
         for (int k = 0; k < 3; ++k)
             dR[3 * j + k] =

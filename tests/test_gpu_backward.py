@@ -332,3 +332,32 @@ def test_equal_colours_have_no_geometry_gradient(gs, spp, n_hits):
                 assert int((got[name] != 0).sum()) == 0, name
     bvh.sync_status()
     bvh.free()
+
+
+@pytest.mark.parametrize("big", [30.0, 42.0, 44.0, 45.0])
+@pytest.mark.parametrize("axis", [0, 1])
+def test_gradients_of_extreme_scales(gs, axis, big):
+    """A Gaussian so long that the square of its scale leaves float32: the
+    tile form's gradients are the per-lane form's (which an explicit stack
+    depth keeps), with the bound of the parity tests."""
+    cloud = scenes.tiny_cloud(4, M=2)
+    cloud.means[:] = ((0.1, -0.05, 0.2), (0.0, 50.0, 0.0))
+    cloud.quats[:] = (1.0, 0.0, 0.0, 0.0)
+    cloud.log_scales[:] = -1.0
+    cloud.log_scales[0, axis] = big
+    cloud.opacity_logits[:] = 0.5
+    cam = scenes.Pinhole(width=20, height=14, eye=(0.3, 0.2, 2.8))
+    g = gs.Gaussians.from_cloud(cloud)
+    d = torch.randn((cam.height, cam.width, 3), device="cuda",
+                    generator=torch.Generator("cuda").manual_seed(1))
+    bvh = gs.build_bvh(g)
+    kw = dict(seed=2, spp=4, bg=(0.2, 0.1, 0.4))
+    ref = gs.trace_backward(bvh, g, cam, d, stack_depth=96, **kw)
+    got = gs.trace_backward(bvh, g, cam, d, **kw)
+    bvh.sync_status()
+    bvh.free()
+    assert ref["log_scales"].abs().max() > 0
+    for name in ref:
+        assert torch.isfinite(ref[name]).all() and torch.isfinite(got[name]).all(), name
+        bound = 1e-4 * ref[name].abs().max() + 1e-6
+        assert (got[name] - ref[name]).abs().max() <= bound, name
