@@ -264,7 +264,8 @@ __device__ void enumerate_packet(const TraceArgs &a, const Ray<N> &r, const floa
             hL = false;
         }
         if (cref.y & kLeafBit) {
-            leaf_gradient<N>(a, r, hR, cref.y & ~kLeafBit, ck, g, Y);
+            // (a single Gaussian is both children of the root and counts once)
+            if (cref.y != cref.x) leaf_gradient<N>(a, r, hR, cref.y & ~kLeafBit, ck, g, Y);
             hR = false;
         }
         const unsigned mL = __ballot_sync(kAll, hL), mR = __ballot_sync(kAll, hR);

@@ -361,3 +361,28 @@ def test_gradients_of_extreme_scales(gs, axis, big):
         assert torch.isfinite(ref[name]).all() and torch.isfinite(got[name]).all(), name
         bound = 1e-4 * ref[name].abs().max() + 1e-6
         assert (got[name] - ref[name]).abs().max() <= bound, name
+
+
+def test_single_gaussian_gradients(gs):
+    """One Gaussian is both children of the root; its gradient counts once,
+    in the tile form and in the per-lane form, as the oracle's does."""
+    cloud = scenes.tiny_cloud(4, M=1)
+    cloud.means[:] = (0.1, -0.05, 0.2)
+    cloud.log_scales[:] = (-0.6, -0.9, -0.4)
+    cam = scenes.default_camera(20, 14)
+    d_rgb = np.random.default_rng(0).normal(size=(cam.width * cam.height, 3))
+    bg = (0.2, 0.1, 0.4)
+    ref = oracle.grad_pinhole(cloud, cam, scenes.TraceSettings(seed=2, spp=4, bg=bg), d_rgb,
+                              mode="estimator")
+    g = gs.Gaussians.from_cloud(cloud)
+    d = torch.from_numpy(d_rgb.astype(np.float32)).cuda().reshape(cam.height, cam.width, 3)
+    for fmt in ("binary", "binary_q8", "wide4"):
+        bvh = gs.build_bvh(g, node_format=fmt)
+        for depth in (0, 96):
+            for spl in (0, 1):
+                got = gs.trace_backward(bvh, g, cam, d, seed=2, spp=4, bg=bg, stack_depth=depth, samples_per_lane=spl)
+                for k, v in got.items():
+                    err = np.abs(v.cpu().numpy().astype(np.float64) - ref[k]).max()
+                    assert err <= 1e-4 * np.abs(ref[k]).max() + 1e-6, (k, fmt, depth)
+        bvh.sync_status()
+        bvh.free()
