@@ -97,6 +97,11 @@ __global__ void __launch_bounds__(kThreads, is_group_fmt(FMT) ? group_min_blocks
     uint32_t *grp_ref = s_ref[pooled ? threadIdx.x >> 5 : 0] + grp_off;
     float *grp_t = s_t[pooled ? threadIdx.x >> 5 : 0] + grp_off;
     float *pyr = s_pyr[tiled ? threadIdx.x >> 5 : 0];
+    // a warp on one pixel of a layout of fewer lanes: the colours (at most 64)
+    // pass through the walk's stack
+    const bool relay = grouped && LG == 5 && !COUNT && a.sum_log2 < 5;
+    float(*colour)[64] = reinterpret_cast<float(*)[64]>(grp_ref);
+    const int sum_lanes = relay ? 1 << a.sum_log2 : L;
     for (;;) {
         uint32_t tile = 0;
         const int more = next_tile(a, tiles_x, n_tiles, tile);
@@ -150,6 +155,7 @@ __global__ void __launch_bounds__(kThreads, is_group_fmt(FMT) ? group_min_blocks
                 else
                     traverse_packet_wide<N, COUNT, FMT>(a, r, pass, stack, stack_t, err, cnt);
             }
+            if (relay) __syncwarp();  // the walk's reads of the stack are done
             if (live) {
                 // shade each slot once (Eq. 6) and accumulate (Eq. 7)
                 float Y[16];
@@ -164,9 +170,13 @@ __global__ void __launch_bounds__(kThreads, is_group_fmt(FMT) ? group_min_blocks
                     } else {
                         c[0] = a.bg[0]; c[1] = a.bg[1]; c[2] = a.bg[2];
                     }
-                    acc[0] += c[0];
-                    acc[1] += c[1];
-                    acc[2] += c[2];
+                    if (relay) {
+                        for (int i = 0; i < 3; ++i) colour[i][s0 + k] = c[i];
+                    } else {
+                        acc[0] += c[0];
+                        acc[1] += c[1];
+                        acc[2] += c[2];
+                    }
                     if (a.hit_id) {
                         const int64_t o = ((int64_t)s0 + k) * npix + pix;
                         a.hit_id[o] = r.slot[k].gid == 0xffffffffu ? -1 : (int32_t)r.slot[k].gid;
@@ -185,9 +195,13 @@ __global__ void __launch_bounds__(kThreads, is_group_fmt(FMT) ? group_min_blocks
                 }
             }
             __syncwarp();
+            if (relay) {
+                add_in_layout(colour, 0, a.n_samples, log2_of(N), a.sum_log2, lane, acc);
+                __syncwarp();
+            }
         }
         // the pixel's lanes add their partial sums (Eq. 7)
-        for (int o = L >> 1; o >= 1; o >>= 1) {
+        for (int o = sum_lanes >> 1; o >= 1; o >>= 1) {
             acc[0] += __shfl_xor_sync(kAll, acc[0], o);
             acc[1] += __shfl_xor_sync(kAll, acc[1], o);
             acc[2] += __shfl_xor_sync(kAll, acc[2], o);
@@ -495,18 +509,10 @@ __global__ void __launch_bounds__(kThreads, 8) k_trace_shared(const __grid_const
                     }
                 }
                 __syncwarp();
-                // the sums of k_trace's lanes (passes of 2^k samples, 2^l
-                // lanes a pixel), in their order: the same image bit for bit
                 float acc[3];
                 for (int i = 0; i < 3; ++i) acc[i] = base > 0 ? m.acc[p][i][lane] : 0.0f;
-                const int L = 1 << a.lpp_log2, end = min(base + 64, a.n_samples);
-                if (lane < L) {
-                    int pass = base >> a.k_log2;
-                    pass += (lane - pass) & (L - 1);
-                    for (; pass << a.k_log2 < end; pass += L)
-                        for (int s = pass << a.k_log2; s < min((pass + 1) << a.k_log2, end); ++s)
-                            for (int i = 0; i < 3; ++i) acc[i] += m.colour[i][s - base];
-                }
+                add_in_layout(m.colour, base, min(base + 64, a.n_samples), a.k_log2, a.sum_log2,
+                              lane, acc);
                 for (int i = 0; i < 3; ++i) m.acc[p][i][lane] = acc[i];
                 __syncwarp();
             }
@@ -518,7 +524,7 @@ __global__ void __launch_bounds__(kThreads, 8) k_trace_shared(const __grid_const
             if (x >= a.width || y >= a.height) continue;
             float acc[3];
             for (int i = 0; i < 3; ++i) acc[i] = m.acc[p][i][lane];
-            for (int o = (1 << a.lpp_log2) >> 1; o >= 1; o >>= 1) {
+            for (int o = (1 << a.sum_log2) >> 1; o >= 1; o >>= 1) {
                 acc[0] += __shfl_xor_sync(kAll, acc[0], o);
                 acc[1] += __shfl_xor_sync(kAll, acc[1], o);
                 acc[2] += __shfl_xor_sync(kAll, acc[2], o);
@@ -668,6 +674,7 @@ gs_status launch_trace(const gs_bvh *b, const gs_gaussians *g, const gs_pinhole 
                        p->stack_depth == 0 && p->counters == nullptr;
     const bool shared = plain && p->samples_per_lane == 0 && (int64_t)p->spp * p->n_hits > 32;
     bool tile = plain && !shared && lpp_log2 < 3;
+    const int sum_log2 = lpp_log2;
     if (tile && tile_warps(cam->width, cam->height, lpp_log2) < resident_warps()) {
         // Too few tiles to fill the chip once: the time is the longest walk
         // of a warp, which evaluates its tile's Gaussians one after the other.
@@ -684,6 +691,7 @@ gs_status launch_trace(const gs_bvh *b, const gs_gaussians *g, const gs_pinhole 
     a.nodes = b->nodes;
     a.wide = b->wide;
     a.lpp_log2 = lpp_log2;
+    a.sum_log2 = sum_log2;
     if (b->link && a.lpp_log2 >= 3) {
         a.grec = b->group[group_tree(a.lpp_log2)].rec;
         a.groot = b->group[group_tree(a.lpp_log2)].ref;

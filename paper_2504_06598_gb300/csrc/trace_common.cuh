@@ -56,6 +56,7 @@ struct TraceArgs {
     const uint32_t *order;
     int region_log2, regions_x, n_regions;
     int lpp_log2;    // log2 of the lanes that trace samples of one pixel
+    int sum_log2;    // log2 of the lanes a pixel has in the layout of its sums
     int k_log2;      // log2 of the slots of a pass (shared walks)
     int depth_mode;  // 0: 1D mean; 1: centre projected on fwd (camera rays)
     int rng_mode;    // 0: Philox; 1: trigonometric hash of the hit point
@@ -84,6 +85,25 @@ inline int lanes_per_pixel_log2(int spp) {
     while (l < 5 && (2 << l) <= spp) ++l;
     return l;
 }
+
+// A form that walks otherwise than its layout says (a warp per pixel of a small
+// image, a walk shared by four pixels) still adds a pixel's samples in the
+// layout's order, so that the image does not depend on the form: the colours of
+// samples [base, end) wait in shared memory ([channel][sample - base]) and lane
+// l < 2^l_log2 adds its passes' (2^k_log2 samples each, dealt to the lanes in
+// turn) one after the other.
+__device__ __forceinline__ void add_in_layout(const float (*colour)[64], int base, int end,
+                                              int k_log2, int l_log2, int lane, float acc[3]) {
+    const int L = 1 << l_log2;
+    if (lane >= L) return;
+    int pass = base >> k_log2;
+    pass += (lane - pass) & (L - 1);
+    for (; pass << k_log2 < end; pass += L)
+        for (int s = pass << k_log2; s < min((pass + 1) << k_log2, end); ++s)
+            for (int i = 0; i < 3; ++i) acc[i] += colour[i][s - base];
+}
+
+__host__ __device__ constexpr int log2_of(int n) { return n <= 1 ? 0 : 1 + log2_of(n >> 1); }
 
 // ---------------------------------------------------------------- Philox
 // Philox-4x32-10 (Salmon et al., SC'11): ten rounds, multipliers

@@ -215,6 +215,9 @@ __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
         g_t = reinterpret_cast<float *>(pool + kTilePool);
         pyr = reinterpret_cast<float *>(pool + 2 * kTilePool);
     }
+    // a warp per pixel: sums in the layout's order (as in k_trace)
+    const bool relay = GLG == 5 && !COUNT && a.sum_log2 < 5;
+    float(*colour)[64] = reinterpret_cast<float(*)[64]>(g_ref);
     const int lg = a.lpp_log2, L = 1 << lg;
     const int tw_lg = tile_w_log2(lg), th_lg = 5 - lg - tw_lg;
     const int sub = lane & (L - 1), pl = lane >> lg;
@@ -395,12 +398,17 @@ __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
                     }
                 }
             }
+            if (relay) __syncwarp();  // the walks' reads of the stack are done
 #pragma unroll
             for (int k = 0; k < K; ++k) {
                 if (!live[k]) continue;
-                acc[0] += c[k][0];
-                acc[1] += c[k][1];
-                acc[2] += c[k][2];
+                if (relay) {
+                    for (int i = 0; i < 3; ++i) colour[i][pass * K + k] = c[k][i];
+                } else {
+                    acc[0] += c[k][0];
+                    acc[1] += c[k][1];
+                    acc[2] += c[k][2];
+                }
                 if (w.samples) {
                     const int64_t o = ((int64_t)(pass * K + k) * w.n_pix + vw.pix_begin + lpix) * 3;
                     w.samples[o] = diag_cam[k];
@@ -409,9 +417,13 @@ __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
                 }
             }
             __syncwarp();
+            if (relay) {
+                add_in_layout(colour, 0, S, log2_of(K), a.sum_log2, lane, acc);
+                __syncwarp();
+            }
         }
         // the pixel's lanes add their partial sums
-        for (int o = L >> 1; o >= 1; o >>= 1) {
+        for (int o = (relay ? 1 << a.sum_log2 : L) >> 1; o >= 1; o >>= 1) {
             acc[0] += __shfl_xor_sync(kAll, acc[0], o);
             acc[1] += __shfl_xor_sync(kAll, acc[1], o);
             acc[2] += __shfl_xor_sync(kAll, acc[2], o);
@@ -933,6 +945,7 @@ gs_status launch_render_views(const gs_bvh *b, const gs_gaussians *g, const gs_p
     a.status = b->status;
     a.work = b->status + 1;
     a.lpp_log2 = whole_warp ? 5 : lanes_lg;
+    a.sum_log2 = lanes_lg;
     if (b->link && (whole_warp || !ungrouped)) {
         a.grec = b->group[group_tree(a.lpp_log2)].rec;
         a.groot = b->group[group_tree(a.lpp_log2)].ref;

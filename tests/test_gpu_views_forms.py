@@ -46,3 +46,16 @@ def test_samples_up_to_64(gs, fmt, spp, size):
         assert torch.equal(got, smp)
         # sums of spp colours in another order
         assert (rgb - ref).abs().max() <= 2 * spp * 2.0 ** -24 * ref.abs().max()
+
+
+@pytest.mark.parametrize("spp", [1, 3, 5, 17, 20, 24, 56, 60])
+def test_small_frames_add_samples_in_the_layouts_order(gs, spp):
+    """A warp per pixel, as small frames take it: the packets' image to the
+    last bit."""
+    g = gs.Gaussians.from_cloud(scenes.shell_cloud(7, M=6000))
+    cams = scenes.wavefront_views(2, seed=4, fixed_res=(31, 23))
+    ex = scenes.ground_and_lights(3, seed=1)
+    ref, smp = _render(gs, g, cams, ex, "wide4", spp=spp)
+    for fmt in ("binary", "binary_q8"):
+        rgb, got = _render(gs, g, cams, ex, fmt, spp=spp)
+        assert torch.equal(got, smp) and torch.equal(rgb, ref), fmt

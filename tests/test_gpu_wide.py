@@ -157,3 +157,23 @@ def test_tile_gradients_equal_packet_gradients(gs, fmt, spp, n_hits, degree):
                     bound = 1e-4 * ref[name].abs().max() + 1e-6
                     assert (got[name] - ref[name]).abs().max() <= bound, (name, M, cam)
         bvh.free()
+
+
+@pytest.mark.parametrize("fmt", ["binary", "binary_q8"])
+@pytest.mark.parametrize("spp,spl,n_hits", [(3, 1, 1), (5, 1, 1), (7, 1, 1), (17, 0, 1), (20, 0, 1), (24, 0, 1), (6, 1, 8),
+                                            (5, 0, 4), (13, 2, 2), (20, 4, 1)])
+def test_small_images_add_samples_in_the_layouts_order(gs, fmt, spp, spl, n_hits):
+    """The warp per pixel of small images adds a pixel's samples in the order
+    of the layout that gs_trace_layout reports: the image of the per-lane walk
+    (which an explicit stack depth keeps) bit for bit."""
+    cloud = scenes.tiny_cloud(5, M=700)
+    cloud.log_scales[:] += 1.0
+    g = gs.Gaussians.from_cloud(cloud)
+    bvh = gs.build_bvh(g, node_format=fmt)
+    for cam in SMALL[:2]:
+        kw = dict(seed=6, spp=spp, n_hits=n_hits, samples_per_lane=spl, bg=(0.3, 0.2, 0.9))
+        rgb = gs.trace_stochastic(bvh, g, cam, **kw)
+        ref = gs.trace_stochastic(bvh, g, cam, stack_depth=96, **kw)
+        assert torch.equal(rgb, ref)
+    bvh.sync_status()
+    bvh.free()
