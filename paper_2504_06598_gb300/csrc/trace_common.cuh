@@ -1200,8 +1200,10 @@ __device__ __forceinline__ void tile_pyramid(const float d[3], bool in, float *p
         tx = fmaxf(tx, __shfl_xor_sync(kAll, tx, o));
         ty = fmaxf(ty, __shfl_xor_sync(kAll, ty, o));
     }
-    // 2^-17 of the distance outward: the roundings here and in the box test
-    // stay below 2^-20 of it
+    // 2^-17 of the distance outward, and 2^-20 of the box's extent along each
+    // axis of the frame: the roundings here and in the box test (its sums and
+    // differences of planes have the box's size, however near its closest
+    // point is) stay below a quarter of the two together
     tx += 0x1p-17f;
     ty += 0x1p-17f;
     __syncwarp();
@@ -1209,11 +1211,11 @@ __device__ __forceinline__ void tile_pyramid(const float d[3], bool in, float *p
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
             pyr[i] = narrow ? r[i] : 0.0f;
-            pyr[3 + i] = narrow ? fabsf(r[i]) : 0.0f;
+            pyr[3 + i] = narrow ? fabsf(r[i]) * (1.0f + 0x1p-20f) : 0.0f;
             pyr[6 + i] = narrow ? u[i] : 0.0f;
-            pyr[9 + i] = narrow ? fabsf(u[i]) : 0.0f;
+            pyr[9 + i] = narrow ? fabsf(u[i]) * (1.0f + 0x1p-20f) : 0.0f;
             pyr[12 + i] = narrow ? f[i] : 0.0f;
-            pyr[15 + i] = narrow ? fabsf(f[i]) : 0.0f;
+            pyr[15 + i] = narrow ? fabsf(f[i]) * (1.0f + 0x1p-20f) : 0.0f;
         }
         pyr[18] = narrow ? tx : 0.0f;
         pyr[19] = narrow ? ty : 0.0f;

@@ -177,3 +177,27 @@ def test_small_images_add_samples_in_the_layouts_order(gs, fmt, spp, spl, n_hits
         assert torch.equal(rgb, ref)
     bvh.sync_status()
     bvh.free()
+
+
+@pytest.mark.parametrize("fmt", ["binary", "binary_q8"])
+@pytest.mark.parametrize("seed", [0, 2, 4, 5])
+def test_far_outliers_hide_nothing(gs, fmt, seed):
+    """Gaussians far outside the scene make nodes as long as they are far; what
+    lies beside them in such a node is still found."""
+    M, n = 4000, 1500
+    cloud = scenes.tiny_cloud(seed, M=M)
+    rng = np.random.default_rng(seed)
+    far = 10.0 ** rng.uniform(0.5, 8, (n, 3)) * rng.choice([-1, 1], (n, 3))
+    cloud.means[:n, 0] = far[:, 0]
+    cloud.log_scales[:] -= 1.0
+    cloud = cloud.subset(rng.permutation(M))
+    g = gs.Gaussians.from_cloud(cloud)
+    bvh = gs.build_bvh(g, node_format=fmt)
+    for cam in LARGE[:1] + SMALL[:2]:
+        for spp in (1, 16, 64):
+            kw = dict(seed=1, spp=spp, want_hits=True)
+            _, a, ta = gs.trace_stochastic(bvh, g, cam, **kw)
+            _, b, tb = gs.trace_stochastic(bvh, g, cam, stack_depth=96, **kw)
+            assert torch.equal(a, b) and torch.equal(ta, tb), (cam, spp)
+    bvh.sync_status()
+    bvh.free()
