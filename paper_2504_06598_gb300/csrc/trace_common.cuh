@@ -1155,14 +1155,17 @@ __device__ __forceinline__ void traverse_group(const TraceArgs &a, Ray<N> &r, in
 // A warp's rays through one apex (camera rays through the eye; shadow rays
 // through their light) as a narrow pyramid: an orthonormal frame (r, u, f)
 // with f inside the rays, and the largest |x / z| and |y / z| of a ray in it.
-// Kept in shared memory, 20 floats per warp: r, |r|, u, |u|, f, |f|, tx, ty.
-constexpr int kTileFloats = 20;
+// Kept in shared memory, 24 floats per warp: r, |r|, u, |u|, f, |f|, tx, ty, twice
+// the distance by which a ray may miss the apex, padding.
+constexpr int kTileFloats = 24;
 constexpr int kTilePool = 256;  // stack entries per warp
 
 // Fills the warp's pyramid from each lane's direction d (away from the apex,
-// any length; `in` marks the lanes that count). false when the rays spread
-// too far for it (or none counts): the caller then traverses otherwise.
-__device__ __forceinline__ void tile_pyramid(const float d[3], bool in, float *pyr) {
+// any length; `in` marks the lanes that count). miss: no ray passes the apex
+// farther away than this. A zero frame, which every box meets, when the rays
+// spread too far (or none counts).
+__device__ __forceinline__ void tile_pyramid(const float d[3], bool in, float *pyr,
+                                             float miss = 0.0f) {
     const uint32_t kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const float n = rsqrtf(fmaf(d[0], d[0], fmaf(d[1], d[1], d[2] * d[2])));
@@ -1219,6 +1222,7 @@ __device__ __forceinline__ void tile_pyramid(const float d[3], bool in, float *p
         }
         pyr[18] = narrow ? tx : 0.0f;
         pyr[19] = narrow ? ty : 0.0f;
+        pyr[20] = 2.0f * miss;
     }
     __syncwarp();
 }
@@ -1227,11 +1231,13 @@ __device__ __forceinline__ void tile_pyramid(const float d[3], bool in, float *p
 // than the clip (squared, g2), and its squared distance from the apex. With
 // c twice the centre and e twice the half extents in the pyramid's frame,
 // the box reaches in front of the apex if cz + ez >= 0 and into the pyramid
-// if |cx| <= ex + tx (cz + ez), likewise y. A NaN box never does.
+// if |cx| <= ex + tx (cz + ez), likewise y; where the rays miss the apex, ex, ey
+// and ez are as much larger. A NaN box never does.
 __device__ __forceinline__ bool tile_box(const float lo[3], const float hi[3], const float *pyr,
                                          float g2, float &d2) {
     const float4 *p = reinterpret_cast<const float4 *>(pyr);
     const float4 p0 = p[0], p1 = p[1], p2 = p[2], p3 = p[3], p4 = p[4];
+    const float miss2 = pyr[20];
     float c[3], e[3], m[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
@@ -1241,11 +1247,11 @@ __device__ __forceinline__ bool tile_box(const float lo[3], const float hi[3], c
     }
     d2 = fmaf(m[0], m[0], fmaf(m[1], m[1], m[2] * m[2]));
     const float cx = fmaf(p0.x, c[0], fmaf(p0.y, c[1], p0.z * c[2]));
-    const float ex = fmaf(p0.w, e[0], fmaf(p1.x, e[1], p1.y * e[2]));
+    const float ex = fmaf(p0.w, e[0], fmaf(p1.x, e[1], fmaf(p1.y, e[2], miss2)));
     const float cy = fmaf(p1.z, c[0], fmaf(p1.w, c[1], p2.x * c[2]));
-    const float ey = fmaf(p2.y, e[0], fmaf(p2.z, e[1], p2.w * e[2]));
+    const float ey = fmaf(p2.y, e[0], fmaf(p2.z, e[1], fmaf(p2.w, e[2], miss2)));
     const float cz = fmaf(p3.x, c[0], fmaf(p3.y, c[1], p3.z * c[2]));
-    const float s = cz + fmaf(p3.w, e[0], fmaf(p4.x, e[1], p4.y * e[2]));
+    const float s = cz + fmaf(p3.w, e[0], fmaf(p4.x, e[1], fmaf(p4.y, e[2], miss2)));
     return s >= 0.0f && fabsf(cx) <= fmaf(p4.z, s, ex) && fabsf(cy) <= fmaf(p4.w, s, ey) && d2 <= g2;
 }
 

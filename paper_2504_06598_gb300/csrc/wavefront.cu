@@ -329,8 +329,13 @@ __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
                 update_clip(sr, sr.t_max);
                 if (!any_need) sr.t_far = -INFINITY;
                 if constexpr (GLG == kTileWarp) {
+                    // a shadow ray starts at its ground point, so it passes the
+                    // light by the rounding of its direction: below 2^-22 of
+                    // the distance, which near the light is all there is
                     const float away[3] = {-omega[0], -omega[1], -omega[2]};
-                    tile_pyramid(away, any_need, pyr);
+                    const uint32_t far =
+                        __reduce_max_sync(kAll, any_need ? __float_as_uint(dist) : 0u);
+                    tile_pyramid(away, any_need, pyr, 0x1p-21f * __uint_as_float(far));
                 }
                 trace_pixel_ray<FMT, GLG, COUNT, K>(a, sr, pass, w.light_pos[l], pyr, stack, stack_t,
                                                     g_ref, g_t, err, cnt);

@@ -59,3 +59,43 @@ def test_small_frames_add_samples_in_the_layouts_order(gs, spp):
     for fmt in ("binary", "binary_q8"):
         rgb, got = _render(gs, g, cams, ex, fmt, spp=spp)
         assert torch.equal(got, smp) and torch.equal(rgb, ref), fmt
+
+
+@pytest.mark.parametrize("fmt", ["binary", "binary_q8"])
+@pytest.mark.parametrize("spp", [1, 3, 4, 16])
+def test_tiles(gs, fmt, spp):
+    """Frames large enough for the tile walk: camera rays and the shadow rays
+    toward lights above the scene, in its middle and close to the ground (whose
+    nearest pixels have no pyramid), at odd sizes."""
+    g = gs.Gaussians.from_cloud(scenes.shell_cloud(7, M=6000))
+    cams = scenes.wavefront_views(2, seed=4, fixed_res=(401, 299))
+    ex = scenes.ground_and_lights(2, seed=1)
+    ex.lights += [((0.0, 0.0, 0.0), (1.0, 2.0, 3.0)), ((0.4, -1.29, 0.3), (0.1, 0.1, 0.1))]
+    ref, smp = _render(gs, g, cams, ex, "wide4", spp=spp)
+    rgb, got = _render(gs, g, cams, ex, fmt, spp=spp)
+    assert torch.equal(got, smp) and torch.equal(rgb, ref)
+
+
+@pytest.mark.parametrize("fmt", ["binary", "binary_q8"])
+@pytest.mark.parametrize("spp", [1, 4])
+@pytest.mark.parametrize("size", [1e-3, 1e-4])
+def test_shadows_of_gaussians_beside_the_light(gs, fmt, spp, size):
+    """A light a hundred units above the ground, inside a cloud as small as
+    `size`: shadow rays pass the light by the rounding of their direction, a
+    length not far below that of the cloud's Gaussians."""
+    cloud = scenes.tiny_cloud(9, M=2000)
+    cloud.means[:] *= np.float32(size)
+    cloud.log_scales[:] += np.float32(np.log(size))
+    g = gs.Gaussians.from_cloud(cloud)
+    cams = [scenes.Pinhole(width=401, height=299, eye=(x, 60.0, 0.1), look_at=(0.0, -100.0, 0.0),
+                           up=(0.0, 0.0, 1.0), ray_id_offset=o) for x, o in ((0.0, 0), (90.0, 401 * 299))]
+    ex = scenes.SceneExtras(lights=[((0.0, 0.0, 0.0), (1.0, 1.0, 1.0))], has_ground=True,
+                            ground_y=-100.0, ground_half_extent=300.0)
+    _, smp = _render(gs, g, cams, ex, "wide4", spp=spp)
+    _, got = _render(gs, g, cams, ex, fmt, spp=spp)
+    lit, got_lit = smp[..., 2] != 0, got[..., 2] != 0
+    assert lit.any() and not lit[smp[..., 0] == -2].all()
+    # a shadow is a hit that was found. (The packets miss a few of these: their
+    # slabs are taken from the ground point, a hundred units away.)
+    assert torch.equal(got[..., :2], smp[..., :2])
+    assert not (got_lit & ~lit).any()
