@@ -97,9 +97,10 @@ __global__ void __launch_bounds__(kThreads, is_group_fmt(FMT) ? group_min_blocks
     uint32_t *grp_ref = s_ref[pooled ? threadIdx.x >> 5 : 0] + grp_off;
     float *grp_t = s_t[pooled ? threadIdx.x >> 5 : 0] + grp_off;
     float *pyr = s_pyr[tiled ? threadIdx.x >> 5 : 0];
-    // a warp on one pixel of a layout of fewer lanes: the colours (at most 64)
-    // pass through the walk's stack
-    const bool relay = grouped && LG == 5 && !COUNT && a.sum_log2 < 5;
+    // a warp on one pixel with more passes than its layout has lanes: the colours
+    // (at most 64) pass through the walk's stack. (Otherwise each pass is a lane's
+    // own in the layout too.)
+    const bool relay = grouped && LG == 5 && !COUNT && a.sum_log2 < 5 && a.spp > 1 << a.sum_log2;
     float(*colour)[64] = reinterpret_cast<float(*)[64]>(grp_ref);
     const int sum_lanes = relay ? 1 << a.sum_log2 : L;
     for (;;) {

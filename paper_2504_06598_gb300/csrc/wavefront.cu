@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
         pyr = reinterpret_cast<float *>(pool + 2 * kTilePool);
     }
     // a warp per pixel: sums in the layout's order (as in k_trace)
-    const bool relay = GLG == 5 && !COUNT && a.sum_log2 < 5;
+    const bool relay = GLG == 5 && !COUNT && a.sum_log2 < 5 && a.spp > 1 << a.sum_log2;
     float(*colour)[64] = reinterpret_cast<float(*)[64]>(g_ref);
     const int lg = a.lpp_log2, L = 1 << lg;
     const int tw_lg = tile_w_log2(lg), th_lg = 5 - lg - tw_lg;
