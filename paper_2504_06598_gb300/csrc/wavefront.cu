@@ -500,10 +500,10 @@ __device__ __forceinline__ void bounce_finish(const WaveArgs &w, const Ray<1> &b
 
 // One step of traverse_lane's walk of the binary nodes, its state (node,
 // stack depth, steps) held by the caller: false once the walk has no node
-// left. Leaves the ray reaches are handed to the caller (their records, the
-// farther one first), at most two a step, instead of being evaluated here.
-template <bool COUNT>
-__device__ __forceinline__ bool lane_step(const TraceArgs &a, const Ray<1> &r, uint32_t &node,
+// left. HOLD: leaves the ray reaches are handed to the caller (their records,
+// the farther one first), at most two a step, instead of being evaluated here.
+template <bool COUNT, bool HOLD>
+__device__ __forceinline__ bool lane_step(const TraceArgs &a, Ray<1> &r, int pass, uint32_t &node,
                                           int &sp, uint32_t &steps, uint32_t *stack,
                                           float *stack_t, uint32_t leaves[2], int &n_leaves,
                                           uint32_t &err, Counts &cnt) {
@@ -526,7 +526,22 @@ __device__ __forceinline__ bool lane_step(const TraceArgs &a, const Ray<1> &r, u
     bool hR = slab(boxR, r.inv, r.oinv, r.t_min, r.t_far, tR);
     const bool leafL = (cref.x & kLeafBit) != 0u, leafR = (cref.y & kLeafBit) != 0u;
     const bool left_first = tL <= tR;
-    {
+    if constexpr (!HOLD) {
+        if ((leafL && hL) || (leafR && hR)) {
+            const bool swap = leafL && leafR && hR && (!hL || tR < tL);
+            for (int li = 0; li < 2; ++li) {
+                const bool right = (li == 0) == swap;
+                if (!(right ? leafR : leafL) || !(right ? hR : hL)) continue;
+                if (COUNT) {
+                    ++cnt.prims;
+                    ++cnt.prim_fetch;
+                }
+                intersect<1, COUNT>(a, r, (right ? cref.y : cref.x) & ~kLeafBit, pass, cnt.draws);
+            }
+        }
+        hL = hL && tL <= r.t_far;
+        hR = hR && tR <= r.t_far;
+    } else {
         const bool l = leafL && hL, q = leafR && hR;
         n_leaves = (int)l + (int)q;
         leaves[0] = l && (!q || !left_first) ? cref.x : cref.y;
@@ -579,17 +594,19 @@ __device__ __forceinline__ bool lane_step(const TraceArgs &a, const Ray<1> &r, u
 // Alg. 1 (two to three times a node step's instructions) for those few. A
 // lane keeps up to kPending of them and walks on while there is room; the
 // warp evaluates one per lane when kEvalLanes lanes hold some, or when no lane
-// can walk on. A clip that moves later than it could only costs node steps:
-// the order of candidates does not change a sample's hit. Each lane shades
-// its ray when the walk ends and writes albedo x radiance to the sample's slot. On
-// 4-wide nodes a warp takes 32 consecutive codes and walks them as a
-// packet.
+// can walk on. A clip that moves later than it could only costs node steps and
+// stack entries: the order of candidates does not change a sample's hit. (HOLD;
+// otherwise a lane evaluates in the step: where the stack is shorter than the
+// deepest tree, a walk that fits it must not overflow for the nodes behind its
+// clip.) Each lane shades its ray when the walk ends and writes albedo x radiance
+// to the sample's slot. On 4-wide nodes a warp takes 32 consecutive codes and
+// walks them as a packet.
 // 16-view frame at spp 16 for 8, 12, 20 and 26 holding lanes: 353.9, 349.4, 352.4
 // and 371.2 ms; with up to six leaves a lane 364.8 (24 lanes).
 constexpr int kPending = 4;
 constexpr int kEvalLanes = 12;
 
-template <int FMT, int STACK, bool COUNT>
+template <int FMT, int STACK, bool COUNT, bool HOLD>
 __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
     k_bounce(const WaveArgs w, const unsigned long long *__restrict__ codes, int64_t n_slots) {
     const TraceArgs &a = w.t;
@@ -634,6 +651,15 @@ __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
                 }
             }
             if (!__any_sync(kAll, active) && !__any_sync(kAll, more)) break;
+            if constexpr (!HOLD) {
+                int nl;
+                if (active && !lane_step<COUNT, false>(a, br, s, node, sp, steps, stack, stack_t,
+                                                       nullptr, nl, err, cnt)) {
+                    active = false;
+                    bounce_finish(w, br, gpix, s);
+                }
+                continue;
+            }
             const bool room = walking && np <= kPending - 2;
             const uint32_t holding = __ballot_sync(kAll, np > 0);
             if (__popc(holding) >= kEvalLanes || !__any_sync(kAll, room)) {
@@ -648,7 +674,8 @@ __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
             } else if (room) {
                 uint32_t leaves[2];
                 int nl;
-                walking = lane_step<COUNT>(a, br, node, sp, steps, stack, stack_t, leaves, nl, err, cnt);
+                walking = lane_step<COUNT, true>(a, br, s, node, sp, steps, stack, stack_t, leaves, nl,
+                                                 err, cnt);
 #pragma unroll
                 for (int k = 0; k < kPending; ++k) {
                     if (nl > 0 && k == np) pend[k] = leaves[0];
@@ -707,14 +734,14 @@ __global__ void k_combine(const WaveArgs w) {
     for (int c = 0; c < 3; ++c) a.rgb[3 * px + c] = fmaf(sum[c], inv_n, a.rgb[3 * px + c]);
 }
 
-template <int FMT, int STACK, bool COUNT>
+template <int FMT, int STACK, bool COUNT, bool HOLD>
 gs_status launch_bounce(const WaveArgs &w, const unsigned long long *codes, int64_t n_slots,
                         int threads, cudaStream_t s) {
     int dev = 0, sms = 0, per = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_bounce<FMT, STACK, COUNT>,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_bounce<FMT, STACK, COUNT, HOLD>,
                                                           threads, 0);
     if (e != cudaSuccess) return cuda_fail(e, "bounce launch setup");
     const int64_t tiles = (n_slots + 31) / 32;
@@ -725,7 +752,7 @@ gs_status launch_bounce(const WaveArgs &w, const unsigned long long *codes, int6
     if (blocks == 0) return GS_OK;
     if ((e = cudaMemsetAsync(w.t.work, 0, sizeof(uint32_t), s)) != cudaSuccess)
         return cuda_fail(e, "reset work counter");
-    k_bounce<FMT, STACK, COUNT><<<blocks, threads, 0, s>>>(w, codes, n_slots);
+    k_bounce<FMT, STACK, COUNT, HOLD><<<blocks, threads, 0, s>>>(w, codes, n_slots);
     k_combine<<<(unsigned)((w.n_pix + 255) / 256), 256, 0, s>>>(w);
     return GS_OK;
 }
@@ -735,10 +762,15 @@ gs_status launch_bounce_f(const WaveArgs &w, const unsigned long long *codes, in
                           int threads, int stack, cudaStream_t s) {
     const bool count = w.counters != nullptr;
     if (stack == 48)
-        return count ? launch_bounce<FMT, 48, true>(w, codes, n_slots, threads, s)
-                     : launch_bounce<FMT, 48, false>(w, codes, n_slots, threads, s);
-    return count ? launch_bounce<FMT, 96, true>(w, codes, n_slots, threads, s)
-                 : launch_bounce<FMT, 96, false>(w, codes, n_slots, threads, s);
+        return count ? launch_bounce<FMT, 48, true, false>(w, codes, n_slots, threads, s)
+                     : launch_bounce<FMT, 48, false, false>(w, codes, n_slots, threads, s);
+    // (a tree has at most 95 levels)
+    if constexpr (FMT == GS_NODES_BINARY)
+        if (w.t.stack_depth == kMaxStack)
+            return count ? launch_bounce<FMT, 96, true, true>(w, codes, n_slots, threads, s)
+                         : launch_bounce<FMT, 96, false, true>(w, codes, n_slots, threads, s);
+    return count ? launch_bounce<FMT, 96, true, false>(w, codes, n_slots, threads, s)
+                 : launch_bounce<FMT, 96, false, false>(w, codes, n_slots, threads, s);
 }
 
 template <int FMT, int STACK, bool COUNT, int GLG, int K = 1>

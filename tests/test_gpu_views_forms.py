@@ -99,3 +99,32 @@ def test_shadows_of_gaussians_beside_the_light(gs, fmt, spp, size):
     # slabs are taken from the ground point, a hundred units away.)
     assert torch.equal(got[..., :2], smp[..., :2])
     assert not (got_lit & ~lit).any()
+
+
+@pytest.mark.parametrize("fmt", ["binary", "binary_q8"])
+def test_bounce_rays_at_a_small_stack(gs, fmt):
+    """An opaque sheet above the ground is the root's left child: a bounce ray
+    that evaluates it first never pushes a node."""
+    cloud = scenes.tiny_cloud(2, M=65)
+    cloud.means[1:, 0] = 0.55 + 0.45 * np.abs(cloud.means[1:, 0])
+    cloud.means[1:, 1] += 2.0
+    cloud.log_scales[1:] += 1.0
+    cloud.means[0] = (0.0, 0.0, 0.0)
+    cloud.log_scales[0] = (5.0, -4.0, 5.0)
+    cloud.quats[0] = (1.0, 0.0, 0.0, 0.0)
+    cloud.opacity_logits[0] = 40.0
+    g = gs.Gaussians.from_cloud(cloud)
+    ex = scenes.SceneExtras(lights=[], has_ground=True, ground_y=-0.5, ground_half_extent=3.0, bounce=True, shadow_eps=1e-4)
+    bvh = gs.build_bvh(g, node_format=fmt)
+    cnt = torch.zeros(4, dtype=torch.int64, device="cuda")
+    # eight rays at a time: too few for the warp to evaluate at once
+    for x in np.linspace(-0.4, 1.2, 60):
+        cams = [scenes.Pinhole(width=1, height=1, eye=(0.3, -0.1, 0.4), look_at=(float(x), -0.5, 0.0))]
+        _, s0 = gs.render_views(bvh, g, cams, ex, seed=1, spp=8, want_samples=True)
+        # (counters: camera rays in groups, which have a stack of their own)
+        _, s1 = gs.render_views(bvh, g, cams, ex, seed=1, spp=8, counters=cnt, stack_depth=1,
+                                want_samples=True)
+        bvh.sync_status()
+        assert torch.equal(s0, s1)
+        assert (s0[..., 1] == 0).any()
+    bvh.free()
