@@ -57,6 +57,7 @@ struct WaveArgs {
     unsigned long long *codes;
     float *bounce_rgb;
     int spl;  // samples per lane of the camera and shadow pass (1, 2, 4 or 8)
+    int eval_lanes;  // lanes holding leaves at which the bounce pass evaluates them
 };
 
 // Sort code of a deferred bounce ray: 28 key bits (direction bin in an
@@ -593,18 +594,23 @@ __device__ __forceinline__ bool lane_step(const TraceArgs &a, Ray<1> &r, int pas
 // at once: about one lane in six reaches one per step, and the warp would run
 // Alg. 1 (two to three times a node step's instructions) for those few. A
 // lane keeps up to kPending of them and walks on while there is room; the
-// warp evaluates one per lane when kEvalLanes lanes hold some, or when no lane
+// warp evaluates one per lane when eval_lanes lanes hold some, or when no lane
 // can walk on. A clip that moves later than it could only costs node steps and
 // stack entries: the order of candidates does not change a sample's hit. (HOLD;
-// otherwise a lane evaluates in the step: where the stack is shorter than the
-// deepest tree, a walk that fits it must not overflow for the nodes behind its
-// clip.) Each lane shades its ray when the walk ends and writes albedo x radiance
+// otherwise a lane evaluates in the step: in small frames, and where the stack is
+// shorter than the deepest tree, since a walk that fits it must not overflow for
+// the nodes behind its clip.) Each lane shades its ray when the walk ends and writes albedo x radiance
 // to the sample's slot. On 4-wide nodes a warp takes 32 consecutive codes and
 // walks them as a packet.
 // 16-view frame at spp 16 for 8, 12, 20 and 26 holding lanes: 353.9, 349.4, 352.4
-// and 371.2 ms; with up to six leaves a lane 364.8 (24 lanes).
+// and 371.2 ms; with up to six leaves a lane 364.8 (24 lanes). The fewer the rays,
+// the less those of a warp have in common, and the more the steps past a clip
+// that has not moved cost. This pass over the 1M shell (ms) with 12 holding lanes,
+// with 4, and with evaluation in the step: 33M samples 37.3, 38.9, 41.9; 8M 12.8,
+// 11.9, 12.2; 0.5M 6.2, 4.6, 3.9.
 constexpr int kPending = 4;
-constexpr int kEvalLanes = 12;
+constexpr int kEvalLanes = 12, kEvalLanesFew = 4;
+constexpr int64_t kHoldSlots = 1 << 21, kManySlots = 12 << 20;
 
 template <int FMT, int STACK, bool COUNT, bool HOLD>
 __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
@@ -662,7 +668,7 @@ __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
             }
             const bool room = walking && np <= kPending - 2;
             const uint32_t holding = __ballot_sync(kAll, np > 0);
-            if (__popc(holding) >= kEvalLanes || !__any_sync(kAll, room)) {
+            if (__popc(holding) >= w.eval_lanes || !__any_sync(kAll, room)) {
                 if (np > 0) {
                     uint32_t leaf = pend[0];
 #pragma unroll
@@ -766,7 +772,7 @@ gs_status launch_bounce_f(const WaveArgs &w, const unsigned long long *codes, in
                      : launch_bounce<FMT, 48, false, false>(w, codes, n_slots, threads, s);
     // (a tree has at most 95 levels)
     if constexpr (FMT == GS_NODES_BINARY)
-        if (w.t.stack_depth == kMaxStack)
+        if (w.t.stack_depth == kMaxStack && n_slots >= kHoldSlots)
             return count ? launch_bounce<FMT, 96, true, true>(w, codes, n_slots, threads, s)
                          : launch_bounce<FMT, 96, false, true>(w, codes, n_slots, threads, s);
     return count ? launch_bounce<FMT, 96, true, false>(w, codes, n_slots, threads, s)
@@ -1045,6 +1051,7 @@ gs_status launch_render_views(const gs_bvh *b, const gs_gaussians *g, const gs_p
         w.deferred = 1;
         w.codes = mb->wave_codes[0];
         w.bounce_rgb = mb->wave_bounce;
+        w.eval_lanes = slots >= kManySlots ? kEvalLanes : kEvalLanesFew;
     }
     switch (b->node_format) {
         case GS_NODES_WIDE4: st = launch_views_f<GS_NODES_WIDE4>(w, threads, stack, s); break;
