@@ -345,13 +345,18 @@ void scan_exclusive(uint32_t *a, int64_t n, uint32_t *sums, cudaStream_t s) {
 // the counts of digit d until a tile whose running total is known. The keys
 // go through shared memory so that each digit's run is stored together.
 // A tile is taken only after the tiles before it, so each waits only on
-// blocks that are already running; the wait is bounded all the same.
+// blocks that are already running; the wait is bounded all the same, and a
+// thread whose wait runs out counts its digit in the tile's keys itself: the
+// order of the keys, which the rest of the build indexes by, never depends on it.
 // Against a histogram, a three-kernel scan and a scatter per digit (40
 // launches for eight digits): the whole rebuild 806 -> 557 us at 1M, 272 -> 132
 // at 1,000. Bound by the chain of a tile, about 20 us a digit at 1M.
 constexpr unsigned long long kTileCounted = 1ull << 62, kTileTotal = 2ull << 62;
 constexpr unsigned long long kTileValue = (1ull << 40) - 1ull;
-constexpr int kLookbackLimit = 1 << 24;
+#ifndef GSRT_LOOKBACK_LIMIT  // (a test builds with 0)
+#define GSRT_LOOKBACK_LIMIT (1 << 24)
+#endif
+constexpr int kLookbackLimit = GSRT_LOOKBACK_LIMIT;
 
 // Four blocks per SM, so that the tiles of 1M keys run at once (three, at 74
 // registers, left a second wave: 21 us a pass).
@@ -360,8 +365,7 @@ __global__ void __launch_bounds__(kSortThreads, 4)
     k_radix_pass(int64_t n, const unsigned long long *__restrict__ kin,
                  const uint32_t *__restrict__ vin, unsigned long long *__restrict__ kout,
                  uint32_t *__restrict__ vout, int pass, const uint32_t *__restrict__ hist,
-                 uint32_t *__restrict__ tickets, unsigned long long *__restrict__ tile_state,
-                 uint32_t *__restrict__ status) {
+                 uint32_t *__restrict__ tickets, unsigned long long *__restrict__ tile_state) {
     constexpr int W = kSortThreads / 32;
     __shared__ unsigned long long s_key[kSortTile];
     __shared__ uint32_t s_val[VALS ? kSortTile : 1];
@@ -431,9 +435,11 @@ __global__ void __launch_bounds__(kSortThreads, 4)
             }
         if (done) break;
         t -= used;
-        if (used == 0 && ++spins > kLookbackLimit) {
-            atomicOr(status, kErrSteps);
-            break;
+        if (used == 0 && spins++ >= kLookbackLimit) {
+            const int64_t end = min((t + 1) * kSortTile, n);
+            for (int64_t i = t * kSortTile; i < end; ++i)
+                prior += ((uint32_t)(kin[i] >> shift) & 255u) == (uint32_t)tid;
+            --t;
         }
     }
     if (tile > 0) *mine = kTileTotal | tag | (prior + count);
@@ -453,7 +459,6 @@ __global__ void __launch_bounds__(kSortThreads, 4)
     for (int i = tid; i < m; i += kSortThreads) {
         const unsigned long long k = s_key[i];
         const int64_t pos = s_shift[(uint32_t)(k >> shift) & 255u] + i;
-        if (pos < 0 || pos >= n) continue;  // after a wait that ran out
         kout[pos] = k;
         if constexpr (VALS) vout[pos] = s_val[i];
     }
@@ -1202,7 +1207,7 @@ constexpr int kBuildCounters = kGroupTrees + 1;
 size_t build_scratch_bytes(int64_t n) { return ZeroScratch(n, n + kBuildCounters).bytes; }
 
 int sort_keys64(unsigned long long *keys[2], int64_t n, int lo_bit, void *scratch,
-                uint32_t *status, cudaStream_t s) {
+                cudaStream_t s) {
     const ZeroScratch z(n, 0);
     unsigned char *base = static_cast<unsigned char *>(scratch);
     uint32_t *hist = reinterpret_cast<uint32_t *>(base + z.hist);
@@ -1216,7 +1221,7 @@ int sort_keys64(unsigned long long *keys[2], int64_t n, int lo_bit, void *scratc
         k_radix_pass<false><<<(unsigned)tiles, kSortThreads, 0, s>>>(
             n, keys[cur], nullptr, keys[1 - cur], nullptr, pass, hist,
             reinterpret_cast<uint32_t *>(base + z.tickets),
-            reinterpret_cast<unsigned long long *>(base + z.states), status);
+            reinterpret_cast<unsigned long long *>(base + z.states));
         cur = 1 - cur;
     }
     return cur;
@@ -1257,7 +1262,7 @@ gs_status build_into(gs_bvh *b, const gs_gaussians *g, cudaStream_t s) {
             k_radix_pass<true><<<(unsigned)tiles, kSortThreads, 0, s>>>(
                 M, b->codes[cur], b->vals[cur], b->codes[1 - cur], b->vals[1 - cur], pass, hist,
                 reinterpret_cast<uint32_t *>(base + z.tickets),
-                reinterpret_cast<unsigned long long *>(base + z.states), b->status);
+                reinterpret_cast<unsigned long long *>(base + z.states));
             cur = 1 - cur;
         }
     }

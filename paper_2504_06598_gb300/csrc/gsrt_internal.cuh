@@ -183,10 +183,10 @@ size_t build_scratch_bytes(int64_t n);
 // Stable LSD radix sort of n 64-bit keys on bits [lo_bit, 64), 8 bits per
 // pass, ping-ponging between keys[0] and keys[1]; returns the index of the
 // buffer holding the result. scratch: sort_scratch_bytes(n) bytes, 256-byte
-// aligned; status: receives kErrSteps if a wait between tiles runs out.
+// aligned.
 size_t sort_scratch_bytes(int64_t n);
 int sort_keys64(unsigned long long *keys[2], int64_t n, int lo_bit, void *scratch,
-                uint32_t *status, cudaStream_t s);
+                cudaStream_t s);
 
 // Batched form (wavefront.cu): grows the handle's deferred-bounce scratch to
 // `slots` sample slots (synchronous allocation; refused while the stream is

@@ -436,7 +436,7 @@ __global__ void __launch_bounds__(kThreads, 8) k_trace_shared(const __grid_const
                     const uint32_t next = __shfl_sync(kAll, ref, nj);
                     const uint32_t others = im & ~(1u << nj);
                     const int npush = __popc(others);
-                    if (sp + npush > kSharedPool) {
+                    if (sp + npush > kSharedPool >> kPoolShift) {
                         full = true;
                         break;
                     }

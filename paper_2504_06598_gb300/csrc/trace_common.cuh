@@ -927,6 +927,11 @@ __device__ __forceinline__ bool group_child(const void *grec, uint32_t node, int
 }
 
 constexpr int kGroupPool = 512;    // stack entries per warp, split among its groups
+// A test builds with the pools' use cut to 1/8, so that walks start over.
+#ifndef GSRT_POOL_SHIFT
+#define GSRT_POOL_SHIFT 0
+#endif
+constexpr int kPoolShift = GSRT_POOL_SHIFT;
 constexpr int kGroupMinBlocks = 8; // resident blocks per SM to build for
 
 // Cooperative traversal of the W-wide hierarchy (W = L = 2^LG, 8 to 32) by a
@@ -946,7 +951,7 @@ __device__ __forceinline__ void traverse_group(const TraceArgs &a, Ray<N> &r, in
                                                uint32_t *s_ref, float *s_t, uint32_t &err,
                                                Counts &cnt) {
     constexpr int L = 1 << LG;
-    constexpr int kCap = kGroupPool >> (5 - LG);  // this group's stack entries
+    constexpr int kCap = (kGroupPool >> (5 - LG)) >> kPoolShift;  // this group's stack entries
     constexpr uint32_t kLaneBits = L == 32 ? 0xffffffffu : ((1u << (L & 31)) - 1u);
     const int lane = threadIdx.x & 31;
     const int base = lane & ~(L - 1);
@@ -1353,7 +1358,7 @@ __device__ __forceinline__ bool traverse_tile(const TraceArgs &a, Ray<N> &r, int
             const uint32_t next = __shfl_sync(kAll, ref, nj);
             const uint32_t others = im & ~(1u << nj);
             const int npush = __popc(others);
-            if (sp + npush > kTilePool) return false;
+            if (sp + npush > kTilePool >> kPoolShift) return false;
             __syncwarp();  // earlier reads of these entries are done
             if (inner && lane != nj) {
                 const int pos = sp + __popc(others & ((1u << lane) - 1u));

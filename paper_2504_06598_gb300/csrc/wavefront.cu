@@ -1062,7 +1062,7 @@ gs_status launch_render_views(const gs_bvh *b, const gs_gaussians *g, const gs_p
     if (st != GS_OK) return st;
     if (slots > 0) {
         gs_bvh *mb = const_cast<gs_bvh *>(b);
-        const int cur = sort_keys64(mb->wave_codes, slots, 32, mb->wave_sort, mb->status, s);
+        const int cur = sort_keys64(mb->wave_codes, slots, 32, mb->wave_sort, s);
         const unsigned long long *sorted = mb->wave_codes[cur];
         switch (b->node_format) {
             case GS_NODES_WIDE4:
