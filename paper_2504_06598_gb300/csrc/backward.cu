@@ -607,15 +607,15 @@ __device__ __forceinline__ int stat_of(int lane) {
 }
 
 // One candidate (record idx, the same for the warp) against every lane's
-// slots. ck: the colours of the slots' winners, [slot and channel][lane] in
-// shared memory (in registers, 24 more at eight slots, they would spill). The
+// slots. ck: the colours of the slots' winners, [slot][lane] in shared memory (in
+// registers, 24 more at eight slots, they would spill). The
 // difference of the colours comes before the product with g: as the difference
 // of the two products the weight had up to 4e-6 of itself in rounding where
 // colours differ by a hundredth, and no exact 0 where they are equal. 1M at
 // 1080p, spp 16, rebuild + image + gradients 19.79 -> 20.15 ms (the same box).
 template <int N>
 __device__ __forceinline__ void tile_gradient(const TraceArgs &a, const Ray<N> &r, uint32_t idx,
-                                              const float (*ck)[32], const float g[3]) {
+                                              const float4 (*ck)[32], const float g[3]) {
     const uint32_t kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const Cand c = eval_cand<true>(a, r.o, r.d, idx);
@@ -634,9 +634,10 @@ __device__ __forceinline__ void tile_gradient(const TraceArgs &a, const Ray<N> &
         float coef = 0.0f;
 #pragma unroll
         for (int k = 0; k < N; ++k)
-            if ((front >> k) & 1u)
-                coef += fmaf(g[0], ci[0] - ck[3 * k][lane],
-                             fmaf(g[1], ci[1] - ck[3 * k + 1][lane], g[2] * (ci[2] - ck[3 * k + 2][lane])));
+            if ((front >> k) & 1u) {
+                const float4 w = ck[k][lane];
+                coef += fmaf(g[0], ci[0] - w.x, fmaf(g[1], ci[1] - w.y, g[2] * (ci[2] - w.z)));
+            }
         // a rejected hit has alpha <= xi < 1
         wa = coef / (1.0f - c.alpha) * c.alpha;
     }
@@ -665,7 +666,7 @@ constexpr int kTileLevels = 128;
 
 template <int N, bool Q8>
 __device__ __forceinline__ void enumerate_tile(const TraceArgs &a, const Ray<N> &r,
-                                               const float (*ck)[32], const float g[3],
+                                               const float4 (*ck)[32], const float g[3],
                                                const float *pyr, uint2 *stack, uint32_t &err) {
     const uint32_t kAll = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -753,7 +754,7 @@ __global__ void __launch_bounds__(kThreads, N >= 8 ? 5 : 6)
     const uint32_t kAll = 0xffffffffu;
     __shared__ __align__(16) float s_pyr[kThreads / 32][kTileFloats];
     __shared__ uint2 s_lvl[kThreads / 32][kTileLevels];
-    __shared__ float s_ck[kThreads / 32][3 * N][32];
+    __shared__ float4 s_ck[kThreads / 32][N][32];
     // the forward traversal's stack, where the winners are traced again
     __shared__ uint32_t s_ref[KEYS ? 1 : kThreads / 32][KEYS ? 1 : kTilePool];
     __shared__ float s_t[KEYS ? 1 : kThreads / 32][KEYS ? 1 : kTilePool];
@@ -852,7 +853,7 @@ __global__ void __launch_bounds__(kThreads, N >= 8 ? 5 : 6)
                         if (first && (gm[0] != 0.0f || gm[1] != 0.0f || gm[2] != 0.0f))
                             add_sh_gradient(a, wid, gm, Y);
                     }
-                    for (int ch = 0; ch < 3; ++ch) s_ck[warp][3 * k + ch][lane] = ck[ch];
+                    s_ck[warp][k][lane] = make_float4(ck[0], ck[1], ck[2], 0.0f);
                 }
             }
             // 3) every Gaussian in front of a winner
