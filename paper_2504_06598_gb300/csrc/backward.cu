@@ -664,7 +664,7 @@ __device__ __forceinline__ void tile_gradient(const TraceArgs &a, const Ray<N> &
 // tree: at most the 95 levels of the binary one.
 constexpr int kTileLevels = 128;
 
-template <int N, bool Q8>
+template <int N, bool Q8, bool LEAF>
 __device__ __forceinline__ void enumerate_tile(const TraceArgs &a, const Ray<N> &r,
                                                const float4 (*ck)[32], const float g[3],
                                                const float *pyr, uint2 *stack, uint32_t &err) {
@@ -675,6 +675,8 @@ __device__ __forceinline__ void enumerate_tile(const TraceArgs &a, const Ray<N> 
     const float G = __uint_as_float(
         __reduce_max_sync(kAll, live ? __float_as_uint(fmaxf(r.t_far, 0.0f)) : 0u));
     const float g2 = G * G;
+    float inv[3];
+    if constexpr (LEAF) tile_inverse(r.d, inv);
     int sp = 0;
     uint32_t node = __ldg(a.troot), steps = 0;
     for (;;) {
@@ -684,11 +686,13 @@ __device__ __forceinline__ void enumerate_tile(const TraceArgs &a, const Ray<N> 
         }
         const int n_child = (int)((node >> kWideCountShift) & 31u) + 1;
         uint32_t ref = kEmpty;
-        float d2 = INFINITY;
+        float d2 = INFINITY, lo[3] = {0.0f, 0.0f, 0.0f}, hi[3] = {0.0f, 0.0f, 0.0f};
         bool hit = false;
-        if (lane < n_child) hit = tile_child<Q8>(a.trec, node, lane, a.eye, pyr, g2, ref, d2);
+        if (lane < n_child) hit = tile_child<Q8>(a.trec, node, lane, a.eye, pyr, g2, ref, d2, lo, hi);
         const bool leaf = (ref & kLeafBit) != 0u;
         for (uint32_t lm = __ballot_sync(kAll, hit && leaf); lm; lm &= lm - 1u) {
+            if constexpr (LEAF)
+                if (!__any_sync(kAll, tile_leaf(lo, hi, __ffs(lm) - 1, inv, 0.0f, r.t_far))) continue;
             const uint32_t idx = __shfl_sync(kAll, ref, __ffs(lm) - 1) & ~kLeafBit;
             tile_gradient<N>(a, r, idx, ck, g);
         }
@@ -747,7 +751,7 @@ __device__ __forceinline__ void add_sh_gradient(const TraceArgs &a, uint32_t gid
 
 // Built for five blocks per SM with eight slots (four: 1M at 1080p, spp 16,
 // rebuild + image + gradients 17.6 -> 16.9 ms) and six with fewer.
-template <int N, bool Q8, bool KEYS>
+template <int N, bool Q8, bool KEYS, bool LEAF>
 __global__ void __launch_bounds__(kThreads, N >= 8 ? 5 : 6)
     k_backward_tile(const __grid_constant__ TraceArgs a) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -824,7 +828,7 @@ __global__ void __launch_bounds__(kThreads, N >= 8 ? 5 : 6)
                     }
                 }
             } else {
-                trace_tile<N, Q8>(a, r, pass, a.eye, pyr, s_ref[warp], s_t[warp], err);
+                trace_tile<N, Q8, LEAF>(a, r, pass, a.eye, pyr, s_ref[warp], s_t[warp], err);
             }
             // 2) colours of the winners; dLoss/dk of the selected Gaussians,
             // once for the slots of a lane that hold the same one
@@ -860,7 +864,7 @@ __global__ void __launch_bounds__(kThreads, N >= 8 ? 5 : 6)
             update_clip(r, a.t_max);
             if (!live) r.t_far = -INFINITY;
             __syncwarp();
-            enumerate_tile<N, Q8>(a, r, s_ck[warp], g, pyr, s_lvl[warp], err);
+            enumerate_tile<N, Q8, LEAF>(a, r, s_ck[warp], g, pyr, s_lvl[warp], err);
             __syncwarp();
         }
     }
@@ -940,13 +944,13 @@ gs_status launch_backward_nl(const TraceArgs &a, cudaStream_t s) {
 }
 
 // Groups of 8 or more lanes on one pixel use the widest copy that fits them.
-template <int N, bool Q8, bool KEYS>
+template <int N, bool Q8, bool KEYS, bool LEAF>
 gs_status launch_backward_tile(const TraceArgs &a, cudaStream_t s) {
     int dev = 0, sms = 0, per = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_backward_tile<N, Q8, KEYS>,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_backward_tile<N, Q8, KEYS, LEAF>,
                                                           kThreads, 0);
     if (e != cudaSuccess) return cuda_fail(e, "backward launch setup");
     const int tw_lg = tile_w_log2(a.lpp_log2), th_lg = 5 - a.lpp_log2 - tw_lg;
@@ -960,16 +964,19 @@ gs_status launch_backward_tile(const TraceArgs &a, cudaStream_t s) {
         return cuda_fail(e, "reset work counter");
     if ((e = cudaMemsetAsync(a.g_stats, 0, (size_t)a.n_gauss * kStats * sizeof(float), s)) != cudaSuccess)
         return cuda_fail(e, "reset gradient sums");
-    k_backward_tile<N, Q8, KEYS><<<blocks, kThreads, 0, s>>>(a);
+    k_backward_tile<N, Q8, KEYS, LEAF><<<blocks, kThreads, 0, s>>>(a);
     k_chain<<<(unsigned)((a.n_gauss + 255) / 256), 256, 0, s>>>(a);
     return GS_OK;
 }
 
 template <int N, bool KEYS>
 gs_status launch_backward_nk(const TraceArgs &a, cudaStream_t s) {
+    if (a.trec != nullptr && a.leaf_test)
+        return a.gq8 ? launch_backward_tile<N, true, KEYS, true>(a, s)
+                     : launch_backward_tile<N, false, KEYS, true>(a, s);
     if (a.trec != nullptr)
-        return a.gq8 ? launch_backward_tile<N, true, KEYS>(a, s)
-                     : launch_backward_tile<N, false, KEYS>(a, s);
+        return a.gq8 ? launch_backward_tile<N, true, KEYS, false>(a, s)
+                     : launch_backward_tile<N, false, KEYS, false>(a, s);
     if (a.grec != nullptr && a.gq8) {
         switch (a.lpp_log2) {
             case 5: return launch_backward_nl<N, 5, true, KEYS>(a, s);
@@ -1076,6 +1083,7 @@ gs_status launch_backward(const gs_bvh *b, const gs_gaussians *g, const gs_pinho
         a.troot = b->group[kWarpTree].ref;
         a.gq8 = b->node_format == GS_NODES_BINARY_Q8;
         a.g_stats = b->grad;
+        a.leaf_test = leaf_test_pays(b->M, (int64_t)cam->width * cam->height);
         a.sh_vec = ((uintptr_t)d_sh & 15u) == 0;
     }
     a.keys = const_cast<gs_sample_key *>(keys);  // read only here

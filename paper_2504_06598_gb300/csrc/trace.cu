@@ -49,9 +49,10 @@ namespace {
 // GS_NODES_*.
 constexpr int kFmtGroup = 8;
 constexpr int kFmtGroupQ8 = 16;
-// Tile traversal of the 32-wide records by a warp of camera rays.
-constexpr int kFmtTile = 6, kFmtTileQ8 = 7;
-__host__ __device__ constexpr bool is_tile_fmt(int f) { return f == kFmtTile || f == kFmtTileQ8; }
+// Tile traversal of the 32-wide records by a warp of camera rays, with and
+// without the test of each leaf's box.
+constexpr int kFmtTileLeaf = 4, kFmtTileLeafQ8 = 5, kFmtTile = 6, kFmtTileQ8 = 7;
+__host__ __device__ constexpr bool is_tile_fmt(int f) { return f >= kFmtTileLeaf && f <= kFmtTileQ8; }
 __host__ __device__ constexpr bool is_group_fmt(int f) { return f >= kFmtGroup + 3; }
 __host__ __device__ constexpr bool is_group_q8(int f) { return f >= kFmtGroupQ8 + 3; }
 
@@ -140,7 +141,7 @@ __global__ void __launch_bounds__(kThreads, is_group_fmt(FMT) ? group_min_blocks
             if (!live) r.t_far = -INFINITY;  // lanes off the image never hit
             if (a.n_nodes > 0) {
                 if constexpr (tiled) {
-                    trace_tile<N, FMT == kFmtTileQ8>(a, r, pass, a.eye, pyr, grp_ref, grp_t, err);
+                    trace_tile<N, (FMT & 1) != 0, FMT <= kFmtTileLeafQ8>(a, r, pass, a.eye, pyr, grp_ref, grp_t, err);
                 } else if constexpr (grouped) {
                     uint32_t e = 0;
                     traverse_group<N, COUNT, LG, true, is_group_q8(FMT)>(a, r, pass, grp_ref,
@@ -387,9 +388,10 @@ __global__ void __launch_bounds__(kThreads, 8) k_trace_shared(const __grid_const
                 }
                 const int n_child = (int)((node >> kWideCountShift) & 31u) + 1;
                 uint32_t ref = kEmpty;
-                float d2 = INFINITY;
+                float d2 = INFINITY, lo[3], hi[3];
                 bool hit = false;
-                if (lane < n_child) hit = tile_child<Q8>(a.trec, node, lane, a.eye, m.pyr, g2, ref, d2);
+                if (lane < n_child)
+                    hit = tile_child<Q8>(a.trec, node, lane, a.eye, m.pyr, g2, ref, d2, lo, hi);
                 const bool leaf = (ref & kLeafBit) != 0u;
                 const uint32_t lm = __ballot_sync(kAll, hit && leaf);
                 if (lm) {
@@ -586,6 +588,9 @@ gs_status launch_nf(const TraceArgs &a, bool count, cudaStream_t s) {
 
 template <int N>
 gs_status launch_n(const TraceArgs &a, int format, bool count, cudaStream_t s) {
+    if (a.trec != nullptr && a.leaf_test)
+        return a.gq8 ? launch_nf<N, kFmtTileLeafQ8>(a, false, s)
+                     : launch_nf<N, kFmtTileLeaf>(a, false, s);
     if (a.trec != nullptr)
         return a.gq8 ? launch_nf<N, kFmtTileQ8>(a, false, s) : launch_nf<N, kFmtTile>(a, false, s);
     // groups of 8 or more lanes on one pixel take the cooperative form
@@ -703,6 +708,7 @@ gs_status launch_trace(const gs_bvh *b, const gs_gaussians *g, const gs_pinhole 
     a.gq8 = b->node_format == GS_NODES_BINARY_Q8;
     a.trec = tile || shared ? b->group[kWarpTree].rec : nullptr;
     a.troot = tile || shared ? b->group[kWarpTree].ref : nullptr;
+    a.leaf_test = leaf_test_pays(b->M, (int64_t)cam->width * cam->height);
     a.prims = b->prims;
     a.sh = g->sh;
     a.n_nodes = b->n_nodes;

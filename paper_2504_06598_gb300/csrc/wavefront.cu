@@ -145,17 +145,19 @@ __device__ __forceinline__ void trace_own_ray(const TraceArgs &a, Ray<1> &r, int
 
 // Camera and shadow rays are one ray for all lanes of a pixel: with groups
 // of 2^GLG >= 8 lanes they take the grouped traversal of the wide copy.
-// GLG = kTileWarp: a warp's rays of one apex take the tile traversal.
-constexpr int kTileWarp = 1;
+// GLG = kTileWarp or kTileLeaf: a warp's rays of one apex take the tile
+// traversal, the latter with the test of each leaf's box.
+constexpr int kTileWarp = 1, kTileLeaf = 2;
+__host__ __device__ constexpr bool is_tile_form(int g) { return g == kTileWarp || g == kTileLeaf; }
 
-template <int FMT, int GLG, bool COUNT, int K = 1>
+template <int FMT, int GLG, bool COUNT, int K = 1, bool SHADOW = false>
 __device__ __forceinline__ void trace_pixel_ray(const TraceArgs &a, Ray<K> &r, int pass,
                                                 const float apex[3], const float *pyr,
                                                 uint32_t *stack, float *stack_t, uint32_t *g_ref,
                                                 float *g_t, uint32_t &err, Counts &cnt) {
     if (a.n_nodes == 0) return;
-    if constexpr (GLG == kTileWarp) {
-        trace_tile<K, FMT == GS_NODES_BINARY_Q8>(a, r, pass, apex, pyr, g_ref, g_t, err);
+    if constexpr (is_tile_form(GLG)) {
+        trace_tile<K, FMT == GS_NODES_BINARY_Q8, GLG == kTileLeaf, SHADOW>(a, r, pass, apex, pyr, g_ref, g_t, err);
     } else if constexpr (GLG >= 3)
     {
         uint32_t e = 0;
@@ -210,7 +212,7 @@ __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
         const int off = (lane >> GLG) * (kGroupPool >> (5 - GLG));
         g_ref = pool + off;
         g_t = reinterpret_cast<float *>(pool + kGroupPool) + off;
-    } else if constexpr (GLG == kTileWarp) {
+    } else if constexpr (is_tile_form(GLG)) {
         uint32_t *pool = wave_smem + (size_t)(threadIdx.x >> 5) * (2 * kTilePool + kTileFloats);
         g_ref = pool;
         g_t = reinterpret_cast<float *>(pool + kTilePool);
@@ -276,7 +278,7 @@ __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
             reset_live_slots<K>(r, pass, S, live);
             update_clip(r, r.t_max);
             if (!live[0]) r.t_far = -INFINITY;
-            if constexpr (GLG == kTileWarp) tile_pyramid(d0, valid, pyr);
+            if constexpr (is_tile_form(GLG)) tile_pyramid(d0, valid, pyr);
             trace_pixel_ray<FMT, GLG, COUNT, K>(a, r, pass, vw.eye, pyr, stack, stack_t, g_ref, g_t,
                                                 err, cnt);
             float c[K][3];
@@ -329,7 +331,7 @@ __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
                 reset_live_slots<K>(sr, pass, S, need);
                 update_clip(sr, sr.t_max);
                 if (!any_need) sr.t_far = -INFINITY;
-                if constexpr (GLG == kTileWarp) {
+                if constexpr (is_tile_form(GLG)) {
                     // a shadow ray starts at its ground point, so it passes the
                     // light by the rounding of its direction: below 2^-22 of
                     // the distance, which near the light is all there is
@@ -338,7 +340,7 @@ __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
                         __reduce_max_sync(kAll, any_need ? __float_as_uint(dist) : 0u);
                     tile_pyramid(away, any_need, pyr, 0x1p-21f * __uint_as_float(far));
                 }
-                trace_pixel_ray<FMT, GLG, COUNT, K>(a, sr, pass, w.light_pos[l], pyr, stack, stack_t,
+                trace_pixel_ray<FMT, GLG, COUNT, K, true>(a, sr, pass, w.light_pos[l], pyr, stack, stack_t,
                                                     g_ref, g_t, err, cnt);
 #pragma unroll
                 for (int k = 0; k < K; ++k) {
@@ -784,7 +786,7 @@ gs_status launch_views(const WaveArgs &w, int threads, cudaStream_t s) {
     int dev = 0, sms = 0, per = 0;
     const size_t smem =
         (size_t)(threads / 32) * sizeof(uint32_t) *
-        (GLG >= 3 ? 2 * kGroupPool : GLG == kTileWarp ? 2 * kTilePool + kTileFloats : 0);
+        (GLG >= 3 ? 2 * kGroupPool : is_tile_form(GLG) ? 2 * kTilePool + kTileFloats : 0);
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
@@ -805,7 +807,7 @@ gs_status launch_views(const WaveArgs &w, int threads, cudaStream_t s) {
 template <int FMT, int GLG>
 gs_status launch_views_g(const WaveArgs &w, int threads, int stack, cudaStream_t s) {
     const bool count = w.counters != nullptr;
-    if constexpr (GLG == kTileWarp) {
+    if constexpr (is_tile_form(GLG)) {
         // (no per-lane stacks but the fallback's own)
         switch (w.spl) {
             case 8: return launch_views<FMT, 48, false, GLG, 8>(w, threads, s);
@@ -850,7 +852,9 @@ gs_status launch_views_f(const WaveArgs &w, int threads, int stack, cudaStream_t
 // Binary handles with wide copies: pixels with 8 or more lanes group.
 template <>
 gs_status launch_views_f<GS_NODES_BINARY>(const WaveArgs &w, int threads, int stack, cudaStream_t s) {
-    if (w.t.trec != nullptr) return launch_views_g<GS_NODES_BINARY, kTileWarp>(w, threads, stack, s);
+    if (w.t.trec != nullptr)
+        return w.t.leaf_test ? launch_views_g<GS_NODES_BINARY, kTileLeaf>(w, threads, stack, s)
+                             : launch_views_g<GS_NODES_BINARY, kTileWarp>(w, threads, stack, s);
     if (w.t.grec != nullptr) {
         switch (w.t.lpp_log2) {
             case 5: return launch_views_g<GS_NODES_BINARY, 5>(w, threads, stack, s);
@@ -868,7 +872,8 @@ template <>
 gs_status launch_views_f<GS_NODES_BINARY_Q8>(const WaveArgs &w, int threads, int stack,
                                              cudaStream_t s) {
     if (w.t.trec != nullptr)
-        return launch_views_g<GS_NODES_BINARY_Q8, kTileWarp>(w, threads, stack, s);
+        return w.t.leaf_test ? launch_views_g<GS_NODES_BINARY_Q8, kTileLeaf>(w, threads, stack, s)
+                             : launch_views_g<GS_NODES_BINARY_Q8, kTileWarp>(w, threads, stack, s);
     if (w.t.grec != nullptr) {
         switch (w.t.lpp_log2) {
             case 5: return launch_views_g<GS_NODES_BINARY_Q8, 5>(w, threads, stack, s);
@@ -997,6 +1002,7 @@ gs_status launch_render_views(const gs_bvh *b, const gs_gaussians *g, const gs_p
     if (tiles_ok && ungrouped && !whole_warp) {
         a.trec = b->group[kWarpTree].rec;
         a.troot = b->group[kWarpTree].ref;
+        a.leaf_test = leaf_test_pays(b->M, all_pix / n_views);
     }
     const int tw_lg = tile_w_log2(a.lpp_log2), th_lg = 5 - a.lpp_log2 - tw_lg;
     uint32_t tiles = 0;

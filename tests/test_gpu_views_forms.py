@@ -128,3 +128,18 @@ def test_bounce_rays_at_a_small_stack(gs, fmt):
         assert torch.equal(s0, s1)
         assert (s0[..., 1] == 0).any()
     bvh.free()
+
+
+@pytest.mark.parametrize("fmt", ["binary", "binary_q8"])
+@pytest.mark.parametrize("spp", [1, 16])
+def test_tiles_that_test_each_leaf(gs, fmt, spp):
+    """More Gaussians than a sixteenth of a view's pixels, a light among them."""
+    cloud = scenes.shell_cloud(7, M=20000)
+    g = gs.Gaussians.from_cloud(cloud)
+    cams = scenes.wavefront_views(2, seed=4, fixed_res=(401, 299))
+    ex = scenes.ground_and_lights(1, seed=1)
+    ex.lights += [((0.0, 0.0, 0.0), (1.0, 2.0, 3.0)),
+                  (tuple(float(v) for v in cloud.means[0] + 0.01), (0.1, 0.1, 0.1))]
+    ref, smp = _render(gs, g, cams, ex, "wide4", spp=spp)
+    rgb, got = _render(gs, g, cams, ex, fmt, spp=spp)
+    assert torch.equal(got, smp) and torch.equal(rgb, ref)
