@@ -81,10 +81,15 @@ constexpr uint32_t kQ8Skip = 1u << 16;  // q1 flag: a child with a non-finite bo
 constexpr int kWideCountShift = 26;
 constexpr uint32_t kWideOffsetMask = (1u << kWideCountShift) - 1u;
 constexpr int kGroupTrees = 2;
-// Their widths: 8 for groups of 8 and 16 lanes, 32 for whole warps. (A 16-wide
-// tree served only groups of 16 lanes, which the library's own choices no
-// longer form; a 4-wide one for rays walked by a lane each made the batched
-// frame slower, 427 ms against 353 on the binary nodes.)
+// Their widths: 8 for groups of 8 and 16 lanes, 32 for whole warps. Groups of 16
+// have half of their lanes idle in the child test and take 1.2 to 1.4 times what
+// they took on a 16-wide tree (1M at 640x480, 16 samples of one a lane 6.1 -> 7.6
+// ms; on the 32-wide one, two children a lane, 5.8, but 0.31 against 0.27 at 1,000
+// Gaussians). That tree cost every rebuild 6% (1M 529 -> 562 us) and 68 bytes a
+// Gaussian, so the library's own choices avoid such groups instead; they remain
+// for 16 to 31 samples with counters, and where the caller sets the samples per
+// lane. (A 4-wide tree for rays walked by a lane each made the batched frame
+// slower, 427 ms against 353 on the binary nodes.)
 __host__ __device__ constexpr uint32_t group_width(int tree) { return tree == 0 ? 8u : 32u; }
 constexpr int kWarpTree = 1;
 constexpr int group_tree(int lanes_log2) { return lanes_log2 >= 5 ? kWarpTree : 0; }
