@@ -510,7 +510,7 @@ __global__ void __launch_bounds__(kThreads, LG >= 3 ? (N >= 4 ? 7 : kGroupMinBlo
                     }
                 }
             } else if constexpr (LG >= 3) {
-                traverse_group<N, false, LG, false, Q8>(a, r, pass, grp_ref, grp_t, err, cnt);
+                traverse_group<N, false, LG, false, Q8, false>(a, r, pass, grp_ref, grp_t, err, cnt);
             } else {
                 traverse_packet<N, false>(a, r, pass, stack, stack_t, err, cnt);
             }

@@ -947,7 +947,7 @@ constexpr int kGroupMinBlocks = 8; // resident blocks per SM to build for
 // and clip, so per-lane results are those of an independent traversal.
 // POP2 selects the two-stage pop of the group stack (below); both pop the
 // same entries. Q8 reads the 8-bit form of the records.
-template <int N, bool COUNT, int LG, bool POP2 = false, bool Q8 = false>
+template <int N, bool COUNT, int LG, bool POP2 = false, bool Q8 = false, bool PAIRED = true>
 __device__ __forceinline__ void traverse_group(const TraceArgs &a, Ray<N> &r, int pass,
                                                uint32_t *s_ref, float *s_t, uint32_t &err,
                                                Counts &cnt) {
@@ -1013,7 +1013,7 @@ __device__ __forceinline__ void traverse_group(const TraceArgs &a, Ray<N> &r, in
                 return __uint_as_float(o ^ ((o & 0x80000000u) ? 0x80000000u : 0xffffffffu));
             };
             bool paired = false;
-            if constexpr (N == 2 && !COUNT) paired = a.rng_mode == 0;
+            if constexpr (PAIRED && N == 2 && !COUNT) paired = a.rng_mode == 0;
             if (paired) {
                 // Two slots a lane use half of a Philox call: lanes 2i and
                 // 2i + 1 need the same one. So candidates go two at a time,
