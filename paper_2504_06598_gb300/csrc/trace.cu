@@ -639,11 +639,6 @@ int auto_samples_per_lane(int spp, int n_hits, int node_format) {
 
 }  // namespace
 
-static int64_t tile_warps(int width, int height, int lpp_log2) {
-    const int tw_lg = tile_w_log2(lpp_log2), th_lg = 5 - lpp_log2 - tw_lg;
-    return (int64_t)((width + (1 << tw_lg) - 1) >> tw_lg) * ((height + (1 << th_lg) - 1) >> th_lg);
-}
-
 // Warps the current device holds at once at 64 registers a thread.
 static int64_t resident_warps() {
     int dev = 0, sms = 0;
@@ -651,6 +646,65 @@ static int64_t resident_warps() {
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return 0;
     return (int64_t)sms * 32;
+}
+
+// The walks of a launch: the layout's own (packets of the binary nodes, or
+// groups of 8 and more lanes), tiles, a warp per pixel, or one walk for four
+// pixels.
+enum class Walk { kLayout, kTile, kWarp, kShared };
+
+// Lines from the times (us) of shells of 10 to 1M Gaussians in images of 64x64 to
+// 1080p, one to 256 samples a pixel.
+static Walk choose_walk(const gs_bvh *b, const gs_pinhole *cam, const gs_trace_params *p, int n_eff,
+                        int passes, int lpp_log2) {
+    // the forms other than the layout's take depths along the ray from the eye
+    // and none of the options that are about the per-lane walk
+    if (!b->link || !(p->t_min >= 0.0f) || p->depth_mode != 0 || p->rng_mode != 0 ||
+        p->stack_depth != 0 || p->counters != nullptr)
+        return Walk::kLayout;
+    const int64_t pix = (int64_t)cam->width * cam->height, T = (int64_t)p->spp * p->n_hits;
+    const double waves = (double)pix / (double)resident_warps();  // of a warp per pixel
+    const bool many = p->samples_per_lane == 0 && T > 32;
+    // A warp per pixel (most lanes without a sample, helping in the walk) evaluates
+    // 32 Gaussians at a time, a tile's warp one after the other, so that the time
+    // of few tiles is the longest tile's; but its work is the pixels'. Its share
+    // of waves before it loses to tiles grows with the scene's size, as the
+    // depth of a tile does: at one slot a lane 4 waves at 1,000 Gaussians (45 against
+    // 62), 15 at 20,000 (233 against 313), 41 at 300,000 (1336 against 1367), 63 at
+    // 1M (3108 against 2919); at eight slots two thirds, against shared walks a
+    // quarter of that.
+    if (lpp_log2 < 3 || (many && T < 64)) {
+        double share = many ? 0.14 : n_eff < 8 ? 0.6 : 0.40 - 0.04 * lpp_log2;
+        // (three or five to seven passes are two rounds of the layout's lanes)
+        if (!many && passes > 1 << lpp_log2) share *= 1.6;
+        if (waves < share * cbrt((double)b->M)) return Walk::kWarp;
+    }
+    // Eight to 31 passes of the caller's samples per lane: a whole warp does in one
+    // round what groups of 8 or 16 lanes do in two, and more than groups of 16 do on
+    // the 8-wide copy (spp 24, one a lane: 20,000 at 640x480 2036 -> 977, 1M 14.6 ->
+    // 4.7 ms; spp 16: 90k 2213 -> 1686).
+    if (!many && lpp_log2 >= 3 && passes < 32 && passes * n_eff <= 64 &&
+        (passes > 1 << lpp_log2 ? b->M >= 4096 : lpp_log2 == 4 && b->M >= 65536))
+        return Walk::kWarp;
+    // Shared walks for 64 samples and more: a second walk for samples 64 to 127, where
+    // the groups of four slots from 128 on still walk once. Below six waves of 2x2
+    // tiles the groups' many small warps win (1M, spp 64: 320x240 1622 against 2305,
+    // 500x400 3841 against 3305).
+    if (many && T >= 64) return T < 128 && waves > 24.0 ? Walk::kShared : Walk::kLayout;
+    // A few hundred Gaussians: the packets' steps are the cheapest, and with them a
+    // launch is little more than its fixed cost (100 at 1080p, spp 4 90 against 119).
+    if (b->M < 512) return Walk::kLayout;
+    if (many) {
+        // 33 to 63 samples are five to eight passes of tiles: with few Gaussians that
+        // costs less than the draws of 64 (1,000 at 1080p 1448 against 1861; 20,000
+        // 4222 against 3947)
+        return b->M < 4096 && waves > 32.0 ? Walk::kTile : Walk::kShared;
+    }
+    if (lpp_log2 >= 3) return Walk::kLayout;
+    // More than three Gaussians a ray of the tile: its farthest clip takes in so many
+    // that packets, which clip per ray, do better (1M at 500x400, spp 8 4502 against
+    // 5533; at 640x480 4428 against 4846).
+    return b->M > 3 * (pix << lpp_log2) ? Walk::kLayout : Walk::kTile;
 }
 
 void trace_layout(const gs_bvh *b, const gs_trace_params *p, int *S_out, int *spp_eff_out,
@@ -674,25 +728,10 @@ gs_status launch_trace(const gs_bvh *b, const gs_gaussians *g, const gs_pinhole 
     bool grouped = false;
     trace_layout(b, p, &S, &spp_eff, &lpp_log2, &grouped);
     const int n_eff = p->n_hits * S;
-    // the tile traversal: fewer than 8 lanes a pixel, depths along the ray
-    // from the eye, and none of the options that are about the per-lane walk
-    const bool plain = b->link && p->t_min >= 0.0f && p->depth_mode == 0 && p->rng_mode == 0 &&
-                       p->stack_depth == 0 && p->counters == nullptr;
-    const bool shared = plain && p->samples_per_lane == 0 && (int64_t)p->spp * p->n_hits > 32;
-    bool tile = plain && !shared && lpp_log2 < 3;
     const int sum_log2 = lpp_log2;
-    if (tile && tile_warps(cam->width, cam->height, lpp_log2) < resident_warps()) {
-        // Too few tiles to fill the chip once: the time is the longest walk
-        // of a warp, which evaluates its tile's Gaussians one after the other.
-        // A whole warp per pixel then (most lanes without a sample, helping in
-        // the walk) evaluates 32 at a time. us, tile -> warp per pixel: 1k
-        // Gaussians, 64x64, spp 1 89 -> 31; 90k, 96x72, spp 1 2662 -> 126 and
-        // spp 16 3350 -> 199; 411x307, spp 1 774 -> 516 (3,900 tiles); above
-        // one wave the tiles win (411x307, spp 16, 7,900 tiles 1004 against
-        // 1204; 1M at 1080p, spp 1 3.1 ms against 13.6).
-        tile = false;
-        lpp_log2 = 5;
-    }
+    const Walk walk = choose_walk(b, cam, p, n_eff, spp_eff, lpp_log2);
+    const bool shared = walk == Walk::kShared, tile = walk == Walk::kTile;
+    if (walk == Walk::kWarp) lpp_log2 = 5;
     TraceArgs a;
     a.nodes = b->nodes;
     a.wide = b->wide;
@@ -761,11 +800,15 @@ gs_status launch_trace(const gs_bvh *b, const gs_gaussians *g, const gs_pinhole 
     gs_status st;
     a.order = nullptr;
     // below three waves the longest tile decides, whatever the order (90k at
-    // 411x307, 1.6 waves: 1119 us by rows, 1147 ordered)
-    if (shared ? (int64_t)((a.width + 1) >> 1) * ((a.height + 1) >> 1) > 3 * resident_warps()
-               : tile && tile_warps(a.width, a.height, a.lpp_log2) > 3 * resident_warps())
-        order_regions(b, a, shared ? 1 : tile_w_log2(a.lpp_log2),
-                      shared ? 1 : 5 - a.lpp_log2 - tile_w_log2(a.lpp_log2), s);
+    // 411x307, 1.6 waves: 1119 us by rows, 1147 ordered), and a launch of 200 us does
+    // not gain the two launches' 20 (1,000 at 1080p, spp 1 119 by rows, 137 ordered,
+    // spp 8 303 and 276)
+    const bool worth = b->M >= 4096 || (b->M >= 512 && (int64_t)p->spp * p->n_hits >= 8);
+    const int tw_lg = shared ? 1 : tile_w_log2(a.lpp_log2), th_lg = shared ? 1 : 5 - a.lpp_log2 - tw_lg;
+    const int64_t tiles = (((int64_t)a.width + (1 << tw_lg) - 1) >> tw_lg) *
+                          (((int64_t)a.height + (1 << th_lg) - 1) >> th_lg);
+    if ((shared || tile) && worth && tiles > 3 * resident_warps())
+        order_regions(b, a, tw_lg, th_lg, s);
     if (shared) {
         st = a.gq8 ? launch_shared<true>(a, s) : launch_shared<false>(a, s);
         if (st != GS_OK) return st;
