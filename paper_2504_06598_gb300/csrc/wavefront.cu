@@ -57,6 +57,7 @@ struct WaveArgs {
     unsigned long long *codes;
     float *bounce_rgb;
     int spl;  // samples per lane of the camera and shadow pass (1, 2, 4 or 8)
+    int few;         // 1: few waves of tiles
     int eval_lanes;  // lanes holding leaves at which the bounce pass evaluates them
 };
 
@@ -147,8 +148,16 @@ __device__ __forceinline__ void trace_own_ray(const TraceArgs &a, Ray<1> &r, int
 // of 2^GLG >= 8 lanes they take the grouped traversal of the wide copy.
 // GLG = kTileWarp or kTileLeaf: a warp's rays of one apex take the tile
 // traversal, the latter with the test of each leaf's box.
-constexpr int kTileWarp = 1, kTileLeaf = 2;
-__host__ __device__ constexpr bool is_tile_form(int g) { return g == kTileWarp || g == kTileLeaf; }
+// kTileFew: kTileLeaf built for two blocks per SM instead of four, for launches
+// of few waves of tiles, where the longest tile's own time counts and not the
+// warps in flight: 100k in two 640x360 views, spp 8 2.49 -> 2.19 ms, 1M in two
+// views, spp 16 8.8 -> 8.2; in four 1080p views 14.5 against 17.4. With one or two
+// samples a lane it gains 2 to 10% and is left out.
+constexpr int kTileWarp = 1, kTileLeaf = 2, kTileFew = 6;
+__host__ __device__ constexpr bool is_tile_form(int g) {
+    return g == kTileWarp || g == kTileLeaf || g == kTileFew;
+}
+__host__ __device__ constexpr bool is_group_form(int g) { return g >= 3 && g <= 5; }
 
 template <int FMT, int GLG, bool COUNT, int K = 1, bool SHADOW = false>
 __device__ __forceinline__ void trace_pixel_ray(const TraceArgs &a, Ray<K> &r, int pass,
@@ -157,9 +166,8 @@ __device__ __forceinline__ void trace_pixel_ray(const TraceArgs &a, Ray<K> &r, i
                                                 float *g_t, uint32_t &err, Counts &cnt) {
     if (a.n_nodes == 0) return;
     if constexpr (is_tile_form(GLG)) {
-        trace_tile<K, FMT == GS_NODES_BINARY_Q8, GLG == kTileLeaf, SHADOW>(a, r, pass, apex, pyr, g_ref, g_t, err);
-    } else if constexpr (GLG >= 3)
-    {
+        trace_tile<K, FMT == GS_NODES_BINARY_Q8, GLG != kTileWarp, SHADOW>(a, r, pass, apex, pyr, g_ref, g_t, err);
+    } else if constexpr (is_group_form(GLG)) {
         uint32_t e = 0;
         traverse_group<K, COUNT, GLG, false, FMT == GS_NODES_BINARY_Q8>(a, r, pass, g_ref, g_t, e, cnt);
         if (!COUNT && __any_sync(0xffffffffu, e & kErrStack)) {
@@ -198,7 +206,7 @@ constexpr int kWaveMinBlocks = 4;
 // frame at spp 8, 16 and 32: 202.4, 381.8 and 737.7 ms against 205.5,
 // 386.9 and 747.4 with three blocks; 423.7 with two at spp 16).
 template <int FMT, int STACK, bool COUNT, int GLG, int K = 1>
-__global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
+__global__ void __launch_bounds__(kWaveMaxThreads, GLG == kTileFew ? 2 : kWaveMinBlocks)
     k_render_views(const __grid_constant__ WaveArgs w) {
     const TraceArgs &a = w.t;
     const int lane = threadIdx.x & 31;
@@ -207,9 +215,10 @@ __global__ void __launch_bounds__(kWaveMaxThreads, kWaveMinBlocks)
     uint32_t *g_ref = nullptr;
     float *g_t = nullptr;
     float *pyr = nullptr;
-    if constexpr (GLG >= 3) {
+    if constexpr (is_group_form(GLG)) {
         uint32_t *pool = wave_smem + (size_t)(threadIdx.x >> 5) * 2 * kGroupPool;
-        const int off = (lane >> GLG) * (kGroupPool >> (5 - GLG));
+        constexpr int LG = is_group_form(GLG) ? GLG : 5;
+        const int off = (lane >> LG) * (kGroupPool >> (5 - LG));
         g_ref = pool + off;
         g_t = reinterpret_cast<float *>(pool + kGroupPool) + off;
     } else if constexpr (is_tile_form(GLG)) {
@@ -786,7 +795,7 @@ gs_status launch_views(const WaveArgs &w, int threads, cudaStream_t s) {
     int dev = 0, sms = 0, per = 0;
     const size_t smem =
         (size_t)(threads / 32) * sizeof(uint32_t) *
-        (GLG >= 3 ? 2 * kGroupPool : is_tile_form(GLG) ? 2 * kTilePool + kTileFloats : 0);
+        (is_group_form(GLG) ? 2 * kGroupPool : is_tile_form(GLG) ? 2 * kTilePool + kTileFloats : 0);
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
@@ -812,9 +821,11 @@ gs_status launch_views_g(const WaveArgs &w, int threads, int stack, cudaStream_t
         switch (w.spl) {
             case 8: return launch_views<FMT, 48, false, GLG, 8>(w, threads, s);
             case 4: return launch_views<FMT, 48, false, GLG, 4>(w, threads, s);
-            case 2: return launch_views<FMT, 48, false, GLG, 2>(w, threads, s);
-            default: return launch_views<FMT, 48, false, GLG, 1>(w, threads, s);
+            default: break;
         }
+        if constexpr (GLG != kTileFew)
+            return w.spl == 2 ? launch_views<FMT, 48, false, GLG, 2>(w, threads, s)
+                              : launch_views<FMT, 48, false, GLG, 1>(w, threads, s);
     }
     // several samples per lane: fewer than 8 lanes a pixel, or a warp per
     // pixel with most lanes idle; never with counters
@@ -853,8 +864,9 @@ gs_status launch_views_f(const WaveArgs &w, int threads, int stack, cudaStream_t
 template <>
 gs_status launch_views_f<GS_NODES_BINARY>(const WaveArgs &w, int threads, int stack, cudaStream_t s) {
     if (w.t.trec != nullptr)
-        return w.t.leaf_test ? launch_views_g<GS_NODES_BINARY, kTileLeaf>(w, threads, stack, s)
-                             : launch_views_g<GS_NODES_BINARY, kTileWarp>(w, threads, stack, s);
+        return !w.t.leaf_test ? launch_views_g<GS_NODES_BINARY, kTileWarp>(w, threads, stack, s)
+               : w.few        ? launch_views_g<GS_NODES_BINARY, kTileFew>(w, threads, stack, s)
+                              : launch_views_g<GS_NODES_BINARY, kTileLeaf>(w, threads, stack, s);
     if (w.t.grec != nullptr) {
         switch (w.t.lpp_log2) {
             case 5: return launch_views_g<GS_NODES_BINARY, 5>(w, threads, stack, s);
@@ -872,8 +884,9 @@ template <>
 gs_status launch_views_f<GS_NODES_BINARY_Q8>(const WaveArgs &w, int threads, int stack,
                                              cudaStream_t s) {
     if (w.t.trec != nullptr)
-        return w.t.leaf_test ? launch_views_g<GS_NODES_BINARY_Q8, kTileLeaf>(w, threads, stack, s)
-                             : launch_views_g<GS_NODES_BINARY_Q8, kTileWarp>(w, threads, stack, s);
+        return !w.t.leaf_test ? launch_views_g<GS_NODES_BINARY_Q8, kTileWarp>(w, threads, stack, s)
+               : w.few        ? launch_views_g<GS_NODES_BINARY_Q8, kTileFew>(w, threads, stack, s)
+                              : launch_views_g<GS_NODES_BINARY_Q8, kTileLeaf>(w, threads, stack, s);
     if (w.t.grec != nullptr) {
         switch (w.t.lpp_log2) {
             case 5: return launch_views_g<GS_NODES_BINARY_Q8, 5>(w, threads, stack, s);
@@ -978,9 +991,18 @@ gs_status launch_render_views(const gs_bvh *b, const gs_gaussians *g, const gs_p
     // samples a lane (8 to 63 samples: up to 8 lanes) are never theirs
     const int lanes_lg = lanes_per_pixel_log2((p->spp + K - 1) / K);
     const bool ungrouped = lanes_lg < 3 || K > 1;
-    // too few tiles to fill the chip once: a warp per pixel (see launch_trace)
-    const bool whole_warp =
-        tiles_ok && ungrouped && (all_pix << lanes_lg) < (int64_t)sms * 32 * 32;
+    // A warp per pixel for few pixels, packets for a few hundred Gaussians or more
+    // than three a ray, tiles between: the lines of choose_walk (trace.cu), the first
+    // a little higher, since a view also has its shadow rays. us, two lights,
+    // packets, tiles, warp per pixel: 5,000 at 160x120, spp 1 466, 360, 132; in two
+    // 320x240 views 352, 290, 591; 1M there 4312, 6030, 2013; 1M in two 640x360
+    // views 3873, 4932, 4395; in four 1080p views 19.2 and 14.3 ms; 100 there 0.47
+    // and 0.62.
+    const double waves = (double)all_pix / ((double)sms * 32.0);
+    const double share = K < 8 ? 0.72 : 0.40 - 0.04 * lanes_lg;
+    const bool whole_warp = tiles_ok && ungrouped && waves < share * cbrt((double)b->M);
+    const bool tiled = tiles_ok && ungrouped && !whole_warp && b->M >= 512 &&
+                       b->M <= 3 * ((all_pix / n_views) << lanes_lg);
     w.spl = K;
     a.spp = (p->spp + K - 1) / K;
     a.n_samples = p->spp;
@@ -999,10 +1021,11 @@ gs_status launch_render_views(const gs_bvh *b, const gs_gaussians *g, const gs_p
         a.groot = b->group[group_tree(a.lpp_log2)].ref;
         a.gq8 = b->node_format == GS_NODES_BINARY_Q8;
     }
-    if (tiles_ok && ungrouped && !whole_warp) {
+    if (tiled) {
         a.trec = b->group[kWarpTree].rec;
         a.troot = b->group[kWarpTree].ref;
         a.leaf_test = leaf_test_pays(b->M, all_pix / n_views);
+        w.few = K >= 4 && (all_pix << lanes_lg) < 6 * (int64_t)sms * 32 * 32;
     }
     const int tw_lg = tile_w_log2(a.lpp_log2), th_lg = 5 - a.lpp_log2 - tw_lg;
     uint32_t tiles = 0;
