@@ -1031,20 +1031,52 @@ gs_status launch_backward(const gs_bvh *b, const gs_gaussians *g, const gs_pinho
                           float *d_sh, cudaStream_t s) {
     // a lane carries S consecutive samples: ceil(spp / S) passes of
     // n_hits * S slots, the same sample indices and keys as the forward
-    const bool tile = b->link && p->t_min >= 0.0f && p->stack_depth == 0;
-    int S = p->samples_per_lane > 0 ? p->samples_per_lane
-                                    : auto_backward_samples_per_lane(p->spp, p->n_hits, tile);
-    if (tile && p->samples_per_lane == 0) {
-        // fewer warps than the chip holds: more lanes a pixel, fewer samples
-        // each, so that a tile covers fewer pixels
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const int64_t pix = (int64_t)cam->width * cam->height;
-        while (S > 1 && (pix << lanes_per_pixel_log2((p->spp + S - 1) / S)) < (int64_t)sms * 16 * 32)
-            S >>= 1;
+    bool tile = b->link && p->t_min >= 0.0f && p->stack_depth == 0;
+    const int64_t pix = (int64_t)cam->width * cam->height;
+    // samples a lane of the tile form or of the others, and the log2 of the lanes a
+    // pixel then has
+    auto lane_samples = [&](bool t) {
+        int n = p->samples_per_lane > 0 ? p->samples_per_lane
+                                        : auto_backward_samples_per_lane(p->spp, p->n_hits, t);
+        if (t && p->samples_per_lane == 0) {
+            // fewer warps than the chip holds: more lanes a pixel, fewer samples
+            // each, so that a tile covers fewer pixels
+            int dev = 0, sms = 0;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            while (n > 1 && (pix << lanes_per_pixel_log2((p->spp + n - 1) / n)) < (int64_t)sms * 16 * 32)
+                n >>= 1;
+        }
+        while (n > 1 && n > p->spp) n >>= 1;
+        return n;
+    };
+    auto lanes_log2 = [&](int n) { return lanes_per_pixel_log2((p->spp + n - 1) / n); };
+    // A tile's warp visits all that its pyramid holds, where packets and groups
+    // visit what a ray meets: with too many Gaussians a tile (tiny images of large
+    // scenes) they are the faster, the sooner the fewer pixels a warp of theirs
+    // has. From stored payloads, ms, tiles and the other form: 1M, spp 1 (packets)
+    // 32x32 19.0 and 6.7, 160x120 5.0 and 3.2, 320x240 2.1 and 2.9; spp 4 (packets of
+    // four samples a lane against tiles of eight pixels) 32x32 7.7 and 11.0; spp 16
+    // (groups) 32x32 1.9 and 1.4, 96x72 1.2 and 1.7.
+    if (tile) {
+        const double size = sqrt((double)b->M);
+        const int lg = lanes_log2(lane_samples(true));
+        const bool groups = lanes_log2(lane_samples(false)) >= 3;
+        tile = (double)b->M * (double)(32 >> lg) / (double)pix <= (groups ? 1.0 : lg == 0 ? 0.8 : 8.0) * size;
+        // without payloads the winners are traced again, in small images on the
+        // tiles' longest chain, which a second round of passes doubles (spp 40
+        // against groups: 1M at 160x120 7.7 and 3.9, at 64x64 4.2 and 3.5; 90k at
+        // 160x120 2.0 and 1.5, at 64x64 1.2 and 1.6)
+        const int passes = (p->spp + lane_samples(true) - 1) / lane_samples(true);
+        if (groups && keys == nullptr && passes > 1 << lg) {
+            int dev = 0, sms = 0;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            tile = tile && (b->M < (lg == 5 ? 500000 : 50000) ||
+                            (double)pix >= 0.14 * cbrt((double)b->M) * sms * 32.0);
+        }
     }
-    while (S > 1 && S > p->spp) S >>= 1;
+    const int S = lane_samples(tile);
     const int spp_eff = (p->spp + S - 1) / S;
     TraceArgs a = {};
     a.nodes = b->nodes;
@@ -1103,7 +1135,9 @@ gs_status launch_backward(const gs_bvh *b, const gs_gaussians *g, const gs_pinho
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (((int64_t)a.width * a.height << a.lpp_log2) > (int64_t)sms * 3 * 16 * 32)
+        // (two launches of 20 us: see launch_trace)
+        const bool worth = b->M >= 4096 || (b->M >= 512 && (int64_t)p->spp * p->n_hits >= 4);
+        if (worth && (pix << a.lpp_log2) > (int64_t)sms * 3 * 16 * 32)
             order_regions(b, a, tile_w_log2(a.lpp_log2), 5 - a.lpp_log2 - tile_w_log2(a.lpp_log2), s);
     }
     gs_status st;

@@ -386,3 +386,18 @@ def test_single_gaussian_gradients(gs):
                     assert err <= 1e-4 * np.abs(ref[k]).max() + 1e-6, (k, fmt, depth)
         bvh.sync_status()
         bvh.free()
+
+
+@pytest.mark.parametrize("M,w,h,spp", [(20000, 9, 7, 1), (20000, 9, 7, 2), (40000, 9, 7, 16),
+                                       (20000, 48, 36, 1)])
+def test_gradients_of_tiny_images_of_large_scenes(gs, M, w, h, spp):
+    """Either side of the lines between tiles and the other gradient forms."""
+    cloud = scenes.shell_cloud(8, M=M, n_clusters=4, sh_degree=1)
+    cam = scenes.default_camera(w, h)
+    rng = np.random.default_rng(5)
+    d_rgb = rng.normal(size=(w * h, 3))
+    a = _gpu_grads(gs, cloud, cam, d_rgb, seed=2, spp=spp)
+    b = _gpu_grads(gs, cloud, cam, d_rgb, seed=2, spp=spp, stack_depth=96)
+    for k in KEYS:
+        assert np.abs(b[k]).max() > 0, k
+        assert np.abs(a[k] - b[k]).max() <= 1e-4 * np.abs(b[k]).max() + 1e-6, k
