@@ -151,8 +151,7 @@ __device__ __forceinline__ void trace_own_ray(const TraceArgs &a, Ray<1> &r, int
 // kTileFew: kTileLeaf built for two blocks per SM instead of four, for launches
 // of few waves of tiles, where the longest tile's own time counts and not the
 // warps in flight: 100k in two 640x360 views, spp 8 2.49 -> 2.19 ms, 1M in two
-// views, spp 16 8.8 -> 8.2; in four 1080p views 14.5 against 17.4. With one or two
-// samples a lane it gains 2 to 10% and is left out.
+// views, spp 16 8.8 -> 8.2; in four 1080p views 14.5 against 17.4.
 constexpr int kTileWarp = 1, kTileLeaf = 2, kTileFew = 6;
 __host__ __device__ constexpr bool is_tile_form(int g) {
     return g == kTileWarp || g == kTileLeaf || g == kTileFew;
@@ -837,11 +836,9 @@ gs_status launch_views_g(const WaveArgs &w, int threads, int stack, cudaStream_t
         switch (w.spl) {
             case 8: return launch_views<FMT, 48, false, GLG, 8>(w, threads, s);
             case 4: return launch_views<FMT, 48, false, GLG, 4>(w, threads, s);
-            default: break;
+            case 2: return launch_views<FMT, 48, false, GLG, 2>(w, threads, s);
+            default: return launch_views<FMT, 48, false, GLG, 1>(w, threads, s);
         }
-        if constexpr (GLG != kTileFew)
-            return w.spl == 2 ? launch_views<FMT, 48, false, GLG, 2>(w, threads, s)
-                              : launch_views<FMT, 48, false, GLG, 1>(w, threads, s);
     }
     // several samples per lane: fewer than 8 lanes a pixel, or a warp per
     // pixel with most lanes idle; never with counters
@@ -982,12 +979,12 @@ gs_status launch_render_views(const gs_bvh *b, const gs_gaussians *g, const gs_p
     a.key1 = (uint32_t)(p->seed >> 32);
     philox_round_keys(a.key0, a.key1, a.rk);
     a.stream_tag = p->stream_tag;
-    // samples per lane of the camera and shadow pass: 8 from spp 8 to 63
-    // (per-lane packets), 4 at spp 4-7, 2 at spp 2-3; one from spp 64 (grouped), with
-    // counters, or with the bounce traced inline. Frame of 16 views 256^2
-    // to 1080p with ground, four lights and a bounce, one sample per lane
-    // -> four -> eight: spp 16 634 -> 472 -> 430 ms, spp 8 -> 269 -> 251,
-    // spp 32 806 (one) -> 770 (eight).
+    // samples per lane of the camera and shadow pass: 8 from spp 8 to 63, 4 at
+    // spp 4-7, 2 at spp 2-3; one from spp 64 (grouped), with counters, or with
+    // the bounce traced inline. Frame of 16 views 256^2 to 1080p with ground,
+    // four lights and a bounce as per-lane packets, one sample per lane -> four ->
+    // eight: spp 16 634 -> 472 -> 430 ms, spp 8 -> 269 -> 251, spp 32 806 (one) ->
+    // 770 (eight).
     const int64_t bounce_slots = wave_slots(cams, n_views, ex, p);
     const bool inline_bounce = ex && ex->bounce && ex->has_ground && bounce_slots == 0;
     int sms = 0, dev = 0;
@@ -1041,7 +1038,7 @@ gs_status launch_render_views(const gs_bvh *b, const gs_gaussians *g, const gs_p
         a.trec = b->group[kWarpTree].rec;
         a.troot = b->group[kWarpTree].ref;
         a.leaf_test = leaf_test_pays(b->M, all_pix / n_views);
-        w.few = K >= 4 && (all_pix << lanes_lg) < 6 * (int64_t)sms * 32 * 32;
+        w.few = (all_pix << lanes_lg) < 6 * (int64_t)sms * 32 * 32;
     }
     const int tw_lg = tile_w_log2(a.lpp_log2), th_lg = 5 - a.lpp_log2 - tw_lg;
     uint32_t tiles = 0;
