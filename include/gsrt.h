@@ -272,11 +272,12 @@ gs_status gs_bvh_export_wide(const gs_bvh *bvh, void *out, int64_t capacity, int
  * child box, evaluates one hit Gaussian's depth and alpha, and draws for its
  * own samples); otherwise each lane traverses the nodes of the handle's
  * format in a warp packet. On binary handles with t_min >= 0 and none of
- * counters, stack_depth, depth_mode and rng_mode set, the warp packet gives
- * way to a tile walk of the 32-wide copy (in small images to a warp per
- * pixel), and above 32 samples with samples_per_lane = 0 one walk serves four
- * pixels. Every form returns the same hits, and the same image for the same
- * S and L.
+ * counters, stack_depth, depth_mode and rng_mode set, the library may walk
+ * otherwise, by the sizes of image and scene: a warp as one tile of the
+ * 32-wide copy, a whole warp per pixel, or, from 33 to 127 samples with
+ * samples_per_lane = 0, one walk for four pixels. Every form returns the same
+ * hits, and adds a pixel's samples in the order of S and L, so that the image
+ * is the same bit for bit.
  * Deterministic: identical inputs give bit-identical outputs. Traces that use
  * the same handle share its tile counter and status word, so they must not
  * overlap on the GPU: issue them on one stream (or order their streams). */
@@ -310,14 +311,17 @@ gs_status gs_trace_stochastic_keys(const gs_bvh *bvh, const gs_gaussians *g,
                                    const gs_pinhole *cam, const gs_trace_params *p, float *rgb_out,
                                    gs_sample_key *keys_out, void *stream);
 
-/* How gs_trace_stochastic(bvh, ..., p, ...) maps samples to lanes (host
- * call, nothing is enqueued). layout_out (host int32[4]) receives
- * {samples per lane S, lanes per pixel L, passes ceil(spp / S) of
- * n_hits * S slots each, 1 if a group of L lanes walks a wide copy
- * together else 0}: one walk
- * of the hierarchy serves L * S samples of one ray when grouped, S samples
- * otherwise. Returns GS_ERR_INVALID_ARG for NULL pointers or options
- * gs_trace_stochastic would reject. */
+/* The layout of gs_trace_stochastic(bvh, ..., p, ...): which samples share a
+ * lane's sum (host call, nothing is enqueued). layout_out (host int32[4])
+ * receives {samples per lane S, lanes per pixel L, passes ceil(spp / S) of
+ * n_hits * S slots each, 1 if the layout has groups of 8 or more lanes on a
+ * wide copy else 0}. A pixel's samples are added in this layout's order
+ * whatever walks the hierarchy. With counters or an explicit stack_depth the
+ * walks are the layout's own: one serves L * S samples of a ray when grouped, S
+ * otherwise; without them the form may differ (see gs_trace_stochastic), which
+ * depends on the image's size and is not reported here. Returns
+ * GS_ERR_INVALID_ARG for NULL pointers or options gs_trace_stochastic would
+ * reject. */
 gs_status gs_trace_layout(const gs_bvh *bvh, const gs_trace_params *p, int32_t *layout_out);
 
 /* Measurement support (the paper has no counterpart): copy `bytes` from

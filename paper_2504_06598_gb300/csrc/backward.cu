@@ -943,7 +943,6 @@ gs_status launch_backward_nl(const TraceArgs &a, cudaStream_t s) {
     return GS_OK;
 }
 
-// Groups of 8 or more lanes on one pixel use the widest copy that fits them.
 template <int N, bool Q8, bool KEYS, bool LEAF>
 gs_status launch_backward_tile(const TraceArgs &a, cudaStream_t s) {
     int dev = 0, sms = 0, per = 0;
@@ -969,6 +968,8 @@ gs_status launch_backward_tile(const TraceArgs &a, cudaStream_t s) {
     return GS_OK;
 }
 
+// Tiles where the launch chose them, else groups of 8 or more lanes on one pixel,
+// else packets.
 template <int N, bool KEYS>
 gs_status launch_backward_nk(const TraceArgs &a, cudaStream_t s) {
     if (a.trec != nullptr && a.leaf_test)

@@ -8,9 +8,11 @@
 // the random draws and the clips they cause; with one pass per pixel the
 // tile is 8x4 pixels. With 8 or more lanes on a pixel the group walks a wide
 // copy together (traverse_group), otherwise the warp traverses as a tile
-// (traverse_tile) or, for the options that are about the per-lane walk, as a
-// packet (traverse_packet). Above 32 samples a pixel one walk serves four
-// pixels (k_trace_shared). Each pass is one traversal of the hierarchy
+// (traverse_tile) or, for the options that are about the per-lane walk and for
+// very small or dense scenes, as a packet (traverse_packet); in small images a
+// warp takes one pixel, and from 33 to 127 samples a pixel one walk may serve
+// four pixels (k_trace_shared); choose_walk has the lines. Each pass is one
+// traversal of the hierarchy
 // (Sec. 3.2) keeping its closest accepted intersections (Sec. 3.5). At every
 // leaf the intersection routine of Alg. 1 runs:
 //   t    mean of the 1D Gaussian along the ray (Sec. 3.1)
@@ -61,10 +63,12 @@ __host__ __device__ constexpr bool is_group_q8(int f) { return f >= kFmtGroupQ8 
 // of its pixels. The grouped form is latency-bound and is built for eight
 // resident blocks per SM with one or two slots per lane (64 registers),
 // seven with four (72: fewer spills of the four slots), five with eight;
-// the per-lane packet form for eight with up to four slots (against five:
-// spp 1 4.77 -> 4.31 ms, spp 16 with four slots 16.9 -> 15.9 ms) and six
-// with eight (85 registers; against one, four, five and eight blocks:
-// spp 16 with eight slots 14.8, 13.3, 12.4, 11.7 and 12.1 ms).
+// the packets for eight with up to four slots (as packets of the 1M shell at
+// 1080p, against five: spp 1 4.77 -> 4.31 ms, spp 16 with four slots 16.9 -> 15.9
+// ms) and six with eight (85 registers; against one, four, five and eight blocks:
+// spp 16 with eight slots 14.8, 13.3, 12.4, 11.7 and 12.1 ms). The tiles have the
+// packets' bounds; seven blocks with eight slots gained 3% at 1080p and cost 4%
+// at 411x307.
 constexpr int group_min_blocks(int n) { return n >= 8 ? 5 : (n >= 4 ? 7 : kGroupMinBlocks); }
 
 template <int N, bool COUNT, int FMT>
@@ -229,7 +233,7 @@ __global__ void __launch_bounds__(kThreads, is_group_fmt(FMT) ? group_min_blocks
 }
 
 // ---------------------------------------------------------------- shared walks
-// Above 32 samples a pixel: a warp holds a 2x2 tile, walks the 32-wide copy
+// From 33 to 127 samples a pixel: a warp holds a 2x2 tile, walks the 32-wide copy
 // once for its four pixels (the pyramid test of traverse_tile), evaluates the
 // surviving Gaussians with a lane per (pixel, Gaussian) pair, eight Gaussians
 // for the four pixels at a time, and then draws for one pixel after the
@@ -614,8 +618,11 @@ gs_status launch_n(const TraceArgs &a, int format, bool count, cudaStream_t s) {
 // Samples one lane carries when the caller leaves the choice to the
 // library (samples_per_lane = 0). The time follows the number of walks a
 // pixel needs and grows slowly with the slots a walk carries. Measured on
-// the 1M-Gaussian shell at 1080p, trace ms for K = n_hits * S slots per
-// lane and T = spp * n_hits samples per pixel (one sample per lane first):
+// the 1M-Gaussian shell at 1080p with packets and groups, which every layout can
+// take (the tiles and shared walks that the library prefers keep the layout's
+// sums but take less: T = 1 2.9 ms, 16 8.4, 64 15.5), trace ms for K = n_hits * S
+// slots per lane and T = spp * n_hits samples per pixel (one sample per lane
+// first):
 //   T = 4:   K 1 14.1, 2 7.6, 4 5.4 (per-lane packets)
 //   T = 8:   K 1 20.1, 4 8.8, 8 7.1
 //   T = 16:  K 1 24.2, 4 15.9, 8 11.7
