@@ -700,9 +700,11 @@ def main():
         the L2 and DRAM levels against this run's copy peaks beside it."""
         key = "n%d_spp%d" % (n_hits, spp)
         bv = binary[n_hits if n_hits in binary else 1]
-        # algorithmic bytes per sample: 64 B per binary node its own
-        # traversal enters, 64 B per Gaussian tested, one SH record per
-        # shaded sample, plus each pixel's 12-byte output
+        # algorithmic bytes per sample of the binary packets (their visit
+        # counts; a launch with counters never takes the tiles and shared walks
+        # that are timed): 64 B per binary node a sample's own traversal
+        # enters, 64 B per Gaussian tested, one SH record per shaded sample,
+        # plus each pixel's 12-byte output
         per_ray = (info["node_bytes"] * bv["nodes"] + info["prim_bytes"] * bv["prims"]
                    + sh_bytes * bv["shaded"]) / (bv["rays"] * bv["spp"])
         alg = per_ray * npix * spp + 12 * npix
@@ -715,10 +717,12 @@ def main():
                "traffic": None, "kernel": "k_trace (%s)" % key,
                "peak_basis": "%d SMs x 4 schedulers x 1 warp-inst/cycle x %.0f MHz sampled"
                              % (n_sms, mhz),
-               "alg_bytes_per_ray": per_ray, "alg_bytes_per_launch": alg,
-               "alg_gbs_useful": alg / sec / 1e9,
-               "binary_nodes_per_ray": bv["nodes"] / (bv["rays"] * bv["spp"]),
-               "gaussians_tested_per_ray": bv["prims"] / (bv["rays"] * bv["spp"])}
+               "packet_visits": {
+                   "what": "per sample, by a counting launch on the binary nodes "
+                           "(not the timed kernel)",
+                   "alg_bytes_per_ray": per_ray, "alg_bytes_per_launch": alg,
+                   "binary_nodes_per_ray": bv["nodes"] / (bv["rays"] * bv["spp"]),
+                   "gaussians_tested_per_ray": bv["prims"] / (bv["rays"] * bv["spp"])}}
         c = recorded_counters(key)
         if c is None:
             out["counters"] = "not captured on this kernel source"
@@ -739,12 +743,9 @@ def main():
         return out
 
     def record(n_hits, spp, steps):
-        """Timing, layout, visit counts and roofline of one trace launch."""
-        v = counted(n_hits, spp)
+        """Timing, layout of the sums, and roofline of one trace launch."""
         r = timed(n_hits, spp, steps)
         lay = gs.trace_layout(bvh, spp=spp, n_hits=n_hits)
-        share = lay["samples_per_lane"] * (lay["lanes_per_pixel"] if lay["grouped"] else 1)
-        walks = npix * -(-spp // share)
         sec = r["trace_ms"] * 1e-3
         return {"spp": spp, "n_hits": n_hits, "ms_per_step": r["step_ms"],
                 "build_ms": r["build_ms"], "trace_ms": r["trace_ms"],
@@ -752,12 +753,6 @@ def main():
                 "msamples_per_s": npix * spp * n_hits * world / (r["step_ms"] * 1e-3) / 1e6,
                 "trace_mrays_per_s": npix * spp / sec / 1e6,
                 "layout": lay,
-                # walks of the hierarchy: one per group of lanes sharing a
-                # ray when grouped, one per lane otherwise
-                "walks_per_s": walks / sec, "samples_per_walk": npix * spp / walks,
-                "visits_per_walk": {"node_records": v["nodes"] / walks,
-                                    "prims": v["prims"] / walks,
-                                    "philox": v["philox"] / walks},
                 "roofline": roof(n_hits, spp, r["trace_ms"], r["clocks"]),
                 "clocks": r["clocks"]}
 
@@ -824,8 +819,7 @@ def main():
         "copy_peaks_gbs": peaks,
         "build_ms": r1["build_ms"], "trace_ms": r1["trace_ms"],
         "trace_mrays_per_s": r1["trace_mrays_per_s"],
-        "layout": r1["layout"], "walks_per_s": r1["walks_per_s"],
-        "samples_per_walk": r1["samples_per_walk"], "visits_per_walk": r1["visits_per_walk"],
+        "layout": r1["layout"],
         "n4": r4,
         "n1_spp1": ladder["n1_spp1"],
         "n1_spp16": ladder["n1_spp16"],
