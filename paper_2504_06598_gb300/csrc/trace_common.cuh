@@ -1238,12 +1238,13 @@ __device__ __forceinline__ void tile_pyramid(const float d[3], bool in, float *p
 // c twice the centre and e twice the half extents in the pyramid's frame,
 // the box reaches in front of the apex if cz + ez >= 0 and into the pyramid
 // if |cx| <= ex + tx (cz + ez), likewise y; where the rays miss the apex, ex, ey
-// and ez are as much larger. A NaN box never does.
+// and ez are as much larger (MISS). A NaN box never does.
+template <bool MISS>
 __device__ __forceinline__ bool tile_box(const float lo[3], const float hi[3], const float *pyr,
                                          float g2, float &d2) {
     const float4 *p = reinterpret_cast<const float4 *>(pyr);
     const float4 p0 = p[0], p1 = p[1], p2 = p[2], p3 = p[3], p4 = p[4];
-    const float miss2 = pyr[20];
+    const float miss2 = MISS ? pyr[20] : 0.0f;
     float c[3], e[3], m[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
@@ -1253,17 +1254,20 @@ __device__ __forceinline__ bool tile_box(const float lo[3], const float hi[3], c
     }
     d2 = fmaf(m[0], m[0], fmaf(m[1], m[1], m[2] * m[2]));
     const float cx = fmaf(p0.x, c[0], fmaf(p0.y, c[1], p0.z * c[2]));
-    const float ex = fmaf(p0.w, e[0], fmaf(p1.x, e[1], fmaf(p1.y, e[2], miss2)));
+    auto dot = [](float x, float y, float z, const float v[3], float w) {
+        return fmaf(x, v[0], fmaf(y, v[1], MISS ? fmaf(z, v[2], w) : z * v[2]));
+    };
+    const float ex = dot(p0.w, p1.x, p1.y, e, miss2);
     const float cy = fmaf(p1.z, c[0], fmaf(p1.w, c[1], p2.x * c[2]));
-    const float ey = fmaf(p2.y, e[0], fmaf(p2.z, e[1], fmaf(p2.w, e[2], miss2)));
+    const float ey = dot(p2.y, p2.z, p2.w, e, miss2);
     const float cz = fmaf(p3.x, c[0], fmaf(p3.y, c[1], p3.z * c[2]));
-    const float s = cz + fmaf(p3.w, e[0], fmaf(p4.x, e[1], fmaf(p4.y, e[2], miss2)));
+    const float s = cz + dot(p3.w, p4.x, p4.y, e, miss2);
     return s >= 0.0f && fabsf(cx) <= fmaf(p4.z, s, ex) && fabsf(cy) <= fmaf(p4.w, s, ey) && d2 <= g2;
 }
 
 // Child `sub` of wide node `node` of the 32-wide copy against the pyramid; lo
 // and hi receive its planes relative to the apex.
-template <bool Q8>
+template <bool Q8, bool MISS = false>
 __device__ __forceinline__ bool tile_child(const void *grec, uint32_t node, int sub,
                                            const float apex[3], const float *pyr, float g2,
                                            uint32_t &ref, float &d2, float lo[3], float hi[3]) {
@@ -1295,7 +1299,7 @@ __device__ __forceinline__ bool tile_child(const void *grec, uint32_t node, int 
         lo[i] -= apex[i];
         hi[i] -= apex[i];
     }
-    return tile_box(lo, hi, pyr, g2, d2) && ok;
+    return tile_box<MISS>(lo, hi, pyr, g2, d2) && ok;
 }
 
 // The pyramid takes in what lies between the rays, and everything up to the
@@ -1377,7 +1381,8 @@ __device__ __forceinline__ bool traverse_tile(const TraceArgs &a, Ray<N> &r, int
         uint32_t ref = kEmpty;
         float d2 = INFINITY, lo[3] = {0.0f, 0.0f, 0.0f}, hi[3] = {0.0f, 0.0f, 0.0f};
         bool hit = false;
-        if (lane < n_child) hit = tile_child<Q8>(a.trec, node, lane, apex, pyr, g2, ref, d2, lo, hi);
+        if (lane < n_child)
+            hit = tile_child<Q8, SHADOW>(a.trec, node, lane, apex, pyr, g2, ref, d2, lo, hi);
         const bool leaf = (ref & kLeafBit) != 0u;
         const uint32_t key = (__float_as_uint(d2) & ~31u) | (uint32_t)lane;
         bool pending = hit && leaf;
