@@ -1004,18 +1004,21 @@ gs_status launch_render_views(const gs_bvh *b, const gs_gaussians *g, const gs_p
     // samples a lane (8 to 63 samples: up to 8 lanes) are never theirs
     const int lanes_lg = lanes_per_pixel_log2((p->spp + K - 1) / K);
     const bool ungrouped = lanes_lg < 3 || K > 1;
-    // A warp per pixel for few pixels, packets for a few hundred Gaussians or more
-    // than three a ray, tiles between: the lines of choose_walk (trace.cu), the first
-    // a little higher, since a view also has its shadow rays. us, two lights,
-    // packets, tiles, warp per pixel: 5,000 at 160x120, spp 1 466, 360, 132; in two
-    // 320x240 views 352, 290, 591; 1M there 4312, 6030, 2013; 1M in two 640x360
-    // views 3873, 4932, 4395; in four 1080p views 19.2 and 14.3 ms; 100 there 0.47
-    // and 0.62.
+    // A warp per pixel for few pixels, packets for a few hundred Gaussians or many
+    // more than pixels, tiles between: as choose_walk (trace.cu), the first line a
+    // little higher, since a view also has its shadow rays. us, two lights, packets,
+    // tiles, warp per pixel: 5,000 at 160x120, spp 1 466, 360, 132; in two 320x240
+    // views 352, 290, 591; 1M there 4312, 6030, 2013; in four 1080p views 19.2 and
+    // 14.3 ms; 100 there 0.47 and 0.62. Dense scenes, ms, four lights, packets and
+    // tiles: 1M in sixteen 320x200 views, spp 1 9.5 and 15.7, spp 8 22.7 and 23.4, spp
+    // 16 26.7 and 22.6; 0.3M there, spp 1 5.7 and 6.8; 1M in four 448x308 views, spp 1
+    // 5.7 and 5.4 (few tiles), in eight 640x480 14.1 and 11.9.
     const double waves = (double)all_pix / ((double)sms * 32.0);
     const double share = K < 8 ? 0.72 : 0.40 - 0.04 * lanes_lg;
     const bool whole_warp = tiles_ok && ungrouped && waves < share * cbrt((double)b->M);
+    w.few = (all_pix << lanes_lg) < 6 * (int64_t)sms * 32 * 32;
     const bool tiled = tiles_ok && ungrouped && !whole_warp && b->M >= 512 &&
-                       b->M <= 3 * ((all_pix / n_views) << lanes_lg);
+                       b->M <= (K >= 8 ? 32 : w.few ? 8 : 4) * (all_pix / n_views);
     w.spl = K;
     a.spp = (p->spp + K - 1) / K;
     a.n_samples = p->spp;
@@ -1038,7 +1041,6 @@ gs_status launch_render_views(const gs_bvh *b, const gs_gaussians *g, const gs_p
         a.trec = b->group[kWarpTree].rec;
         a.troot = b->group[kWarpTree].ref;
         a.leaf_test = leaf_test_pays(b->M, all_pix / n_views);
-        w.few = (all_pix << lanes_lg) < 6 * (int64_t)sms * 32 * 32;
     }
     const int tw_lg = tile_w_log2(a.lpp_log2), th_lg = 5 - a.lpp_log2 - tw_lg;
     uint32_t tiles = 0;
