@@ -1063,7 +1063,7 @@ gs_status launch_backward(const gs_bvh *b, const gs_gaussians *g, const gs_pinho
         const double size = sqrt((double)b->M);
         const int lg = lanes_log2(lane_samples(true));
         const bool groups = lanes_log2(lane_samples(false)) >= 3;
-        tile = (double)b->M * (double)(32 >> lg) / (double)pix <= (groups ? 1.0 : lg == 0 ? 0.8 : 8.0) * size;
+        tile = (double)b->M * (double)(32 >> lg) / field_pixels(cam) <= (groups ? 1.0 : lg == 0 ? 0.8 : 8.0) * size;
         // without payloads the winners are traced again, in small images on the
         // tiles' longest chain, which a second round of passes doubles (spp 40
         // against groups: 1M at 160x120 7.7 and 3.9, at 64x64 4.2 and 3.5; 90k at
@@ -1119,7 +1119,7 @@ gs_status launch_backward(const gs_bvh *b, const gs_gaussians *g, const gs_pinho
         a.troot = b->group[kWarpTree].ref;
         a.gq8 = b->node_format == GS_NODES_BINARY_Q8;
         a.g_stats = b->grad;
-        a.leaf_test = leaf_test_pays(b->M, (int64_t)cam->width * cam->height);
+        a.leaf_test = leaf_test_pays(b->M, field_pixels(cam));
         a.sh_vec = ((uintptr_t)d_sh & 15u) == 0;
     }
     a.keys = const_cast<gs_sample_key *>(keys);  // read only here

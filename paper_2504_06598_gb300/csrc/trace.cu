@@ -671,6 +671,7 @@ static Walk choose_walk(const gs_bvh *b, const gs_pinhole *cam, const gs_trace_p
         return Walk::kLayout;
     const int64_t pix = (int64_t)cam->width * cam->height, T = (int64_t)p->spp * p->n_hits;
     const double waves = (double)pix / (double)resident_warps();  // of a warp per pixel
+    const double field = field_pixels(cam);
     const bool many = p->samples_per_lane == 0 && T > 32;
     // A warp per pixel (most lanes without a sample, helping in the walk) evaluates
     // 32 Gaussians at a time, a tile's warp one after the other, so that the time
@@ -684,7 +685,7 @@ static Walk choose_walk(const gs_bvh *b, const gs_pinhole *cam, const gs_trace_p
         double share = many ? 0.14 : n_eff < 8 ? 0.6 : 0.40 - 0.04 * lpp_log2;
         // (three or five to seven passes are two rounds of the layout's lanes)
         if (!many && passes > 1 << lpp_log2) share *= 1.6;
-        if (waves < share * cbrt((double)b->M)) return Walk::kWarp;
+        if (waves < warp_waves(share, b->M, field, (double)resident_warps())) return Walk::kWarp;
     }
     // Eight to 31 passes of the caller's samples per lane: a whole warp does in one
     // round what groups of 8 or 16 lanes do in two, and more than groups of 16 do on
@@ -711,7 +712,7 @@ static Walk choose_walk(const gs_bvh *b, const gs_pinhole *cam, const gs_trace_p
     // More than three Gaussians a ray of the tile: its farthest clip takes in so many
     // that packets, which clip per ray, do better (1M at 500x400, spp 8 4502 against
     // 5533; at 640x480 4428 against 4846).
-    return b->M > 3 * (pix << lpp_log2) ? Walk::kLayout : Walk::kTile;
+    return (double)b->M > 3.0 * field * (double)(1 << lpp_log2) ? Walk::kLayout : Walk::kTile;
 }
 
 void trace_layout(const gs_bvh *b, const gs_trace_params *p, int *S_out, int *spp_eff_out,
@@ -754,7 +755,7 @@ gs_status launch_trace(const gs_bvh *b, const gs_gaussians *g, const gs_pinhole 
     a.gq8 = b->node_format == GS_NODES_BINARY_Q8;
     a.trec = tile || shared ? b->group[kWarpTree].rec : nullptr;
     a.troot = tile || shared ? b->group[kWarpTree].ref : nullptr;
-    a.leaf_test = leaf_test_pays(b->M, (int64_t)cam->width * cam->height);
+    a.leaf_test = leaf_test_pays(b->M, field_pixels(cam));
     a.prims = b->prims;
     a.sh = g->sh;
     a.n_nodes = b->n_nodes;

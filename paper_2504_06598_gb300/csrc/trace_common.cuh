@@ -1308,9 +1308,28 @@ __device__ __forceinline__ bool tile_child(const void *grec, uint32_t node, int 
 // packets, gradients at 96x72 20.6 against 4.8. So (LEAF) a leaf's box is tested by
 // every lane, at a quarter of an evaluation's instructions, before the warp
 // evaluates it: 4.9 and 7.3 ms; 1M at 1080p, spp 1 3.91 -> 3.47, spp 16 9.44 -> 8.94.
-// With fewer Gaussians than a sixteenth of the pixels most leaves of a tile are met
+// With fewer Gaussians than a sixteenth of field_pixels most leaves of a tile are met
 // and the test only costs (5,000 in four 1080p views 9%): a form without it.
-inline int leaf_test_pays(int64_t M, int64_t pix) { return M > pix / 16 ? 1 : 0; }
+inline int leaf_test_pays(int64_t M, double field) { return (double)M > field / 16.0 ? 1 : 0; }
+
+// How dense a scene of M Gaussians is in an image depends on the camera's
+// resolution and not on how much of its field the image's width takes in: M over
+// the pixels that a 4:3 image of 60 degrees has at this resolution.
+inline double field_pixels(const gs_pinhole *cam) {
+    const double h = cam->height * 0.57735026918962573 /
+                     tan((double)cam->fov_y_deg * 3.14159265358979323846 / 360.0);
+    return 4.0 / 3.0 * h * h;
+}
+
+// Waves of a warp per pixel (of `resident` warps) up to which that form beats tiles:
+// `share` of the scene's depth, which grows with the cube root of its size, and
+// less where the resolution is so high that the same scene fills larger tiles'
+// counts less (measured in images of 4:3 to 16:9, and of 70x957 and 237x930: 0.91M
+// there 14 waves 2.2 ms against 3.1, 0.47M 45 waves 5.0 against 2.4).
+inline double warp_waves(double share, int64_t M, double field, double resident) {
+    const double w = share * cbrt((double)M), f = field / resident;
+    return f > w ? w * pow(w / f, 0.6) : w;
+}
 
 // Whether a lane's ray can hit what the box of lane src's child holds: its
 // direction away from the apex (inv: the reciprocals) meets the box, no farther

@@ -1015,10 +1015,16 @@ gs_status launch_render_views(const gs_bvh *b, const gs_gaussians *g, const gs_p
     // 5.7 and 5.4 (few tiles), in eight 640x480 14.1 and 11.9.
     const double waves = (double)all_pix / ((double)sms * 32.0);
     const double share = K < 8 ? 0.72 : 0.40 - 0.04 * lanes_lg;
-    const bool whole_warp = tiles_ok && ungrouped && waves < share * cbrt((double)b->M);
+    double field = 0.0;
+    for (int v = 0; v < n_views; ++v) field += field_pixels(&cams[v]) / n_views;
+    const bool whole_warp = tiles_ok && ungrouped &&
+                            waves < warp_waves(share, b->M, n_views * field, (double)sms * 32.0);
     w.few = (all_pix << lanes_lg) < 6 * (int64_t)sms * 32 * 32;
+    // (many tiles of four and more samples a lane spill: below 16,384 Gaussians the
+    // packets are the better then, 5,000 in four 1080p views, spp 8 4.5 and 4.9 ms)
     const bool tiled = tiles_ok && ungrouped && !whole_warp && b->M >= 512 &&
-                       b->M <= (K >= 8 ? 32 : w.few ? 8 : 4) * (all_pix / n_views);
+                       (K < 4 || w.few || b->M >= 16384) &&
+                       (double)b->M <= (K >= 8 ? 32.0 : w.few ? 8.0 : 4.0) * field;
     w.spl = K;
     a.spp = (p->spp + K - 1) / K;
     a.n_samples = p->spp;
@@ -1040,7 +1046,7 @@ gs_status launch_render_views(const gs_bvh *b, const gs_gaussians *g, const gs_p
     if (tiled) {
         a.trec = b->group[kWarpTree].rec;
         a.troot = b->group[kWarpTree].ref;
-        a.leaf_test = leaf_test_pays(b->M, all_pix / n_views);
+        a.leaf_test = leaf_test_pays(b->M, field);
     }
     const int tw_lg = tile_w_log2(a.lpp_log2), th_lg = 5 - a.lpp_log2 - tw_lg;
     uint32_t tiles = 0;

@@ -36,6 +36,7 @@ CASES = [
     (5000, 613, 401, 40, 1), (5000, 613, 401, 64, 1), (1025, 613, 401, 127, 1), (33, 613, 401, 25, 4),  # shared
     (300, 613, 401, 4, 1), (5000, 160, 121, 100, 1), (1025, 613, 401, 129, 1),  # the layout's own
     (1000000, 500, 403, 8, 1),  # packets of a dense scene
+    (70000, 61, 930, 2, 1), (70000, 930, 61, 2, 1),  # narrow and wide: tiles, warp per pixel
 ]
 
 
