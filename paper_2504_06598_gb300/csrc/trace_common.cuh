@@ -1322,10 +1322,11 @@ inline double field_pixels(const gs_pinhole *cam) {
 }
 
 // Waves of a warp per pixel (of `resident` warps) up to which that form beats tiles:
-// `share` of the scene's depth, which grows with the cube root of its size, and
-// less where the resolution is so high that the same scene fills larger tiles'
-// counts less (measured in images of 4:3 to 16:9, and of 70x957 and 237x930: 0.91M
-// there 14 waves 2.2 ms against 3.1, 0.47M 45 waves 5.0 against 2.4).
+// `share` of the scene's depth, which grows with the cube root of its size. At a
+// higher resolution a tile covers less of the scene, holds fewer Gaussians and is
+// the cheaper: fewer waves then. (0.91M in 70x957, 14 waves: 2.2 ms against 3.1 in
+// tiles; 0.47M in 237x930, 45 waves: 5.0 against 2.4. The exponent was fitted to
+// these two and to images of 4:3 to 16:9.)
 inline double warp_waves(double share, int64_t M, double field, double resident) {
     const double w = share * cbrt((double)M), f = field / resident;
     return f > w ? w * pow(w / f, 0.6) : w;
